@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "../../include/chem.h"
+#include "fx_mech.h"
 
 namespace chem {
 
@@ -87,6 +88,8 @@ struct chem_mech_s {
   void* d_blob = nullptr;                 // device copy of the shared-memory blob
   void* d_jac = nullptr;                  // device allocation holding the JacProgram arrays
   chem::JacProgram jac{};
+  chem::FxLayout fx{};                    // fixed-point form (integrator_cell.cu), bytes = 0: none
+  void* d_fx = nullptr;
 };
 
 namespace chem {

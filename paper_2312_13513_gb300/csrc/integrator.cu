@@ -32,42 +32,27 @@
 
 #include "chem_internal.h"
 #include "fastexp.cuh"
+#include "queue.cuh"
 
 namespace chem {
+
+// one thread per cell (integrator_cell.cu)
+bool cell_kernel_fits(const chem_mech_s* m);
+int launch_cell_advance(const chem_mech_s* m, const QueueParams& Q, const chem_options* opt, cudaStream_t stream);
+int launch_cell_eval(const chem_mech_s* m, const double* T, const double* p, const double* Y, int64_t ld, int64_t n,
+                     double* f, double* J, cudaStream_t stream);
 
 // Cells claimed per work-queue access: two consecutive cells for sub-warp groups (16 bytes per
 // row of the SoA state: the state traffic is far below HBM bandwidth, shared memory per cell is
 // what limits residency), one cell for groups of a warp or more, whose cells take milliseconds
 // each
 // (a time-sliced launch then overruns its budget by at most one cell).
-__host__ __device__ constexpr int chunk_cells(int G) { return G >= 32 ? 1 : 2; }
+__host__ __device__ constexpr int chunk_cells(int G) { return G >= 32 || G == 1 ? 1 : 2; }
 
 // Threads per CTA at most.  Two-thread groups are few per CTA (shared memory per cell bounds
 // them near 80), so their kernels are compiled for 256 threads and one CTA per SM, which lifts
 // the register cap from 128 to 255 per thread: the inlined rate evaluation does not spill.
 __host__ __device__ constexpr int max_threads(int G) { return G == 2 ? 256 : 512; }
-
-// Rodas4 coefficients, transformed (u-variable) form:
-//   (I/(gamma h) - J) u_s = f(y + sum_j A[s][j] u_j) + sum_j (C[s][j]/h) u_j,
-//   y_new = y + sum_s M[s] u_s,  error = u_5.
-__constant__ double kRA[6][6] = {
-    {0, 0, 0, 0, 0, 0},
-    {1.544, 0, 0, 0, 0, 0},
-    {0.9466785280815826, 0.2557011698983284, 0, 0, 0, 0},
-    {3.314825187068521, 2.896124015972201, 0.9986419139977817, 0, 0, 0},
-    {1.221224509226641, 6.019134481288629, 12.53708332932087, -0.6878860361058950, 0, 0},
-    {1.221224509226641, 6.019134481288629, 12.53708332932087, -0.6878860361058950, 1.0, 0}};
-__constant__ double kRC[6][6] = {
-    {0, 0, 0, 0, 0, 0},
-    {-5.6688, 0, 0, 0, 0, 0},
-    {-2.430093356833875, -0.2063599157091915, 0, 0, 0, 0},
-    {-0.1073529058151375, -9.594562251023355, -20.47028614809616, 0, 0, 0},
-    {7.496443313967647, -10.24680431464352, -33.99990352819905, 11.70890893206160, 0, 0},
-    {8.083246795921522, -7.981132988064893, -31.52159432874371, 16.31930543123136,
-     -6.058818238834054, 0}};
-__constant__ double kRM[6] = {1.221224509226641, 6.019134481288629, 12.53708332932087,
-                              -0.6878860361058950, 1.0, 1.0};
-constexpr double kGamma = 0.25;
 
 // ---------------------------------------------------------------------------------------
 // mechanism view (shared memory)
@@ -281,14 +266,6 @@ __device__ __forceinline__ void gsum_lead(const Grp<G>& g, double (&v)[K], doubl
 // length up to 1625, far beyond a matrix that fits in shared memory.
 __device__ __forceinline__ unsigned div_magic(unsigned d) { return 0xFFFFFFFFu / d + 1u; }
 __device__ __forceinline__ int div_by(int e, unsigned magic) { return (int)__umulhi((unsigned)e, magic); }
-
-// Pivot key of a matrix entry: the bit pattern of |a| read as an unsigned integer.  For
-// non-negative doubles the integer order is the numeric order, so the pivot search runs on the
-// integer pipes instead of FP64 compares (the FP64 pipe is the scarce one).  NaN maps to 0.
-__device__ __forceinline__ unsigned long long pivot_key(double a) {
-  const unsigned long long k = (unsigned long long)__double_as_longlong(a) & 0x7fffffffffffffffull;
-  return k > 0x7ff0000000000000ull ? 0ull : k;
-}
 
 __device__ __forceinline__ void argmax_merge(unsigned long long& best, int& bi, unsigned long long ob, int oi) {
   if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
@@ -939,47 +916,12 @@ __device__ void lu_solve(const Grp<G>& g, const double* M, int N, int LD, const 
 // ---------------------------------------------------------------------------------------
 // kernels
 // ---------------------------------------------------------------------------------------
-// One independent set of cells advanced by a launch: its own state arrays, step and
-// tolerances, optional index list and outputs.  A launch walks the chunks of all its segments
-// through one work queue (iteration-level batching of several requests).
-struct Segment {
-  double* T;
-  const double* p;
-  double* Y;
-  int64_t ld, ncells;
-  const int32_t* idx;
-  int8_t* status;
-  int32_t* nsub;
-  int32_t* nrej;
-  double dt, rtol, atol;
-  long long chunk_begin;           // first queue entry of this segment
-};
-
-constexpr int kMaxSegs = kMaxSegsPerLaunch;   // segments per launch (kernel-parameter space)
-
-struct AdvanceParams {
+struct AdvanceParams : QueueParams {
   MechLayout lay;
   WsLayout ws;
   JacArgs jp;
   const unsigned char* blob;
-  Segment segs[kMaxSegs];
-  int nseg;
-  long long total_chunks;
-  int max_steps;
-  unsigned long long* counter;
-  const unsigned int* ncells_dev;  // single segment: cell count read from device memory
-  unsigned long long budget_ns = 0;  // > 0: stop claiming chunks this long after the group started
-  // time-sliced launches: a nonzero *stop (device memory, set by the caller while the slice runs)
-  // also stops the claiming, once the group has run min_ns
-  const unsigned int* stop = nullptr;
-  unsigned long long min_ns = 0;
 };
-
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
 
 __device__ __forceinline__ void stage_mech(const unsigned char* src, unsigned char* dst, int bytes) {
   const int4* s = (const int4*)src;
@@ -1073,16 +1015,6 @@ struct ChunkPos {
   long long total;      // queue entries (chunks) of the launch
   unsigned long long t0;  // group start time (time-sliced launches)
 };
-
-__device__ __forceinline__ int64_t cell_of(const Segment* S, long long base, int c) {
-  return S->idx ? (int64_t)S->idx[base + c] : (int64_t)(base + c);
-}
-
-__device__ __forceinline__ const Segment* segment_of(const AdvanceParams& P, long long chunk) {
-  int s = 0;
-  while (s + 1 < P.nseg && P.segs[s + 1].chunk_begin <= chunk) ++s;
-  return &P.segs[s];
-}
 
 // Move to the next cell: store a finished chunk, claim and load the next one when needed.
 // Loads the cell's state into w.y and returns its pressure; false when the queue is empty.
@@ -1320,7 +1252,8 @@ __global__ void __launch_bounds__(max_threads(G)) eval_kernel(const EvalParams P
 namespace {
 
 struct LaunchShape {
-  int G, groups, threads;
+  const chem_mech_s* m;
+  int G, groups, threads;    // G = 1: one thread per cell (integrator_cell.cu)
   size_t smem;
   WsLayout ws;
 };
@@ -1328,6 +1261,11 @@ struct LaunchShape {
 
 int pick_shape(const chem_mech_s* m, const chem_options* opt, LaunchShape* s) {
   const int N = m->ns + 1;
+  s->m = m;
+  if (!(opt && opt->group_threads) && cell_kernel_fits(m)) {
+    s->G = 1;
+    return CHEM_OK;
+  }
   int G = (opt && opt->group_threads) ? opt->group_threads : (N <= 16 ? 2 : 128);
   if (G != 2 && G != 4 && G != 8 && G != 16 && G != 32 && G != 64 && G != 128 && G != 256) {
     set_error("group_threads must be 2, 4, 8, 16, 32, 64, 128 or 256 (got %d)", G);
@@ -1407,6 +1345,7 @@ int launch_eval_t(const LaunchShape& s, const EvalParams& P, cudaStream_t stream
 int dispatch_adv(const LaunchShape& s, const AdvanceParams& P, const chem_options* opt,
                  cudaStream_t stream) {
   switch (s.G) {
+    case 1: return launch_cell_advance(s.m, P, opt, stream);
     case 2: return launch_adv_t<2>(s, P, opt, stream);
     case 4: return launch_adv_t<4>(s, P, opt, stream);
     case 8: return launch_adv_t<8>(s, P, opt, stream);
@@ -1764,6 +1703,7 @@ extern "C" int chem_eval_rhs_jac(chem_mech_t m, const double* T, const double* p
   LaunchShape s;
   int rc = pick_shape(m, nullptr, &s);
   if (rc) return rc;
+  if (s.G == 1) return launch_cell_eval(m, T, p, Y, ld, ncells, f, J, (cudaStream_t)stream);
   EvalParams P;
   P.lay = m->lay; P.ws = s.ws; P.jp = jac_args(m); P.blob = (const unsigned char*)m->d_blob;
   P.T = T; P.p = p; P.Y = Y; P.ld = ld; P.ncells = ncells; P.f = f; P.J = J;

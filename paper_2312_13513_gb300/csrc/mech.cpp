@@ -19,6 +19,7 @@
 
 #include "chem_internal.h"
 #include "exp_table.h"
+#include "fixed.cuh"
 
 namespace chem {
 
@@ -85,6 +86,176 @@ void reorder_reactions(const chem_mech_desc* in, Reordered* o) {
     o->d.has_t2 = o->has_t2.data(); o->d.A = o->A.data(); o->d.b = o->b.data(); o->d.Ea = o->Ea.data();
     o->d.troe = o->troe.data(); o->d.eff = o->eff.data();
   }
+}
+
+// The fixed-point form of the mechanism (reactions in the order of the blob).  Returns the bytes;
+// L->bytes = 0 where a number lies outside the formats.  No polynomial can leave Q11.52 (its
+// coefficients' magnitudes sum to at most 2000), and every base-2 exponent that the kernel forms
+// stays below 3074 in magnitude (|log2 kf| <= 600 + 32 * 12 + 1900; |log2 kr| <= 1023 + 2000 by
+// the bound on Delta G below), so that a wrapped sum is always recognised as out of range
+// (exp2_in_range) and never mistaken for a small one.
+std::vector<unsigned char> build_fx(const chem_mech_desc* d, const chem_mech_s* m,
+                                    const std::vector<std::vector<int>>& nu, FxLayout* L) {
+  const int ns = d->n_species, nr = d->n_reactions;
+  *L = FxLayout{};
+  std::vector<unsigned char> none;
+  if (ns > 15 || nr > 1024) return none;
+  bool ok = true;
+  auto q = [&](double v, int frac, double lim) -> int64_t {
+    if (!(std::fabs(v) <= lim)) { ok = false; return 0; }
+    return (int64_t)std::nearbyintl((long double)v * (long double)std::ldexp(1.0, frac));
+  };
+  const long double l2 = std::log(2.0L);
+  auto q52l = [&](long double v, double lim) -> int64_t {
+    if (!(std::fabs((double)v) <= lim)) { ok = false; return 0; }
+    return (int64_t)std::nearbyintl(v * 4503599627370496.0L);
+  };
+  Builder B;
+  int ntb = 0, ntroe = 0;
+  for (int j = 0; j < nr; ++j) { ntb += d->rtype[j] != 0; ntroe += d->rtype[j] == 2; }
+  std::vector<int> effoff(1, 0);
+  std::vector<double> effv, eff;
+  std::vector<int16_t> effidx;
+  for (int j = 0; j < nr; ++j) {
+    if (d->rtype[j] == 0) continue;
+    for (int k = 0; k < ns; ++k) {
+      const double e = d->eff[(size_t)j * ns + k];
+      eff.push_back(e);
+      if (e != 1.0) { effidx.push_back((int16_t)k); effv.push_back(e - 1.0); }
+    }
+    effoff.push_back((int)effidx.size());
+  }
+  L->ns = ns; L->nr = nr; L->ntb = ntb;
+  L->o_exp2 = B.add(8 * 256);
+  L->o_lg = B.add(8 * 128);
+  L->o_rcp = B.add(4 * 128);
+  L->o_sp = B.add(2 * ns * (int)sizeof(FxSpecies));
+  L->o_W = B.add(8 * ns);
+  L->o_invW = B.add(8 * ns);
+  L->o_nu = B.add(8 * 16);
+  L->o_reac = B.add(nr * (int)sizeof(FxReac));
+  L->o_troe = B.add(ntroe * (int)sizeof(FxTroe));
+  L->o_effv = B.add(8 * (int)effv.size());
+  L->o_eff = B.add(8 * (int)eff.size());
+  L->o_effidx = B.add(2 * (int)effidx.size());
+  L->o_effoff = B.add(4 * (int)effoff.size());
+  static const fx::u64 e2[256] = {CHEM_FX_EXP2_VALUES};
+  static const fx::u64 lg[128] = {CHEM_FX_LOG2_VALUES};
+  static const uint32_t rc[128] = {CHEM_FX_RCP_VALUES};
+  memcpy(B.at<unsigned char>(L->o_exp2), e2, sizeof(e2));
+  memcpy(B.at<unsigned char>(L->o_lg), lg, sizeof(lg));
+  memcpy(B.at<unsigned char>(L->o_rcp), rc, sizeof(rc));
+  for (int r = 0; r < 2; ++r)
+    for (int k = 0; k < ns; ++k) {
+      const double* a = (r == 0 ? d->nasa_lo : d->nasa_hi) + 7 * k;
+      FxSpecies* S = B.at<FxSpecies>(L->o_sp) + r * ns + k;
+      const int sh = r == 0 ? kFxR0 : kFxR1;
+      long double p = 1.0L;
+      for (int i = 0; i < 5; ++i, p *= std::ldexp(1.0L, sh)) {
+        // i-th coefficients of h/RT, s/R (the constant is a7, the T-free part of a1 (1 - ln T) is
+        // a1) and cp/R in powers of tau
+        S->c[i] = q52l((long double)a[i] * p, 500.0);
+        S->h[i] = q52l((long double)a[i] / (i + 1) * p, 500.0);
+        const long double s = i == 0 ? (long double)a[6] : (long double)a[i] / i * p;
+        const long double g = (i == 0 ? (long double)a[0] : (long double)a[i] / (i + 1) * p) - s;
+        S->g[i] = q52l(g / l2, 1000.0);
+      }
+      S->ha6 = q52l((long double)a[5] / 128.0L, 1900.0);
+      S->ga6 = q52l((long double)a[5] / 128.0L / l2, 1900.0);
+      S->gl = q(-a[0], 56, 100.0);
+      double sg = std::fabs((double)S->ga6), sh_ = std::fabs((double)S->ha6), sc = 0.0;
+      for (int i = 0; i < 5; ++i) {
+        sg += std::fabs((double)S->g[i]); sh_ += std::fabs((double)S->h[i]);
+        sc += std::max(1, i) * std::fabs((double)S->c[i]);
+      }
+      if (!(std::max(std::max(sg + 12.0 * std::fabs((double)S->gl) / 16.0, sh_), sc) <= 2000.0 * 4503599627370496.0)) ok = false;
+    }
+  for (int k = 0; k < ns; ++k) {
+    B.at<double>(L->o_W)[k] = m->W[k];
+    B.at<double>(L->o_invW)[k] = 1.0 / m->W[k];
+  }
+  for (int c = 0; c < 16; ++c) B.at<double>(L->o_nu)[c] = (double)(c - 8);
+  L->lpr0 = q52l(std::log((long double)PATM / (long double)RU) / l2, 1000.0);
+  int tb = 0, tr = 0;
+  for (int j = 0; j < nr; ++j) {
+    FxReac* R = B.at<FxReac>(L->o_reac) + j;
+    R->type = (uint8_t)d->rtype[j];
+    R->tb = R->type ? (int16_t)tb++ : (int16_t)-1;
+    R->troe = R->type == 2 ? (int16_t)tr++ : (int16_t)-1;
+    R->b = d->b[j];
+    R->TaK = d->Ea[j] / RC;
+    auto rate = [&](double A, double b, double Ea, int64_t* o) {
+      const long double lnA = A > 0.0 ? std::log((long double)A) / l2 : 1e9L;
+      const long double Ta = (long double)Ea / (long double)RC / l2 / 128.0L;
+      if (!(std::fabs((double)lnA) <= 600.0) || !(std::fabs(b) <= 32.0) || !(std::fabs((double)Ta) <= 1900.0)) {
+        R->slow = 1;
+        o[0] = o[1] = o[2] = 0;
+        return;
+      }
+      o[0] = q52l(lnA, 600.0);
+      o[1] = q(b, 56, 32.0);
+      o[2] = q52l(Ta, 1900.0);
+    };
+    int64_t o[3];
+    rate(d->A[j], d->b[j], d->Ea[j], o);
+    R->lnA = o[0]; R->beta = o[1]; R->Ta = o[2];
+    if (R->type == 2) {
+      const double* t = d->troe + 7 * j;
+      FxTroe* F = B.at<FxTroe>(L->o_troe) + R->troe;
+      rate(t[0], t[1], t[2], o);
+      F->lnA0 = o[0]; F->b0 = o[1]; F->Ta0 = o[2];
+      F->b0d = t[1]; F->Ta0K = t[2] / RC;
+      F->a = t[3]; F->iT3 = 1.0 / t[4]; F->iT1 = 1.0 / t[5]; F->T2 = t[6];
+      F->has_t2 = d->has_t2[j] ? 1.0 : 0.0;
+    }
+    int dnu = 0;
+    for (int i = 0; i < 3; ++i) {
+      if (d->reac[3 * j + i] >= 0) { R->re[R->nre++] = (uint8_t)d->reac[3 * j + i]; --dnu; }
+      if (d->prod[3 * j + i] >= 0) { R->pr[R->npr++] = (uint8_t)d->prod[3 * j + i]; ++dnu; }
+    }
+    R->dnu = (int8_t)dnu;
+    for (int k = 0; k < ns; ++k)
+      if (nu[j][k] != 0) { R->sp[R->nnet] = (uint8_t)k; R->nu[R->nnet++] = (int8_t)nu[j][k]; }
+  }
+  // |Delta G / (RT ln 2)| of a reaction over [kTlo, kThi): on 512 log-spaced pieces, the value at
+  // the left end plus the change of every (monotone) term across the piece; above 2000: slow
+  for (int j = 0; j < nr; ++j) {
+    FxReac* R = B.at<FxReac>(L->o_reac) + j;
+    double worst = 0.0;
+    const double step = std::pow(fx::kThi / fx::kTlo, 1.0 / 512.0);
+    double T = fx::kTlo;
+    for (int i = 0; i < 512; ++i, T *= step) {
+      const double T1 = T * step;
+      for (int r = (T1 < TMID ? 0 : (T >= TMID ? 1 : 0)); r <= (T1 < TMID ? 0 : 1); ++r) {
+        const double* nasa = r == 0 ? d->nasa_lo : d->nasa_hi;
+        double c[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+        for (int k = 0; k < ns; ++k)
+          for (int t = 0; t < 7; ++t) c[t] += nu[j][k] * nasa[7 * k + t];
+        auto terms = [&](double x, double* o) {
+          double p = 1.0;
+          for (int t = 0; t < 5; ++t, p *= x)
+            o[t] = t == 0 ? c[0] * (1.0 - std::log(x)) - c[6] : -c[t] * p / (t * (t + 1));
+          o[5] = c[5] / x;
+          o[6] = R->dnu * (std::log(x) - std::log(PATM / RU));
+        };
+        double a0[7], a1[7], v = 0.0, w = 0.0;
+        terms(T, a0);
+        terms(T1, a1);
+        for (int t = 0; t < 7; ++t) { v += a0[t]; w += std::fabs(a1[t] - a0[t]); }
+        worst = std::max(worst, std::fabs(v) + w);
+      }
+    }
+    if (!(worst / std::log(2.0) <= 2000.0)) R->slow = 1;
+  }
+  for (size_t i = 0; i < effv.size(); ++i) {
+    B.at<double>(L->o_effv)[i] = effv[i];
+    B.at<int16_t>(L->o_effidx)[i] = effidx[i];
+  }
+  for (size_t i = 0; i < eff.size(); ++i) B.at<double>(L->o_eff)[i] = eff[i];
+  for (size_t i = 0; i < effoff.size(); ++i) B.at<int>(L->o_effoff)[i] = effoff[i];
+  if (!ok) return none;
+  L->bytes = (int)B.buf.size();
+  return B.buf;
 }
 
 int build(const chem_mech_desc* din, chem_mech_s* m) {
@@ -284,7 +455,12 @@ int build(const chem_mech_desc* din, chem_mech_s* m) {
   }
   P.nterm = (int)src.size();
 
+  const std::vector<unsigned char> fxb = build_fx(d, m, nu, &m->fx);
   CHEM_CUDA_TRY(cudaGetDevice(&m->device));
+  if (m->fx.bytes) {
+    CHEM_CUDA_TRY(cudaMalloc(&m->d_fx, m->fx.bytes));
+    CHEM_CUDA_TRY(cudaMemcpy(m->d_fx, fxb.data(), m->fx.bytes, cudaMemcpyHostToDevice));
+  }
   CHEM_CUDA_TRY(cudaMalloc(&m->d_blob, L.bytes));
   CHEM_CUDA_TRY(cudaMemcpy(m->d_blob, B.buf.data(), L.bytes, cudaMemcpyHostToDevice));
   size_t o_off = 0;
@@ -478,6 +654,7 @@ extern "C" int chem_free_mechanism(chem_mech_t m) {
   if (!m) { set_error("NULL mechanism"); return CHEM_EINVAL; }
   if (m->d_blob) cudaFree(m->d_blob);
   if (m->d_jac) cudaFree(m->d_jac);
+  if (m->d_fx) cudaFree(m->d_fx);
   delete m;
   return CHEM_OK;
 }
