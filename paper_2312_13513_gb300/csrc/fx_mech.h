@@ -7,40 +7,60 @@
 
 namespace chem {
 
-// one reaction; species slots beyond nre / npr are 0 and unread
+// Signed constants that multiply a temperature quantity are stored biased (fx::biased).
+
+// One reaction with at most two species per side.  Species are byte offsets k * 256 of a cell's
+// workspace columns (32 lanes of 8 bytes); an empty slot is species ns, whose concentration reads
+// 1 and whose Gibbs energy 0.  The net production goes to four distinct species: those of the
+// reaction, padded with others at coefficient 0, so that the four updates never alias.
+struct alignas(16) FxRate {
+  int64_t lnA;                // log2 A (Q11.52); 2000: the FP64 rate expressions take the reaction
+  uint64_t beta;              // b (Q7.56), biased
+  uint64_t Ta;                // Ea / (Rc ln 2) / 128 (Q11.52), biased
+  uint16_t c[4];              // two reactants, two products
+  uint16_t w[4];              // species of the net production ...
+  int16_t dnu, id, tb, troe;  // id: index in the FP64 form; third-body set and Troe record, -1: none
+  double nu[4];               // ... and its coefficients
+  double b, TaK;              // b and Ea / Rc, for the temperature derivative
+};
+
+// any reaction (up to three species per side, six net species): what FxRate cannot hold
 struct alignas(16) FxReac {
-  int64_t lnA, beta, Ta;      // log2 A (Q11.52), b (Q7.56), Ea / (Rc ln 2) / 128 (Q11.52)
-  double b, TaK;              // b and Ea / Rc in FP64, for the temperature derivative
-  uint8_t re[3], pr[3];       // species of each side
-  uint8_t nre, npr;
-  uint8_t sp[6];              // net production: nnet distinct species ...
-  int8_t nu[6];               // ... with their coefficients
-  uint8_t nnet, type, slow;
-  int8_t dnu;
-  int16_t tb, troe;           // third-body set and Troe record, -1: none
+  int64_t lnA;
+  uint64_t beta, Ta;
+  double b, TaK;
+  uint8_t re[3], pr[3], nre, npr;   // species of each side
+  uint8_t sp[6];                    // net production: nnet distinct species ...
+  int8_t nu[6];                     // ... with their coefficients
+  uint8_t nnet, type;
+  int16_t dnu, id, tb, troe;
 };
 
 struct alignas(16) FxTroe {
-  int64_t lnA0, b0, Ta0;      // low-pressure limit, as FxReac
+  int64_t lnA0;               // low-pressure limit, as FxRate
+  uint64_t b0, Ta0;
   double b0d, Ta0K;
   double a, iT3, iT1, T2, has_t2;
 };
 
 // one species in one temperature range; the polynomial variable is tau = T / 2^r (r = 10 below
-// TMID, 12 above), all Q11.52 except gl (Q7.56)
+// TMID, 12 above), all Q11.52 except gl (Q7.56); the leading coefficients g[4], h[4], c[4] and
+// ga6, gl, ha6 are biased
 struct FxSpecies {
   int64_t g[5], ga6, gl;      // g/RT/ln 2 = g(tau) + ga6 (128 / T) + gl log2 T
   int64_t h[5], ha6;          // h/RT
   int64_t c[5];               // cp/R
+  int64_t d3, d2;             // 4 c[4] (biased) and 3 c[3] of d(cp/R)/dtau
 };
 
 struct FxLayout {
-  int ns, nr, ntb, bytes;     // bytes = 0: no fixed-point form
+  int ns, ntb, bytes;         // bytes = 0: no fixed-point form
   int o_exp2, o_lg, o_rcp;    // tables of fixed.cuh
   int o_sp;                   // FxSpecies [2][ns]
   int o_W, o_invW;            // [ns]
   int o_nu;                   // double [16]: coefficient of code c is c - 8
-  int o_reac, o_troe;
+  int o_rate, o_reac, o_troe;   // FxRate [n_plain + n_tb + n_fo] in that order, FxReac [n_gen]
+  int n_plain, n_tb, n_fo, n_gen;
   int o_effv, o_eff;          // sparse (efficiency - 1); dense efficiencies [ntb][ns]
   int o_effidx, o_effoff;
   int64_t lpr0;               // log2(p_atm / R), Q11.52

@@ -1,6 +1,6 @@
 """Writes fixed_tables.h: the constants of the fixed-point exponential and logarithm (fixed.cuh).
 
-* 2^(j / 256) for j = 0 .. 255 as 64-bit mantissas (value times 2^63, rounded to nearest);
+* 2^(j / 256) for j = 0 .. 255 as 64-bit mantissas (value times 2^62, rounded to nearest);
 * for j = 0 .. 127 a 16-bit reciprocal c_j of the midpoint of [1 + j / 128, 1 + (j + 1) / 128)
   (value times 2^16), and -log2(c_j) times 2^60, rounded to nearest;
 * the Taylor coefficients of 2^x and of log2(1 + x) at the scales fixed.cuh states.
@@ -29,9 +29,9 @@ def main() -> None:
     u64 = lambda n: f"0x{n:016x}ull"
     out = ["// Generated by gen_fixed_tables.py; do not edit.",
            "#pragma once",
-           "// 2^(j / 256) times 2^63, j = 0 .. 255",
+           "// 2^(j / 256) times 2^62, j = 0 .. 255",
            "#define CHEM_FX_EXP2_VALUES \\"]
-    out += rows([u64(nearest((ln2 * j / 256).exp() * 2 ** 63)) for j in range(256)])
+    out += rows([u64(nearest((ln2 * j / 256).exp() * 2 ** 62)) for j in range(256)])
     c = [nearest(Decimal(2 ** 16) / (1 + (Decimal(j) + Decimal("0.5")) / 128)) for j in range(128)]
     out += ["", "// reciprocals c_j times 2^16 and their logarithms -log2(c_j) times 2^60, j = 0 .. 127",
             "#define CHEM_FX_RCP_VALUES \\"]

@@ -26,13 +26,13 @@ namespace chem {
 namespace cell {
 
 // workspace elements of one cell (doubles): state, six stage vectors, the iteration matrix,
-// concentrations, Gibbs energies and enthalpies
+// concentrations and Gibbs energies (each with the empty slot's 1 and 0 at the end), enthalpies
 template <int NS>
 struct Ws {
   static constexpr int N = NS + 1;
-  static constexpr int Y = 0, U = N, M = 7 * N, C = M + N * N, G = C + NS, H = G + NS, TOTAL = H + NS;
+  static constexpr int Y = 0, U = N, M = 7 * N, C = M + N * N, G = C + N, H = G + N, TOTAL = H + NS;
   // scratch inside the stage vectors while the Jacobian is formed (u_0 holds the rates)
-  static constexpr int DWDT = U + N, CP = U + 2 * N, RK = U + 3 * N, HM = U + 4 * N;
+  static constexpr int DWDT = U + N, CP = U + 2 * N, RK = U + 3 * N, WK = U + 4 * N;
 };
 
 struct View {
@@ -40,11 +40,12 @@ struct View {
   const uint32_t* rc;
   const FxSpecies* sp;
   const double *W, *invW, *nu, *effv, *eff;
+  const FxRate* rate;
   const FxReac* reac;
   const FxTroe* troe;
   const int16_t* effidx;
   const int* effoff;
-  int nr;
+  int n_plain, n_tb, n_fo, n_gen;
   fx::i64 lpr0;
   const unsigned char* blob;     // FP64 form in global memory (rates outside the fixed-point range)
   const MechLayout* lay;
@@ -62,11 +63,12 @@ __device__ __forceinline__ View bind(const unsigned char* s, const FxLayout& L, 
   v.nu = (const double*)(s + L.o_nu);
   v.effv = (const double*)(s + L.o_effv);
   v.eff = (const double*)(s + L.o_eff);
+  v.rate = (const FxRate*)(s + L.o_rate);
   v.reac = (const FxReac*)(s + L.o_reac);
   v.troe = (const FxTroe*)(s + L.o_troe);
   v.effidx = (const int16_t*)(s + L.o_effidx);
   v.effoff = (const int*)(s + L.o_effoff);
-  v.nr = L.nr;
+  v.n_plain = L.n_plain; v.n_tb = L.n_tb; v.n_fo = L.n_fo; v.n_gen = L.n_gen;
   v.lpr0 = L.lpr0;
   v.blob = blob;
   v.lay = lay;
@@ -109,6 +111,7 @@ __device__ __forceinline__ bool positive_normal(double x) {
 struct Temp {
   double T, invT;
   fx::u64 L, iT, tau;    // log2 T (Q4.60), 128 / T and T / 2^r (Q0.64)
+  fx::i64 L2, iT2, tau2; // halves of the three (fx::biased products)
   int rg;
   bool fast;             // T in [kTlo, kThi): fixed point
 };
@@ -125,6 +128,7 @@ __device__ __forceinline__ Temp temp_of(double T, const View& m, bool need_inv) 
   t.rg = T < TMID ? 0 : 1;
   const int rr = t.fast ? t.rg : 1;
   t.tau = mant >> ((rr == 0 ? kFxR0 - 1 : kFxR1 - 1) - e);
+  t.L2 = (fx::i64)(t.L >> 1); t.iT2 = (fx::i64)(t.iT >> 1); t.tau2 = (fx::i64)(t.tau >> 1);
   t.invT = 0.0;
   if (need_inv) t.invT = t.fast ? fx::to_double((fx::i64)(t.iT >> 1), 63 + fx::kTloExp) : 1.0 / T;
   return t;
@@ -136,26 +140,28 @@ __device__ __forceinline__ double g_of(double raw, bool fast) {
 }
 
 // Rate constants in FP64 for what the fixed-point path leaves out: cells whose temperature is
-// outside its range, reactions whose exponents are.  kf (the high-pressure limit of a fall-off
-// reaction) and 1 / Kc; k0 of a fall-off reaction.
+// outside its range, reactions whose exponents are.  Reaction id of the FP64 form: kf (the
+// high-pressure limit of a fall-off reaction), 1 / Kc, and k0 of a fall-off reaction.
 template <int NS>
-__device__ __noinline__ void slow_k(const View& m, const double* col, int j, double T, bool fast, double* kf,
+__device__ __noinline__ void slow_k(const View& m, const double* col, int id, double T, bool fast, double* kf,
                                     double* invKc, double* k0) {
   using w = Ws<NS>;
-  const FxReac& R = m.reac[j];
   const MechLayout& L = *m.lay;
   const double lnT = log(T), invT = 1.0 / T;
   const double* lnA = (const double*)(m.blob + L.o_lnA);
-  *kf = exp(lnA[j] + R.b * lnT - R.TaK * invT);
-  if (R.type == 2) {
-    const double* tr = (const double*)(m.blob + L.o_troe) + 8 * R.troe;
+  const double* beta = (const double*)(m.blob + L.o_beta);
+  const double* Ta = (const double*)(m.blob + L.o_Ta);
+  const short4 re = ((const short4*)(m.blob + L.o_reac))[id], pr = ((const short4*)(m.blob + L.o_prod))[id];
+  const short4 ri = ((const short4*)(m.blob + L.o_rinfo))[id];
+  *kf = exp(lnA[id] + beta[id] * lnT - Ta[id] * invT);
+  if (ri.x == 2) {
+    const double* tr = (const double*)(m.blob + L.o_troe) + 8 * ri.w;
     *k0 = exp(tr[0] + tr[1] * lnT - tr[2] * invT);
   }
-  double dG = 0.0;
-  for (int i = 0; i < R.nre; ++i) dG -= g_of(col[(w::G + R.re[i]) * 32], fast);
-  for (int i = 0; i < R.npr; ++i) dG += g_of(col[(w::G + R.pr[i]) * 32], fast);
+  auto g = [&](int k) { return k >= 0 ? g_of(col[(w::G + k) * 32], fast) : 0.0; };
+  const double dG = g(pr.x) + g(pr.y) + g(pr.z) - g(re.x) - g(re.y) - g(re.z);
   const double* cst = (const double*)(m.blob + L.o_const);
-  *invKc = exp(dG - (double)R.dnu * (cst[kC_LNPR0] - lnT));
+  *invKc = exp(dG - (double)ri.y * (cst[kC_LNPR0] - lnT));
 }
 
 // Species thermo in FP64 (temperatures outside the fixed-point range): g/RT and h/RT (cp/R with
@@ -275,7 +281,120 @@ __device__ __forceinline__ bool troe_fast(const View& m, const FxTroe& t, const 
   return true;
 }
 
-// Right-hand side f(T, Y) into u (workspace elements uoff ..), and with JAC the NEGATED analytic
+// Base-2 exponents of a reaction's forward and reverse rate constants: log2 kf = log2 A + b log2 T -
+// Ta / (T ln 2), log2 kr = log2 kf + Delta G / (RT ln 2) - dnu log2(p_atm / (R T)); shift = iT2 - L2
+// of the biased products, D = log2 T - log2(p_atm / R).
+template <class R>
+__device__ __forceinline__ fx::i64 exponent_f(const R& r, const Temp& t, fx::i64 shift) {
+  return r.lnA + (fx::i64)(fx::umulhi3(r.beta, t.L) - fx::umulhi3(r.Ta, t.iT)) + shift;
+}
+
+// The slots of an FxRate, warp-uniform, in registers
+struct Slots {
+  unsigned r0, r1, p0, p1;
+};
+__device__ __forceinline__ Slots slots(const uint16_t* c) {
+  const uint2 v = *reinterpret_cast<const uint2*>(c);
+  return Slots{v.x & 0xffffu, v.x >> 16, v.y & 0xffffu, v.y >> 16};
+}
+__device__ __forceinline__ double* at(double* col, unsigned off) {
+  return reinterpret_cast<double*>(reinterpret_cast<unsigned char*>(col) + off);
+}
+
+// FP64 rate constants of a reaction that (or whose cell) is outside the fixed-point range; JAC
+// also d ln kf/dT, d kf/d[M] and 1 / Kc
+template <int NS>
+__device__ __noinline__ void slow_rate(const View& m, const double* col, int id, int troe, double T, bool fast,
+                                       double Mc, double* kf, double* kr, double* dlnkf, double* dkfdM,
+                                       double* invKc) {
+  double k0 = 0.0;
+  slow_k<NS>(m, col, id, T, fast, kf, invKc, &k0);
+  if (troe >= 0) {
+    const double kinf = *kf;
+    slow_troe(m.troe[troe], T, kinf, k0, Mc, *dlnkf, kf, dlnkf, dkfdM);
+  }
+  *kr = *kf * *invKc;
+}
+
+// collision-partner concentration sum_k eff_k C_k of third-body set tb
+template <int NS>
+__device__ __forceinline__ double partners(const View& m, const double* col, int tb, double Ctot) {
+  double Mc = Ctot;
+  const int e1 = m.effoff[tb + 1];
+  for (int e = m.effoff[tb]; e < e1; ++e) Mc = fma(m.effv[e], col[(Ws<NS>::C + m.effidx[e]) * 32], Mc);
+  return Mc;
+}
+
+// Any reaction (FxReac): three species on a side, up to six net species.  Adds its production rates
+// and, with JAC, its derivatives.
+template <int NS, bool JAC>
+__device__ __noinline__ void general_reaction(const View& m, double* col, const FxReac& R, const Temp& t, double T,
+                                              fx::i64 shift, fx::i64 D, double Ctot, int uoff) {
+  using w = Ws<NS>;
+  constexpr int N = w::N;
+  const int nre = R.nre, npr = R.npr, nn = R.nnet;
+  const double* Cc = col + w::C * 32;
+  const double* Gc = col + w::G * 32;
+  const fx::i64 Xf = exponent_f(R, t, shift);
+  fx::i64 Xr = Xf + (fx::i64)R.dnu * D;
+  double a[3] = {1.0, 1.0, 1.0}, b[3] = {1.0, 1.0, 1.0};
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    if (i < nre) { a[i] = Cc[R.re[i] * 32]; Xr -= __double_as_longlong(Gc[R.re[i] * 32]); }
+    if (i < npr) { b[i] = Cc[R.pr[i] * 32]; Xr += __double_as_longlong(Gc[R.pr[i] * 32]); }
+  }
+  const double Mc = R.type != 0 ? partners<NS>(m, col, R.tb, Ctot) : 1.0;
+  double dlnkf = JAC ? fma(R.TaK * t.invT, t.invT, R.b * t.invT) : 0.0;
+  double kf = 0.0, kr = 0.0, dMr = 0.0, dkfdM = 0.0, invKc = 0.0;
+  bool fastk = t.fast && fx::exp2_in_range(Xf) && fx::exp2_in_range(Xr);
+  if (fastk) {
+    kf = fx::exp2_q52(Xf, m.e2);
+    kr = fx::exp2_q52(Xr, m.e2);
+    if (R.type == 2) {
+      const FxTroe& F = m.troe[R.troe];
+      const fx::i64 Xk = F.lnA0 + (fx::i64)(fx::umulhi3(F.b0, t.L) - fx::umulhi3(F.Ta0, t.iT)) + shift - Xf;
+      double fac = 1.0, dl = 0.0;
+      fastk = troe_fast<JAC>(m, F, t, Xk, Mc, dlnkf, &fac, &dl, &dMr);
+      kf *= fac;
+      kr *= fac;
+      if (JAC && fastk) dlnkf = dl;
+    }
+  }
+  if (!fastk)
+    slow_rate<NS>(m, col, R.id, R.type == 2 ? R.troe : -1, T, t.fast, Mc, &kf, &kr, &dlnkf, &dkfdM, &invKc);
+  const double Pf = a[0] * a[1] * a[2], Pr = b[0] * b[1] * b[2];
+  const double mult = R.type == 1 ? Mc : 1.0;
+  const double fwd = kf * Pf, rev = kr * Pr, net = fwd - rev;
+  double dqdT = 0.0;
+  if (JAC) {
+    double dH = -(double)R.dnu;
+    for (int i = 0; i < nre; ++i) dH -= col[(w::H + R.re[i]) * 32];
+    for (int i = 0; i < npr; ++i) dH += col[(w::H + R.pr[i]) * 32];
+    dqdT = mult * fma(net, dlnkf, rev * (dH * t.invT));
+  }
+  double* Jm = col + (w::M + N + 1) * 32;
+  for (int i = 0; i < nn; ++i) {
+    const double nu = m.nu[R.nu[i] + 8];
+    double* x = col + (uoff + 1 + R.sp[i]) * 32;
+    *x = fma(nu, mult * net, *x);
+    if (!JAC) continue;
+    double* y = col + (w::DWDT + R.sp[i]) * 32;
+    *y = fma(nu, dqdT, *y);
+    double* row = Jm + R.sp[i] * N * 32;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      if (q < nre) row[R.re[q] * 32] = fma(-nu, mult * kf * a[(q + 1) % 3] * a[(q + 2) % 3], row[R.re[q] * 32]);
+      if (q < npr) row[R.pr[q] * 32] = fma(nu, mult * kr * b[(q + 1) % 3] * b[(q + 2) % 3], row[R.pr[q] * 32]);
+    }
+    if (R.type != 0) {
+      const double X = R.type == 1 ? net : (fastk ? dMr * net : dkfdM * (Pf - Pr * invKc));
+      const double* ef = m.eff + R.tb * NS;
+      for (int mm = 0; mm < NS; ++mm) row[mm * 32] = fma(-nu * X, ef[mm], row[mm * 32]);
+    }
+  }
+}
+
+// Right-hand side f(T, Y) into workspace elements uoff .., and with JAC the NEGATED analytic
 // Jacobian -df/dy into the matrix.  Yk(k) returns the mass fraction of species k; p and 1 / p of
 // the cell.  Writes the concentrations, Gibbs energies and enthalpies of the workspace.
 template <int NS, bool JAC, class YF>
@@ -293,30 +412,32 @@ __device__ __forceinline__ void rhs(const View& m, double* col, double T, YF Yk,
   }
   if (t.fast) {
     const FxSpecies* sp = m.sp + t.rg * NS;
+    const fx::u64 B = 0x8000000000000000ull;
+    const fx::i64 gT = t.iT2 + t.L2;
 #pragma unroll 3
     for (int k = 0; k < NS; ++k) {
       const FxSpecies& s = sp[k];
-      fx::i64 g = s.g[4], h = s.h[4], cp = s.c[4];
+      fx::u64 g = (fx::u64)s.g[4], h = (fx::u64)s.h[4], cp = (fx::u64)s.c[4];   // biased
 #pragma unroll
       for (int i = 3; i >= 0; --i) {
-        g = fx::mulhi_su(g, t.tau) + s.g[i];
-        h = fx::mulhi_su(h, t.tau) + s.h[i];
-        cp = fx::mulhi_su(cp, t.tau) + s.c[i];
+        const fx::u64 b = i ? B : 0ull;                                        // the last one unbiased
+        g = (fx::umulhi3(g, t.tau) + (fx::u64)(s.g[i] - t.tau2)) ^ b;
+        h = (fx::umulhi3(h, t.tau) + (fx::u64)(s.h[i] - t.tau2)) ^ b;
+        cp = (fx::umulhi3(cp, t.tau) + (fx::u64)(s.c[i] - t.tau2)) ^ b;
       }
-      g += fx::mulhi_su(s.ga6, t.iT) + fx::mulhi_su(s.gl, t.L);
-      h += fx::mulhi_su(s.ha6, t.iT);
-      col[(w::G + k) * 32] = __longlong_as_double(g);
-      col[(w::H + k) * 32] = fx::to_double(h, 52);
-      const double cpd = fx::to_double(cp, 52);
+      g += fx::umulhi3((fx::u64)s.ga6, t.iT) + fx::umulhi3((fx::u64)s.gl, t.L) - (fx::u64)gT;
+      h += fx::umulhi3((fx::u64)s.ha6, t.iT) - (fx::u64)t.iT2;
+      col[(w::G + k) * 32] = __longlong_as_double((fx::i64)g);
+      col[(w::H + k) * 32] = fx::to_double((fx::i64)h, 52);
+      const double cpd = fx::to_double((fx::i64)cp, 52);
       const double ck = col[(w::C + k) * 32];
       cps = fma(ck, cpd, cps);
       if (JAC) {
         // d(cp/R)/dT 2^r = sum_i i c_i tau^(i-1)
-        fx::i64 dc = s.c[4] * 4;
-        dc = fx::mulhi_su(dc, t.tau) + s.c[3] * 3;
-        dc = fx::mulhi_su(dc, t.tau) + s.c[2] * 2;
-        dc = fx::mulhi_su(dc, t.tau) + s.c[1];
-        dcps = fma(ck, fx::to_double(dc, 52 + (t.rg == 0 ? kFxR0 : kFxR1)), dcps);
+        fx::u64 dc = (fx::umulhi3((fx::u64)s.d3, t.tau) + (fx::u64)(s.d2 - t.tau2)) ^ B;
+        dc = (fx::umulhi3(dc, t.tau) + (fx::u64)(s.c[2] * 2 - t.tau2)) ^ B;
+        dc = fx::umulhi3(dc, t.tau) + (fx::u64)(s.c[1] - t.tau2);
+        dcps = fma(ck, fx::to_double((fx::i64)dc, 52 + (t.rg == 0 ? kFxR0 : kFxR1)), dcps);
         col[(w::CP + k) * 32] = cpd;
       }
     }
@@ -331,158 +452,162 @@ __device__ __forceinline__ void rhs(const View& m, double* col, double T, YF Yk,
     col[(uoff + 1 + k) * 32] = 0.0;
     if (JAC) col[(w::DWDT + k) * 32] = 0.0;
   }
+  col[(w::C + NS) * 32] = 1.0;                 // the empty slot
+  col[(w::G + NS) * 32] = 0.0;
   if (JAC) {
 #pragma unroll
     for (int e = 0; e < NS * NS; ++e) col[(w::M + (1 + e / NS) * N + 1 + e % NS) * 32] = 0.0;
   }
   const double Ctot = rho * S;
-  const fx::i64 L52 = (fx::i64)((t.L + 128ull) >> 8);
-  double* Jm = col + (w::M + N + 1) * 32;      // row 1 (species 0), column 1
+  const fx::i64 D = (fx::i64)((t.L + 128ull) >> 8) - m.lpr0;
+  const fx::i64 shift = t.iT2 - t.L2;
+  double* const Cc = col + w::C * 32;
+  double* const Gc = col + w::G * 32;
+  double* const wd = col + (uoff + 1) * 32;
+  double* const Jm = col + (w::M + N + 1) * 32;      // row 1 (species 0), column 1
 
-  for (int j = 0; j < m.nr; ++j) {
-    const FxReac& R = m.reac[j];
-    const int nre = R.nre, npr = R.npr;
-    const fx::i64 Xf = R.lnA + fx::mulhi_su(R.beta, t.L) - fx::mulhi_su(R.Ta, t.iT);
-    const double* cr0 = col + (w::C + R.re[0]) * 32;
-    const double* cp0 = col + (w::C + R.pr[0]) * 32;
-    double a0 = cr0[0], b0 = cp0[0], a1 = 1.0, a2 = 1.0, b1 = 1.0, b2 = 1.0;
-    fx::i64 Xr = Xf + __double_as_longlong(cp0[NS * 32]) - __double_as_longlong(cr0[NS * 32]);   // G follows C
-    double Pf = a0, Pr = b0;
-    if (nre > 1) {
-      const double* q = col + (w::C + R.re[1]) * 32;
-      a1 = q[0]; Xr -= __double_as_longlong(q[NS * 32]); Pf *= a1;
-      if (nre > 2) {
-        const double* q2 = col + (w::C + R.re[2]) * 32;
-        a2 = q2[0]; Xr -= __double_as_longlong(q2[NS * 32]); Pf *= a2;
-      }
-    }
-    if (npr > 1) {
-      const double* q = col + (w::C + R.pr[1]) * 32;
-      b1 = q[0]; Xr += __double_as_longlong(q[NS * 32]); Pr *= b1;
-      if (npr > 2) {
-        const double* q2 = col + (w::C + R.pr[2]) * 32;
-        b2 = q2[0]; Xr += __double_as_longlong(q2[NS * 32]); Pr *= b2;
-      }
-    }
-    const int dnu = R.dnu;
-    Xr += (fx::i64)dnu * (L52 - m.lpr0);
-    double Mc = 1.0;
-    if (R.type != 0) {
-      Mc = Ctot;
-      const int e1 = m.effoff[R.tb + 1];
-      for (int e = m.effoff[R.tb]; e < e1; ++e) Mc = fma(m.effv[e], col[(w::C + m.effidx[e]) * 32], Mc);
-    }
-    double dlnkf = 0.0;
-    if (JAC) dlnkf = fma(R.TaK * t.invT, t.invT, R.b * t.invT);
-    double kf, kr, k0 = 0.0, dMr = 0.0;        // dMr: (d kf / d[M]) / kf of a fall-off reaction
-    double dkfdM = 0.0, invKc = 0.0;
-    bool done = t.fast && !R.slow && fx::exp2_in_range(Xf) && fx::exp2_in_range(Xr);
-    if (done) {
-      kf = fx::exp2_q52(Xf, m.e2);
-      kr = fx::exp2_q52(Xr, m.e2);
-      if (R.type == 2) {
-        const FxTroe& F = m.troe[R.troe];
-        const fx::i64 Xk = F.lnA0 + fx::mulhi_su(F.b0, t.L) - fx::mulhi_su(F.Ta0, t.iT) - Xf;
-        double fac = 1.0, dl = 0.0;
-        done = troe_fast<JAC>(m, F, t, Xk, Mc, dlnkf, &fac, &dl, &dMr);
-        kf *= fac;
-        kr *= fac;
-        if (JAC && done) dlnkf = dl;
-      }
-    }
-    const bool fastk = done;
-    if (!fastk) {
-      slow_k<NS>(m, col, j, T, t.fast, &kf, &invKc, &k0);
-      if (R.type == 2) {
-        const double kinf = kf;
-        double dl;
-        slow_troe(m.troe[R.troe], T, kinf, k0, Mc, dlnkf, &kf, &dl, &dkfdM);
-        dlnkf = dl;
-      }
-      kr = kf * invKc;
-    }
-    double* wd = col + (uoff + 1) * 32;
-    if (!JAC) {
-      double q = fma(kf, Pf, -(kr * Pr));
-      if (R.type == 1) q *= Mc;
-      const int nn = R.nnet;
-      for (int i = 0; i < nn; ++i) {
-        double* x = wd + R.sp[i] * 32;
-        *x = fma(m.nu[R.nu[i] + 8], q, *x);
-      }
-    } else {
-      const double fwd = kf * Pf, rev = kr * Pr, net = fwd - rev;
-      const double mult = R.type == 1 ? Mc : 1.0;
-      double dH = -(double)dnu;
-      for (int i = 0; i < nre; ++i) dH -= col[(w::H + R.re[i]) * 32];
-      for (int i = 0; i < npr; ++i) dH += col[(w::H + R.pr[i]) * 32];
-      const double dlnKc = dH * t.invT;
-      double dqdT = fma(net, dlnkf, rev * dlnKc);
-      double q = net, ka = kf, kb = kr;
-      if (R.type == 1) { q *= mult; dqdT *= mult; ka *= mult; kb *= mult; }
-      const int nn = R.nnet;
-      for (int i = 0; i < nn; ++i) {
-        const double nu = m.nu[R.nu[i] + 8];
-        double* x = wd + R.sp[i] * 32;
-        *x = fma(nu, q, *x);
-        double* y = col + (w::DWDT + R.sp[i]) * 32;
-        *y = fma(nu, dqdT, *y);
-      }
-      // d(wdot)/dC, negated: a slot's derivative times the net coefficient of every species
-      auto slot = [&](int sp, double d) {
-        for (int i = 0; i < nn; ++i) {
-          double* x = Jm + (R.sp[i] * N + sp) * 32;
-          *x = fma(-m.nu[R.nu[i] + 8], d, *x);
-        }
-      };
-      if (nre == 1) {
-        slot(R.re[0], ka);
-      } else if (nre == 2) {
-        slot(R.re[0], ka * a1);
-        slot(R.re[1], ka * a0);
-      } else {
-        slot(R.re[0], ka * a1 * a2);
-        slot(R.re[1], ka * a0 * a2);
-        slot(R.re[2], ka * a0 * a1);
-      }
-      if (npr == 1) {
-        slot(R.pr[0], -kb);
-      } else if (npr == 2) {
-        slot(R.pr[0], -kb * b1);
-        slot(R.pr[1], -kb * b0);
-      } else {
-        slot(R.pr[0], -kb * b1 * b2);
-        slot(R.pr[1], -kb * b0 * b2);
-        slot(R.pr[2], -kb * b0 * b1);
-      }
-      if (R.type != 0) {
-        double X;
-        if (R.type == 1) X = net;
-        else X = fastk ? dMr * net : dkfdM * (Pf - Pr * invKc);
-        const double* ef = m.eff + R.tb * NS;
-        for (int i = 0; i < nn; ++i) {
-          const double nx = -m.nu[R.nu[i] + 8] * X;
-          double* x = Jm + R.sp[i] * N * 32;
+  // exponents and concentration products of an FxRate
+  auto prepare = [&](const FxRate& R, const Slots& s, fx::i64& Xf, fx::i64& Xr) {
+    Xf = exponent_f(R, t, shift);
+    Xr = Xf + (__double_as_longlong(*at(Gc, s.p0)) + __double_as_longlong(*at(Gc, s.p1))) -
+         (__double_as_longlong(*at(Gc, s.r0)) + __double_as_longlong(*at(Gc, s.r1)));
+  };
+  auto in_range = [&](fx::i64 Xf, fx::i64 Xr) { return t.fast && fx::exp2_in_range(Xf) && fx::exp2_in_range(Xr); };
+  auto scatter = [&](const FxRate& R, double q) {
+    const Slots s = slots(R.w);
+    double *a0 = at(wd, s.r0), *a1 = at(wd, s.r1), *a2 = at(wd, s.p0), *a3 = at(wd, s.p1);
+    const double v0 = fma(R.nu[0], q, *a0), v1 = fma(R.nu[1], q, *a1);
+    const double v2 = fma(R.nu[2], q, *a2), v3 = fma(R.nu[3], q, *a3);
+    *a0 = v0; *a1 = v1; *a2 = v2; *a3 = v3;
+  };
+  // Jacobian share of an FxRate with rate constants already times the collision partner: q and dq/dT
+  // into the production rates, the slots' derivatives into d(wdot)/dC (negated)
+  auto derivatives = [&](const FxRate& R, const Slots& s, double ka, double kb, double a0, double a1, double b0,
+                         double b1, double q, double dqdT) {
+    scatter(R, q);
+    const Slots x = slots(R.w);
+    const unsigned row[4] = {x.r0, x.r1, x.p0, x.p1};
 #pragma unroll
-          for (int mm = 0; mm < NS; ++mm) x[mm * 32] = fma(nx, ef[mm], x[mm * 32]);
-        }
+    for (int i = 0; i < 4; ++i) {
+      double* y = at(col + w::DWDT * 32, row[i]);
+      *y = fma(R.nu[i], dqdT, *y);
+    }
+    auto column = [&](unsigned sp, double d) {
+      double v[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v[i] = fma(-R.nu[i], d, *at(Jm, row[i] * N + sp));
+#pragma unroll
+      for (int i = 0; i < 4; ++i) *at(Jm, row[i] * N + sp) = v[i];
+    };
+    column(s.r0, ka * a1);
+    if (s.r1 != NS * 256u) column(s.r1, ka * a0);
+    column(s.p0, -kb * b1);
+    if (s.p1 != NS * 256u) column(s.p1, -kb * b0);
+  };
+  auto dlnkf_of = [&](double b, double TaK) { return fma(TaK * t.invT, t.invT, b * t.invT); };
+  auto dlnKc_of = [&](const Slots& s, int dnu) {
+    const double* Hc = col + w::H * 32;
+    double dH = *at(const_cast<double*>(Hc), s.p0) - *at(const_cast<double*>(Hc), s.r0);
+    if (s.p1 != NS * 256u) dH += *at(const_cast<double*>(Hc), s.p1);
+    if (s.r1 != NS * 256u) dH -= *at(const_cast<double*>(Hc), s.r1);
+    if (dnu) dH -= (double)dnu;
+    return dH * t.invT;
+  };
+  // d(wdot)/dC through the collision partners: X times the efficiencies of set tb
+  auto partner_rows = [&](const FxRate& R, double X) {
+    const double* ef = m.eff + R.tb * NS;
+    const Slots x = slots(R.w);
+    const unsigned row[4] = {x.r0, x.r1, x.p0, x.p1};
+    for (int i = 0; i < 4; ++i) {
+      if (R.nu[i] == 0.0) continue;
+      const double nx = -R.nu[i] * X;
+      double* y = at(Jm, row[i] * N);
+#pragma unroll
+      for (int mm = 0; mm < NS; ++mm) y[mm * 32] = fma(nx, ef[mm], y[mm * 32]);
+    }
+  };
+
+  const FxRate* R = m.rate;
+  // ---- plain reactions, two at a time: four independent exponentials hide the integer latency ----
+  int j = 0;
+  if (!JAC) {
+    for (; j + 1 < m.n_plain; j += 2, R += 2) {
+      const Slots s0 = slots(R[0].c), s1 = slots(R[1].c);
+      fx::i64 Xf0, Xr0, Xf1, Xr1;
+      prepare(R[0], s0, Xf0, Xr0);
+      prepare(R[1], s1, Xf1, Xr1);
+      if (R[0].dnu) Xr0 += (fx::i64)R[0].dnu * D;
+      if (R[1].dnu) Xr1 += (fx::i64)R[1].dnu * D;
+      double kf0 = fx::exp2_q52(Xf0, m.e2), kr0 = fx::exp2_q52(Xr0, m.e2);
+      double kf1 = fx::exp2_q52(Xf1, m.e2), kr1 = fx::exp2_q52(Xr1, m.e2);
+      const bool ok0 = in_range(Xf0, Xr0), ok1 = in_range(Xf1, Xr1);
+      if (!(ok0 && ok1)) {
+        double x = 0.0, y, z;
+        if (!ok0) slow_rate<NS>(m, col, R[0].id, -1, T, t.fast, 1.0, &kf0, &kr0, &x, &y, &z);
+        if (!ok1) slow_rate<NS>(m, col, R[1].id, -1, T, t.fast, 1.0, &kf1, &kr1, &x, &y, &z);
       }
+      const double q0 = fma(kf0, *at(Cc, s0.r0) * *at(Cc, s0.r1), -(kr0 * (*at(Cc, s0.p0) * *at(Cc, s0.p1))));
+      const double q1 = fma(kf1, *at(Cc, s1.r0) * *at(Cc, s1.r1), -(kr1 * (*at(Cc, s1.p0) * *at(Cc, s1.p1))));
+      scatter(R[0], q0);
+      scatter(R[1], q1);
     }
   }
+  // ---- the rest of the plain ones, third-body and fall-off reactions (stored in that order) ----
+  const int n2 = m.n_plain + m.n_tb, n3 = n2 + m.n_fo;
+  for (; j < n3; ++j, ++R) {
+    const Slots s = slots(R->c);
+    fx::i64 Xf, Xr;
+    prepare(*R, s, Xf, Xr);
+    if (R->dnu) Xr += (fx::i64)R->dnu * D;
+    const double a0 = *at(Cc, s.r0), a1 = *at(Cc, s.r1), b0 = *at(Cc, s.p0), b1 = *at(Cc, s.p1);
+    double Mc = 1.0;
+    if (j >= m.n_plain) Mc = partners<NS>(m, col, R->tb, Ctot);
+    double dlnkf = JAC ? dlnkf_of(R->b, R->TaK) : 0.0;
+    double kf = fx::exp2_q52(Xf, m.e2), kr = fx::exp2_q52(Xr, m.e2);
+    double dMr = 0.0, dkfdM = 0.0, invKc = 0.0;   // (d kf/d[M]) / kf; d kf/d[M] and 1 / Kc of the FP64 form
+    bool fastk = in_range(Xf, Xr);
+    if (j >= n2 && fastk) {
+      const FxTroe& F = m.troe[R->troe];
+      const fx::i64 Xk = F.lnA0 + (fx::i64)(fx::umulhi3(F.b0, t.L) - fx::umulhi3(F.Ta0, t.iT)) + shift - Xf;
+      double fac = 1.0, dl = 0.0;
+      fastk = troe_fast<JAC>(m, F, t, Xk, Mc, dlnkf, &fac, &dl, &dMr);
+      kf *= fac;
+      kr *= fac;
+      if (JAC && fastk) dlnkf = dl;
+    }
+    if (!fastk)
+      slow_rate<NS>(m, col, R->id, j >= n2 ? R->troe : -1, T, t.fast, Mc, &kf, &kr, &dlnkf, &dkfdM, &invKc);
+    const bool third = j >= m.n_plain && j < n2;
+    if (!JAC) {
+      double q = fma(kf, a0 * a1, -(kr * (b0 * b1)));
+      if (third) q *= Mc;
+      scatter(*R, q);
+    } else {
+      const double fwd = kf * (a0 * a1), rev = kr * (b0 * b1), net = fwd - rev;
+      double dqdT = fma(net, dlnkf, rev * dlnKc_of(s, R->dnu));
+      double q = net, ka = kf, kb = kr;
+      if (third) { q *= Mc; dqdT *= Mc; ka *= Mc; kb *= Mc; }
+      derivatives(*R, s, ka, kb, a0, a1, b0, b1, q, dqdT);
+      if (third) partner_rows(*R, net);
+      else if (j >= n2) partner_rows(*R, fastk ? dMr * net : dkfdM * (a0 * a1 - b0 * b1 * invKc));
+    }
+  }
+  // ---- reactions with three species on a side or more than four net species ----
+  for (int i = 0; i < m.n_gen; ++i) general_reaction<NS, JAC>(m, col, m.reac[i], t, T, shift, D, Ctot, uoff);
 
   // species and temperature rows: f_k = W_k w_k / rho, f_0 = -T sum h/RT w / (rho cp/R)
   double Q = 0.0, r31 = 0.0, r32 = 0.0;
-  double wk[NS];
 #pragma unroll
   for (int k = 0; k < NS; ++k) {
-    wk[k] = col[(uoff + 1 + k) * 32];
+    const double wk = col[(uoff + 1 + k) * 32];
     const double h = col[(w::H + k) * 32];
-    Q = fma(h, wk[k], Q);
+    Q = fma(h, wk, Q);
     if (JAC) {
-      r31 = fma(col[(w::CP + k) * 32], wk[k], r31);
+      r31 = fma(col[(w::CP + k) * 32], wk, r31);
       r32 = fma(h, col[(w::DWDT + k) * 32], r32);
+      col[(w::WK + k) * 32] = wk;
     }
-    col[(uoff + 1 + k) * 32] = m.W[k] * (wk[k] * invrho);
+    col[(uoff + 1 + k) * 32] = m.W[k] * (wk * invrho);
   }
   const double ircp = rcp(rho * cps);         // 1 / (rho cp/R)
   col[uoff * 32] = -(T * Q) * ircp;
@@ -494,13 +619,13 @@ __device__ __forceinline__ void rhs(const View& m, double* col, double T, YF Yk,
   const double iS = rcp(S);
   const double rS = invrho * iS;
   double Rh = 0.0;
-#pragma unroll
+#pragma unroll 2
   for (int k = 0; k < NS; ++k) {
     double s = 0.0;
 #pragma unroll
     for (int mm = 0; mm < NS; ++mm) s = fma(Jm[(k * N + mm) * 32], col[(w::C + mm) * 32], s);
     Rh = fma(-col[(w::H + k) * 32], s, Rh);
-    const double dk = -s - wk[k];
+    const double dk = -s - col[(w::WK + k) * 32];
     col[(w::RK + k) * 32] = dk * rS;
     Jm[(k * N - 1) * 32] = -(m.W[k] * invrho * (col[(w::DWDT + k) * 32] - dk * t.invT));
   }
@@ -508,7 +633,7 @@ __device__ __forceinline__ void rhs(const View& m, double* col, double T, YF Yk,
   const double Qr = TQ * ircp;                 // -f_0
   col[w::M * 32] = (r31 + T * r32 - Rh) * ircp + Qr * (cps * t.invT - dcps) * (rho * ircp);
   const double RhS = TRh * iS, cpS = cps * iS, Qrr = Qr * rho;
-#pragma unroll
+#pragma unroll 2
   for (int mm = 0; mm < NS; ++mm) {
     double s = 0.0;
 #pragma unroll
@@ -516,7 +641,7 @@ __device__ __forceinline__ void rhs(const View& m, double* col, double T, YF Yk,
     const double Hm = T * s;
     Jm[(mm - N) * 32] = m.invW[mm] * ircp * ((rho * Hm - RhS) - Qrr * (col[(w::CP + mm) * 32] - cpS));
   }
-#pragma unroll
+#pragma unroll 2
   for (int k = 0; k < NS; ++k) {
     const double rk = col[(w::RK + k) * 32], Wk = m.W[k];
 #pragma unroll

@@ -125,7 +125,17 @@ std::vector<unsigned char> build_fx(const chem_mech_desc* d, const chem_mech_s* 
     }
     effoff.push_back((int)effidx.size());
   }
-  L->ns = ns; L->nr = nr; L->ntb = ntb;
+  L->ns = ns; L->ntb = ntb;
+  // at most two species per side and four net species: FxRate, by type; the rest: FxReac
+  std::vector<int> order[4];
+  for (int j = 0; j < nr; ++j) {
+    int nre = 0, npr = 0, nn = 0;
+    for (int i = 0; i < 3; ++i) { nre += d->reac[3 * j + i] >= 0; npr += d->prod[3 * j + i] >= 0; }
+    for (int k = 0; k < ns; ++k) nn += nu[j][k] != 0;
+    order[nre <= 2 && npr <= 2 && nn <= 4 && ns >= 4 ? d->rtype[j] : 3].push_back(j);
+  }
+  L->n_plain = (int)order[0].size(); L->n_tb = (int)order[1].size(); L->n_fo = (int)order[2].size();
+  L->n_gen = (int)order[3].size();
   L->o_exp2 = B.add(8 * 256);
   L->o_lg = B.add(8 * 128);
   L->o_rcp = B.add(4 * 128);
@@ -133,7 +143,8 @@ std::vector<unsigned char> build_fx(const chem_mech_desc* d, const chem_mech_s* 
   L->o_W = B.add(8 * ns);
   L->o_invW = B.add(8 * ns);
   L->o_nu = B.add(8 * 16);
-  L->o_reac = B.add(nr * (int)sizeof(FxReac));
+  L->o_rate = B.add((nr - L->n_gen) * (int)sizeof(FxRate));
+  L->o_reac = B.add(L->n_gen * (int)sizeof(FxReac));
   L->o_troe = B.add(ntroe * (int)sizeof(FxTroe));
   L->o_effv = B.add(8 * (int)effv.size());
   L->o_eff = B.add(8 * (int)eff.size());
@@ -163,12 +174,15 @@ std::vector<unsigned char> build_fx(const chem_mech_desc* d, const chem_mech_s* 
       S->ha6 = q52l((long double)a[5] / 128.0L, 1900.0);
       S->ga6 = q52l((long double)a[5] / 128.0L / l2, 1900.0);
       S->gl = q(-a[0], 56, 100.0);
+      S->d3 = S->c[4] * 4;
+      S->d2 = S->c[3] * 3;
       double sg = std::fabs((double)S->ga6), sh_ = std::fabs((double)S->ha6), sc = 0.0;
       for (int i = 0; i < 5; ++i) {
         sg += std::fabs((double)S->g[i]); sh_ += std::fabs((double)S->h[i]);
         sc += std::max(1, i) * std::fabs((double)S->c[i]);
       }
       if (!(std::max(std::max(sg + 12.0 * std::fabs((double)S->gl) / 16.0, sh_), sc) <= 2000.0 * 4503599627370496.0)) ok = false;
+      for (int64_t* x : {&S->g[4], &S->h[4], &S->c[4], &S->ga6, &S->gl, &S->ha6, &S->d3}) *x = (int64_t)fx::biased(*x);
     }
   for (int k = 0; k < ns; ++k) {
     B.at<double>(L->o_W)[k] = m->W[k];
@@ -176,57 +190,15 @@ std::vector<unsigned char> build_fx(const chem_mech_desc* d, const chem_mech_s* 
   }
   for (int c = 0; c < 16; ++c) B.at<double>(L->o_nu)[c] = (double)(c - 8);
   L->lpr0 = q52l(std::log((long double)PATM / (long double)RU) / l2, 1000.0);
-  int tb = 0, tr = 0;
-  for (int j = 0; j < nr; ++j) {
-    FxReac* R = B.at<FxReac>(L->o_reac) + j;
-    R->type = (uint8_t)d->rtype[j];
-    R->tb = R->type ? (int16_t)tb++ : (int16_t)-1;
-    R->troe = R->type == 2 ? (int16_t)tr++ : (int16_t)-1;
-    R->b = d->b[j];
-    R->TaK = d->Ea[j] / RC;
-    auto rate = [&](double A, double b, double Ea, int64_t* o) {
-      const long double lnA = A > 0.0 ? std::log((long double)A) / l2 : 1e9L;
-      const long double Ta = (long double)Ea / (long double)RC / l2 / 128.0L;
-      if (!(std::fabs((double)lnA) <= 600.0) || !(std::fabs(b) <= 32.0) || !(std::fabs((double)Ta) <= 1900.0)) {
-        R->slow = 1;
-        o[0] = o[1] = o[2] = 0;
-        return;
-      }
-      o[0] = q52l(lnA, 600.0);
-      o[1] = q(b, 56, 32.0);
-      o[2] = q52l(Ta, 1900.0);
-    };
-    int64_t o[3];
-    rate(d->A[j], d->b[j], d->Ea[j], o);
-    R->lnA = o[0]; R->beta = o[1]; R->Ta = o[2];
-    if (R->type == 2) {
-      const double* t = d->troe + 7 * j;
-      FxTroe* F = B.at<FxTroe>(L->o_troe) + R->troe;
-      rate(t[0], t[1], t[2], o);
-      F->lnA0 = o[0]; F->b0 = o[1]; F->Ta0 = o[2];
-      F->b0d = t[1]; F->Ta0K = t[2] / RC;
-      F->a = t[3]; F->iT3 = 1.0 / t[4]; F->iT1 = 1.0 / t[5]; F->T2 = t[6];
-      F->has_t2 = d->has_t2[j] ? 1.0 : 0.0;
-    }
-    int dnu = 0;
-    for (int i = 0; i < 3; ++i) {
-      if (d->reac[3 * j + i] >= 0) { R->re[R->nre++] = (uint8_t)d->reac[3 * j + i]; --dnu; }
-      if (d->prod[3 * j + i] >= 0) { R->pr[R->npr++] = (uint8_t)d->prod[3 * j + i]; ++dnu; }
-    }
-    R->dnu = (int8_t)dnu;
-    for (int k = 0; k < ns; ++k)
-      if (nu[j][k] != 0) { R->sp[R->nnet] = (uint8_t)k; R->nu[R->nnet++] = (int8_t)nu[j][k]; }
-  }
   // |Delta G / (RT ln 2)| of a reaction over [kTlo, kThi): on 512 log-spaced pieces, the value at
-  // the left end plus the change of every (monotone) term across the piece; above 2000: slow
-  for (int j = 0; j < nr; ++j) {
-    FxReac* R = B.at<FxReac>(L->o_reac) + j;
+  // the left end plus the change of every (monotone) term across the piece
+  auto worst_dG = [&](int j, int dnu) {
     double worst = 0.0;
     const double step = std::pow(fx::kThi / fx::kTlo, 1.0 / 512.0);
     double T = fx::kTlo;
     for (int i = 0; i < 512; ++i, T *= step) {
       const double T1 = T * step;
-      for (int r = (T1 < TMID ? 0 : (T >= TMID ? 1 : 0)); r <= (T1 < TMID ? 0 : 1); ++r) {
+      for (int r = T >= TMID ? 1 : 0; r <= (T1 < TMID ? 0 : 1); ++r) {
         const double* nasa = r == 0 ? d->nasa_lo : d->nasa_hi;
         double c[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
         for (int k = 0; k < ns; ++k)
@@ -236,7 +208,7 @@ std::vector<unsigned char> build_fx(const chem_mech_desc* d, const chem_mech_s* 
           for (int t = 0; t < 5; ++t, p *= x)
             o[t] = t == 0 ? c[0] * (1.0 - std::log(x)) - c[6] : -c[t] * p / (t * (t + 1));
           o[5] = c[5] / x;
-          o[6] = R->dnu * (std::log(x) - std::log(PATM / RU));
+          o[6] = dnu * (std::log(x) - std::log(PATM / RU));
         };
         double a0[7], a1[7], v = 0.0, w = 0.0;
         terms(T, a0);
@@ -245,7 +217,70 @@ std::vector<unsigned char> build_fx(const chem_mech_desc* d, const chem_mech_s* 
         worst = std::max(worst, std::fabs(v) + w);
       }
     }
-    if (!(worst / std::log(2.0) <= 2000.0)) R->slow = 1;
+    return worst / std::log(2.0);
+  };
+  auto in_formats = [&](double A, double b, double Ea) {
+    return A > 0.0 && std::fabs(std::log2(A)) <= 599.0 && std::fabs(b) <= 32.0 && std::fabs(Ea / RC) <= 160000.0;
+  };
+  auto low_fits = [&](int j) {                 // the low-pressure limit of a fall-off reaction
+    const double* t = d->troe + 7 * j;
+    return d->rtype[j] != 2 || in_formats(t[0], t[1], t[2]);
+  };
+  // log2 A, b and Ta in the formats; log2 A = 2000 (never in range) where one does not fit
+  auto rate = [&](double A, double b, double Ea, bool fits, int64_t* lnA_, uint64_t* beta, uint64_t* Ta_) {
+    fits = fits && in_formats(A, b, Ea);
+    *lnA_ = fits ? q52l(std::log((long double)A) / l2, 600.0) : (int64_t)2000 << 52;
+    *beta = fx::biased(fits ? q(b, 56, 32.0) : 0);
+    *Ta_ = fx::biased(fits ? q52l((long double)Ea / (long double)RC / l2 / 128.0L, 1900.0) : 0);
+  };
+  std::vector<int16_t> tb_of(nr, -1), troe_of(nr, -1);
+  for (int j = 0, tb = 0, tr = 0; j < nr; ++j) {
+    if (d->rtype[j] != 0) tb_of[j] = (int16_t)tb++;
+    if (d->rtype[j] == 2) troe_of[j] = (int16_t)tr++;
+  }
+  FxRate* R = B.at<FxRate>(L->o_rate);
+  for (int cls = 0; cls < 3; ++cls)
+    for (int j : order[cls]) {
+      int dnu = 0, nr_ = 0, np_ = 2;
+      for (int i = 0; i < 4; ++i) R->c[i] = (uint16_t)(ns * 256);
+      for (int i = 0; i < 3; ++i) {
+        if (d->reac[3 * j + i] >= 0) { R->c[nr_++] = (uint16_t)(d->reac[3 * j + i] * 256); --dnu; }
+        if (d->prod[3 * j + i] >= 0) { R->c[np_++] = (uint16_t)(d->prod[3 * j + i] * 256); ++dnu; }
+      }
+      R->dnu = (int16_t)dnu; R->id = (int16_t)j; R->tb = tb_of[j]; R->troe = troe_of[j];
+      rate(d->A[j], d->b[j], d->Ea[j], worst_dG(j, dnu) <= 2000.0 && low_fits(j), &R->lnA, &R->beta, &R->Ta);
+      R->b = d->b[j];
+      R->TaK = d->Ea[j] / RC;
+      int n = 0;
+      for (int pass = 0; pass < 2; ++pass)                      // net species first, then fillers
+        for (int k = 0; k < ns && n < 4; ++k)
+          if ((nu[j][k] != 0) == (pass == 0)) { R->w[n] = (uint16_t)(k * 256); R->nu[n++] = nu[j][k]; }
+      ++R;
+    }
+  FxReac* G = B.at<FxReac>(L->o_reac);
+  for (int j : order[3]) {
+    int dnu = 0;
+    for (int i = 0; i < 3; ++i) {
+      if (d->reac[3 * j + i] >= 0) { G->re[G->nre++] = (uint8_t)d->reac[3 * j + i]; --dnu; }
+      if (d->prod[3 * j + i] >= 0) { G->pr[G->npr++] = (uint8_t)d->prod[3 * j + i]; ++dnu; }
+    }
+    G->dnu = (int16_t)dnu; G->id = (int16_t)j; G->tb = tb_of[j]; G->troe = troe_of[j];
+    G->type = (uint8_t)d->rtype[j];
+    rate(d->A[j], d->b[j], d->Ea[j], worst_dG(j, dnu) <= 2000.0 && low_fits(j), &G->lnA, &G->beta, &G->Ta);
+    G->b = d->b[j];
+    G->TaK = d->Ea[j] / RC;
+    for (int k = 0; k < ns; ++k)
+      if (nu[j][k] != 0) { G->sp[G->nnet] = (uint8_t)k; G->nu[G->nnet++] = (int8_t)nu[j][k]; }
+    ++G;
+  }
+  for (int j = 0; j < nr; ++j) {
+    if (troe_of[j] < 0) continue;
+    const double* t = d->troe + 7 * j;
+    FxTroe* F = B.at<FxTroe>(L->o_troe) + troe_of[j];
+    rate(t[0], t[1], t[2], true, &F->lnA0, &F->b0, &F->Ta0);
+    F->b0d = t[1]; F->Ta0K = t[2] / RC;
+    F->a = t[3]; F->iT3 = 1.0 / t[4]; F->iT1 = 1.0 / t[5]; F->T2 = t[6];
+    F->has_t2 = d->has_t2[j] ? 1.0 : 0.0;
   }
   for (size_t i = 0; i < effv.size(); ++i) {
     B.at<double>(L->o_effv)[i] = effv[i];
