@@ -90,6 +90,11 @@ struct chem_mech_s {
   chem::JacProgram jac{};
   chem::FxLayout fx{};                    // fixed-point form (integrator_cell.cu), bytes = 0: none
   void* d_fx = nullptr;
+  chem::GxLayout gx{};                    // the group kernels' fixed-point form, bytes = 0: none
+  chem::GxJac gxj{};
+  void *d_gx = nullptr, *d_gxj = nullptr; // blob; Jacobian program, then log2 and reciprocal tables
+  const unsigned long long* d_lg = nullptr;
+  const unsigned int* d_rc = nullptr;
 };
 
 namespace chem {

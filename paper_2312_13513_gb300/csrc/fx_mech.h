@@ -50,7 +50,6 @@ struct FxSpecies {
   int64_t g[5], ga6, gl;      // g/RT/ln 2 = g(tau) + ga6 (128 / T) + gl log2 T
   int64_t h[5], ha6;          // h/RT
   int64_t c[5];               // cp/R
-  int64_t d3, d2;             // 4 c[4] (biased) and 3 c[3] of d(cp/R)/dtau
 };
 
 struct FxLayout {
@@ -64,6 +63,36 @@ struct FxLayout {
   int o_effv, o_eff;          // sparse (efficiency - 1); dense efficiencies [ntb][ns]
   int o_effidx, o_effoff;
   int64_t lpr0;               // log2(p_atm / R), Q11.52
+};
+
+// The same for the group kernels (integrator.cu): one lane per reaction, so the records are arrays;
+// species slots are indices, ns in an empty one.
+struct GxLayout {
+  int ns, nr, ntb, npieces, bytes;      // bytes = 0: no fixed-point form
+  int o_exp2, o_sp, o_W, o_invW, o_nu;
+  int o_lnA, o_beta, o_Ta;              // [nr] as FxRate
+  int o_reac, o_prod, o_rinfo;          // short4 [nr]: species; type, dnu, third-body set, Troe record
+  int o_troe, o_effv, o_effidx, o_effoff;
+  int o_wpk, o_pterm, o_poff;           // production lists, as MechLayout
+  int64_t lpr0;
+};
+
+// Jacobian-assembly program of the group kernels with the fixed-point form (global memory): entry
+// e covers row ent_row[e], column ent_col[e] and sums slot terms slot_off[e] .. slot_off[e + 1) and
+// partner terms part_off[e] .. part_off[e + 1).  A slot term is the derivative of one direction of reaction j with
+// respect to one of its species: slot_src = (2 j + side) << 4 | (nu + 8), times the concentrations
+// of the side's other species slot_oth = o1 | o2 << 16.  Collision partners: d(wdot_k)/dC_m =
+// sum_j nu_kj X_j eff_jm = R_k + sum_j nu_kj X_j (eff_jm - 1), with R_k = sum_j nu_kj X_j the same
+// for every column: only the sparse deviations are terms (part_tb = set, part_coef = nu (eff - 1)),
+// R_k (row_off, row_src = set << 4 | (nu + 8)) joins the chain rule.  For the 53-species mechanism
+// this leaves 4.4 k slot and 2.8 k partner terms of 13.1 k.
+struct GxJac {
+  int nent = 0;
+  const int *slot_off = nullptr, *part_off = nullptr;      // [nent + 1]
+  const int16_t *ent_row = nullptr, *ent_col = nullptr;    // [nent]
+  const int *slot_src = nullptr, *slot_oth = nullptr, *part_tb = nullptr;
+  const double* part_coef = nullptr;
+  const int *row_off = nullptr, *row_src = nullptr;        // [ns + 1], terms of R_k
 };
 
 constexpr int kFxR0 = 10, kFxR1 = 12;

@@ -32,6 +32,7 @@
 
 #include "chem_internal.h"
 #include "fastexp.cuh"
+#include "fx_rates.cuh"
 #include "queue.cuh"
 
 namespace chem {
@@ -91,11 +92,50 @@ __device__ __forceinline__ MechView bind_mech(const unsigned char* s, const Mech
   return m;
 }
 
+// the fixed-point form (GxLayout), with the FP64 form behind it for what the formats leave out
+struct GxView : fx::Ctx {
+  int ns, nr, N, npieces;
+  const FxSpecies* sp;
+  const double *W, *invW, *nu, *effv;
+  const fx::i64* lnA;
+  const fx::u64 *beta, *Ta;
+  const short4 *reac, *prod, *rinfo;
+  const FxTroe* troe;
+  const int16_t* effidx;
+  const int *effoff, *wpk, *pterm, *poff;
+  fx::i64 lpr0;
+};
+
+__device__ __forceinline__ GxView bind_gx(const unsigned char* s, const GxLayout& L) {
+  GxView m;
+  m.ns = L.ns; m.nr = L.nr; m.N = L.ns + 1; m.npieces = L.npieces;
+  m.e2 = (const fx::u64*)(s + L.o_exp2);
+  m.sp = (const FxSpecies*)(s + L.o_sp);
+  m.W = (const double*)(s + L.o_W);
+  m.invW = (const double*)(s + L.o_invW);
+  m.nu = (const double*)(s + L.o_nu);
+  m.effv = (const double*)(s + L.o_effv);
+  m.lnA = (const fx::i64*)(s + L.o_lnA);
+  m.beta = (const fx::u64*)(s + L.o_beta);
+  m.Ta = (const fx::u64*)(s + L.o_Ta);
+  m.reac = (const short4*)(s + L.o_reac);
+  m.prod = (const short4*)(s + L.o_prod);
+  m.rinfo = (const short4*)(s + L.o_rinfo);
+  m.troe = (const FxTroe*)(s + L.o_troe);
+  m.effidx = (const int16_t*)(s + L.o_effidx);
+  m.effoff = (const int*)(s + L.o_effoff);
+  m.wpk = (const int*)(s + L.o_wpk);
+  m.pterm = (const int*)(s + L.o_pterm);
+  m.poff = (const int*)(s + L.o_poff);
+  m.lpr0 = L.lpr0;
+  return m;
+}
+
 // Per-cell scalars that a multi-warp group evaluates on its first warp only and shares through
 // the workspace (slot indices into w.sc).
 enum : int {
   S_LNT, S_INVT, S_RHO, S_INVRHO, S_GSHIFT, S_EP1, S_IEP1, S_S, S_CP, S_DCP, S_Q, S_IRCP,
-  S_RS, S_QOR2R, S_RHS, S_CPS, S_J00, S_IG, S_INVH, S_EN, S_FAC, S_NSC
+  S_RS, S_QOR2R, S_RHS, S_CPS, S_J00, S_IG, S_INVH, S_EN, S_FAC, S_HR, S_L, S_IT, S_TAU, S_NSC
 };
 
 // per-group workspace layout (doubles unless noted); offsets in doubles.  The Jacobian is
@@ -105,11 +145,13 @@ struct WsLayout {
   int LD;                  // leading dimension of the N x N matrix
   int y, ynew, ys, fs, f0, u, M, invd, tmp;
   int C, hRT, gRT, cpR, wdot, dwdT, rk, Hm;
-  int q, dqdT, dq, wpart, dwpart, red, sc, stage, ctl, perm;
+  int q, dqdT, dq, row, wpart, dwpart, red, sc, stage, ctl, perm;
   int total;               // doubles
 };
 
-inline WsLayout make_ws(int ns, int nr, int npieces, int G) {
+// fx: the layout of the fixed-point form (per reaction the two slot derivatives, per third-body set
+// the collision-partner factor; a row constant per species)
+inline WsLayout make_ws(int ns, int nr, int npieces, int G, bool fx, int ntb) {
   WsLayout w{};
   const int N = ns + 1;
   // a group wider than a warp reads matrix columns across rows: an odd leading dimension keeps
@@ -121,7 +163,7 @@ inline WsLayout make_ws(int ns, int nr, int npieces, int G) {
   // solve's scratch and the new state share its storage
   w.y = take(N); w.f0 = take(N); w.ys = take(N); w.ynew = w.ys; w.tmp = w.ys; w.fs = take(N);
   w.u = take(6 * N); w.M = take(N * w.LD); w.invd = take(N);
-  w.C = take(ns + 1); w.hRT = take(ns); w.gRT = take(ns); w.cpR = take(ns);
+  w.C = take(ns + 1); w.hRT = take(ns); w.gRT = take(ns + 1); w.cpR = take(ns);
   w.wdot = take(ns); w.dwdT = take(ns); w.rk = take(ns); w.Hm = take(ns);
   // dq/dT per reaction is only needed inside a Jacobian evaluation, before the assembly writes the
   // matrix buffer (whose previous content, the last LU, is dead by then): it borrows that buffer
@@ -130,7 +172,9 @@ inline WsLayout make_ws(int ns, int nr, int npieces, int G) {
   // evaluation, at the start of an attempt, when the stage buffers ys, fs and u (contiguous
   // above) are dead: small mechanisms keep them there
   const int stage_span = w.M - w.ys;
-  w.dq = 3 * nr <= stage_span ? w.ys : take(3 * nr);
+  const int ndq = fx ? 2 * nr + ntb : 3 * nr;
+  w.dq = ndq <= stage_span ? w.ys : take(ndq);
+  w.row = take(fx ? ns : 0);
   // partial production sums of the balanced pieces (groups wider than a warp)
   w.wpart = take(G > 32 ? npieces : 0); w.dwpart = take(G > 32 ? npieces : 0);
   // cross-warp reductions and shared scalars exist only for groups wider than a warp
@@ -146,7 +190,7 @@ inline WsLayout make_ws(int ns, int nr, int npieces, int G) {
 struct WsPtr {
   double *y, *ynew, *ys, *fs, *f0, *u, *M, *invd, *tmp;
   double *C, *hRT, *gRT, *cpR, *wdot, *dwdT, *rk, *Hm;
-  double *q, *dqdT, *dq, *wpart, *dwpart, *red, *sc, *stage;
+  double *q, *dqdT, *dq, *row, *wpart, *dwpart, *red, *sc, *stage;
   unsigned long long* ctl;
   int* perm;
 };
@@ -158,6 +202,7 @@ __device__ __forceinline__ WsPtr bind_ws(double* b, const WsLayout& w) {
   p.C = b + w.C; p.hRT = b + w.hRT; p.gRT = b + w.gRT; p.cpR = b + w.cpR;
   p.wdot = b + w.wdot; p.dwdT = b + w.dwdT; p.rk = b + w.rk; p.Hm = b + w.Hm;
   p.q = b + w.q; p.dqdT = b + w.dqdT; p.dq = b + w.dq; p.red = b + w.red; p.sc = b + w.sc;
+  p.row = b + w.row;
   p.wpart = b + w.wpart; p.dwpart = b + w.dwpart;
   p.stage = b + w.stage;
   p.ctl = (unsigned long long*)(b + w.ctl);
@@ -627,6 +672,299 @@ __device__ __forceinline__ void eval_fj(const Grp<G>& g, const MechView& m, cons
   g.sync();
 }
 
+// The same right-hand side and (negated) Jacobian from the mechanism's fixed-point form, for groups
+// of several warps.  The FP64 pipe bounds the group kernels (65 % busy with 289 k lane slots per
+// attempt of the 53-species mechanism); here the exponentials, logarithms and NASA-7 polynomials
+// run on the integer pipe (fixed.cuh), kr = 2^(log2 kf + Delta G) replaces the products of 1/Kc
+// factors, and the Jacobian's collision-partner part is a row constant plus sparse deviations
+// (GxJac).  FP64 left per reaction and evaluation: 5 instructions instead of about 24.
+template <int G>
+__device__ __forceinline__ void eval_fx(const Grp<G>& g, const GxView& m, const WsPtr& w, const GxJac& jp, int LD,
+                                        const double* y, double p, double* f, double* Jneg) {
+  static_assert(G > 32, "groups of several warps");
+  const bool lead = is_lead(g);
+  const bool jac = Jneg != nullptr;
+  const int ns = m.ns, nr = m.nr;
+  const double T = y[0];
+  if (lead) {
+    const fx::Temp t = fx::temp_of(T, m, false);
+    if (g.tid == 0) {
+      w.sc[S_L] = __longlong_as_double((long long)t.L);
+      w.sc[S_IT] = __longlong_as_double((long long)t.iT);
+      w.sc[S_TAU] = __longlong_as_double((long long)t.tau);
+    }
+  }
+  g.sync();
+  fx::Temp t;
+  t.T = T;
+  t.fast = (unsigned)__double2hiint(T) - 0x40600000u < 0x40b00000u - 0x40600000u;
+  t.rg = (__double2hiint(T) < 0x408f4000) ? 0 : 1;          // T < 1000 (for T > 0)
+  t.L = (fx::u64)__double_as_longlong(w.sc[S_L]);
+  t.iT = (fx::u64)__double_as_longlong(w.sc[S_IT]);
+  t.tau = (fx::u64)__double_as_longlong(w.sc[S_TAU]);
+  t.L2 = (fx::i64)(t.L >> 1); t.iT2 = (fx::i64)(t.iT >> 1); t.tau2 = (fx::i64)(t.tau >> 1);
+  t.invT = 0.0;
+  if (jac) t.invT = t.fast ? fx::to_double(t.iT2, 63 + fx::kTloExp) : 1.0 / T;
+
+  // species thermo (A2): g/RT (Q11.52 / ln 2 in fast cells), h/RT, cp/R
+  double acc[3] = {0.0, 0.0, 0.0};
+  const fx::u64 B = 0x8000000000000000ull;
+  for (int k = g.tid; k < ns; k += G) {
+    const double yw = y[1 + k] * m.invW[k];
+    double cp, d = 0.0;
+    if (t.fast) {
+      const FxSpecies& s = m.sp[t.rg * ns + k];
+      fx::u64 gg = (fx::u64)s.g[4], h = (fx::u64)s.h[4], c = (fx::u64)s.c[4];
+#pragma unroll
+      for (int i = 3; i >= 0; --i) {
+        const fx::u64 b = i ? B : 0ull;
+        gg = (fx::umulhi3(gg, t.tau) + (fx::u64)(s.g[i] - t.tau2)) ^ b;
+        h = (fx::umulhi3(h, t.tau) + (fx::u64)(s.h[i] - t.tau2)) ^ b;
+        c = (fx::umulhi3(c, t.tau) + (fx::u64)(s.c[i] - t.tau2)) ^ b;
+      }
+      gg += fx::umulhi3((fx::u64)s.ga6, t.iT) + fx::umulhi3((fx::u64)s.gl, t.L) - (fx::u64)(t.iT2 + t.L2);
+      h += fx::umulhi3((fx::u64)s.ha6, t.iT) - (fx::u64)t.iT2;
+      w.gRT[k] = __longlong_as_double((long long)gg);
+      w.hRT[k] = fx::to_double((fx::i64)h, 52);
+      cp = fx::to_double((fx::i64)c, 52);
+      if (jac) {
+        fx::u64 dc = fx::biased((fx::i64)(((fx::u64)s.c[4] ^ B) << 2));
+        dc = (fx::umulhi3(dc, t.tau) + (fx::u64)(s.c[3] * 3 - t.tau2)) ^ B;
+        dc = (fx::umulhi3(dc, t.tau) + (fx::u64)(s.c[2] * 2 - t.tau2)) ^ B;
+        dc = fx::umulhi3(dc, t.tau) + (fx::u64)(s.c[1] - t.tau2);
+        d = fx::to_double((fx::i64)dc, 52 + (t.rg == 0 ? kFxR0 : kFxR1));
+      }
+    } else {
+      const int rg = T < TMID ? 0 : 1;
+      const double lnT = log(T), invT = 1.0 / T;
+      const double* hc = (const double*)(m.blob + m.lay->o_hc) + (rg * ns + k) * 6;
+      const double* sc = (const double*)(m.blob + m.lay->o_sc) + (rg * ns + k) * 6;
+      const double* cc = (const double*)(m.blob + m.lay->o_cpc) + (rg * ns + k) * 5;
+      const double h = hc[0] + T * (hc[1] + T * (hc[2] + T * (hc[3] + T * hc[4]))) + hc[5] * invT;
+      const double s = sc[0] * lnT + T * (sc[1] + T * (sc[2] + T * (sc[3] + T * sc[4]))) + sc[5];
+      cp = cc[0] + T * (cc[1] + T * (cc[2] + T * (cc[3] + T * cc[4])));
+      d = cc[1] + T * (2.0 * cc[2] + T * (3.0 * cc[3] + T * (4.0 * cc[4])));
+      w.gRT[k] = h - s;
+      w.hRT[k] = h;
+    }
+    w.C[k] = yw;
+    acc[0] += yw;
+    acc[1] = fma(yw, cp, acc[1]);
+    if (jac) {
+      w.cpR[k] = cp;
+      acc[2] = fma(yw, d, acc[2]);
+    }
+  }
+  if (jac) {
+    gsum_lead<G, 3>(g, acc, w.red, ns);
+  } else {
+    double a2[2] = {acc[0], acc[1]};
+    gsum_lead<G, 2>(g, a2, w.red, ns);
+    acc[0] = a2[0]; acc[1] = a2[1];
+  }
+  // mixture scalars: S = sum Y/W, cp/R, d(cp/R)/dT, density
+  double S = 0.0, cp = 0.0, dcp = 0.0, rho = 0.0, invrho = 0.0;
+  if (lead) {
+    S = acc[0]; cp = acc[1]; dcp = acc[2];
+    rho = p * fx::rcp(RU * T * S);
+    invrho = fx::rcp(rho);
+    if (g.tid == 0) {
+      w.sc[S_S] = S; w.sc[S_CP] = cp; w.sc[S_DCP] = dcp; w.sc[S_RHO] = rho; w.sc[S_INVRHO] = invrho;
+      w.C[ns] = 1.0;                                        // the empty slot
+      w.gRT[ns] = 0.0;
+    }
+  }
+  g.sync();
+  S = w.sc[S_S]; cp = w.sc[S_CP]; dcp = w.sc[S_DCP]; rho = w.sc[S_RHO]; invrho = w.sc[S_INVRHO];
+  for (int k = g.tid; k < ns; k += G) w.C[k] = rho * w.C[k];
+  g.sync();
+
+  // rates of progress (A3)
+  const double Ctot = rho * S;
+  const fx::i64 D = (fx::i64)((t.L + 128ull) >> 8) - m.lpr0;
+  const fx::i64 shift = t.iT2 - t.L2;
+  for (int j = g.tid; j < nr; j += G) {
+    const short4 ri = m.rinfo[j], re = m.reac[j], pr = m.prod[j];
+    const fx::i64 Xf = m.lnA[j] + (fx::i64)(fx::umulhi3(m.beta[j], t.L) - fx::umulhi3(m.Ta[j], t.iT)) + shift;
+    fx::i64 Xr = Xf + (__double_as_longlong(w.gRT[pr.x]) + __double_as_longlong(w.gRT[pr.y])) -
+                 (__double_as_longlong(w.gRT[re.x]) + __double_as_longlong(w.gRT[re.y])) + (fx::i64)ri.y * D;
+    double Pf = w.C[re.x] * w.C[re.y], Pr = w.C[pr.x] * w.C[pr.y];
+    if (re.z != ns) { Pf *= w.C[re.z]; Xr -= __double_as_longlong(w.gRT[re.z]); }
+    if (pr.z != ns) { Pr *= w.C[pr.z]; Xr += __double_as_longlong(w.gRT[pr.z]); }
+    double kf = fx::exp2_q52(Xf, m.e2), kr = fx::exp2_q52(Xr, m.e2);
+    double Mc = 1.0;
+    if (ri.x != 0) {
+      Mc = Ctot;
+      for (int e = m.effoff[ri.z]; e < m.effoff[ri.z + 1]; ++e) Mc = fma(m.effv[e], w.C[m.effidx[e]], Mc);
+    }
+    double dlnkf = 0.0, dMr = 0.0, dkfdM = 0.0, invKc = 0.0;
+    if (jac) {
+      const double b = fx::to_double((fx::i64)(m.beta[j] ^ B), 56);
+      const double TaT = fx::to_double((fx::i64)(m.Ta[j] ^ B), 52) * (128.0 * fx::kLn2) * t.invT;
+      dlnkf = (b + TaT) * t.invT;
+    }
+    bool fastk = t.fast && fx::exp2_in_range(Xf) && fx::exp2_in_range(Xr);
+    if (ri.x == 2 && fastk) {
+      const FxTroe& F = m.troe[ri.w];
+      const fx::i64 Xk = F.lnA0 + (fx::i64)(fx::umulhi3(F.b0, t.L) - fx::umulhi3(F.Ta0, t.iT)) + shift - Xf;
+      double fac = 1.0, dl = 0.0;
+      fastk = jac ? fx::troe_fast<true>(m, F, t, Xk, Mc, dlnkf, &fac, &dl, &dMr)
+                  : fx::troe_fast<false>(m, F, t, Xk, Mc, dlnkf, &fac, &dl, &dMr);
+      kf *= fac;
+      kr *= fac;
+      if (jac && fastk) dlnkf = dl;
+    }
+    if (!fastk) {
+      if (jac) {                                            // the derivative from the FP64 constants
+        const double invT = 1.0 / T;
+        dlnkf = ((const double*)(m.blob + m.lay->o_beta))[j] * invT +
+                ((const double*)(m.blob + m.lay->o_Ta))[j] * invT * invT;
+      }
+      fx::slow_rate(m, w.gRT, 1, j, ri.x == 2 ? m.troe + ri.w : nullptr, T, t.fast, Mc, &kf, &kr, &dlnkf, &dkfdM,
+                    &invKc);
+    }
+    if (!jac) {
+      double q = fma(kf, Pf, -(kr * Pr));
+      if (ri.x == 1) q *= Mc;
+      w.q[j] = q;
+      continue;
+    }
+    const double fwd = kf * Pf, rev = kr * Pr, net = fwd - rev;
+    const double mult = ri.x == 1 ? Mc : 1.0;
+    double dH = (w.hRT[pr.x] - w.hRT[re.x]) - (double)ri.y;
+    if (pr.y != ns) dH += w.hRT[pr.y];
+    if (pr.z != ns) dH += w.hRT[pr.z];
+    if (re.y != ns) dH -= w.hRT[re.y];
+    if (re.z != ns) dH -= w.hRT[re.z];
+    w.q[j] = mult * net;
+    w.dqdT[j] = mult * fma(net, dlnkf, rev * (dH * t.invT));
+    w.dq[2 * j] = mult * kf;
+    w.dq[2 * j + 1] = -mult * kr;
+    if (ri.x != 0) w.dq[2 * nr + ri.z] = ri.x == 1 ? net : (fastk ? dMr * net : dkfdM * (Pf - Pr * invKc));
+  }
+  g.sync();
+
+  // production rates and right-hand side (A4): balanced pieces, then each species' pieces
+  for (int pc = g.tid; pc < m.npieces; pc += G) {
+    double a = 0.0, b = 0.0;
+    for (int e = m.pterm[pc]; e < m.pterm[pc + 1]; ++e) {
+      const int pk = m.wpk[e];
+      const double nu = m.nu[pk & 15];
+      const int j = pk >> 4;
+      a = fma(nu, w.q[j], a);
+      if (jac) b = fma(nu, w.dqdT[j], b);
+    }
+    w.wpart[pc] = a;
+    if (jac) w.dwpart[pc] = b;
+  }
+  g.sync();
+  double r3[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int k = g.tid; k < ns; k += G) {
+    double wk = 0.0, dwk = 0.0;
+    for (int pc = m.poff[k]; pc < m.poff[k + 1]; ++pc) {
+      wk += w.wpart[pc];
+      if (jac) dwk += w.dwpart[pc];
+    }
+    const double hk = w.hRT[k];
+    r3[0] = fma(hk, wk, r3[0]);
+    f[1 + k] = m.W[k] * (wk * invrho);
+    if (jac) {
+      w.wdot[k] = wk;
+      w.dwdT[k] = dwk;
+      r3[1] = fma(w.cpR[k], wk, r3[1]);
+      r3[2] = fma(hk, dwk, r3[2]);
+      // R_k, the column-independent part of the collision partners' derivatives
+      double R = 0.0;
+      const int t1 = __ldg(jp.row_off + k + 1);
+      for (int e = __ldg(jp.row_off + k); e < t1; ++e) {
+        const int src = __ldg(jp.row_src + e);
+        R = fma(m.nu[src & 15], w.dq[2 * nr + (src >> 4)], R);
+      }
+      w.row[k] = R;
+      r3[3] = fma(hk, R, r3[3]);
+    }
+  }
+  if (!jac) {
+    double q1[1] = {r3[0]};
+    gsum_lead<G, 1>(g, q1, w.red, ns);
+    if (lead) {
+      const double f0 = -(T * q1[0]) * fx::rcp(rho * cp);
+      if (g.tid == 0) f[0] = f0;
+    }
+    g.sync();
+    return;
+  }
+  gsum_lead<G, 4>(g, r3, w.red, ns);
+  const double Q = T * r3[0];                               // in units of R, as cp and h below
+  double ircp = 0.0;
+  if (lead) ircp = fx::rcp(rho * cp);
+  if (g.tid == 0) f[0] = -Q * ircp;
+
+  // analytic Jacobian (A5): d(wdot)/dC by the assembly program ...
+  double* Jm = Jneg;
+  const unsigned mns = div_magic((unsigned)ns);
+  for (int e = g.tid; e < ns * ns; e += G) {
+    const int k = div_by(e, mns);
+    Jm[(1 + k) * LD + 1 + (e - k * ns)] = 0.0;
+  }
+  g.sync();
+  for (int e = g.tid; e < jp.nent; e += G) {
+    double s = 0.0;
+    const int t1 = __ldg(jp.slot_off + e + 1);
+    for (int i = __ldg(jp.slot_off + e); i < t1; ++i) {
+      const int src = __ldg(jp.slot_src + i), oth = __ldg(jp.slot_oth + i);
+      double d = w.dq[src >> 4];
+      if ((oth & 0xffff) != ns) d *= w.C[oth & 0xffff];
+      if ((oth >> 16) != ns) d *= w.C[oth >> 16];
+      s = fma(m.nu[src & 15], d, s);
+    }
+    const int p1 = __ldg(jp.part_off + e + 1);
+    for (int i = __ldg(jp.part_off + e); i < p1; ++i)
+      s = fma(__ldg(jp.part_coef + i), w.dq[2 * nr + __ldg(jp.part_tb + i)], s);
+    Jm[(1 + __ldg(jp.ent_row + e)) * LD + 1 + __ldg(jp.ent_col + e)] = s;
+  }
+  if (g.tid == 0) w.sc[S_IRCP] = ircp;
+  g.sync();
+  ircp = w.sc[S_IRCP];
+  // ... then the chain rule through C(T, Y) and rho(T, Y) (eval_fj), with R_k added on the way
+  const double iS = fx::rcp(S);
+  const double rS = invrho * iS;
+  double rh[1] = {0.0};
+  for (int k = g.tid; k < ns; k += G) {
+    double s = w.row[k] * Ctot;
+    for (int mm = 0; mm < ns; ++mm) s = fma(Jm[(1 + k) * LD + 1 + mm], w.C[mm], s);
+    rh[0] = fma(w.hRT[k], s, rh[0]);
+    const double dk = s - w.wdot[k];
+    w.rk[k] = dk * rS - w.row[k];
+    Jm[(1 + k) * LD] = -(m.W[k] * invrho * (w.dwdT[k] - dk * t.invT));
+  }
+  for (int mm = g.tid; mm < ns; mm += G) {
+    double s = 0.0;
+    for (int k = 0; k < ns; ++k) s = fma(w.hRT[k], Jm[(1 + k) * LD + 1 + mm], s);
+    w.Hm[mm] = s;
+  }
+  gsum_lead<G, 1>(g, rh, w.red, ns);
+  if (lead) {
+    const double Rh = T * rh[0], Qr = Q * ircp;
+    if (g.tid == 0) {
+      Jm[0] = (r3[1] + T * r3[2] - rh[0]) * ircp + Qr * (cp * t.invT - dcp) * (rho * ircp);
+      w.sc[S_RHS] = Rh * iS; w.sc[S_CPS] = cp * iS; w.sc[S_QOR2R] = Qr * rho; w.sc[S_HR] = r3[3];
+    }
+  }
+  g.sync();
+  const double RhS = w.sc[S_RHS], cpS = w.sc[S_CPS], Qrr = w.sc[S_QOR2R], HR = w.sc[S_HR];
+  for (int e = g.tid; e < ns * ns; e += G) {
+    const int k = div_by(e, mns), mm = e - k * ns;
+    double* Jkm = Jm + (1 + k) * LD + 1 + mm;
+    *Jkm = m.W[k] * m.invW[mm] * (w.rk[k] - *Jkm);
+  }
+  for (int mm = g.tid; mm < ns; mm += G) {
+    const double Hm = T * (w.Hm[mm] + HR);
+    Jm[1 + mm] = m.invW[mm] * ircp * ((rho * Hm - RhS) - Qrr * (w.cpR[mm] - cpS));
+  }
+  g.sync();
+}
+
 // ---------------------------------------------------------------------------------------
 // dense LU with partial pivoting (A6) and triangular solves
 // ---------------------------------------------------------------------------------------
@@ -660,7 +998,7 @@ __device__ bool lu_factor(const Grp<G>& g, double* M, int N, int LD, int* perm, 
     if (best == 0ull) return false;
     if (is_lead(g)) {
       const int pk = perm[bi], pb = perm[k];
-      const double ip = 1.0 / M[pk * LD + k];
+      const double ip = fx::rcp(M[pk * LD + k]);
       for (int i = k + 1 + g.tid; i < N; i += W) {
         const int ph = (i == bi) ? pb : perm[i];
         M[ph * LD + k] *= ip;
@@ -726,7 +1064,7 @@ __device__ bool lu_factor_panel(const Grp<G>& g, double* M, int N, int LD, int* 
     warp_argmax<G>(g, best, bi);
     for (int i = l; i < N; i += 32) pbuf[i] = i == 0 ? bi : (i == bi ? 0 : i);
     if (best != 0ull) {
-      const double ip = 1.0 / M[bi * LD];
+      const double ip = fx::rcp(M[bi * LD]);
       for (int i = 1 + l; i < N; i += 32) {
         const int ph = i == bi ? 0 : i;
         M[ph * LD] *= ip;
@@ -765,7 +1103,7 @@ __device__ bool lu_factor_panel(const Grp<G>& g, double* M, int N, int LD, int* 
       if (best != 0ull) {
         const int src = bi - (k + 1);
         const double piv = __shfl_sync(F, src < 32 ? v0 : v1, src & 31);
-        const double ip = 1.0 / piv;
+        const double ip = fx::rcp(piv);
         if (ph0 >= 0) M[ph0 * LD + k + 1] = ph0 == pnew ? v0 : v0 * ip;
         if (ph1 >= 0) M[ph1 * LD + k + 1] = ph1 == pnew ? v1 : v1 * ip;
         if (l == 0) { invd[k + 1] = ip; perm[k + 1] = pnew; }
@@ -916,11 +1254,50 @@ __device__ void lu_solve(const Grp<G>& g, const double* M, int N, int LD, const 
 // ---------------------------------------------------------------------------------------
 // kernels
 // ---------------------------------------------------------------------------------------
-struct AdvanceParams : QueueParams {
+// mechanism arguments of the group kernels: the FP64 form, and the fixed-point form where there is one
+struct MechArgs {
   MechLayout lay;
+  GxLayout gx;
   WsLayout ws;
   JacArgs jp;
-  const unsigned char* blob;
+  GxJac gj;
+  const unsigned char *blob, *gxblob;
+  const fx::u64* lg;
+  const uint32_t* rc;
+};
+
+struct AdvanceParams : QueueParams, MechArgs {};
+
+// the view a kernel instance works with (staged by stage_mech), and its right-hand side
+template <bool FX>
+struct Form;
+template <>
+struct Form<false> {
+  using View = MechView;
+  static __device__ __forceinline__ int bytes(const MechArgs& A) { return A.lay.bytes; }
+  static __device__ __forceinline__ const unsigned char* src(const MechArgs& A) { return A.blob; }
+  static __device__ __forceinline__ View bind(const unsigned char* s, const MechArgs& A) { return bind_mech(s, A.lay); }
+  template <int G>
+  static __device__ __forceinline__ void eval(const Grp<G>& g, const View& m, const WsPtr& w, const MechArgs& A,
+                                              const double* y, double p, double* f, double* Jneg) {
+    eval_fj<G>(g, m, w, A.jp, A.ws.LD, y, p, f, Jneg);
+  }
+};
+template <>
+struct Form<true> {
+  using View = GxView;
+  static __device__ __forceinline__ int bytes(const MechArgs& A) { return A.gx.bytes; }
+  static __device__ __forceinline__ const unsigned char* src(const MechArgs& A) { return A.gxblob; }
+  static __device__ __forceinline__ View bind(const unsigned char* s, const MechArgs& A) {
+    View m = bind_gx(s, A.gx);
+    m.lg = A.lg; m.rc = A.rc; m.blob = A.blob; m.lay = &A.lay;
+    return m;
+  }
+  template <int G>
+  static __device__ __forceinline__ void eval(const Grp<G>& g, const View& m, const WsPtr& w, const MechArgs& A,
+                                              const double* y, double p, double* f, double* Jneg) {
+    eval_fx<G>(g, m, w, A.gj, A.ws.LD, y, p, f, Jneg);
+  }
 };
 
 __device__ __forceinline__ void stage_mech(const unsigned char* src, unsigned char* dst, int bytes) {
@@ -933,8 +1310,8 @@ __device__ __forceinline__ void stage_mech(const unsigned char* src, unsigned ch
 // exactly singular iteration matrix; otherwise *en receives the error norm and *fac the step-size
 // factor 0.9 en^(-1/4) (clamped below at 0.2; 0.2 for a non-finite norm), evaluated once per
 // group.
-template <int G>
-__device__ bool rodas4_attempt(const Grp<G>& g, const MechView& m, const WsPtr& w,
+template <int G, bool FX>
+__device__ bool rodas4_attempt(const Grp<G>& g, const typename Form<FX>::View& m, const WsPtr& w,
                                const AdvanceParams& P, double p, double h, double rtol, double atol,
                                double* en, double* fac) {
   constexpr bool kMulti = G > 32;
@@ -942,7 +1319,7 @@ __device__ bool rodas4_attempt(const Grp<G>& g, const MechView& m, const WsPtr& 
   double ig = 0.0, invh = 0.0;
   if (is_lead(g)) { ig = 1.0 / (kGamma * h); invh = 1.0 / h; }
   if (kMulti && g.tid == 0) { w.sc[S_IG] = ig; w.sc[S_INVH] = invh; }
-  eval_fj<G>(g, m, w, P.jp, LD, w.y, p, w.f0, w.M);      // M = -J; synchronises
+  Form<FX>::template eval<G>(g, m, w, P, w.y, p, w.f0, w.M);      // M = -J; synchronises
   if (kMulti) { ig = w.sc[S_IG]; invh = w.sc[S_INVH]; }
   for (int i = g.tid; i < N; i += G) w.M[i * LD + i] += ig;   // M = I / (gamma h) - J
   g.sync();
@@ -963,7 +1340,7 @@ __device__ bool rodas4_attempt(const Grp<G>& g, const MechView& m, const WsPtr& 
         w.ys[i] = v;
       }
       g.sync();
-      eval_fj<G>(g, m, w, P.jp, LD, w.ys, p, w.fs, nullptr);
+      Form<FX>::template eval<G>(g, m, w, P, w.ys, p, w.fs, nullptr);
       src = w.fs;
     }
     double* us = w.u + s * N;
@@ -1018,8 +1395,8 @@ struct ChunkPos {
 
 // Move to the next cell: store a finished chunk, claim and load the next one when needed.
 // Loads the cell's state into w.y and returns its pressure; false when the queue is empty.
-template <int G>
-__device__ bool next_cell(const Grp<G>& g, const MechView& m, const WsPtr& w,
+template <int G, class View>
+__device__ bool next_cell(const Grp<G>& g, const View& m, const WsPtr& w,
                           const AdvanceParams& P, ChunkPos& q, double* p) {
   constexpr int CHUNK = chunk_cells(G);
   const int N = m.N;
@@ -1091,16 +1468,16 @@ __device__ bool next_cell(const Grp<G>& g, const MechView& m, const WsPtr& w,
 // cell changes happen between iterations.  For sub-warp groups every group of a warp executes
 // the attempt body each iteration (an idle group works on a dummy state whose results are
 // discarded), so the warp's FP64 instructions stay converged across its groups.
-template <int G>
+template <int G, bool FX>
 __global__ void __launch_bounds__(max_threads(G), 1) advance_kernel(const __grid_constant__ AdvanceParams P) {
   extern __shared__ __align__(16) unsigned char smem[];
   if (blockDim.x % G != 0 || blockDim.x < G) return;   // a block of whole groups only
-  stage_mech(P.blob, smem, P.lay.bytes);
+  stage_mech(Form<FX>::src(P), smem, Form<FX>::bytes(P));
   __syncthreads();
-  const MechView m = bind_mech(smem, P.lay);
+  const typename Form<FX>::View m = Form<FX>::bind(smem, P);
   Grp<G> g;
   g.init();
-  double* wbase = (double*)(smem + P.lay.bytes) + (size_t)g.gid * P.ws.total;
+  double* wbase = (double*)(smem + Form<FX>::bytes(P)) + (size_t)g.gid * P.ws.total;
   const WsPtr w = bind_ws(wbase, P.ws);
   const int N = m.N;
   // benign dummy state for groups without a cell
@@ -1166,7 +1543,7 @@ __global__ void __launch_bounds__(max_threads(G), 1) advance_kernel(const __grid
     bool finished = false;
     if (run || G < 32) {
       double en = 0.0, fac = 0.2;
-      const bool ok = rodas4_attempt<G>(g, m, w, P, p, run ? h : dt, rtol, atol, &en, &fac);
+      const bool ok = rodas4_attempt<G, FX>(g, m, w, P, p, run ? h : dt, rtol, atol, &en, &fac);
       if (run) {
         if (!ok) {
           stop = true; status = CHEM_CELL_SINGULAR_LU;
@@ -1208,11 +1585,7 @@ __global__ void __launch_bounds__(max_threads(G), 1) advance_kernel(const __grid
   }
 }
 
-struct EvalParams {
-  MechLayout lay;
-  WsLayout ws;
-  JacArgs jp;
-  const unsigned char* blob;
+struct EvalParams : MechArgs {
   const double* T;
   const double* p;
   const double* Y;
@@ -1221,23 +1594,23 @@ struct EvalParams {
   double* J;
 };
 
-template <int G>
-__global__ void __launch_bounds__(max_threads(G)) eval_kernel(const EvalParams P) {
+template <int G, bool FX>
+__global__ void __launch_bounds__(max_threads(G)) eval_kernel(const __grid_constant__ EvalParams P) {
   extern __shared__ __align__(16) unsigned char smem[];
   if (blockDim.x % G != 0 || blockDim.x < G) return;   // a block of whole groups only
-  stage_mech(P.blob, smem, P.lay.bytes);
+  stage_mech(Form<FX>::src(P), smem, Form<FX>::bytes(P));
   __syncthreads();
-  const MechView m = bind_mech(smem, P.lay);
+  const typename Form<FX>::View m = Form<FX>::bind(smem, P);
   Grp<G> g;
   g.init();
   const int gpb = blockDim.x / G;
-  double* wbase = (double*)(smem + P.lay.bytes) + (size_t)g.gid * P.ws.total;
+  double* wbase = (double*)(smem + Form<FX>::bytes(P)) + (size_t)g.gid * P.ws.total;
   const WsPtr w = bind_ws(wbase, P.ws);
   const int N = m.N, LD = P.ws.LD;
   for (int64_t c = (int64_t)blockIdx.x * gpb + g.gid; c < P.ncells; c += (int64_t)gridDim.x * gpb) {
     for (int i = g.tid; i < N; i += G) w.y[i] = i == 0 ? P.T[c] : P.Y[(int64_t)(i - 1) * P.ld + c];
     g.sync();
-    eval_fj<G>(g, m, w, P.jp, LD, w.y, P.p[c], w.f0, P.J ? w.M : nullptr);
+    Form<FX>::template eval<G>(g, m, w, P, w.y, P.p[c], w.f0, P.J ? w.M : nullptr);
     for (int i = g.tid; i < N; i += G) P.f[(int64_t)i * P.ld + c] = w.f0[i];
     if (P.J)     // the kernel assembles -J (exact negation back)
       for (int e = g.tid; e < N * N; e += G)
@@ -1254,6 +1627,7 @@ namespace {
 struct LaunchShape {
   const chem_mech_s* m;
   int G, groups, threads;    // G = 1: one thread per cell (integrator_cell.cu)
+  bool fx;                   // the fixed-point form
   size_t smem;
   WsLayout ws;
 };
@@ -1272,13 +1646,16 @@ int pick_shape(const chem_mech_s* m, const chem_options* opt, LaunchShape* s) {
     return CHEM_EINVAL;
   }
   s->G = G;
-  s->ws = make_ws(m->ns, m->nr, m->lay.npieces, G);
+  // the fixed-point form has an instance for 128-thread groups, the large mechanisms' default; the
+  // other group sizes are a caller's option and keep the FP64 form
+  s->fx = G == 128 && m->gx.bytes > 0;
+  s->ws = make_ws(m->ns, m->nr, m->lay.npieces, G, s->fx, s->fx ? m->gx.ntb : 0);
   int dev = 0;
   CHEM_CUDA_TRY(cudaGetDevice(&dev));
   int smem_max = 0;
   CHEM_CUDA_TRY(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   const size_t per_group = (size_t)s->ws.total * 8;
-  const size_t fixed = (size_t)m->lay.bytes;
+  const size_t fixed = (size_t)(s->fx ? m->gx.bytes : m->lay.bytes);
   const int unit = G < 32 ? 32 / G : 1;          // groups per warp: whole warps only
   int groups = (opt && opt->groups_per_cta) ? opt->groups_per_cta : max_threads(G) / G;
   groups = std::min(groups, max_threads(G) / G);
@@ -1296,15 +1673,15 @@ int pick_shape(const chem_mech_s* m, const chem_options* opt, LaunchShape* s) {
   return CHEM_OK;
 }
 
-template <int G>
+template <int G, bool FX = false>
 int launch_adv_t(const LaunchShape& s, const AdvanceParams& P, const chem_options* opt,
                  cudaStream_t stream) {
-  CHEM_CUDA_TRY(cudaFuncSetAttribute(advance_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  CHEM_CUDA_TRY(cudaFuncSetAttribute((advance_kernel<G, FX>), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)s.smem));
   int dev = 0, sms = 0, per_sm = 0;
   CHEM_CUDA_TRY(cudaGetDevice(&dev));
   CHEM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  CHEM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, advance_kernel<G>, s.threads, s.smem));
+  CHEM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (advance_kernel<G, FX>), s.threads, s.smem));
   if (per_sm < 1) { set_error("kernel does not fit on an SM"); return CHEM_EINVAL; }
   int64_t chunks = P.total_chunks;     // an upper bound when the count is read on the device
   int64_t grid = (int64_t)sms * per_sm;
@@ -1326,18 +1703,18 @@ int launch_adv_t(const LaunchShape& s, const AdvanceParams& P, const chem_option
     grid = std::min<int64_t>(grid, (chunks + s.groups - 1) / s.groups);
   }
   if (grid < 1) grid = 1;
-  advance_kernel<G><<<(unsigned)grid, threads, smem, stream>>>(P);
+  advance_kernel<G, FX><<<(unsigned)grid, threads, smem, stream>>>(P);
   CHEM_CUDA_TRY(cudaGetLastError());
   return CHEM_OK;
 }
 
-template <int G>
+template <int G, bool FX = false>
 int launch_eval_t(const LaunchShape& s, const EvalParams& P, cudaStream_t stream) {
-  CHEM_CUDA_TRY(cudaFuncSetAttribute(eval_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  CHEM_CUDA_TRY(cudaFuncSetAttribute((eval_kernel<G, FX>), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)s.smem));
   int64_t grid = (P.ncells + s.groups - 1) / s.groups;
   grid = std::min<int64_t>(grid, 65535);
-  eval_kernel<G><<<(unsigned)grid, s.threads, s.smem, stream>>>(P);
+  eval_kernel<G, FX><<<(unsigned)grid, s.threads, s.smem, stream>>>(P);
   CHEM_CUDA_TRY(cudaGetLastError());
   return CHEM_OK;
 }
@@ -1352,10 +1729,18 @@ int dispatch_adv(const LaunchShape& s, const AdvanceParams& P, const chem_option
     case 16: return launch_adv_t<16>(s, P, opt, stream);
     case 32: return launch_adv_t<32>(s, P, opt, stream);
     case 64: return launch_adv_t<64>(s, P, opt, stream);
-    case 128: return launch_adv_t<128>(s, P, opt, stream);
+    case 128: return s.fx ? launch_adv_t<128, true>(s, P, opt, stream) : launch_adv_t<128>(s, P, opt, stream);
     case 256: return launch_adv_t<256>(s, P, opt, stream);
     default: set_error("no kernel for group_threads %d", s.G); return CHEM_EINVAL;
   }
+}
+
+JacArgs jac_args(const chem_mech_s* m);
+
+void mech_args(const chem_mech_s* m, const LaunchShape& s, MechArgs* A) {
+  A->lay = m->lay; A->gx = m->gx; A->ws = s.ws; A->jp = jac_args(m); A->gj = m->gxj;
+  A->blob = (const unsigned char*)m->d_blob; A->gxblob = (const unsigned char*)m->d_gx;
+  A->lg = m->d_lg; A->rc = m->d_rc;
 }
 
 JacArgs jac_args(const chem_mech_s* m) {
@@ -1391,7 +1776,7 @@ int launch_advance(chem_mech_s* m, double* T, const double* p, double* Y, int64_
   CHEM_CUDA_TRY(cudaMallocAsync((void**)&counter, sizeof(unsigned long long), stream));
   CHEM_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(unsigned long long), stream));
   AdvanceParams P;
-  P.lay = m->lay; P.ws = s.ws; P.jp = jac_args(m); P.blob = (const unsigned char*)m->d_blob;
+  mech_args(m, s, &P);
   P.segs[0] = Segment{T, p, Y, ld, ncells, idx, status, nsub, nrej, dt, rtol, atol, 0};
   P.nseg = 1;
   P.total_chunks = (ncells + chunk_cells(s.G) - 1) / chunk_cells(s.G);
@@ -1420,7 +1805,7 @@ int launch_advance_counted(chem_mech_s* m, double* T, const double* p, double* Y
   CHEM_CUDA_TRY(cudaMallocAsync((void**)&counter, sizeof(unsigned long long), stream));
   CHEM_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(unsigned long long), stream));
   AdvanceParams P;
-  P.lay = m->lay; P.ws = s.ws; P.jp = jac_args(m); P.blob = (const unsigned char*)m->d_blob;
+  mech_args(m, s, &P);
   P.segs[0] = Segment{T, p, Y, ld, capacity, idx, nullptr, nullptr, nullptr, dt, rtol, atol, 0};
   P.nseg = 1;
   P.total_chunks = (capacity + chunk_cells(s.G) - 1) / chunk_cells(s.G);
@@ -1454,7 +1839,7 @@ int launch_advance_batch(chem_mech_s* m, const chem_segment* segs, int nseg, cud
   for (int first = 0; first < nseg; first += kMaxSegs) {
     const int cnt = std::min(kMaxSegs, nseg - first);
     AdvanceParams P;
-    P.lay = m->lay; P.ws = s.ws; P.jp = jac_args(m); P.blob = (const unsigned char*)m->d_blob;
+    mech_args(m, s, &P);
     long long total = 0;
     for (int i = 0; i < cnt; ++i) {
       const chem_segment& a = segs[first + i];
@@ -1501,7 +1886,7 @@ int launch_advance_slice(chem_mech_s* m, const chem_segment* segs, int nseg, uns
   int rc = pick_shape(m, nullptr, &s);
   if (rc) return rc;
   AdvanceParams P;
-  P.lay = m->lay; P.ws = s.ws; P.jp = jac_args(m); P.blob = (const unsigned char*)m->d_blob;
+  mech_args(m, s, &P);
   long long total = 0;
   for (int i = 0; i < nseg; ++i) {
     const chem_segment& a = segs[i];
@@ -1651,7 +2036,7 @@ int launch_advance_noalloc(chem_mech_s* m, double* T, const double* p, double* Y
   unsigned long long* counter = (unsigned long long*)scratch;
   CHEM_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(unsigned long long), stream));
   AdvanceParams P;
-  P.lay = m->lay; P.ws = s.ws; P.jp = jac_args(m); P.blob = (const unsigned char*)m->d_blob;
+  mech_args(m, s, &P);
   P.segs[0] = Segment{T, p, Y, ld, ncells, nullptr, status, nsub, nrej, dt, rtol, atol, 0};
   P.nseg = 1;
   P.total_chunks = (ncells + chunk_cells(s.G) - 1) / chunk_cells(s.G);
@@ -1705,7 +2090,7 @@ extern "C" int chem_eval_rhs_jac(chem_mech_t m, const double* T, const double* p
   if (rc) return rc;
   if (s.G == 1) return launch_cell_eval(m, T, p, Y, ld, ncells, f, J, (cudaStream_t)stream);
   EvalParams P;
-  P.lay = m->lay; P.ws = s.ws; P.jp = jac_args(m); P.blob = (const unsigned char*)m->d_blob;
+  mech_args(m, s, &P);
   P.T = T; P.p = p; P.Y = Y; P.ld = ld; P.ncells = ncells; P.f = f; P.J = J;
   cudaStream_t st = (cudaStream_t)stream;
   switch (s.G) {
@@ -1715,7 +2100,7 @@ extern "C" int chem_eval_rhs_jac(chem_mech_t m, const double* T, const double* p
     case 16: return launch_eval_t<16>(s, P, st);
     case 32: return launch_eval_t<32>(s, P, st);
     case 64: return launch_eval_t<64>(s, P, st);
-    case 128: return launch_eval_t<128>(s, P, st);
+    case 128: return s.fx ? launch_eval_t<128, true>(s, P, st) : launch_eval_t<128>(s, P, st);
     case 256: return launch_eval_t<256>(s, P, st);
     default: set_error("no kernel for group_threads %d", s.G); return CHEM_EINVAL;
   }

@@ -47,7 +47,7 @@ __device__ __forceinline__ bool attempt(const cell::View& m, double* col, double
                                         double atol, double* e2) {
   using w = Ws<NS>;
   constexpr int N = w::N;
-  const double invh = cell::rcp(h), ig = invh * (1.0 / kGamma);
+  const double invh = fx::rcp(h), ig = invh * (1.0 / kGamma);
   cell::rhs<NS, true>(m, col, col[w::Y * 32], [&](int k) { return col[(w::Y + 1 + k) * 32]; }, p, invp, w::U);
   double* M = col + w::M * 32;
 #pragma unroll
@@ -81,7 +81,7 @@ __device__ __forceinline__ bool attempt(const cell::View& m, double* col, double
         rp = row[i]; row[i] = row[k];
       }
     row[k] = rp;
-    const double ip = cell::rcp(piv);
+    const double ip = fx::rcp(piv);
     M[rp + k * 32] = ip;
     double u[N];
 #pragma unroll
@@ -144,8 +144,8 @@ __device__ __forceinline__ bool attempt(const cell::View& m, double* col, double
     double v = y;
 #pragma unroll
     for (int s = 0; s < 6; ++s) v = fma(kRM[s], col[(w::U + s * N + i) * 32], v);
-    const double sc = fma(rtol, cell::max_pos(fabs(y), fabs(v)), atol);
-    const double r = col[(w::U + 5 * N + i) * 32] * cell::rcp(sc);
+    const double sc = fma(rtol, fx::max_pos(fabs(y), fabs(v)), atol);
+    const double r = col[(w::U + 5 * N + i) * 32] * fx::rcp(sc);
     acc = fma(r, r, acc);
     col[(w::U + 5 * N + i) * 32] = v;
   }
@@ -157,7 +157,7 @@ __device__ __forceinline__ bool attempt(const cell::View& m, double* col, double
 // norm.  2^(-log2(e2) / 8) in fixed point (pow is 83 FP64 instructions).
 __device__ __forceinline__ double step_factor(double e2, const cell::View& m) {
   if (!isfinite(e2)) return 0.2;
-  if (!cell::positive_normal(e2)) return 1e30;             // e2 = 0: the caller's facmax bounds it
+  if (!fx::positive_normal(e2)) return 1e30;             // e2 = 0: the caller's facmax bounds it
   const fx::i64 X = -(fx::log2_q52(e2, m.rc, m.lg) >> 3);
   const double f = 0.9 * fx::exp2_q52(X, m.e2);
   return f < 0.2 ? 0.2 : f;

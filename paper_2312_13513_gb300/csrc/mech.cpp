@@ -88,126 +88,53 @@ void reorder_reactions(const chem_mech_desc* in, Reordered* o) {
   }
 }
 
-// The fixed-point form of the mechanism (reactions in the order of the blob).  Returns the bytes;
-// L->bytes = 0 where a number lies outside the formats.  No polynomial can leave Q11.52 (its
-// coefficients' magnitudes sum to at most 2000), and every base-2 exponent that the kernel forms
-// stays below 3074 in magnitude (|log2 kf| <= 600 + 32 * 12 + 1900; |log2 kr| <= 1023 + 2000 by
-// the bound on Delta G below), so that a wrapped sum is always recognised as out of range
-// (exp2_in_range) and never mistaken for a small one.
-std::vector<unsigned char> build_fx(const chem_mech_desc* d, const chem_mech_s* m,
-                                    const std::vector<std::vector<int>>& nu, FxLayout* L) {
-  const int ns = d->n_species, nr = d->n_reactions;
-  *L = FxLayout{};
-  std::vector<unsigned char> none;
-  if (ns > 15 || nr > 1024) return none;
+const fx::u64 kExp2Tab[256] = {CHEM_FX_EXP2_VALUES};
+const fx::u64 kLog2Tab[128] = {CHEM_FX_LOG2_VALUES};
+const uint32_t kRcpTab[128] = {CHEM_FX_RCP_VALUES};
+
+// The numbers of a mechanism in the fixed-point formats (fixed.cuh, fx_mech.h).  ok = false where a
+// species' polynomials leave them.  No polynomial can leave Q11.52 (its coefficients' magnitudes
+// sum to at most 2000), and every base-2 exponent that a kernel forms stays below 3074 in magnitude
+// (|log2 kf| <= 600 + 32 * 12 + 1900; |log2 kr| <= 1023 + 2000 by the bound on Delta G), so that a
+// wrapped sum is always recognised as out of range (exp2_in_range) and never mistaken for a small
+// one.
+struct FxNumbers {
   bool ok = true;
-  auto q = [&](double v, int frac, double lim) -> int64_t {
-    if (!(std::fabs(v) <= lim)) { ok = false; return 0; }
-    return (int64_t)std::nearbyintl((long double)v * (long double)std::ldexp(1.0, frac));
-  };
+  std::vector<FxSpecies> sp;                       // [2][ns]
+  std::vector<int64_t> lnA;                        // [nr]; 2000 where a reaction is left to FP64
+  std::vector<uint64_t> beta, Ta;
+  std::vector<FxTroe> troe;
+  int64_t lpr0 = 0;
   const long double l2 = std::log(2.0L);
-  auto q52l = [&](long double v, double lim) -> int64_t {
+
+  int64_t q52l(long double v, double lim) {
     if (!(std::fabs((double)v) <= lim)) { ok = false; return 0; }
     return (int64_t)std::nearbyintl(v * 4503599627370496.0L);
-  };
-  Builder B;
-  int ntb = 0, ntroe = 0;
-  for (int j = 0; j < nr; ++j) { ntb += d->rtype[j] != 0; ntroe += d->rtype[j] == 2; }
-  std::vector<int> effoff(1, 0);
-  std::vector<double> effv, eff;
-  std::vector<int16_t> effidx;
-  for (int j = 0; j < nr; ++j) {
-    if (d->rtype[j] == 0) continue;
-    for (int k = 0; k < ns; ++k) {
-      const double e = d->eff[(size_t)j * ns + k];
-      eff.push_back(e);
-      if (e != 1.0) { effidx.push_back((int16_t)k); effv.push_back(e - 1.0); }
-    }
-    effoff.push_back((int)effidx.size());
   }
-  L->ns = ns; L->ntb = ntb;
-  // at most two species per side and four net species: FxRate, by type; the rest: FxReac
-  std::vector<int> order[4];
-  for (int j = 0; j < nr; ++j) {
-    int nre = 0, npr = 0, nn = 0;
-    for (int i = 0; i < 3; ++i) { nre += d->reac[3 * j + i] >= 0; npr += d->prod[3 * j + i] >= 0; }
-    for (int k = 0; k < ns; ++k) nn += nu[j][k] != 0;
-    order[nre <= 2 && npr <= 2 && nn <= 4 && ns >= 4 ? d->rtype[j] : 3].push_back(j);
-  }
-  L->n_plain = (int)order[0].size(); L->n_tb = (int)order[1].size(); L->n_fo = (int)order[2].size();
-  L->n_gen = (int)order[3].size();
-  L->o_exp2 = B.add(8 * 256);
-  L->o_lg = B.add(8 * 128);
-  L->o_rcp = B.add(4 * 128);
-  L->o_sp = B.add(2 * ns * (int)sizeof(FxSpecies));
-  L->o_W = B.add(8 * ns);
-  L->o_invW = B.add(8 * ns);
-  L->o_nu = B.add(8 * 16);
-  L->o_rate = B.add((nr - L->n_gen) * (int)sizeof(FxRate));
-  L->o_reac = B.add(L->n_gen * (int)sizeof(FxReac));
-  L->o_troe = B.add(ntroe * (int)sizeof(FxTroe));
-  L->o_effv = B.add(8 * (int)effv.size());
-  L->o_eff = B.add(8 * (int)eff.size());
-  L->o_effidx = B.add(2 * (int)effidx.size());
-  L->o_effoff = B.add(4 * (int)effoff.size());
-  static const fx::u64 e2[256] = {CHEM_FX_EXP2_VALUES};
-  static const fx::u64 lg[128] = {CHEM_FX_LOG2_VALUES};
-  static const uint32_t rc[128] = {CHEM_FX_RCP_VALUES};
-  memcpy(B.at<unsigned char>(L->o_exp2), e2, sizeof(e2));
-  memcpy(B.at<unsigned char>(L->o_lg), lg, sizeof(lg));
-  memcpy(B.at<unsigned char>(L->o_rcp), rc, sizeof(rc));
-  for (int r = 0; r < 2; ++r)
-    for (int k = 0; k < ns; ++k) {
-      const double* a = (r == 0 ? d->nasa_lo : d->nasa_hi) + 7 * k;
-      FxSpecies* S = B.at<FxSpecies>(L->o_sp) + r * ns + k;
-      const int sh = r == 0 ? kFxR0 : kFxR1;
-      long double p = 1.0L;
-      for (int i = 0; i < 5; ++i, p *= std::ldexp(1.0L, sh)) {
-        // i-th coefficients of h/RT, s/R (the constant is a7, the T-free part of a1 (1 - ln T) is
-        // a1) and cp/R in powers of tau
-        S->c[i] = q52l((long double)a[i] * p, 500.0);
-        S->h[i] = q52l((long double)a[i] / (i + 1) * p, 500.0);
-        const long double s = i == 0 ? (long double)a[6] : (long double)a[i] / i * p;
-        const long double g = (i == 0 ? (long double)a[0] : (long double)a[i] / (i + 1) * p) - s;
-        S->g[i] = q52l(g / l2, 1000.0);
-      }
-      S->ha6 = q52l((long double)a[5] / 128.0L, 1900.0);
-      S->ga6 = q52l((long double)a[5] / 128.0L / l2, 1900.0);
-      S->gl = q(-a[0], 56, 100.0);
-      S->d3 = S->c[4] * 4;
-      S->d2 = S->c[3] * 3;
-      double sg = std::fabs((double)S->ga6), sh_ = std::fabs((double)S->ha6), sc = 0.0;
-      for (int i = 0; i < 5; ++i) {
-        sg += std::fabs((double)S->g[i]); sh_ += std::fabs((double)S->h[i]);
-        sc += std::max(1, i) * std::fabs((double)S->c[i]);
-      }
-      if (!(std::max(std::max(sg + 12.0 * std::fabs((double)S->gl) / 16.0, sh_), sc) <= 2000.0 * 4503599627370496.0)) ok = false;
-      for (int64_t* x : {&S->g[4], &S->h[4], &S->c[4], &S->ga6, &S->gl, &S->ha6, &S->d3}) *x = (int64_t)fx::biased(*x);
-    }
-  for (int k = 0; k < ns; ++k) {
-    B.at<double>(L->o_W)[k] = m->W[k];
-    B.at<double>(L->o_invW)[k] = 1.0 / m->W[k];
-  }
-  for (int c = 0; c < 16; ++c) B.at<double>(L->o_nu)[c] = (double)(c - 8);
-  L->lpr0 = q52l(std::log((long double)PATM / (long double)RU) / l2, 1000.0);
-  // |Delta G / (RT ln 2)| of a reaction over [kTlo, kThi): on 512 log-spaced pieces, the value at
+  int64_t q56(double v) { return (int64_t)std::nearbyintl((long double)v * 72057594037927936.0L); }
+
+  // |Delta G / (RT ln 2)| of a reaction over [kTlo, kThi): on 128 log-spaced pieces, the value at
   // the left end plus the change of every (monotone) term across the piece
-  auto worst_dG = [&](int j, int dnu) {
+  static double worst_dG(const chem_mech_desc* d, const std::vector<int>& nu, int dnu) {
+    const int ns = d->n_species;
+    double c[2][7] = {};
+    for (int k = 0; k < ns; ++k)
+      if (nu[k])
+        for (int t = 0; t < 7; ++t) {
+          c[0][t] += nu[k] * d->nasa_lo[7 * k + t];
+          c[1][t] += nu[k] * d->nasa_hi[7 * k + t];
+        }
     double worst = 0.0;
-    const double step = std::pow(fx::kThi / fx::kTlo, 1.0 / 512.0);
+    const double step = std::pow(fx::kThi / fx::kTlo, 1.0 / 128.0);
     double T = fx::kTlo;
-    for (int i = 0; i < 512; ++i, T *= step) {
+    for (int i = 0; i < 128; ++i, T *= step) {
       const double T1 = T * step;
       for (int r = T >= TMID ? 1 : 0; r <= (T1 < TMID ? 0 : 1); ++r) {
-        const double* nasa = r == 0 ? d->nasa_lo : d->nasa_hi;
-        double c[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-        for (int k = 0; k < ns; ++k)
-          for (int t = 0; t < 7; ++t) c[t] += nu[j][k] * nasa[7 * k + t];
         auto terms = [&](double x, double* o) {
           double p = 1.0;
           for (int t = 0; t < 5; ++t, p *= x)
-            o[t] = t == 0 ? c[0] * (1.0 - std::log(x)) - c[6] : -c[t] * p / (t * (t + 1));
-          o[5] = c[5] / x;
+            o[t] = t == 0 ? c[r][0] * (1.0 - std::log(x)) - c[r][6] : -c[r][t] * p / (t * (t + 1));
+          o[5] = c[r][5] / x;
           o[6] = dnu * (std::log(x) - std::log(PATM / RU));
         };
         double a0[7], a1[7], v = 0.0, w = 0.0;
@@ -218,26 +145,141 @@ std::vector<unsigned char> build_fx(const chem_mech_desc* d, const chem_mech_s* 
       }
     }
     return worst / std::log(2.0);
-  };
-  auto in_formats = [&](double A, double b, double Ea) {
+  }
+
+  static bool in_formats(double A, double b, double Ea) {
     return A > 0.0 && std::fabs(std::log2(A)) <= 599.0 && std::fabs(b) <= 32.0 && std::fabs(Ea / RC) <= 160000.0;
-  };
-  auto low_fits = [&](int j) {                 // the low-pressure limit of a fall-off reaction
-    const double* t = d->troe + 7 * j;
-    return d->rtype[j] != 2 || in_formats(t[0], t[1], t[2]);
-  };
-  // log2 A, b and Ta in the formats; log2 A = 2000 (never in range) where one does not fit
-  auto rate = [&](double A, double b, double Ea, bool fits, int64_t* lnA_, uint64_t* beta, uint64_t* Ta_) {
+  }
+  void rate(double A, double b, double Ea, bool fits, int64_t* lnA_, uint64_t* beta_, uint64_t* Ta_) {
     fits = fits && in_formats(A, b, Ea);
     *lnA_ = fits ? q52l(std::log((long double)A) / l2, 600.0) : (int64_t)2000 << 52;
-    *beta = fx::biased(fits ? q(b, 56, 32.0) : 0);
+    *beta_ = fx::biased(fits ? q56(b) : 0);
     *Ta_ = fx::biased(fits ? q52l((long double)Ea / (long double)RC / l2 / 128.0L, 1900.0) : 0);
-  };
-  std::vector<int16_t> tb_of(nr, -1), troe_of(nr, -1);
-  for (int j = 0, tb = 0, tr = 0; j < nr; ++j) {
-    if (d->rtype[j] != 0) tb_of[j] = (int16_t)tb++;
-    if (d->rtype[j] == 2) troe_of[j] = (int16_t)tr++;
   }
+
+  FxNumbers(const chem_mech_desc* d, const std::vector<std::vector<int>>& nu) {
+    const int ns = d->n_species, nr = d->n_reactions;
+    sp.resize(2 * (size_t)ns);
+    for (int r = 0; r < 2; ++r)
+      for (int k = 0; k < ns; ++k) {
+        const double* a = (r == 0 ? d->nasa_lo : d->nasa_hi) + 7 * k;
+        FxSpecies& S = sp[(size_t)r * ns + k];
+        const int sh = r == 0 ? kFxR0 : kFxR1;
+        long double p = 1.0L;
+        for (int i = 0; i < 5; ++i, p *= std::ldexp(1.0L, sh)) {
+          // i-th coefficients of h/RT, s/R (the constant is a7, the T-free part of a1 (1 - ln T) is
+          // a1) and cp/R in powers of tau
+          S.c[i] = q52l((long double)a[i] * p, 500.0);
+          S.h[i] = q52l((long double)a[i] / (i + 1) * p, 500.0);
+          const long double s = i == 0 ? (long double)a[6] : (long double)a[i] / i * p;
+          const long double g = (i == 0 ? (long double)a[0] : (long double)a[i] / (i + 1) * p) - s;
+          S.g[i] = q52l(g / l2, 1000.0);
+        }
+        S.ha6 = q52l((long double)a[5] / 128.0L, 1900.0);
+        S.ga6 = q52l((long double)a[5] / 128.0L / l2, 1900.0);
+        if (!(std::fabs(a[0]) <= 100.0)) ok = false;
+        S.gl = ok ? q56(-a[0]) : 0;
+        double sg = std::fabs((double)S.ga6), sh_ = std::fabs((double)S.ha6), sc = 0.0;
+        for (int i = 0; i < 5; ++i) {
+          sg += std::fabs((double)S.g[i]); sh_ += std::fabs((double)S.h[i]);
+          sc += std::max(1, i) * std::fabs((double)S.c[i]);
+        }
+        sg += 12.0 * std::fabs((double)S.gl) / 16.0;
+        if (!(std::max(std::max(sg, sh_), sc) <= 2000.0 * 4503599627370496.0)) ok = false;
+        for (int64_t* x : {&S.g[4], &S.h[4], &S.c[4], &S.ga6, &S.gl, &S.ha6}) *x = (int64_t)fx::biased(*x);
+      }
+    lpr0 = q52l(std::log((long double)PATM / (long double)RU) / l2, 1000.0);
+    lnA.resize(nr); beta.resize(nr); Ta.resize(nr);
+    for (int j = 0; j < nr; ++j) {
+      int dnu = 0;
+      for (int k = 0; k < ns; ++k) dnu += nu[j][k];
+      bool fits = worst_dG(d, nu[j], dnu) <= 2000.0;
+      if (d->rtype[j] == 2) {
+        const double* t = d->troe + 7 * j;
+        fits = fits && in_formats(t[0], t[1], t[2]);
+        FxTroe F{};
+        rate(t[0], t[1], t[2], fits, &F.lnA0, &F.b0, &F.Ta0);
+        F.b0d = t[1]; F.Ta0K = t[2] / RC;
+        F.a = t[3]; F.iT3 = 1.0 / t[4]; F.iT1 = 1.0 / t[5]; F.T2 = t[6];
+        F.has_t2 = d->has_t2[j] ? 1.0 : 0.0;
+        troe.push_back(F);
+      }
+      rate(d->A[j], d->b[j], d->Ea[j], fits, &lnA[j], &beta[j], &Ta[j]);
+    }
+  }
+};
+
+// third-body sets in reaction order: sparse (efficiency - 1) and, dense, the efficiencies
+struct Partners {
+  std::vector<int> off{0};
+  std::vector<int16_t> idx;
+  std::vector<double> val, dense;
+  std::vector<int16_t> tb_of, troe_of;
+  int ntb = 0, ntroe = 0;
+  explicit Partners(const chem_mech_desc* d) : tb_of(d->n_reactions, -1), troe_of(d->n_reactions, -1) {
+    const int ns = d->n_species;
+    for (int j = 0; j < d->n_reactions; ++j) {
+      if (d->rtype[j] == 0) continue;
+      tb_of[j] = (int16_t)ntb++;
+      if (d->rtype[j] == 2) troe_of[j] = (int16_t)ntroe++;
+      for (int k = 0; k < ns; ++k) {
+        const double e = d->eff[(size_t)j * ns + k];
+        dense.push_back(e);
+        if (e != 1.0) { idx.push_back((int16_t)k); val.push_back(e - 1.0); }
+      }
+      off.push_back((int)idx.size());
+    }
+  }
+};
+
+template <class T>
+void put(Builder& B, int off, const std::vector<T>& v) {
+  if (!v.empty()) memcpy(B.at<unsigned char>(off), v.data(), v.size() * sizeof(T));
+}
+
+// Blob of the cell-per-thread kernel (fx_mech.h); L->bytes = 0 where there is none.
+std::vector<unsigned char> build_fx(const chem_mech_desc* d, const chem_mech_s* m, const FxNumbers& F,
+                                    const std::vector<std::vector<int>>& nu, FxLayout* L) {
+  const int ns = d->n_species, nr = d->n_reactions;
+  *L = FxLayout{};
+  if (!F.ok || ns > 15 || nr > 1024) return {};
+  const Partners T(d);
+  Builder B;
+  L->ns = ns; L->ntb = T.ntb; L->lpr0 = F.lpr0;
+  // at most two species per side and four net species: FxRate, by type; the rest: FxReac
+  std::vector<int> order[4];
+  for (int j = 0; j < nr; ++j) {
+    int nre = 0, npr = 0, nn = 0;
+    for (int i = 0; i < 3; ++i) { nre += d->reac[3 * j + i] >= 0; npr += d->prod[3 * j + i] >= 0; }
+    for (int k = 0; k < ns; ++k) nn += nu[j][k] != 0;
+    order[nre <= 2 && npr <= 2 && nn <= 4 && ns >= 4 ? d->rtype[j] : 3].push_back(j);
+  }
+  L->n_plain = (int)order[0].size(); L->n_tb = (int)order[1].size(); L->n_fo = (int)order[2].size();
+  L->n_gen = (int)order[3].size();
+  L->o_exp2 = B.add(sizeof(kExp2Tab));
+  L->o_lg = B.add(sizeof(kLog2Tab));
+  L->o_rcp = B.add(sizeof(kRcpTab));
+  L->o_sp = B.add(2 * ns * (int)sizeof(FxSpecies));
+  L->o_W = B.add(8 * ns);
+  L->o_invW = B.add(8 * ns);
+  L->o_nu = B.add(8 * 16);
+  L->o_rate = B.add((nr - L->n_gen) * (int)sizeof(FxRate));
+  L->o_reac = B.add(L->n_gen * (int)sizeof(FxReac));
+  L->o_troe = B.add(T.ntroe * (int)sizeof(FxTroe));
+  L->o_effv = B.add(8 * (int)T.val.size());
+  L->o_eff = B.add(8 * (int)T.dense.size());
+  L->o_effidx = B.add(2 * (int)T.idx.size());
+  L->o_effoff = B.add(4 * (int)T.off.size());
+  memcpy(B.at<unsigned char>(L->o_exp2), kExp2Tab, sizeof(kExp2Tab));
+  memcpy(B.at<unsigned char>(L->o_lg), kLog2Tab, sizeof(kLog2Tab));
+  memcpy(B.at<unsigned char>(L->o_rcp), kRcpTab, sizeof(kRcpTab));
+  put(B, L->o_sp, F.sp); put(B, L->o_troe, F.troe); put(B, L->o_effv, T.val); put(B, L->o_eff, T.dense);
+  put(B, L->o_effidx, T.idx); put(B, L->o_effoff, T.off);
+  for (int k = 0; k < ns; ++k) {
+    B.at<double>(L->o_W)[k] = m->W[k];
+    B.at<double>(L->o_invW)[k] = 1.0 / m->W[k];
+  }
+  for (int c = 0; c < 16; ++c) B.at<double>(L->o_nu)[c] = (double)(c - 8);
   FxRate* R = B.at<FxRate>(L->o_rate);
   for (int cls = 0; cls < 3; ++cls)
     for (int j : order[cls]) {
@@ -247,8 +289,8 @@ std::vector<unsigned char> build_fx(const chem_mech_desc* d, const chem_mech_s* 
         if (d->reac[3 * j + i] >= 0) { R->c[nr_++] = (uint16_t)(d->reac[3 * j + i] * 256); --dnu; }
         if (d->prod[3 * j + i] >= 0) { R->c[np_++] = (uint16_t)(d->prod[3 * j + i] * 256); ++dnu; }
       }
-      R->dnu = (int16_t)dnu; R->id = (int16_t)j; R->tb = tb_of[j]; R->troe = troe_of[j];
-      rate(d->A[j], d->b[j], d->Ea[j], worst_dG(j, dnu) <= 2000.0 && low_fits(j), &R->lnA, &R->beta, &R->Ta);
+      R->dnu = (int16_t)dnu; R->id = (int16_t)j; R->tb = T.tb_of[j]; R->troe = T.troe_of[j];
+      R->lnA = F.lnA[j]; R->beta = F.beta[j]; R->Ta = F.Ta[j];
       R->b = d->b[j];
       R->TaK = d->Ea[j] / RC;
       int n = 0;
@@ -264,33 +306,131 @@ std::vector<unsigned char> build_fx(const chem_mech_desc* d, const chem_mech_s* 
       if (d->reac[3 * j + i] >= 0) { G->re[G->nre++] = (uint8_t)d->reac[3 * j + i]; --dnu; }
       if (d->prod[3 * j + i] >= 0) { G->pr[G->npr++] = (uint8_t)d->prod[3 * j + i]; ++dnu; }
     }
-    G->dnu = (int16_t)dnu; G->id = (int16_t)j; G->tb = tb_of[j]; G->troe = troe_of[j];
+    G->dnu = (int16_t)dnu; G->id = (int16_t)j; G->tb = T.tb_of[j]; G->troe = T.troe_of[j];
     G->type = (uint8_t)d->rtype[j];
-    rate(d->A[j], d->b[j], d->Ea[j], worst_dG(j, dnu) <= 2000.0 && low_fits(j), &G->lnA, &G->beta, &G->Ta);
+    G->lnA = F.lnA[j]; G->beta = F.beta[j]; G->Ta = F.Ta[j];
     G->b = d->b[j];
     G->TaK = d->Ea[j] / RC;
     for (int k = 0; k < ns; ++k)
       if (nu[j][k] != 0) { G->sp[G->nnet] = (uint8_t)k; G->nu[G->nnet++] = (int8_t)nu[j][k]; }
     ++G;
   }
-  for (int j = 0; j < nr; ++j) {
-    if (troe_of[j] < 0) continue;
-    const double* t = d->troe + 7 * j;
-    FxTroe* F = B.at<FxTroe>(L->o_troe) + troe_of[j];
-    rate(t[0], t[1], t[2], true, &F->lnA0, &F->b0, &F->Ta0);
-    F->b0d = t[1]; F->Ta0K = t[2] / RC;
-    F->a = t[3]; F->iT3 = 1.0 / t[4]; F->iT1 = 1.0 / t[5]; F->T2 = t[6];
-    F->has_t2 = d->has_t2[j] ? 1.0 : 0.0;
-  }
-  for (size_t i = 0; i < effv.size(); ++i) {
-    B.at<double>(L->o_effv)[i] = effv[i];
-    B.at<int16_t>(L->o_effidx)[i] = effidx[i];
-  }
-  for (size_t i = 0; i < eff.size(); ++i) B.at<double>(L->o_eff)[i] = eff[i];
-  for (size_t i = 0; i < effoff.size(); ++i) B.at<int>(L->o_effoff)[i] = effoff[i];
-  if (!ok) return none;
   L->bytes = (int)B.buf.size();
   return B.buf;
+}
+
+// Blob of the group kernels' fixed-point form, and their Jacobian program with the log2 and
+// reciprocal tables behind it (one global allocation each, uploaded here).
+int build_gx(const chem_mech_desc* d, chem_mech_s* m, const FxNumbers& F, const std::vector<std::vector<int>>& nu,
+             const MechLayout& ML, const Builder& MB) {
+  const int ns = d->n_species, nr = d->n_reactions;
+  m->gx = GxLayout{};
+  if (!F.ok) return CHEM_OK;
+  const Partners T(d);
+  GxLayout L{};
+  Builder B;
+  L.ns = ns; L.nr = nr; L.ntb = T.ntb; L.npieces = ML.npieces; L.lpr0 = F.lpr0;
+  L.o_exp2 = B.add(sizeof(kExp2Tab));
+  L.o_sp = B.add(2 * ns * (int)sizeof(FxSpecies));
+  L.o_W = B.add(8 * ns);
+  L.o_invW = B.add(8 * ns);
+  L.o_nu = B.add(8 * 16);
+  L.o_lnA = B.add(8 * nr);
+  L.o_beta = B.add(8 * nr);
+  L.o_Ta = B.add(8 * nr);
+  L.o_reac = B.add(8 * nr);
+  L.o_prod = B.add(8 * nr);
+  L.o_rinfo = B.add(8 * nr);
+  L.o_troe = B.add(T.ntroe * (int)sizeof(FxTroe));
+  L.o_effv = B.add(8 * (int)T.val.size());
+  L.o_effidx = B.add(2 * (int)T.idx.size());
+  L.o_effoff = B.add(4 * (int)T.off.size());
+  const int np = ML.nprod;
+  L.o_wpk = B.add(4 * np);
+  L.o_pterm = B.add(4 * (ML.npieces + 1));
+  L.o_poff = B.add(4 * (ns + 1));
+  memcpy(B.at<unsigned char>(L.o_exp2), kExp2Tab, sizeof(kExp2Tab));
+  put(B, L.o_sp, F.sp); put(B, L.o_lnA, F.lnA); put(B, L.o_beta, F.beta); put(B, L.o_Ta, F.Ta);
+  put(B, L.o_troe, F.troe); put(B, L.o_effv, T.val); put(B, L.o_effidx, T.idx); put(B, L.o_effoff, T.off);
+  memcpy(B.at<unsigned char>(L.o_W), MB.buf.data() + ML.o_W, 8 * ns);
+  memcpy(B.at<unsigned char>(L.o_invW), MB.buf.data() + ML.o_invW, 8 * ns);
+  for (int c = 0; c < 16; ++c) B.at<double>(L.o_nu)[c] = (double)(c - 8);
+  memcpy(B.at<unsigned char>(L.o_reac), MB.buf.data() + ML.o_reac, 8 * (size_t)nr);
+  memcpy(B.at<unsigned char>(L.o_prod), MB.buf.data() + ML.o_prod, 8 * (size_t)nr);
+  memcpy(B.at<unsigned char>(L.o_rinfo), MB.buf.data() + ML.o_rinfo, 8 * (size_t)nr);
+  for (int e = 0; e < 4 * nr; ++e) {
+    int16_t* r = B.at<int16_t>(L.o_reac) + e;
+    int16_t* p = B.at<int16_t>(L.o_prod) + e;
+    if (*r < 0) *r = (int16_t)ns;
+    if (*p < 0) *p = (int16_t)ns;
+  }
+  memcpy(B.at<unsigned char>(L.o_wpk), MB.buf.data() + ML.o_wpk, 4 * (size_t)np);
+  memcpy(B.at<unsigned char>(L.o_pterm), MB.buf.data() + ML.o_pterm, 4 * (size_t)(ML.npieces + 1));
+  memcpy(B.at<unsigned char>(L.o_poff), MB.buf.data() + ML.o_poff, 4 * (size_t)(ns + 1));
+  L.bytes = (int)B.buf.size();
+
+  struct Entry {
+    std::vector<std::pair<int, int>> slot;       // (src, oth)
+    std::vector<std::pair<int, double>> part;    // (set, coef)
+  };
+  std::map<std::pair<int, int>, Entry> ent;
+  std::vector<std::vector<int>> rows(ns);
+  for (int j = 0; j < nr; ++j)
+    for (int k = 0; k < ns; ++k) {
+      if (nu[j][k] == 0) continue;
+      for (int s = 0; s < 6; ++s) {
+        const int* side = s < 3 ? d->reac + 3 * j : d->prod + 3 * j;
+        const int sl = s % 3;
+        if (side[sl] < 0) continue;
+        const int a1 = sl == 0 ? 1 : 0, a2 = sl == 2 ? 1 : 2;
+        const int o1 = side[a1] >= 0 ? side[a1] : ns, o2 = side[a2] >= 0 ? side[a2] : ns;
+        ent[{k, side[sl]}].slot.push_back({((2 * j + (s >= 3)) << 4) | (nu[j][k] + 8), o1 | (o2 << 16)});
+      }
+      if (T.tb_of[j] < 0) continue;
+      rows[k].push_back((T.tb_of[j] << 4) | (nu[j][k] + 8));
+      for (int e = T.off[T.tb_of[j]]; e < T.off[T.tb_of[j] + 1]; ++e)
+        ent[{k, T.idx[e]}].part.push_back({T.tb_of[j], nu[j][k] * T.val[e]});
+    }
+  // entries with much work first: threads take consecutive entries, so a warp's are alike
+  std::vector<const std::pair<const std::pair<int, int>, Entry>*> order;
+  for (auto& kv : ent) order.push_back(&kv);
+  std::stable_sort(order.begin(), order.end(), [](const auto* a, const auto* b) {
+    return 2 * a->second.slot.size() + a->second.part.size() > 2 * b->second.slot.size() + b->second.part.size();
+  });
+  std::vector<int> so(1, 0), po(1, 0), ss, sx, pt, ro(1, 0), rs;
+  std::vector<double> pc;
+  std::vector<int16_t> er, ec;
+  for (const auto* kv : order) {
+    er.push_back((int16_t)kv->first.first);
+    ec.push_back((int16_t)kv->first.second);
+    for (auto& t : kv->second.slot) { ss.push_back(t.first); sx.push_back(t.second); }
+    for (auto& t : kv->second.part) { pt.push_back(t.first); pc.push_back(t.second); }
+    so.push_back((int)ss.size());
+    po.push_back((int)pt.size());
+  }
+  for (int k = 0; k < ns; ++k) { rs.insert(rs.end(), rows[k].begin(), rows[k].end()); ro.push_back((int)rs.size()); }
+  Builder J;
+  const int o_so = J.add(4 * (int)so.size()), o_po = J.add(4 * (int)po.size()), o_er = J.add(2 * (int)er.size()),
+            o_ec = J.add(2 * (int)ec.size()), o_ss = J.add(4 * (int)ss.size()), o_sx = J.add(4 * (int)sx.size()),
+            o_pt = J.add(4 * (int)pt.size()), o_pc = J.add(8 * (int)pc.size()), o_ro = J.add(4 * (int)ro.size()),
+            o_rs = J.add(4 * (int)rs.size()), o_lg = J.add(sizeof(kLog2Tab)), o_rc = J.add(sizeof(kRcpTab));
+  put(J, o_so, so); put(J, o_po, po); put(J, o_er, er); put(J, o_ec, ec); put(J, o_ss, ss); put(J, o_sx, sx);
+  put(J, o_pt, pt); put(J, o_pc, pc); put(J, o_ro, ro); put(J, o_rs, rs);
+  memcpy(J.at<unsigned char>(o_lg), kLog2Tab, sizeof(kLog2Tab));
+  memcpy(J.at<unsigned char>(o_rc), kRcpTab, sizeof(kRcpTab));
+  CHEM_CUDA_TRY(cudaMalloc(&m->d_gx, B.buf.size()));
+  CHEM_CUDA_TRY(cudaMemcpy(m->d_gx, B.buf.data(), B.buf.size(), cudaMemcpyHostToDevice));
+  CHEM_CUDA_TRY(cudaMalloc(&m->d_gxj, J.buf.size()));
+  CHEM_CUDA_TRY(cudaMemcpy(m->d_gxj, J.buf.data(), J.buf.size(), cudaMemcpyHostToDevice));
+  const unsigned char* g = (const unsigned char*)m->d_gxj;
+  m->gxj = GxJac{(int)er.size(),           (const int*)(g + o_so),     (const int*)(g + o_po),
+                 (const int16_t*)(g + o_er), (const int16_t*)(g + o_ec), (const int*)(g + o_ss),
+                 (const int*)(g + o_sx),     (const int*)(g + o_pt),     (const double*)(g + o_pc),
+                 (const int*)(g + o_ro),     (const int*)(g + o_rs)};
+  m->d_lg = (const unsigned long long*)(g + o_lg);
+  m->d_rc = (const unsigned int*)(g + o_rc);
+  m->gx = L;
+  return CHEM_OK;
 }
 
 int build(const chem_mech_desc* din, chem_mech_s* m) {
@@ -490,8 +630,13 @@ int build(const chem_mech_desc* din, chem_mech_s* m) {
   }
   P.nterm = (int)src.size();
 
-  const std::vector<unsigned char> fxb = build_fx(d, m, nu, &m->fx);
+  const FxNumbers fxn(d, nu);
+  const std::vector<unsigned char> fxb = build_fx(d, m, fxn, nu, &m->fx);
   CHEM_CUDA_TRY(cudaGetDevice(&m->device));
+  {
+    const int rc = build_gx(d, m, fxn, nu, L, B);
+    if (rc) return rc;
+  }
   if (m->fx.bytes) {
     CHEM_CUDA_TRY(cudaMalloc(&m->d_fx, m->fx.bytes));
     CHEM_CUDA_TRY(cudaMemcpy(m->d_fx, fxb.data(), m->fx.bytes, cudaMemcpyHostToDevice));
@@ -690,6 +835,8 @@ extern "C" int chem_free_mechanism(chem_mech_t m) {
   if (m->d_blob) cudaFree(m->d_blob);
   if (m->d_jac) cudaFree(m->d_jac);
   if (m->d_fx) cudaFree(m->d_fx);
+  if (m->d_gx) cudaFree(m->d_gx);
+  if (m->d_gxj) cudaFree(m->d_gxj);
   delete m;
   return CHEM_OK;
 }
