@@ -3,6 +3,7 @@
 // the formats' range has none (FxLayout::bytes = 0) and runs on the FP64 kernels, a single
 // reaction outside it carries FxReac::slow and takes the FP64 rate expressions.
 #pragma once
+#include <cuda_runtime.h>
 #include <stdint.h>
 
 namespace chem {
@@ -77,20 +78,25 @@ struct GxLayout {
   int64_t lpr0;
 };
 
-// Jacobian-assembly program of the group kernels with the fixed-point form (global memory): entry
-// e covers row ent_row[e], column ent_col[e] and sums slot terms slot_off[e] .. slot_off[e + 1) and
-// partner terms part_off[e] .. part_off[e + 1).  A slot term is the derivative of one direction of reaction j with
-// respect to one of its species: slot_src = (2 j + side) << 4 | (nu + 8), times the concentrations
-// of the side's other species slot_oth = o1 | o2 << 16.  Collision partners: d(wdot_k)/dC_m =
-// sum_j nu_kj X_j eff_jm = R_k + sum_j nu_kj X_j (eff_jm - 1), with R_k = sum_j nu_kj X_j the same
-// for every column: only the sparse deviations are terms (part_tb = set, part_coef = nu (eff - 1)),
-// R_k (row_off, row_src = set << 4 | (nu + 8)) joins the chain rule.  For the 53-species mechanism
-// this leaves 4.4 k slot and 2.8 k partner terms of 13.1 k.
+// Jacobian-assembly program of the group kernels with the fixed-point form (global memory).  Entry e
+// (row, column of d(wdot)/dC at ent_pos = row << 16 | column, -1: none) is lane e % kGxLanes of
+// chunk e / kGxLanes; chunk = (first slot row, slot rows, first partner row, partner rows), and term
+// row r of lane t lies at r * kGxLanes + t: coalesced loads without dependent offsets (entries
+// sorted by their term counts, short ones padded with terms of coefficient 0).  A slot term is the
+// derivative of one direction of reaction j with respect to one of its species: slot.x =
+// (2 j + side) << 4 | (nu + 8), times the concentrations of the side's other species slot.y =
+// o1 | o2 << 16.  Collision partners: d(wdot_k)/dC_m = sum_j nu_kj X_j eff_jm = R_k +
+// sum_j nu_kj X_j (eff_jm - 1), with R_k = sum_j nu_kj X_j the same for every column: only the sparse
+// deviations are terms (part_tb = set, part_coef = nu (eff - 1)); R_k (row_off, row_src =
+// set << 4 | (nu + 8)) joins the chain rule.  For the 53-species mechanism this leaves 4.4 k slot
+// and 2.8 k partner terms of 13.1 k.
+constexpr int kGxLanes = 128;
 struct GxJac {
-  int nent = 0;
-  const int *slot_off = nullptr, *part_off = nullptr;      // [nent + 1]
-  const int16_t *ent_row = nullptr, *ent_col = nullptr;    // [nent]
-  const int *slot_src = nullptr, *slot_oth = nullptr, *part_tb = nullptr;
+  int nchunk = 0;
+  const int4* chunk = nullptr;
+  const int* ent_pos = nullptr;
+  const int2* slot = nullptr;
+  const int* part_tb = nullptr;
   const double* part_coef = nullptr;
   const int *row_off = nullptr, *row_src = nullptr;        // [ns + 1], terms of R_k
 };

@@ -328,6 +328,19 @@ __device__ __forceinline__ void warp_argmax(const Grp<G>& g, unsigned long long&
   }
 }
 
+// The same over a whole warp by integer reductions (redux.sync, one instruction each): the largest
+// high word, then among its lanes the largest low word and the lowest index.  A few tens of cycles
+// where the shuffle butterfly's five dependent rounds take over 200, on the LU's critical path.
+__device__ __forceinline__ void warp_argmax_redux(unsigned long long& best, int& bi) {
+  constexpr unsigned F = 0xffffffffu;
+  const unsigned hi = (unsigned)(best >> 32);
+  const unsigned mh = __reduce_max_sync(F, hi);
+  const unsigned lo = hi == mh ? (unsigned)best : 0u;
+  const unsigned ml = __reduce_max_sync(F, lo);
+  bi = (int)__reduce_min_sync(F, hi == mh && lo == ml ? (unsigned)bi : 0xffffffffu);
+  best = (unsigned long long)mh << 32 | ml;
+}
+
 // ---------------------------------------------------------------------------------------
 // right-hand side and analytic Jacobian at state y (group-cooperative)
 // ---------------------------------------------------------------------------------------
@@ -908,20 +921,23 @@ __device__ __forceinline__ void eval_fx(const Grp<G>& g, const GxView& m, const 
     Jm[(1 + k) * LD + 1 + (e - k * ns)] = 0.0;
   }
   g.sync();
-  for (int e = g.tid; e < jp.nent; e += G) {
+  for (int c = 0; c < jp.nchunk; ++c) {
+    const int4 h = __ldg(jp.chunk + c);                     // first slot row, slot rows, partner rows
+    const int pos = __ldg(jp.ent_pos + c * kGxLanes + g.tid);
     double s = 0.0;
-    const int t1 = __ldg(jp.slot_off + e + 1);
-    for (int i = __ldg(jp.slot_off + e); i < t1; ++i) {
-      const int src = __ldg(jp.slot_src + i), oth = __ldg(jp.slot_oth + i);
-      double d = w.dq[src >> 4];
-      if ((oth & 0xffff) != ns) d *= w.C[oth & 0xffff];
-      if ((oth >> 16) != ns) d *= w.C[oth >> 16];
-      s = fma(m.nu[src & 15], d, s);
+#pragma unroll 4
+    for (int i = 0; i < h.y; ++i) {
+      const int2 tm = __ldg(jp.slot + (size_t)(h.x + i) * kGxLanes + g.tid);
+      double d = w.dq[tm.x >> 4] * w.C[tm.y & 0xffff];
+      if ((tm.y >> 16) != ns) d *= w.C[tm.y >> 16];
+      s = fma(m.nu[tm.x & 15], d, s);
     }
-    const int p1 = __ldg(jp.part_off + e + 1);
-    for (int i = __ldg(jp.part_off + e); i < p1; ++i)
-      s = fma(__ldg(jp.part_coef + i), w.dq[2 * nr + __ldg(jp.part_tb + i)], s);
-    Jm[(1 + __ldg(jp.ent_row + e)) * LD + 1 + __ldg(jp.ent_col + e)] = s;
+#pragma unroll 4
+    for (int i = 0; i < h.w; ++i) {
+      const size_t o = (size_t)(h.z + i) * kGxLanes + g.tid;
+      s = fma(__ldg(jp.part_coef + o), w.dq[2 * nr + __ldg(jp.part_tb + o)], s);
+    }
+    if (pos >= 0) Jm[(1 + (pos >> 16)) * LD + 1 + (pos & 0xffff)] = s;
   }
   if (g.tid == 0) w.sc[S_IRCP] = ircp;
   g.sync();
@@ -938,7 +954,8 @@ __device__ __forceinline__ void eval_fx(const Grp<G>& g, const GxView& m, const 
     w.rk[k] = dk * rS - w.row[k];
     Jm[(1 + k) * LD] = -(m.W[k] * invrho * (w.dwdT[k] - dk * t.invT));
   }
-  for (int mm = g.tid; mm < ns; mm += G) {
+  // the column sums on the group's second half while the first half still forms the row sums
+  for (int mm = (g.tid + G / 2) % G; mm < ns; mm += G) {
     double s = 0.0;
     for (int k = 0; k < ns; ++k) s = fma(w.hRT[k], Jm[(1 + k) * LD + 1 + mm], s);
     w.Hm[mm] = s;
@@ -1061,7 +1078,7 @@ __device__ bool lu_factor_panel(const Grp<G>& g, double* M, int N, int LD, int* 
     unsigned long long best = 0ull;
     int bi = 0;
     for (int i = l; i < N; i += 32) argmax_merge(best, bi, pivot_key(M[i * LD]), i);
-    warp_argmax<G>(g, best, bi);
+    warp_argmax_redux(best, bi);
     for (int i = l; i < N; i += 32) pbuf[i] = i == 0 ? bi : (i == bi ? 0 : i);
     if (best != 0ull) {
       const double ip = fx::rcp(M[bi * LD]);
@@ -1097,7 +1114,7 @@ __device__ bool lu_factor_panel(const Grp<G>& g, double* M, int N, int LD, int* 
         v1 = fma(-M[ph1 * LD + k], ukj, M[ph1 * LD + k + 1]);
         argmax_merge(best, bi, pivot_key(v1), i1);
       }
-      warp_argmax<G>(g, best, bi);
+      warp_argmax_redux(best, bi);
       const int pnew = Pk[bi], pold = Pk[k + 1];
       for (int i = k + 1 + l; i < N; i += 32) Pn[i] = i == k + 1 ? pnew : (i == bi ? pold : Pk[i]);
       if (best != 0ull) {
@@ -1218,12 +1235,136 @@ __device__ void lu_solve_regs(const Grp<G>& g, const double* M, int N, int LD, c
   g.sync();
 }
 
+// Triangular solves of a 128-thread group (N <= 64) by blocks of eight unknowns.  The six solves of
+// an attempt are its longest dependent chains: one warp sweeping row by row (lu_solve_regs) takes
+// about 200 FP64 instructions of 64 cycles in one sub-partition plus a shuffle and a shared-memory
+// round trip per unknown, 52 k cycles of the 53-species cell's 117 k per solve-and-stage; here the
+// diagonal blocks of L and U are inverted once per attempt, so a block's unknowns are one small
+// matrix-vector product in the warp that owns its rows, and every warp then updates its rows with
+// the block: 7 steps per sweep instead of 54.
+//
+// invert_diag_blocks: in place, L's (strictly lower part, unit diagonal implied) and U's (diagonal
+// included) 8 x 8 diagonal blocks replaced by their inverses, one column per lane (lanes 0-63: L,
+// 64-127: U), by substitution.
+__device__ void invert_diag_blocks(const Grp<128>& g, double* M, int N, int LD, const int* perm, const double* invd) {
+  const int q = g.tid & 63, c = q & 7, i0 = q & ~7, nb = N - i0;
+  const bool upper = g.tid >= 64, mine = c < nb;
+  double v[8];
+  int ro[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    ro[i] = i < nb ? perm[i0 + i] * LD + i0 : 0;
+    v[i] = 0.0;
+  }
+  if (mine) {
+    if (!upper) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        double s = 0.0;
+#pragma unroll
+        for (int k = 0; k < i; ++k) s = fma(i < nb ? M[ro[i] + k] : 0.0, v[k], s);
+        v[i] = i == c ? 1.0 : -s;                    // zero above the diagonal: s = 0 there
+      }
+    } else {
+#pragma unroll
+      for (int i = 7; i >= 0; --i) {
+        double s = 0.0;
+#pragma unroll
+        for (int k = 7; k > i; --k) s = fma(k < nb ? M[ro[i] + k] : 0.0, v[k], s);
+        const double d = i < nb ? invd[i0 + i] : 0.0;
+        v[i] = i == c ? d : -s * d;
+      }
+    }
+  }
+  g.sync();
+  if (mine) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (i < nb && (upper ? i <= c : i > c)) M[ro[i] + c] = v[i];
+  }
+  g.sync();
+}
+
+// b (length N, shared) is overwritten with the solution; xs: N doubles of scratch.  Row i belongs
+// to lanes 2 i and 2 i + 1 (one warp), each with half of a block's columns and of the row's sum.
+__device__ void lu_solve_blocks(const Grp<128>& g, const double* M, int N, int LD, const int* perm, double* b,
+                                double* xs) {
+  constexpr unsigned F = 0xffffffffu;
+  const int i = g.tid >> 1, h = g.tid & 1, warp = g.tid >> 5, il = i & 7;
+  const bool valid = i < N;
+  const int pr = valid ? perm[i] : 0;
+  const double* row = M + pr * LD + 4 * h;
+  const int nblk = (N + 7) >> 3, lane0 = (g.tid & 16) + 8 * h;    // first lane of the block's columns 4 h ..
+  double r = valid && h == 0 ? b[pr] : 0.0;
+  for (int bk = 0; bk < nblk; ++bk) {                // L y = P b
+    const bool later = valid && i >= 8 * bk + 8;
+    double m[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) m[k] = later || (valid && (i >> 3) == bk && 4 * h + k < il) ? row[8 * bk + k] : 0.0;
+    if (warp == bk >> 1) {
+      const double s = r + __shfl_xor_sync(F, r, 1);
+      double a = 0.0;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const double rk = __shfl_sync(F, s, lane0 + 2 * k);
+        a = fma((i >> 3) == bk ? m[k] : 0.0, rk, a);
+      }
+      a += __shfl_xor_sync(F, a, 1);
+      if ((i >> 3) == bk) {
+        r = h == 0 ? s + a : 0.0;                    // y_i
+        if (valid && h == 0) xs[i] = r;
+      }
+    }
+    g.sync();
+    if (later) {
+      const double2 x01 = *reinterpret_cast<const double2*>(xs + 8 * bk + 4 * h);
+      const double2 x23 = *reinterpret_cast<const double2*>(xs + 8 * bk + 4 * h + 2);
+      r = fma(-m[0], x01.x, r);
+      r = fma(-m[1], x01.y, r);
+      r = fma(-m[2], x23.x, r);
+      r = fma(-m[3], x23.y, r);
+    }
+  }
+  for (int bk = nblk - 1; bk >= 0; --bk) {           // U x = y; r still holds y_i (lane 2 i) and 0
+    const bool earlier = valid && i < 8 * bk;
+    double m[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const bool in = 8 * bk + 4 * h + k < N;
+      m[k] = in && (earlier || (valid && (i >> 3) == bk && 4 * h + k >= il)) ? row[8 * bk + k] : 0.0;
+    }
+    if (warp == bk >> 1) {
+      const double s = r + __shfl_xor_sync(F, r, 1);
+      double a = 0.0;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const double rk = __shfl_sync(F, s, lane0 + 2 * k);
+        a = fma((i >> 3) == bk ? m[k] : 0.0, rk, a);
+      }
+      a += __shfl_xor_sync(F, a, 1);
+      if (valid && (i >> 3) == bk && h == 0) { xs[i] = a; b[i] = a; }
+    }
+    g.sync();
+    if (earlier) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (8 * bk + 4 * h + k < N) r = fma(-m[k], xs[8 * bk + 4 * h + k], r);
+    }
+  }
+}
+
 // Solves A x = b with the factors of lu_factor; b (length N) is overwritten with x.  t: N-double
 // scratch holding the permuted right-hand side during the two triangular sweeps.  The division
 // by the diagonal of U happens once per row, in the thread that finishes that row.
 template <int G>
 __device__ void lu_solve(const Grp<G>& g, const double* M, int N, int LD, const int* perm,
                          const double* invd, double* b, double* t) {
+  if constexpr (G == 128) {
+    if (N <= 64) {                                   // after invert_diag_blocks
+      lu_solve_blocks(g, M, N, LD, perm, b, t);
+      return;
+    }
+  }
   if constexpr (G >= 32) {
     if (N <= 64) {
       lu_solve_regs<G>(g, M, N, LD, perm, invd, b, t);
@@ -1331,6 +1472,9 @@ __device__ bool rodas4_attempt(const Grp<G>& g, const typename Form<FX>::View& m
     regular = lu_factor<G>(g, w.M, N, LD, w.perm, w.invd, w.red);
   }
   if (!regular) return false;
+  if constexpr (G == 128) {
+    if (N <= 64) invert_diag_blocks(g, w.M, N, LD, w.perm, w.invd);
+  }
   for (int s = 0; s < 6; ++s) {
     const double* src = w.f0;
     if (s > 0) {

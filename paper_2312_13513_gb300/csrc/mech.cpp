@@ -391,31 +391,48 @@ int build_gx(const chem_mech_desc* d, chem_mech_s* m, const FxNumbers& F, const 
       for (int e = T.off[T.tb_of[j]]; e < T.off[T.tb_of[j] + 1]; ++e)
         ent[{k, T.idx[e]}].part.push_back({T.tb_of[j], nu[j][k] * T.val[e]});
     }
-  // entries with much work first: threads take consecutive entries, so a warp's are alike
+  // entries with many terms first, so that the lanes of a chunk have similar counts
   std::vector<const std::pair<const std::pair<int, int>, Entry>*> order;
   for (auto& kv : ent) order.push_back(&kv);
   std::stable_sort(order.begin(), order.end(), [](const auto* a, const auto* b) {
-    return 2 * a->second.slot.size() + a->second.part.size() > 2 * b->second.slot.size() + b->second.part.size();
+    if (a->second.slot.size() != b->second.slot.size()) return a->second.slot.size() > b->second.slot.size();
+    return a->second.part.size() > b->second.part.size();
   });
-  std::vector<int> so(1, 0), po(1, 0), ss, sx, pt, ro(1, 0), rs;
+  const int nchunk = (int)((order.size() + kGxLanes - 1) / kGxLanes);
+  std::vector<int4> chunk;
+  std::vector<int> pos((size_t)nchunk * kGxLanes, -1), pt, ro(1, 0), rs;
+  std::vector<int2> ss;
   std::vector<double> pc;
-  std::vector<int16_t> er, ec;
-  for (const auto* kv : order) {
-    er.push_back((int16_t)kv->first.first);
-    ec.push_back((int16_t)kv->first.second);
-    for (auto& t : kv->second.slot) { ss.push_back(t.first); sx.push_back(t.second); }
-    for (auto& t : kv->second.part) { pt.push_back(t.first); pc.push_back(t.second); }
-    so.push_back((int)ss.size());
-    po.push_back((int)pt.size());
+  for (int c = 0; c < nchunk; ++c) {
+    const size_t e0 = (size_t)c * kGxLanes, e1 = std::min(order.size(), e0 + kGxLanes);
+    size_t nsl = 0, npt = 0;
+    for (size_t e = e0; e < e1; ++e) {
+      nsl = std::max(nsl, order[e]->second.slot.size());
+      npt = std::max(npt, order[e]->second.part.size());
+      pos[e] = (order[e]->first.first << 16) | order[e]->first.second;
+    }
+    const size_t s0 = ss.size() / kGxLanes, p0 = pt.size() / kGxLanes;
+    chunk.push_back(int4{(int)s0, (int)nsl, (int)p0, (int)npt});
+    ss.resize(ss.size() + nsl * kGxLanes, int2{8, ns | (ns << 16)});
+    pt.resize(pt.size() + npt * kGxLanes, 0);
+    pc.resize(pc.size() + npt * kGxLanes, 0.0);
+    for (size_t e = e0; e < e1; ++e) {
+      const Entry& E = order[e]->second;
+      for (size_t i = 0; i < E.slot.size(); ++i)
+        ss[(s0 + i) * kGxLanes + (e - e0)] = int2{E.slot[i].first, E.slot[i].second};
+      for (size_t i = 0; i < E.part.size(); ++i) {
+        pt[(p0 + i) * kGxLanes + (e - e0)] = E.part[i].first;
+        pc[(p0 + i) * kGxLanes + (e - e0)] = E.part[i].second;
+      }
+    }
   }
   for (int k = 0; k < ns; ++k) { rs.insert(rs.end(), rows[k].begin(), rows[k].end()); ro.push_back((int)rs.size()); }
   Builder J;
-  const int o_so = J.add(4 * (int)so.size()), o_po = J.add(4 * (int)po.size()), o_er = J.add(2 * (int)er.size()),
-            o_ec = J.add(2 * (int)ec.size()), o_ss = J.add(4 * (int)ss.size()), o_sx = J.add(4 * (int)sx.size()),
+  const int o_ch = J.add(16 * (int)chunk.size()), o_ep = J.add(4 * (int)pos.size()), o_ss = J.add(8 * (int)ss.size()),
             o_pt = J.add(4 * (int)pt.size()), o_pc = J.add(8 * (int)pc.size()), o_ro = J.add(4 * (int)ro.size()),
             o_rs = J.add(4 * (int)rs.size()), o_lg = J.add(sizeof(kLog2Tab)), o_rc = J.add(sizeof(kRcpTab));
-  put(J, o_so, so); put(J, o_po, po); put(J, o_er, er); put(J, o_ec, ec); put(J, o_ss, ss); put(J, o_sx, sx);
-  put(J, o_pt, pt); put(J, o_pc, pc); put(J, o_ro, ro); put(J, o_rs, rs);
+  put(J, o_ch, chunk); put(J, o_ep, pos); put(J, o_ss, ss); put(J, o_pt, pt); put(J, o_pc, pc); put(J, o_ro, ro);
+  put(J, o_rs, rs);
   memcpy(J.at<unsigned char>(o_lg), kLog2Tab, sizeof(kLog2Tab));
   memcpy(J.at<unsigned char>(o_rc), kRcpTab, sizeof(kRcpTab));
   CHEM_CUDA_TRY(cudaMalloc(&m->d_gx, B.buf.size()));
@@ -423,10 +440,14 @@ int build_gx(const chem_mech_desc* d, chem_mech_s* m, const FxNumbers& F, const 
   CHEM_CUDA_TRY(cudaMalloc(&m->d_gxj, J.buf.size()));
   CHEM_CUDA_TRY(cudaMemcpy(m->d_gxj, J.buf.data(), J.buf.size(), cudaMemcpyHostToDevice));
   const unsigned char* g = (const unsigned char*)m->d_gxj;
-  m->gxj = GxJac{(int)er.size(),           (const int*)(g + o_so),     (const int*)(g + o_po),
-                 (const int16_t*)(g + o_er), (const int16_t*)(g + o_ec), (const int*)(g + o_ss),
-                 (const int*)(g + o_sx),     (const int*)(g + o_pt),     (const double*)(g + o_pc),
-                 (const int*)(g + o_ro),     (const int*)(g + o_rs)};
+  m->gxj = GxJac{nchunk,
+                 (const int4*)(g + o_ch),
+                 (const int*)(g + o_ep),
+                 (const int2*)(g + o_ss),
+                 (const int*)(g + o_pt),
+                 (const double*)(g + o_pc),
+                 (const int*)(g + o_ro),
+                 (const int*)(g + o_rs)};
   m->d_lg = (const unsigned long long*)(g + o_lg);
   m->d_rc = (const unsigned int*)(g + o_rc);
   m->gx = L;
