@@ -92,8 +92,9 @@ struct chem_mech_s {
   void* d_fx = nullptr;
   chem::GxLayout gx{};                    // the group kernels' fixed-point form, bytes = 0: none
   chem::GxJac gxj{};
-  void *d_gx = nullptr, *d_gxj = nullptr; // blob; Jacobian program, then log2 and reciprocal tables
-  const unsigned long long* d_lg = nullptr;
+  void *d_gx = nullptr, *d_gxj = nullptr; // blob; Jacobian program
+  void* d_tab = nullptr;                  // tables of fixed.cuh
+  const unsigned long long *d_e2 = nullptr, *d_lg = nullptr;
   const unsigned int* d_rc = nullptr;
 };
 

@@ -78,25 +78,25 @@ struct GxLayout {
   int64_t lpr0;
 };
 
-// Jacobian-assembly program of the group kernels with the fixed-point form (global memory).  Entry e
-// (row, column of d(wdot)/dC at ent_pos = row << 16 | column, -1: none) is lane e % kGxLanes of
-// chunk e / kGxLanes; chunk = (first slot row, slot rows, first partner row, partner rows), and term
-// row r of lane t lies at r * kGxLanes + t: coalesced loads without dependent offsets (entries
-// sorted by their term counts, short ones padded with terms of coefficient 0).  A slot term is the
-// derivative of one direction of reaction j with respect to one of its species: slot.x =
-// (2 j + side) << 4 | (nu + 8), times the concentrations of the side's other species slot.y =
-// o1 | o2 << 16.  Collision partners: d(wdot_k)/dC_m = sum_j nu_kj X_j eff_jm = R_k +
-// sum_j nu_kj X_j (eff_jm - 1), with R_k = sum_j nu_kj X_j the same for every column: only the sparse
-// deviations are terms (part_tb = set, part_coef = nu (eff - 1)); R_k (row_off, row_src =
-// set << 4 | (nu + 8)) joins the chain rule.  For the 53-species mechanism this leaves 4.4 k slot
-// and 2.8 k partner terms of 13.1 k.
+// Jacobian-assembly program of the group kernels with the fixed-point form (global memory).  The
+// entries of d(wdot)/dC, sorted by their term counts, are dealt to the kGxLanes lanes of a group in
+// chunks of kGxLanes; a chunk is as many term rows as its longest entry needs (terms of coefficient
+// 0 fill the others), and term row r of lane t lies at r * kGxLanes + t, chunk after chunk: one
+// coalesced stream that a lane can read ahead.  A lane's entry ends with the row whose z (slot) or
+// y (part) is not -1: its place row << 16 | column.
+// A slot term is the derivative of one direction of reaction j with respect to one of its species
+// for one unit of net coefficient: x = (2 j + side) << 1 | (coefficient negative), a null term points
+// at the zero behind the 2 nr derivatives; y = o1 | o2 << 16, the side's other species.
+// Collision partners: d(wdot_k)/dC_m = sum_j nu_kj X_j eff_jm = R_k + sum_j nu_kj X_j (eff_jm - 1),
+// with R_k = sum_j nu_kj X_j the same for every column: only the sparse deviations are terms
+// (x = set, coefficient nu (eff - 1)); R_k (row_off, row_src = set << 4 | (nu + 8)) joins the chain
+// rule.  For the 53-species mechanism this leaves 4.4 k slot and 2.8 k partner terms of 13.1 k.
 constexpr int kGxLanes = 128;
+constexpr int kGxUnroll = 4;                               // term rows are a multiple of this
 struct GxJac {
-  int nchunk = 0;
-  const int4* chunk = nullptr;
-  const int* ent_pos = nullptr;
-  const int2* slot = nullptr;
-  const int* part_tb = nullptr;
+  int nslot = 0, npart = 0;                                // term rows
+  const int4* slot = nullptr;
+  const int2* part = nullptr;
   const double* part_coef = nullptr;
   const int *row_off = nullptr, *row_src = nullptr;        // [ns + 1], terms of R_k
 };

@@ -52,6 +52,16 @@ __device__ __forceinline__ bool positive_normal(double x) {
   return (unsigned)__double2hiint(x) - 0x00100000u < 0x7ff00000u - 0x00100000u;
 }
 
+// Step-size factor 0.9 e^(-1/4) of an error norm e = sqrt(en2), at least 0.2; 0.2 for a non-finite
+// norm.  2^(-log2(en2) / 8) in fixed point (sqrt and pow are 92 FP64 instructions).
+__device__ __forceinline__ double step_factor(double en2, const u64* e2, const uint32_t* rc, const u64* lg) {
+  if (((unsigned)__double2hiint(en2) & 0x7ff00000u) == 0x7ff00000u) return 0.2;
+  if (!positive_normal(en2)) return 1e30;                  // en2 = 0: the caller's limit bounds it
+  const i64 X = -(log2_q52(en2, rc, lg) >> 3);
+  const double f = 0.9 * exp2_q52(X, e2);
+  return f < 0.2 ? 0.2 : f;
+}
+
 // thermo state of a right-hand side at one temperature
 struct Temp {
   double T, invT;

@@ -172,7 +172,7 @@ inline WsLayout make_ws(int ns, int nr, int npieces, int G, bool fx, int ntb) {
   // evaluation, at the start of an attempt, when the stage buffers ys, fs and u (contiguous
   // above) are dead: small mechanisms keep them there
   const int stage_span = w.M - w.ys;
-  const int ndq = fx ? 2 * nr + ntb : 3 * nr;
+  const int ndq = fx ? 2 * nr + 1 + ntb : 3 * nr;       // a zero for null terms in between
   w.dq = ndq <= stage_span ? w.ys : take(ndq);
   w.row = take(fx ? ns : 0);
   // partial production sums of the balanced pieces (groups wider than a warp)
@@ -793,6 +793,7 @@ __device__ __forceinline__ void eval_fx(const Grp<G>& g, const GxView& m, const 
   g.sync();
 
   // rates of progress (A3)
+  if (jac && g.tid == 0) w.dq[2 * nr] = 0.0;
   const double Ctot = rho * S;
   const fx::i64 D = (fx::i64)((t.L + 128ull) >> 8) - m.lpr0;
   const fx::i64 shift = t.iT2 - t.L2;
@@ -853,7 +854,7 @@ __device__ __forceinline__ void eval_fx(const Grp<G>& g, const GxView& m, const 
     w.dqdT[j] = mult * fma(net, dlnkf, rev * (dH * t.invT));
     w.dq[2 * j] = mult * kf;
     w.dq[2 * j + 1] = -mult * kr;
-    if (ri.x != 0) w.dq[2 * nr + ri.z] = ri.x == 1 ? net : (fastk ? dMr * net : dkfdM * (Pf - Pr * invKc));
+    if (ri.x != 0) w.dq[2 * nr + 1 + ri.z] = ri.x == 1 ? net : (fastk ? dMr * net : dkfdM * (Pf - Pr * invKc));
   }
   g.sync();
 
@@ -891,7 +892,7 @@ __device__ __forceinline__ void eval_fx(const Grp<G>& g, const GxView& m, const 
       const int t1 = __ldg(jp.row_off + k + 1);
       for (int e = __ldg(jp.row_off + k); e < t1; ++e) {
         const int src = __ldg(jp.row_src + e);
-        R = fma(m.nu[src & 15], w.dq[2 * nr + (src >> 4)], R);
+        R = fma(m.nu[src & 15], w.dq[2 * nr + 1 + (src >> 4)], R);
       }
       w.row[k] = R;
       r3[3] = fma(hk, R, r3[3]);
@@ -921,23 +922,56 @@ __device__ __forceinline__ void eval_fx(const Grp<G>& g, const GxView& m, const 
     Jm[(1 + k) * LD + 1 + (e - k * ns)] = 0.0;
   }
   g.sync();
-  for (int c = 0; c < jp.nchunk; ++c) {
-    const int4 h = __ldg(jp.chunk + c);                     // first slot row, slot rows, partner rows
-    const int pos = __ldg(jp.ent_pos + c * kGxLanes + g.tid);
+  {
+    // four term rows are read while the previous four are summed
     double s = 0.0;
-#pragma unroll 4
-    for (int i = 0; i < h.y; ++i) {
-      const int2 tm = __ldg(jp.slot + (size_t)(h.x + i) * kGxLanes + g.tid);
-      double d = w.dq[tm.x >> 4] * w.C[tm.y & 0xffff];
-      if ((tm.y >> 16) != ns) d *= w.C[tm.y >> 16];
-      s = fma(m.nu[tm.x & 15], d, s);
+    int4 cur[kGxUnroll];
+    const int4* sp = jp.slot + g.tid;
+#pragma unroll
+    for (int i = 0; i < kGxUnroll; ++i) cur[i] = __ldg(sp + i * kGxLanes);
+    for (int r = 0; r < jp.nslot; r += kGxUnroll) {
+      int4 nxt[kGxUnroll];
+      sp += kGxUnroll * kGxLanes;
+      const bool more = r + kGxUnroll < jp.nslot;
+#pragma unroll
+      for (int i = 0; i < kGxUnroll; ++i) nxt[i] = more ? __ldg(sp + i * kGxLanes) : cur[i];
+#pragma unroll
+      for (int i = 0; i < kGxUnroll; ++i) {
+        const int4 tm = cur[i];
+        double d = w.dq[tm.x >> 1];
+        d = __hiloint2double(__double2hiint(d) ^ (int)((unsigned)tm.x << 31), __double2loint(d));
+        if ((tm.y >> 16) != ns) d *= w.C[tm.y >> 16];
+        s = fma(d, w.C[tm.y & 0xffff], s);
+        if (tm.z != -1) {
+          Jm[(1 + (tm.z >> 16)) * LD + 1 + (tm.z & 0xffff)] = s;
+          s = 0.0;
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < kGxUnroll; ++i) cur[i] = nxt[i];
     }
-#pragma unroll 4
-    for (int i = 0; i < h.w; ++i) {
-      const size_t o = (size_t)(h.z + i) * kGxLanes + g.tid;
-      s = fma(__ldg(jp.part_coef + o), w.dq[2 * nr + __ldg(jp.part_tb + o)], s);
+    // the partner terms: a lane adds to the entries it wrote itself
+    s = 0.0;
+#pragma unroll 1
+    for (int r = 0; r < jp.npart; r += kGxUnroll) {
+      int2 tm[kGxUnroll];
+      double co[kGxUnroll];
+#pragma unroll
+      for (int i = 0; i < kGxUnroll; ++i) {
+        const size_t o = (size_t)(r + i) * kGxLanes + g.tid;
+        tm[i] = __ldg(jp.part + o);
+        co[i] = __ldg(jp.part_coef + o);
+      }
+#pragma unroll
+      for (int i = 0; i < kGxUnroll; ++i) {
+        s = fma(co[i], w.dq[2 * nr + 1 + tm[i].x], s);
+        if (tm[i].y != -1) {
+          double* x = Jm + (1 + (tm[i].y >> 16)) * LD + 1 + (tm[i].y & 0xffff);
+          *x += s;
+          s = 0.0;
+        }
+      }
     }
-    if (pos >= 0) Jm[(1 + (pos >> 16)) * LD + 1 + (pos & 0xffff)] = s;
   }
   if (g.tid == 0) w.sc[S_IRCP] = ircp;
   g.sync();
@@ -1109,7 +1143,7 @@ __device__ bool lu_factor_panel(const Grp<G>& g, double* M, int N, int LD, int* 
         v0 = fma(-M[ph0 * LD + k], ukj, M[ph0 * LD + k + 1]);
         argmax_merge(best, bi, pivot_key(v0), i0);
       }
-      if (i1 < N) {
+      if (k + 33 < N && i1 < N) {
         ph1 = Pk[i1];
         v1 = fma(-M[ph1 * LD + k], ukj, M[ph1 * LD + k + 1]);
         argmax_merge(best, bi, pivot_key(v1), i1);
@@ -1303,7 +1337,7 @@ __device__ void lu_solve_blocks(const Grp<128>& g, const double* M, int N, int L
     for (int k = 0; k < 4; ++k) m[k] = later || (valid && (i >> 3) == bk && 4 * h + k < il) ? row[8 * bk + k] : 0.0;
     if (warp == bk >> 1) {
       const double s = r + __shfl_xor_sync(F, r, 1);
-      double a = 0.0;
+      double a = h == 0 ? s : 0.0;                   // the unit diagonal
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         const double rk = __shfl_sync(F, s, lane0 + 2 * k);
@@ -1311,7 +1345,7 @@ __device__ void lu_solve_blocks(const Grp<128>& g, const double* M, int N, int L
       }
       a += __shfl_xor_sync(F, a, 1);
       if ((i >> 3) == bk) {
-        r = h == 0 ? s + a : 0.0;                    // y_i
+        r = h == 0 ? a : 0.0;                        // y_i
         if (valid && h == 0) xs[i] = r;
       }
     }
@@ -1403,7 +1437,7 @@ struct MechArgs {
   JacArgs jp;
   GxJac gj;
   const unsigned char *blob, *gxblob;
-  const fx::u64* lg;
+  const fx::u64 *e2, *lg;      // the tables of fixed.cuh in global memory
   const uint32_t* rc;
 };
 
@@ -1448,7 +1482,7 @@ __device__ __forceinline__ void stage_mech(const unsigned char* src, unsigned ch
 }
 
 // One Rodas4 attempt from w.y with step h (f and J re-evaluated at w.y).  Returns false on an
-// exactly singular iteration matrix; otherwise *en receives the error norm and *fac the step-size
+// exactly singular iteration matrix; otherwise *en receives the squared error norm and *fac the step-size
 // factor 0.9 en^(-1/4) (clamped below at 0.2; 0.2 for a non-finite norm), evaluated once per
 // group.
 template <int G, bool FX>
@@ -1458,7 +1492,7 @@ __device__ bool rodas4_attempt(const Grp<G>& g, const typename Form<FX>::View& m
   constexpr bool kMulti = G > 32;
   const int N = m.N, LD = P.ws.LD;
   double ig = 0.0, invh = 0.0;
-  if (is_lead(g)) { ig = 1.0 / (kGamma * h); invh = 1.0 / h; }
+  if (is_lead(g)) { invh = fx::rcp(h); ig = invh * (1.0 / kGamma); }
   if (kMulti && g.tid == 0) { w.sc[S_IG] = ig; w.sc[S_INVH] = invh; }
   Form<FX>::template eval<G>(g, m, w, P, w.y, p, w.f0, w.M);      // M = -J; synchronises
   if (kMulti) { ig = w.sc[S_IG]; invh = w.sc[S_INVH]; }
@@ -1480,7 +1514,7 @@ __device__ bool rodas4_attempt(const Grp<G>& g, const typename Form<FX>::View& m
     if (s > 0) {
       for (int i = g.tid; i < N; i += G) {
         double v = w.y[i];
-        for (int j = 0; j < s; ++j) v += kRA[s][j] * w.u[j * N + i];
+        for (int j = 0; j < s; ++j) v = fma(kRA[s][j], w.u[j * N + i], v);
         w.ys[i] = v;
       }
       g.sync();
@@ -1489,9 +1523,9 @@ __device__ bool rodas4_attempt(const Grp<G>& g, const typename Form<FX>::View& m
     }
     double* us = w.u + s * N;
     for (int i = g.tid; i < N; i += G) {
-      double v = src[i];
-      for (int j = 0; j < s; ++j) v += (kRC[s][j] * invh) * w.u[j * N + i];
-      us[i] = v;
+      double v = 0.0;
+      for (int j = 0; j < s; ++j) v = fma(kRC[s][j], w.u[j * N + i], v);
+      us[i] = fma(v, invh, src[i]);
     }
     g.sync();
     lu_solve<G>(g, w.M, N, LD, w.perm, w.invd, us, w.tmp);
@@ -1500,21 +1534,17 @@ __device__ bool rodas4_attempt(const Grp<G>& g, const typename Form<FX>::View& m
   for (int i = g.tid; i < N; i += G) {
     double v = w.y[i];
 #pragma unroll
-    for (int s = 0; s < 6; ++s) v += kRM[s] * w.u[s * N + i];
+    for (int s = 0; s < 6; ++s) v = fma(kRM[s], w.u[s * N + i], v);
     w.ynew[i] = v;
-    const double sc = atol + rtol * fmax(fabs(w.y[i]), fabs(v));
-    const double r = w.u[5 * N + i] / sc;
-    acc[0] += r * r;
+    const double sc = fma(rtol, fx::max_pos(fabs(w.y[i]), fabs(v)), atol);
+    const double r = w.u[5 * N + i] * fx::rcp(sc);
+    acc[0] = fma(r, r, acc[0]);
   }
   gsum_lead<G, 1>(g, acc, w.red, N);
   double e = 0.0, f = 0.0;
   if (is_lead(g)) {
-    e = sqrt(acc[0] / (double)N);
-    f = 0.2;
-    if (isfinite(e)) {
-      f = 0.9 * pow(e, -0.25);
-      if (f < 0.2) f = 0.2;
-    }
+    e = acc[0] * (1.0 / (double)N);                  // the squared norm
+    f = fx::step_factor(e, P.e2, P.rc, P.lg);
   }
   if (kMulti) {
     if (g.tid == 0) { w.sc[S_EN] = e; w.sc[S_FAC] = f; }
@@ -1884,7 +1914,7 @@ JacArgs jac_args(const chem_mech_s* m);
 void mech_args(const chem_mech_s* m, const LaunchShape& s, MechArgs* A) {
   A->lay = m->lay; A->gx = m->gx; A->ws = s.ws; A->jp = jac_args(m); A->gj = m->gxj;
   A->blob = (const unsigned char*)m->d_blob; A->gxblob = (const unsigned char*)m->d_gx;
-  A->lg = m->d_lg; A->rc = m->d_rc;
+  A->e2 = m->d_e2; A->lg = m->d_lg; A->rc = m->d_rc;
 }
 
 JacArgs jac_args(const chem_mech_s* m) {

@@ -153,16 +153,6 @@ __device__ __forceinline__ bool attempt(const cell::View& m, double* col, double
   return !singular;
 }
 
-// Step-size factor 0.9 e^(-1/4) of an error norm e = sqrt(e2), at least 0.2; 0.2 for a non-finite
-// norm.  2^(-log2(e2) / 8) in fixed point (pow is 83 FP64 instructions).
-__device__ __forceinline__ double step_factor(double e2, const cell::View& m) {
-  if (!isfinite(e2)) return 0.2;
-  if (!fx::positive_normal(e2)) return 1e30;             // e2 = 0: the caller's facmax bounds it
-  const fx::i64 X = -(fx::log2_q52(e2, m.rc, m.lg) >> 3);
-  const double f = 0.9 * fx::exp2_q52(X, m.e2);
-  return f < 0.2 ? 0.2 : f;
-}
-
 template <int NS>
 __global__ void __launch_bounds__(128, 1) cell_advance_kernel(const __grid_constant__ CellParams P) {
   using w = Ws<NS>;
@@ -260,7 +250,7 @@ __global__ void __launch_bounds__(128, 1) cell_advance_kernel(const __grid_const
         stop = true; status = CHEM_CELL_SINGULAR_LU;
       } else {
         ++attempts;
-        const double fac = step_factor(e2, m);
+        const double fac = fx::step_factor(e2, m.e2, m.rc, m.lg);
         if (e2 <= 1.0) {
 #pragma unroll
           for (int i = 0; i < N; ++i) col[(w::Y + i) * 32] = col[(w::U + 5 * N + i) * 32];

@@ -319,8 +319,8 @@ std::vector<unsigned char> build_fx(const chem_mech_desc* d, const chem_mech_s* 
   return B.buf;
 }
 
-// Blob of the group kernels' fixed-point form, and their Jacobian program with the log2 and
-// reciprocal tables behind it (one global allocation each, uploaded here).
+// Blob of the group kernels' fixed-point form, and their Jacobian program (one global allocation
+// each, uploaded here).
 int build_gx(const chem_mech_desc* d, chem_mech_s* m, const FxNumbers& F, const std::vector<std::vector<int>>& nu,
              const MechLayout& ML, const Builder& MB) {
   const int ns = d->n_species, nr = d->n_reactions;
@@ -384,7 +384,8 @@ int build_gx(const chem_mech_desc* d, chem_mech_s* m, const FxNumbers& F, const 
         if (side[sl] < 0) continue;
         const int a1 = sl == 0 ? 1 : 0, a2 = sl == 2 ? 1 : 2;
         const int o1 = side[a1] >= 0 ? side[a1] : ns, o2 = side[a2] >= 0 ? side[a2] : ns;
-        ent[{k, side[sl]}].slot.push_back({((2 * j + (s >= 3)) << 4) | (nu[j][k] + 8), o1 | (o2 << 16)});
+        for (int u = 0; u < std::abs(nu[j][k]); ++u)
+          ent[{k, side[sl]}].slot.push_back({((2 * j + (s >= 3)) << 1) | (nu[j][k] < 0), o1 | (o2 << 16)});
       }
       if (T.tb_of[j] < 0) continue;
       rows[k].push_back((T.tb_of[j] << 4) | (nu[j][k] + 8));
@@ -398,58 +399,54 @@ int build_gx(const chem_mech_desc* d, chem_mech_s* m, const FxNumbers& F, const 
     if (a->second.slot.size() != b->second.slot.size()) return a->second.slot.size() > b->second.slot.size();
     return a->second.part.size() > b->second.part.size();
   });
-  const int nchunk = (int)((order.size() + kGxLanes - 1) / kGxLanes);
-  std::vector<int4> chunk;
-  std::vector<int> pos((size_t)nchunk * kGxLanes, -1), pt, ro(1, 0), rs;
-  std::vector<int2> ss;
+  std::vector<int> ro(1, 0), rs;
+  std::vector<int4> ss;
+  std::vector<int2> pt;
   std::vector<double> pc;
-  for (int c = 0; c < nchunk; ++c) {
-    const size_t e0 = (size_t)c * kGxLanes, e1 = std::min(order.size(), e0 + kGxLanes);
-    size_t nsl = 0, npt = 0;
+  for (size_t e0 = 0; e0 < order.size(); e0 += kGxLanes) {
+    const size_t e1 = std::min(order.size(), e0 + kGxLanes);
+    size_t nsl = 1, npt = 0;                         // every entry is written by the slot pass
     for (size_t e = e0; e < e1; ++e) {
       nsl = std::max(nsl, order[e]->second.slot.size());
       npt = std::max(npt, order[e]->second.part.size());
-      pos[e] = (order[e]->first.first << 16) | order[e]->first.second;
     }
-    const size_t s0 = ss.size() / kGxLanes, p0 = pt.size() / kGxLanes;
-    chunk.push_back(int4{(int)s0, (int)nsl, (int)p0, (int)npt});
-    ss.resize(ss.size() + nsl * kGxLanes, int2{8, ns | (ns << 16)});
-    pt.resize(pt.size() + npt * kGxLanes, 0);
-    pc.resize(pc.size() + npt * kGxLanes, 0.0);
+    const size_t s0 = ss.size(), p0 = pt.size();
+    ss.resize(s0 + nsl * kGxLanes, int4{(2 * nr) << 1, ns | (ns << 16), -1, 0});
+    pt.resize(p0 + npt * kGxLanes, int2{0, -1});
+    pc.resize(p0 + npt * kGxLanes, 0.0);
     for (size_t e = e0; e < e1; ++e) {
       const Entry& E = order[e]->second;
-      for (size_t i = 0; i < E.slot.size(); ++i)
-        ss[(s0 + i) * kGxLanes + (e - e0)] = int2{E.slot[i].first, E.slot[i].second};
-      for (size_t i = 0; i < E.part.size(); ++i) {
-        pt[(p0 + i) * kGxLanes + (e - e0)] = E.part[i].first;
-        pc[(p0 + i) * kGxLanes + (e - e0)] = E.part[i].second;
+      const int pos = (order[e]->first.first << 16) | order[e]->first.second;
+      for (size_t i = 0; i < E.slot.size(); ++i) {
+        int4& t = ss[s0 + i * kGxLanes + (e - e0)];
+        t.x = E.slot[i].first;
+        t.y = E.slot[i].second;
       }
+      ss[s0 + (nsl - 1) * kGxLanes + (e - e0)].z = pos;
+      for (size_t i = 0; i < E.part.size(); ++i) {
+        pt[p0 + i * kGxLanes + (e - e0)].x = E.part[i].first;
+        pc[p0 + i * kGxLanes + (e - e0)] = E.part[i].second;
+      }
+      if (npt && !E.part.empty()) pt[p0 + (npt - 1) * kGxLanes + (e - e0)].y = pos;
     }
   }
+  const size_t unit = (size_t)kGxLanes * kGxUnroll;
+  ss.resize((ss.size() + unit - 1) / unit * unit, int4{(2 * nr) << 1, ns | (ns << 16), -1, 0});
+  pt.resize((pt.size() + unit - 1) / unit * unit, int2{0, -1});
+  pc.resize(pt.size(), 0.0);
   for (int k = 0; k < ns; ++k) { rs.insert(rs.end(), rows[k].begin(), rows[k].end()); ro.push_back((int)rs.size()); }
   Builder J;
-  const int o_ch = J.add(16 * (int)chunk.size()), o_ep = J.add(4 * (int)pos.size()), o_ss = J.add(8 * (int)ss.size()),
-            o_pt = J.add(4 * (int)pt.size()), o_pc = J.add(8 * (int)pc.size()), o_ro = J.add(4 * (int)ro.size()),
-            o_rs = J.add(4 * (int)rs.size()), o_lg = J.add(sizeof(kLog2Tab)), o_rc = J.add(sizeof(kRcpTab));
-  put(J, o_ch, chunk); put(J, o_ep, pos); put(J, o_ss, ss); put(J, o_pt, pt); put(J, o_pc, pc); put(J, o_ro, ro);
-  put(J, o_rs, rs);
-  memcpy(J.at<unsigned char>(o_lg), kLog2Tab, sizeof(kLog2Tab));
-  memcpy(J.at<unsigned char>(o_rc), kRcpTab, sizeof(kRcpTab));
+  const int o_ss = J.add(16 * (int)ss.size()), o_pt = J.add(8 * (int)pt.size()), o_pc = J.add(8 * (int)pc.size()),
+            o_ro = J.add(4 * (int)ro.size()), o_rs = J.add(4 * (int)rs.size());
+  put(J, o_ss, ss); put(J, o_pt, pt); put(J, o_pc, pc); put(J, o_ro, ro); put(J, o_rs, rs);
   CHEM_CUDA_TRY(cudaMalloc(&m->d_gx, B.buf.size()));
   CHEM_CUDA_TRY(cudaMemcpy(m->d_gx, B.buf.data(), B.buf.size(), cudaMemcpyHostToDevice));
   CHEM_CUDA_TRY(cudaMalloc(&m->d_gxj, J.buf.size()));
   CHEM_CUDA_TRY(cudaMemcpy(m->d_gxj, J.buf.data(), J.buf.size(), cudaMemcpyHostToDevice));
   const unsigned char* g = (const unsigned char*)m->d_gxj;
-  m->gxj = GxJac{nchunk,
-                 (const int4*)(g + o_ch),
-                 (const int*)(g + o_ep),
-                 (const int2*)(g + o_ss),
-                 (const int*)(g + o_pt),
-                 (const double*)(g + o_pc),
-                 (const int*)(g + o_ro),
+  m->gxj = GxJac{(int)(ss.size() / kGxLanes), (int)(pt.size() / kGxLanes), (const int4*)(g + o_ss),
+                 (const int2*)(g + o_pt),     (const double*)(g + o_pc),   (const int*)(g + o_ro),
                  (const int*)(g + o_rs)};
-  m->d_lg = (const unsigned long long*)(g + o_lg);
-  m->d_rc = (const unsigned int*)(g + o_rc);
   m->gx = L;
   return CHEM_OK;
 }
@@ -651,6 +648,20 @@ int build(const chem_mech_desc* din, chem_mech_s* m) {
   }
   P.nterm = (int)src.size();
 
+  {
+    // the tables of fixed.cuh in global memory: step control of every kernel, temperature functions
+    Builder T;
+    const int o0 = T.add(sizeof(kExp2Tab)), o1 = T.add(sizeof(kLog2Tab)), o2 = T.add(sizeof(kRcpTab));
+    memcpy(T.at<unsigned char>(o0), kExp2Tab, sizeof(kExp2Tab));
+    memcpy(T.at<unsigned char>(o1), kLog2Tab, sizeof(kLog2Tab));
+    memcpy(T.at<unsigned char>(o2), kRcpTab, sizeof(kRcpTab));
+    CHEM_CUDA_TRY(cudaMalloc(&m->d_tab, T.buf.size()));
+    CHEM_CUDA_TRY(cudaMemcpy(m->d_tab, T.buf.data(), T.buf.size(), cudaMemcpyHostToDevice));
+    const unsigned char* t = (const unsigned char*)m->d_tab;
+    m->d_e2 = (const unsigned long long*)(t + o0);
+    m->d_lg = (const unsigned long long*)(t + o1);
+    m->d_rc = (const unsigned int*)(t + o2);
+  }
   const FxNumbers fxn(d, nu);
   const std::vector<unsigned char> fxb = build_fx(d, m, fxn, nu, &m->fx);
   CHEM_CUDA_TRY(cudaGetDevice(&m->device));
@@ -856,6 +867,7 @@ extern "C" int chem_free_mechanism(chem_mech_t m) {
   if (m->d_blob) cudaFree(m->d_blob);
   if (m->d_jac) cudaFree(m->d_jac);
   if (m->d_fx) cudaFree(m->d_fx);
+  if (m->d_tab) cudaFree(m->d_tab);
   if (m->d_gx) cudaFree(m->d_gx);
   if (m->d_gxj) cudaFree(m->d_gxj);
   delete m;
