@@ -73,6 +73,28 @@ __device__ __forceinline__ void mixture_nasa(const unsigned char* blob, const Me
   }
 }
 
+// mixture_nasa for the composition Y[k * ld + cell] in global memory
+__device__ __forceinline__ void mixture_nasa_cell(const unsigned char* blob, const MechLayout& L, int rg,
+                                                  const double* Y, int64_t ld, int64_t cell, double (&Ah)[6],
+                                                  double (&Ac)[5]) {
+  const int ns = L.ns;
+  const double* hc = (const double*)(blob + L.o_hc) + rg * ns * 6;
+  const double* cc = (const double*)(blob + L.o_cpc) + rg * ns * 5;
+  const double* invW = (const double*)(blob + L.o_invW);
+#pragma unroll
+  for (int i = 0; i < 6; ++i) Ah[i] = 0.0;
+#pragma unroll
+  for (int i = 0; i < 5; ++i) Ac[i] = 0.0;
+#pragma unroll 3
+  for (int k = 0; k < ns; ++k) {
+    const double yw = Y[k * ld + cell] * __ldg(invW + k);
+#pragma unroll
+    for (int i = 0; i < 6; ++i) Ah[i] = fma(yw, __ldg(hc + k * 6 + i), Ah[i]);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) Ac[i] = fma(yw, __ldg(cc + k * 5 + i), Ac[i]);
+  }
+}
+
 // h and cp of a mixture polynomial at T; h = R (Ah5 + Ah0 T + ... + Ah4 T^5), no division by T
 __device__ __forceinline__ void h_cp_from_mixture(const double Ah[6], const double Ac[5], double T, double* h,
                                                   double* cp) {

@@ -7,11 +7,16 @@
 //   unchanged).
 // * chem_transport_eval: mixture-averaged viscosity (Wilke), conductivity (Mathur-Saxena) and
 //   diffusion coefficients D_km = (1 - Y_k) / sum_{j != k} X_j / D_jk from cubic fits in ln T.
-//   A group of G threads owns a cell (G = 4 for small mechanisms, 32 for CH4-sized ones): lanes
-//   first evaluate the inverse binary diffusion coefficients once per unordered species pair
-//   (one exponential each, kept in shared memory), then split the species rows of the Wilke and
-//   diffusion sums (ns^2 terms); the per-cell scalars are formed once per group.  Fits, the
-//   pair list and the Wilke weight tables stay in global memory behind the read-only cache.
+//   The FP64 pipe bounds it (19 SM cycles a warp instruction), so
+//   - the fits and their exponentials run in fixed point on the integer pipe (fixed.cuh): no FP64
+//     instruction per pair instead of 13;
+//   - Wilke's sum is expanded: with s = mu^(1/2), sum_j X_j (1 + s_k wq_jk / s_j)^2 cw_kj =
+//     sum_j cw_kj X_j + 2 s_k sum_j (cw wq)_kj X_j / s_j + s_k^2 sum_j (cw wq^2)_kj X_j / s_j^2, three
+//     matrix-vector products with constant matrices: 3 FP64 instructions a pair instead of 5 (all
+//     terms have one sign for non-negative X, nothing cancels);
+//   - small mechanisms (ns <= 15) take one thread per cell, with the cell's vectors in a warp's
+//     interleaved shared memory (conflict-free, no shuffles, no idle lanes); larger ones a warp per
+//     cell, lanes over species and pairs.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -21,7 +26,8 @@
 #include <vector>
 
 #include "chem_internal.h"
-#include "fastexp.cuh"
+#include "fixed.cuh"
+#include "fx_rates.cuh"
 #include "thermo.cuh"
 
 using namespace chem;
@@ -34,9 +40,13 @@ struct chem_transport_s {
   const double* lam_poly = nullptr;    // [ns][4]
   const double* diff_poly = nullptr;   // [ns][ns][4]
   const double* invW = nullptr;        // [ns]
-  const double* wq = nullptr;          // [ns][ns]: (W_j / W_k)^(1/4) at [j * ns + k]
-  const double* cw = nullptr;          // [ns][ns]: (8 (1 + W_k / W_j))^(-1/2) at [k * ns + j]
+  // Wilke's constants cw wq^i, i = 0, 1, 2, of the pair (k, j) at [(i * ns + j) * ns + k], with
+  // wq = (W_j / W_k)^(1/4) and cw = (8 (1 + W_k / W_j))^(-1/2)
+  const double* wilke = nullptr;
   const int* pairs = nullptr;          // [ns (ns - 1) / 2]: j | k << 16, j < k, row-major upper triangle
+  // the fits as base-2 exponents, cubic in log2(T) / 16, Q11.52 with the leading coefficient biased
+  // (fixed.cuh): mu / 2 and lambda per species, -D per pair; null where a coefficient does not fit
+  const long long *mu_fx = nullptr, *lam_fx = nullptr, *diff_fx = nullptr;
 };
 
 namespace {
@@ -60,10 +70,16 @@ __global__ void temperature_from_h_kernel(const unsigned char* blob, MechLayout 
     double Tn = T[c];
     bool conv = false;
     if (isfinite(target) && Tn >= 200.0 && Tn <= 6000.0) {
+      // the composition is fixed during the iteration: its mixture polynomial once per temperature
+      // range visited (11 FP64 instructions a species), then 9 an iteration instead of 13 a species
+      double Ah[6], Ac[5];
+      int rg = -1;
       for (int it = 0; it < 50; ++it) {
+        const int r = Tn < TMID ? 0 : 1;
+        if (r != rg) { rg = r; mixture_nasa_cell(blob, L, rg, Y, ld, c, Ah, Ac); }
         double hh, cp;
-        h_cp_mass(blob, L, Tn, Y, ld, c, nullptr, &hh, &cp);
-        const double dT = (hh - target) / cp;
+        h_cp_from_mixture(Ah, Ac, Tn, &hh, &cp);
+        const double dT = (hh - target) * fx::rcp(cp);
         Tn -= dT;
         if (!(Tn >= 200.0 && Tn <= 6000.0)) break;
         if (fabs(dT) < 1e-9 * Tn) { conv = true; break; }
@@ -74,29 +90,15 @@ __global__ void temperature_from_h_kernel(const unsigned char* blob, MechLayout 
   }
 }
 
-template <int G>
-struct TGrp {
-  int tid, gid;
-  unsigned mask;
-  __device__ void init() {
-    tid = threadIdx.x % G;
-    gid = threadIdx.x / G;
-    mask = G >= 32 ? 0xffffffffu : (((1u << G) - 1u) << ((threadIdx.x & 31) & ~(G - 1)));
-  }
-  __device__ void sync() const { __syncwarp(mask); }
-  __device__ double sum(double v) const {
-#pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
-    return v;
-  }
-};
-
 struct TrParams {
   const double *T, *p, *Y;
   int64_t ld, n;
   double *mu, *lam, *Dm;
-  const double *mu_poly, *lam_poly, *diff_poly, *invW, *wq, *cw;
+  const double *mu_poly, *lam_poly, *diff_poly, *invW, *wilke;
   const int* pairs;
+  const long long *mu_fx, *lam_fx, *diff_fx;
+  const fx::u64 *e2, *lg;
+  const uint32_t* rc;
   int ns;
 };
 
@@ -107,79 +109,239 @@ __device__ __forceinline__ double poly3(const double* c, double x) {
   return __ldg(c) + x * (__ldg(c + 1) + x * (__ldg(c + 2) + x * __ldg(c + 3)));
 }
 
-// G <= 32: a group lives inside one warp, so its synchronisation is a warp-level one
-template <int G>
-__global__ void __launch_bounds__(256) transport_kernel(const TrParams P) {
-  extern __shared__ double tsm[];
-  double* etab = tsm;                        // 2^(j/64) of the table-driven exponential
-  stage_exp_table(etab);
+// Temperature of a cell: in fixed point log2(T) / 16 (Q0.64) for T in [1, 65536), otherwise ln T
+struct FitT {
+  bool fast;
+  fx::u64 l;
+  fx::i64 l2;
+  double lnT;
+};
+
+__device__ __forceinline__ FitT fit_t(double T, const TrParams& P) {
+  FitT t;
+  t.fast = P.mu_fx && (unsigned)__double2hiint(T) - 0x3ff00000u < 0x40f00000u - 0x3ff00000u;
+  int e;
+  const fx::u64 m = fx::mantissa(t.fast ? T : 1024.0, e);
+  const fx::u64 L = ((fx::u64)e << 60) + fx::log2_mant_q60(m, P.rc, P.lg);
+  t.l = e == 0 && (fx::i64)L < 0 ? 0ull : L;               // a few units below zero at T = 1
+  t.l2 = (fx::i64)(t.l >> 1);
+  t.lnT = t.fast ? 0.0 : log(T);
+  return t;
+}
+
+// a fit's base-2 exponent at t: c = 4 coefficients in fixed point
+__device__ __forceinline__ fx::i64 fit_x(const long long* c, const FitT& t) {
+  const fx::u64 B = 0x8000000000000000ull;
+  fx::u64 a = (fx::umulhi3((fx::u64)c[3], t.l) + (fx::u64)(c[2] - t.l2)) ^ B;
+  a = (fx::umulhi3(a, t.l) + (fx::u64)(c[1] - t.l2)) ^ B;
+  return (fx::i64)(fx::umulhi3(a, t.l) + (fx::u64)(c[0] - t.l2));
+}
+__device__ __forceinline__ double exp2_any(fx::i64 X, const fx::u64* e2) {
+  return fx::exp2_in_range(X) ? fx::exp2_q52(X, e2) : exp(fx::to_double(X, 52) * fx::kLn2);
+}
+
+// mu^(1/2) and its inverse, lambda and its inverse, of species k
+__device__ __forceinline__ void pure_species(const TrParams& P, const long long* mu_fx, const long long* lam_fx,
+                                             const fx::u64* e2, const FitT& t, int k, double& s, double& is, double& l,
+                                             double& il) {
+  if (t.fast) {
+    const fx::i64 x = fit_x(mu_fx + 4 * k, t), y = fit_x(lam_fx + 4 * k, t);
+    s = exp2_any(x, e2); is = exp2_any(-x, e2);
+    l = exp2_any(y, e2); il = exp2_any(-y, e2);
+  } else {
+    const double x = 0.5 * poly3(P.mu_poly + 4 * k, t.lnT), y = poly3(P.lam_poly + 4 * k, t.lnT);
+    s = exp(x); is = exp(-x);
+    l = exp(y); il = exp(-y);
+  }
+}
+
+// D_km from its sum; 1 / D_jk(p) = pr / D_jk(p_atm).  A cell holding species k alone takes the
+// self-diffusion fit.
+__device__ __forceinline__ double mixture_d(const TrParams& P, double dsum, double y, double pr, double T, int k) {
+  if (dsum > 0.0) return (1.0 - y) * fx::rcp(dsum * pr);
+  return exp(poly3(P.diff_poly + 4 * (k * P.ns + k), log(T))) / pr;
+}
+
+// One thread per cell (ns <= 15).  Shared memory: exp2 table, the fits and Wilke's constants (read
+// by warp-uniform addresses), then per warp the cells' vectors, element e of a lane at e * 32.
+__global__ void __launch_bounds__(256, 1) transport_cell_kernel(const TrParams P) {
+  extern __shared__ __align__(16) double tsm[];
+  const int ns = P.ns, npair = ns * (ns - 1) / 2;
+  fx::u64* e2 = (fx::u64*)tsm;
+  long long* mu_fx = (long long*)(tsm + 256);
+  long long* lam_fx = mu_fx + 4 * ns;
+  long long* diff_fx = lam_fx + 4 * ns;
+  double* wk = (double*)(diff_fx + 4 * npair);
+  double* invW = wk + 3 * ns * ns;
+  for (int i = threadIdx.x; i < 256; i += blockDim.x) e2[i] = P.e2[i];
+  for (int i = threadIdx.x; i < 4 * ns && P.mu_fx; i += blockDim.x) { mu_fx[i] = P.mu_fx[i]; lam_fx[i] = P.lam_fx[i]; }
+  for (int i = threadIdx.x; i < 4 * npair && P.mu_fx; i += blockDim.x) diff_fx[i] = P.diff_fx[i];
+  for (int i = threadIdx.x; i < 3 * ns * ns; i += blockDim.x) wk[i] = P.wilke[i];
+  for (int i = threadIdx.x; i < ns; i += blockDim.x) invW[i] = P.invW[i];
   __syncthreads();
-  TGrp<G> g;
-  g.init();
-  const int ns = P.ns;
-  const int gpb = blockDim.x / G;
-  const int npair = ns * (ns - 1) / 2;
-  double* X = tsm + 64 + (size_t)g.gid * (4 * ns + npair);   // mole fractions
-  double* s = X + ns;                        // mu_k^(1/2)
-  double* is = s + ns;                       // mu_k^(-1/2)
-  double* Yc = is + ns;                      // mass fractions of the cell
-  double* E = Yc + ns;                       // 1 / D_jk(p_atm) per unordered pair
-  for (int64_t c = (int64_t)blockIdx.x * gpb + g.gid; c < P.n; c += (int64_t)gridDim.x * gpb) {
+  const int lane = threadIdx.x & 31;
+  double* X = invW + ns + (ns & 1) + (size_t)(threadIdx.x >> 5) * (4 * ns + npair) * 32 + lane;   // mole fractions
+  double* X1 = X + ns * 32;                  // X / s
+  double* X2 = X1 + ns * 32;                 // X / s^2
+  double* s = X2 + ns * 32;                  // mu_k^(1/2)
+  double* E = s + ns * 32;                   // 1 / D_jk(p_atm) per unordered pair
+  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < P.n; c += (int64_t)gridDim.x * blockDim.x) {
     const double T = P.T[c];
-    const double lnT = log(T);
-    const double pr = P.p[c] / kPatm;          // D_jk(p) = D_jk(p_atm) / pr
-    // pure-species properties, mole fractions, Mathur sums
-    double yw = 0.0;
-    for (int k = g.tid; k < ns; k += G) {
-      const double y = P.Y[(int64_t)k * P.ld + c];
-      Yc[k] = y;
-      const double a = 0.5 * poly3(P.mu_poly + 4 * k, lnT);
-      s[k] = exp_tab(a, etab);
-      is[k] = exp_tab(-a, etab);
-      X[k] = y * __ldg(P.invW + k);
-      yw += X[k];
+    const FitT t = fit_t(T, P);
+    const double pr = P.p[c] / kPatm;
+    double S = 0.0;
+    for (int k = 0; k < ns; ++k) {
+      const double x = P.Y[(int64_t)k * P.ld + c] * invW[k];
+      X[k * 32] = x;
+      S += x;
     }
-    const double S = g.sum(yw);
+    const double iS = 1.0 / S;
     double lx = 0.0, lxi = 0.0;
-    for (int k = g.tid; k < ns; k += G) {
-      const double x = X[k] / S;
-      X[k] = x;
-      const double pl = poly3(P.lam_poly + 4 * k, lnT);
-      lx += x * exp_tab(pl, etab);
-      lxi += x * exp_tab(-pl, etab);
+#pragma unroll 2
+    for (int k = 0; k < ns; ++k) {
+      double sk, is, l, il;
+      pure_species(P, mu_fx, lam_fx, e2, t, k, sk, is, l, il);
+      const double x = X[k * 32] * iS;
+      const double x1 = x * is;
+      X[k * 32] = x;
+      X1[k * 32] = x1;
+      X2[k * 32] = x1 * is;
+      s[k * 32] = sk;
+      lx = fma(x, l, lx);
+      lxi = fma(x, il, lxi);
     }
-    lx = g.sum(lx);
-    lxi = g.sum(lxi);
-    if (P.Dm)
-      for (int q = g.tid; q < npair; q += G) {
-        const int jk = __ldg(P.pairs + q);
-        E[q] = exp_tab(-poly3(P.diff_poly + 4 * ((jk & 0xffff) * ns + (jk >> 16)), lnT), etab);
+    if (P.Dm) {
+      if (t.fast) {
+#pragma unroll 4
+        for (int q = 0; q < npair; ++q) E[q * 32] = exp2_any(fit_x(diff_fx + 4 * q, t), e2);
+      } else {
+        for (int q = 0; q < npair; ++q) {
+          const int jk = __ldg(P.pairs + q);
+          E[q * 32] = exp(-poly3(P.diff_poly + 4 * ((jk & 0xffff) * ns + (jk >> 16)), t.lnT));
+        }
       }
-    g.sync();
-    // Wilke viscosity and mixture-averaged diffusion: row k per lane
+    }
     double num = 0.0;
-    for (int k = g.tid; k < ns; k += G) {
-      double den = 0.0, dsum = 0.0;
-      const double sk = s[k];
-      for (int j = 0; j < ns; ++j) {
-        const double xj = X[j];
-        const double t = 1.0 + sk * is[j] * __ldg(P.wq + j * ns + k);
-        den += xj * t * t * __ldg(P.cw + k * ns + j);
-        if (P.Dm && j != k) dsum += xj * E[j < k ? pair_index(j, k, ns) : pair_index(k, j, ns)];
+    for (int k = 0; k < ns; ++k) {
+      double a = 0.0, b = 0.0, d = 0.0;
+      if (P.mu) {
+#pragma unroll 3
+        for (int j = 0; j < ns; ++j) {
+          a = fma(wk[j * ns + k], X[j * 32], a);
+          b = fma(wk[(ns + j) * ns + k], X1[j * 32], b);
+          d = fma(wk[(2 * ns + j) * ns + k], X2[j * 32], d);
+        }
+        const double sk = s[k * 32];
+        const double den = fma(sk, fma(sk, d, b + b), a);
+        num = fma(X[k * 32] * sk, sk * fx::rcp(den), num);
       }
-      num += X[k] * sk * sk / den;
       if (P.Dm) {
-        // 1 / D_jk(p) = pr / D_jk(p_atm); a cell holding species k alone takes the self-diffusion fit
-        const double D = dsum > 0.0 ? (1.0 - Yc[k]) / (dsum * pr) : exp(poly3(P.diff_poly + 4 * (k * ns + k), lnT)) / pr;
-        P.Dm[(int64_t)k * P.ld + c] = D;
+        double dsum = 0.0;
+        for (int j = 0; j < k; ++j) dsum = fma(X[j * 32], E[pair_index(j, k, ns) * 32], dsum);
+#pragma unroll 3
+        for (int j = k + 1; j < ns; ++j) dsum = fma(X[j * 32], E[pair_index(k, j, ns) * 32], dsum);
+        P.Dm[(int64_t)k * P.ld + c] = mixture_d(P, dsum, P.Y[(int64_t)k * P.ld + c], pr, T, k);
       }
     }
-    num = g.sum(num);
-    if (g.tid == 0) {
-      if (P.mu) P.mu[c] = num;
-      if (P.lam) P.lam[c] = 0.5 * (lx + 1.0 / lxi);
+    if (P.mu) P.mu[c] = num;
+    if (P.lam) P.lam[c] = 0.5 * (lx + fx::rcp(lxi));
+  }
+}
+
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// One warp per cell: lanes over species, and over pairs for the binary coefficients
+__global__ void __launch_bounds__(256) transport_warp_kernel(const TrParams P) {
+  extern __shared__ __align__(16) double tsm[];
+  const int ns = P.ns, npair = ns * (ns - 1) / 2;
+  fx::u64* e2 = (fx::u64*)tsm;
+  for (int i = threadIdx.x; i < 256; i += blockDim.x) e2[i] = P.e2[i];
+  __syncthreads();
+  const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+  double* X = tsm + 256 + (size_t)(threadIdx.x >> 5) * (4 * ns + npair);   // as transport_cell_kernel
+  double* X1 = X + ns;
+  double* X2 = X1 + ns;
+  double* s = X2 + ns;
+  double* E = s + ns;
+  for (int64_t c = (int64_t)blockIdx.x * wpb + (threadIdx.x >> 5); c < P.n; c += (int64_t)gridDim.x * wpb) {
+    const double T = P.T[c];
+    const FitT t = fit_t(T, P);
+    const double pr = P.p[c] / kPatm;
+    double yw = 0.0;
+    for (int k = lane; k < ns; k += 32) {
+      const double x = P.Y[(int64_t)k * P.ld + c] * __ldg(P.invW + k);
+      X[k] = x;
+      yw += x;
     }
-    g.sync();
+    const double iS = fx::rcp(warp_sum(yw));
+    double lx = 0.0, lxi = 0.0;
+    for (int k = lane; k < ns; k += 32) {
+      double sk, is, l, il;
+      pure_species(P, P.mu_fx, P.lam_fx, e2, t, k, sk, is, l, il);
+      const double x = X[k] * iS;
+      const double x1 = x * is;
+      X[k] = x;
+      X1[k] = x1;
+      X2[k] = x1 * is;
+      s[k] = sk;
+      lx = fma(x, l, lx);
+      lxi = fma(x, il, lxi);
+    }
+    if (P.lam) {
+      lx = warp_sum(lx);
+      lxi = warp_sum(lxi);
+      if (lane == 0) P.lam[c] = 0.5 * (lx + fx::rcp(lxi));
+    }
+    if (P.Dm) {
+      if (t.fast) {
+#pragma unroll 2
+        for (int q = lane; q < npair; q += 32) {
+          const longlong2 c01 = __ldg(reinterpret_cast<const longlong2*>(P.diff_fx + 4 * q));
+          const longlong2 c23 = __ldg(reinterpret_cast<const longlong2*>(P.diff_fx + 4 * q + 2));
+          const long long cc[4] = {c01.x, c01.y, c23.x, c23.y};
+          E[q] = exp2_any(fit_x(cc, t), e2);
+        }
+      } else {
+        for (int q = lane; q < npair; q += 32) {
+          const int jk = __ldg(P.pairs + q);
+          E[q] = exp(-poly3(P.diff_poly + 4 * ((jk & 0xffff) * ns + (jk >> 16)), t.lnT));
+        }
+      }
+    }
+    __syncwarp();
+    double num = 0.0;
+    for (int k = lane; k < ns; k += 32) {
+      double a = 0.0, b = 0.0, d = 0.0, dsum = 0.0;
+      const double* w0 = P.wilke + k;
+      const double* w1 = w0 + ns * ns;
+      const double* w2 = w1 + ns * ns;
+      int q = k - 1;                         // pair_index(j, k) for j < k, then of (k, j)
+#pragma unroll 4
+      for (int j = 0; j < ns; ++j) {
+        const double x = X[j];
+        a = fma(__ldg(w0 + j * ns), x, a);
+        b = fma(__ldg(w1 + j * ns), X1[j], b);
+        d = fma(__ldg(w2 + j * ns), X2[j], d);
+        if (P.Dm) {
+          dsum = fma(x, j == k ? 0.0 : E[q], dsum);
+          q += j < k - 1 ? ns - 2 - j : (j == k - 1 ? 0 : (j == k ? 0 : 1));
+          if (j == k) q = pair_index(k, k + 1, ns);
+        }
+      }
+      const double sk = s[k];
+      const double den = fma(sk, fma(sk, d, b + b), a);
+      num = fma(X[k] * sk, sk * fx::rcp(den), num);
+      if (P.Dm) P.Dm[(int64_t)k * P.ld + c] = mixture_d(P, dsum, P.Y[(int64_t)k * P.ld + c], pr, T, k);
+    }
+    if (P.mu) {
+      num = warp_sum(num);
+      if (lane == 0) P.mu[c] = num;
+    }
+    __syncwarp();
   }
 }
 
@@ -228,29 +390,52 @@ extern "C" int chem_transport_create(chem_mech_t m, const chem_transport_desc* d
   }
   const size_t n1 = (size_t)ns * 4, n2 = (size_t)ns * ns * 4, nw = (size_t)ns * ns;
   const size_t npair = (size_t)ns * (ns - 1) / 2;
-  std::vector<double> h(2 * n1 + n2 + ns + 2 * nw + (npair + 1) / 2);   // the pair list rides along as ints
-  double* p = h.data();
   for (size_t i = 0; i < n1; ++i) {
     if (!std::isfinite(d->mu_poly[i]) || !std::isfinite(d->lambda_poly[i])) {
       set_error("non-finite transport fit");
       return CHEM_EINVAL;
     }
   }
+  // one buffer of 8-byte words: the FP64 tables, the pair list (as ints), the fixed-point fits
+  const size_t o_lam = n1, o_diff = 2 * n1, o_invw = o_diff + n2, o_wilke = o_invw + ns, o_pairs = o_wilke + 3 * nw;
+  const size_t o_fx = (o_pairs + (npair + 1) / 2 + 1) & ~(size_t)1;      // 16-byte aligned
+  std::vector<double> h(o_fx + 2 * n1 + 4 * npair);
+  double* p = h.data();
   std::copy(d->mu_poly, d->mu_poly + n1, p);
-  std::copy(d->lambda_poly, d->lambda_poly + n1, p + n1);
-  std::copy(d->diff_poly, d->diff_poly + n2, p + 2 * n1);
-  double* invW = p + 2 * n1 + n2;
-  double* wq = invW + ns;
-  double* cw = wq + nw;
-  for (int k = 0; k < ns; ++k) invW[k] = 1.0 / m->W[k];
+  std::copy(d->lambda_poly, d->lambda_poly + n1, p + o_lam);
+  std::copy(d->diff_poly, d->diff_poly + n2, p + o_diff);
+  for (int k = 0; k < ns; ++k) p[o_invw + k] = 1.0 / m->W[k];
   for (int j = 0; j < ns; ++j)
     for (int k = 0; k < ns; ++k) {
-      wq[j * ns + k] = std::pow(m->W[j] / m->W[k], 0.25);
-      cw[k * ns + j] = 1.0 / std::sqrt(8.0 * (1.0 + m->W[k] / m->W[j]));
+      const double wq = std::pow(m->W[j] / m->W[k], 0.25), cw = 1.0 / std::sqrt(8.0 * (1.0 + m->W[k] / m->W[j]));
+      p[o_wilke + (size_t)j * ns + k] = cw;
+      p[o_wilke + nw + (size_t)j * ns + k] = cw * wq;
+      p[o_wilke + 2 * nw + (size_t)j * ns + k] = cw * wq * wq;
     }
-  int* pairs = reinterpret_cast<int*>(cw + nw);
+  int* pairs = reinterpret_cast<int*>(p + o_pairs);
   for (int j = 0, q = 0; j < ns; ++j)
     for (int k = j + 1; k < ns; ++k) pairs[q++] = j | (k << 16);
+  // f * poly(ln T) / ln 2 in powers of log2(T) / 16; no partial sum can leave Q11.52 where the
+  // coefficients' magnitudes sum to at most 2000
+  bool fits = true;
+  long long* fxw = reinterpret_cast<long long*>(p + o_fx);
+  const long double l2 = std::log(2.0L);
+  auto fixed = [&](const double* c, double f, long long* o) {
+    long double scale = 1.0L / l2, sum = 0.0L;
+    for (int i = 0; i < 4; ++i, scale *= 16.0L * l2) {
+      const long double v = (long double)f * c[i] * scale;
+      sum += std::fabs(v);
+      o[i] = std::fabs(v) <= 2000.0L ? (long long)std::nearbyintl(v * 4503599627370496.0L) : 0;
+    }
+    o[3] = (long long)fx::biased(o[3]);
+    if (!(sum <= 2000.0L)) fits = false;
+  };
+  for (int k = 0; k < ns; ++k) {
+    fixed(d->mu_poly + 4 * k, 0.5, fxw + 4 * k);
+    fixed(d->lambda_poly + 4 * k, 1.0, fxw + n1 + 4 * k);
+  }
+  for (size_t q = 0; q < npair; ++q)
+    fixed(d->diff_poly + 4 * ((size_t)(pairs[q] & 0xffff) * ns + (pairs[q] >> 16)), -1.0, fxw + 2 * n1 + 4 * q);
   chem_transport_s* t = new chem_transport_s();
   t->mech = m;
   t->ns = ns;
@@ -262,12 +447,16 @@ extern "C" int chem_transport_create(chem_mech_t m, const chem_transport_desc* d
     return rc;
   }
   t->mu_poly = t->d;
-  t->lam_poly = t->d + n1;
-  t->diff_poly = t->d + 2 * n1;
-  t->invW = t->d + 2 * n1 + n2;
-  t->wq = t->invW + ns;
-  t->cw = t->wq + nw;
-  t->pairs = reinterpret_cast<const int*>(t->cw + nw);
+  t->lam_poly = t->d + o_lam;
+  t->diff_poly = t->d + o_diff;
+  t->invW = t->d + o_invw;
+  t->wilke = t->d + o_wilke;
+  t->pairs = reinterpret_cast<const int*>(t->d + o_pairs);
+  if (fits) {
+    t->mu_fx = reinterpret_cast<const long long*>(t->d + o_fx);
+    t->lam_fx = t->mu_fx + n1;
+    t->diff_fx = t->mu_fx + 2 * n1;
+  }
   *out = t;
   return CHEM_OK;
 }
@@ -281,21 +470,31 @@ extern "C" int chem_transport_eval(chem_transport_t t, const double* T, const do
   TrParams P;
   P.T = T; P.p = p; P.Y = Y; P.ld = ld; P.n = ncells; P.mu = mu; P.lam = lambda; P.Dm = Dmix;
   P.mu_poly = t->mu_poly; P.lam_poly = t->lam_poly; P.diff_poly = t->diff_poly; P.invW = t->invW;
-  P.wq = t->wq; P.cw = t->cw; P.pairs = t->pairs; P.ns = t->ns;
-  const int G = t->ns + 1 <= 16 ? 4 : 32;
-  const int threads = 256, gpb = threads / G;
-  const size_t per_group = (size_t)(4 * t->ns + t->ns * (t->ns - 1) / 2) * sizeof(double);
-  const size_t smem = 64 * sizeof(double) + (size_t)gpb * per_group;
-  static size_t smem_set = 48 * 1024;
-  if (smem > smem_set) {
-    if (smem > 200 * 1024) { set_error("mechanism too large for the transport kernel"); return CHEM_EINVAL; }
-    CHEM_CUDA_TRY(cudaFuncSetAttribute(transport_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    CHEM_CUDA_TRY(cudaFuncSetAttribute(transport_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    smem_set = smem;
+  P.wilke = t->wilke; P.pairs = t->pairs; P.ns = t->ns;
+  P.mu_fx = t->mu_fx; P.lam_fx = t->lam_fx; P.diff_fx = t->diff_fx;
+  P.e2 = t->mech->d_e2; P.lg = t->mech->d_lg; P.rc = t->mech->d_rc;
+  const int ns = t->ns, npair = ns * (ns - 1) / 2;
+  int dev = 0, sms = 0;
+  CHEM_CUDA_TRY(cudaGetDevice(&dev));
+  CHEM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  constexpr size_t kSmem = 200 * 1024;
+  if (ns <= 15) {
+    // as many warps as an SM's shared memory holds, up to eight (two per sub-partition: one warp's
+    // integer work runs beside the other's FP64); fewer where that leaves SMs without a warp
+    const size_t fixed = (256 + 8 * (size_t)ns + 4 * npair + 3 * (size_t)ns * ns + ns + (ns & 1)) * 8;
+    const size_t per = (size_t)(4 * ns + npair) * 256;
+    const int64_t need = (ncells + 31) / 32;
+    const int warps = (int)std::max<int64_t>(1, std::min<int64_t>({8, (int64_t)((kSmem - fixed) / per), (need + sms - 1) / sms}));
+    const size_t smem = fixed + per * warps;
+    CHEM_CUDA_TRY(cudaFuncSetAttribute(transport_cell_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const unsigned grid = (unsigned)std::min<int64_t>((need + warps - 1) / warps, sms);
+    transport_cell_kernel<<<grid, 32 * warps, smem, (cudaStream_t)stream>>>(P);
+  } else {
+    const size_t smem = (256 + 8 * (size_t)(4 * ns + npair)) * sizeof(double);
+    if (smem > kSmem) { set_error("mechanism too large for the transport kernel"); return CHEM_EINVAL; }
+    CHEM_CUDA_TRY(cudaFuncSetAttribute(transport_warp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    transport_warp_kernel<<<grid_cells(ncells, 8), 256, smem, (cudaStream_t)stream>>>(P);
   }
-  const unsigned grid = grid_cells(ncells, gpb);
-  if (G == 4) transport_kernel<4><<<grid, threads, smem, (cudaStream_t)stream>>>(P);
-  else transport_kernel<32><<<grid, threads, smem, (cudaStream_t)stream>>>(P);
   CHEM_CUDA_TRY(cudaGetLastError());
   return CHEM_OK;
 }
