@@ -10,16 +10,15 @@
 // matrix in CSR form for a linear solver (the paper converts ldu to CSR for AmgX).
 //
 // Design.  Alg. 1 assembles face by face and accumulates the diagonal with atomicAdd, with one
-// kernel per boundary patch captured in a CUDA graph.  Here one kernel does everything: a thread
-// per cell walks the cell's faces through a cell-to-face index built once per mesh, computes each
-// face coefficient itself (an internal face is evaluated by both of its cells, identically), sums
-// the diagonal in registers and writes the upper entry of the faces it owns and the lower entry of
-// the faces it neighbours.  No atomics, one launch whatever the patch count, and results that are
-// bitwise reproducible run to run.  On GB300 the FP64 pipe, not HBM, bounds this gather (ncu: FP64
-// pipe 85 % busy at 20 % of DRAM bandwidth), so the FP64 work per face visit is kept small: the
-// geometric factor |S_f| delta_f is multiplied once per mesh, the interpolation is one FMA
-// (gamma_f = gamma_n + w (gamma_o - gamma_n)), the upwind choice tests the flux's sign bit with
-// integer arithmetic, and 1/dt is formed once per launch.
+// kernel per boundary patch captured in a CUDA graph.  Here two kernels do everything, whatever the
+// patch count.  The first takes a thread per pair of internal faces: with c = gamma_f |S_f| delta_f
+// (one FMA for the interpolation, the geometric factor multiplied once per mesh) and upwind
+// convection, upper = min(F, 0) - c and lower = -max(F, 0) - c, four FP64 instructions a face.  The
+// second takes a thread per cell and walks its faces through a cell-to-face index built once per
+// mesh: what face f adds to the diagonal of its owner is -lower_f and to that of its neighbour
+// -upper_f, one FP64 addition a visit.  No atomics, and results that are bitwise reproducible run
+// to run.  One kernel that evaluates every face from both of its cells was bound by the FP64 pipe
+// (85 % busy, 224 us on the 128^3 box): 46 FP64 instructions a cell against 26 here.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -28,6 +27,7 @@
 #include <vector>
 
 #include "chem_internal.h"
+#include "fx_rates.cuh"
 
 struct chem_fvmesh_s {
   int64_t n_cells = 0, n_faces = 0, n_bfaces = 0, nnz = 0;
@@ -54,7 +54,53 @@ struct FvmArgs {
   double *lower, *upper, *diag, *source;
 };
 
-__global__ void fvm_assemble_kernel(const FvmArgs a) {
+// internal face: its two matrix entries; F = 0 without convection, c = 0 without diffusion
+__device__ __forceinline__ void face_entries(const FvmArgs& a, int o, int n, double w, double sd, double F, double& up,
+                                             double& lo) {
+  double mc = 0.0;                                           // -c
+  if (a.gamma) {
+    const double gn = a.gamma[n];
+    mc = -(fma(w, a.gamma[o] - gn, gn) * sd);                // w g_own + (1 - w) g_nei
+  }
+  up = mc;
+  lo = mc;
+  if (a.phi) {
+    const double t = mc - fabs(F);
+    if (__double2hiint(F) < 0) up = t; else lo = t;          // the upwind choice reads the sign bit
+  }
+}
+
+// VEC: the caller's arrays allow 16-byte accesses
+template <bool VEC>
+__global__ void __launch_bounds__(256) fvm_face_kernel(const FvmArgs a, int64_t nf) {
+  const int64_t npair = (nf + 1) >> 1;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < npair; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t f = 2 * i;
+    if (VEC && f + 1 < nf) {
+      const int2 o = *reinterpret_cast<const int2*>(a.owner + f), n = *reinterpret_cast<const int2*>(a.neighbour + f);
+      double2 w = make_double2(0.0, 0.0), sd = w, F = w, up, lo;
+      if (a.gamma) {
+        w = *reinterpret_cast<const double2*>(a.weight + f);
+        sd = *reinterpret_cast<const double2*>(a.sd + f);
+      }
+      if (a.phi) F = *reinterpret_cast<const double2*>(a.phi + f);
+      face_entries(a, o.x, n.x, w.x, sd.x, F.x, up.x, lo.x);
+      face_entries(a, o.y, n.y, w.y, sd.y, F.y, up.y, lo.y);
+      *reinterpret_cast<double2*>(a.upper + f) = up;
+      *reinterpret_cast<double2*>(a.lower + f) = lo;
+    } else {
+      for (int64_t g = f; g < min(f + 2, nf); ++g) {
+        double up, lo;
+        face_entries(a, a.owner[g], a.neighbour[g], a.gamma ? a.weight[g] : 0.0, a.gamma ? a.sd[g] : 0.0,
+                     a.phi ? a.phi[g] : 0.0, up, lo);
+        a.upper[g] = up;
+        a.lower[g] = lo;
+      }
+    }
+  }
+}
+
+__global__ void __launch_bounds__(256) fvm_cell_kernel(const FvmArgs a) {
   for (int64_t P = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; P < a.n; P += (int64_t)gridDim.x * blockDim.x) {
     const double V = a.volume[P];
     double dg = 0.0, src = 0.0;
@@ -63,54 +109,75 @@ __global__ void fvm_assemble_kernel(const FvmArgs a) {
       dg = a.rho[P] * vdt;
       src = a.rho_old[P] * a.Y_old[P] * vdt;
     }
-    const double gP = a.gamma ? a.gamma[P] : 0.0;
+    if (a.S) src += V * (a.kappa ? a.kappa[P] : 1.0) * a.S[P];
     const int e1 = a.cell_ptr[P + 1];
-    for (int e = a.cell_ptr[P]; e < e1; ++e) {
-      const int code = a.cell_face[e];
-      const int kind = code & 3, f = code >> 2;
-      if (kind < 2) {                                        // internal face; kind 0: P owns it
-        double off = 0.0;
-        if (a.phi) {
-          // mass flux out of P (the sign flip and the upwind test are bit operations)
-          const double F = a.phi[f];
-          const double Fout = __hiloint2double(__double2hiint(F) ^ (kind == 0 ? 0 : (int)0x80000000),
-                                               __double2loint(F));
-          if (__double2hiint(Fout) >= 0) dg += Fout; else off += Fout;   // outflow carries Y_P
-        }
-        if (a.gamma) {
-          const int other = kind == 0 ? a.neighbour[f] : a.owner[f];
-          const double gO = a.gamma[other];
-          const double g_own = kind == 0 ? gP : gO, g_nei = kind == 0 ? gO : gP;
-          const double gf = fma(a.weight[f], g_own - g_nei, g_nei);     // w g_own + (1 - w) g_nei
-          const double c = gf * a.sd[f];
-          dg += c;
-          off -= c;
-        }
-        if (kind == 0) a.upper[f] = off; else a.lower[f] = off;
-      } else {                                               // boundary face
-        if (a.phi_b) {
-          const double Fb = a.phi_b[f];
-          if (__double2hiint(Fb) >= 0) dg += Fb; else src -= Fb * a.Y_b[f];
-        }
-        if (a.gamma && a.b_type[f] == 1) {
-          const double c = a.gamma_b[f] * a.b_sd[f];
-          dg += c;
-          src += c * a.Y_b[f];
+    for (int e = a.cell_ptr[P]; e < e1; e += 4) {
+      // four faces at a time: their loads are independent
+      int code[4];
+      double v[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) code[q] = e + q < e1 ? a.cell_face[e + q] : 3;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int kind = code[q] & 3, f = code[q] >> 2;
+        v[q] = kind == 0 ? a.lower[f] : (kind == 1 ? a.upper[f] : 0.0);
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int kind = code[q] & 3, f = code[q] >> 2;
+        if (kind < 2) {
+          dg -= v[q];
+        } else if (kind == 2) {                              // boundary face
+          if (a.phi_b) {
+            const double Fb = a.phi_b[f];
+            if (__double2hiint(Fb) >= 0) dg += Fb; else src -= Fb * a.Y_b[f];
+          }
+          if (a.gamma && a.b_type[f] == 1) {
+            const double c = a.gamma_b[f] * a.b_sd[f];
+            dg += c;
+            src += c * a.Y_b[f];
+          }
         }
       }
     }
-    if (a.S) src += V * (a.kappa ? a.kappa[P] : 1.0) * a.S[P];
     a.diag[P] = dg;
     if (a.source) a.source[P] = src;
   }
 }
 
-__global__ void fvm_to_csr_kernel(int64_t nnz, const int32_t* row_of, const int32_t* src, const double* lower,
-                                  const double* upper, const double* diag, double* vals) {
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nnz; e += (int64_t)gridDim.x * blockDim.x) {
-    const int s = src[e];
-    vals[e] = s < 0 ? diag[row_of[e]] : ((s & 1) ? lower[s >> 1] : upper[s >> 1]);
+// Four entries per thread, a grid stride apart: coalesced, with four independent gathers in flight
+__global__ void __launch_bounds__(256) fvm_to_csr_kernel(int64_t nnz, const int32_t* row_of, const int32_t* src,
+                                                         const double* lower, const double* upper, const double* diag,
+                                                         double* vals) {
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nnz; e += 4 * step) {
+    int s[4];
+    double v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) s[q] = e + q * step < nnz ? src[e + q * step] : 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      v[q] = 0.0;
+      if (e + q * step < nnz)
+        v[q] = s[q] < 0 ? diag[row_of[e + q * step]] : ((s[q] & 1) ? lower[s[q] >> 1] : upper[s[q] >> 1]);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (e + q * step < nnz) vals[e + q * step] = v[q];
   }
+}
+
+// sqrt(a / b) for positive normal a, b with a normal product, as a (a b)^(-1/2): the reciprocal
+// square root approximation y (20 bits) and one third-order step y (1 + e / 2 + 3 e^2 / 8),
+// e = 1 - x y^2 (the binomial series), six FP64 instructions where the library's division and
+// square root take about 17
+__device__ __forceinline__ double sqrt_ratio(double a, double b) {
+  const double x = a * b;
+  if (!((unsigned)__double2hiint(x) - 0x08000000u < 0x70000000u)) return sqrt(a / b);
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x * y, y, 1.0);
+  return a * fma(y * e, fma(e, 0.375, 0.5), y);
 }
 
 // kappa = tau_c / (tau_c + tau_mix), tau_mix = C_mix sqrt(mu_eff / (rho eps)),
@@ -125,8 +192,8 @@ __global__ void pasr_kernel(int64_t n, const double* tau_c, const double* rho, c
     const double eps = nu * s * s;
     double k = 1.0;
     if (eps > 0.0) {
-      const double tmix = c_mix * sqrt((mu[i] + rho[i] * nu) / (rho[i] * eps));
-      k = tau_c[i] / (tau_c[i] + tmix);
+      const double tmix = c_mix * sqrt_ratio(fma(rho[i], nu, mu[i]), rho[i] * eps);
+      k = tau_c[i] * fx::rcp(tau_c[i] + tmix);
     }
     kappa[i] = k;
   }
@@ -262,7 +329,13 @@ extern "C" int chem_fvm_assemble(chem_fvmesh_t m, const chem_fvm_terms* t, doubl
   a.inv_dt = t->dt > 0.0 ? 1.0 / t->dt : 0.0; a.rho = t->rho; a.rho_old = t->rho_old; a.Y_old = t->Y_old; a.phi = t->phi; a.phi_b = t->phi_b;
   a.gamma = t->gamma; a.gamma_b = t->gamma_b; a.Y_b = t->Y_b; a.S = t->S; a.kappa = t->kappa;
   a.lower = lower; a.upper = upper; a.diag = diag; a.source = source;
-  fvm_assemble_kernel<<<grid_for(a.n), 256, 0, (cudaStream_t)stream>>>(a);
+  if (m->n_faces > 0) {
+    const bool vec = (((uintptr_t)lower | (uintptr_t)upper | (uintptr_t)t->phi) & 15) == 0;
+    const unsigned grid = grid_for((m->n_faces + 1) / 2);
+    if (vec) fvm_face_kernel<true><<<grid, 256, 0, (cudaStream_t)stream>>>(a, m->n_faces);
+    else fvm_face_kernel<false><<<grid, 256, 0, (cudaStream_t)stream>>>(a, m->n_faces);
+  }
+  fvm_cell_kernel<<<grid_for(a.n), 256, 0, (cudaStream_t)stream>>>(a);
   CHEM_CUDA_TRY(cudaGetLastError());
   return CHEM_OK;
 }
@@ -271,7 +344,7 @@ extern "C" int chem_fvm_to_csr(chem_fvmesh_t m, const double* lower, const doubl
                                double* vals, chem_stream_t stream) {
   if (!m || !diag || !vals || (m->n_faces && (!lower || !upper))) { set_error("NULL argument"); return CHEM_EINVAL; }
   // the row of each nonzero, for the diagonal entries: col_idx holds the row there
-  fvm_to_csr_kernel<<<grid_for(m->nnz), 256, 0, (cudaStream_t)stream>>>(m->nnz, m->col_idx, m->csr_src, lower,
+  fvm_to_csr_kernel<<<grid_for((m->nnz + 3) / 4), 256, 0, (cudaStream_t)stream>>>(m->nnz, m->col_idx, m->csr_src, lower,
                                                                          upper, diag, vals);
   CHEM_CUDA_TRY(cudaGetLastError());
   return CHEM_OK;

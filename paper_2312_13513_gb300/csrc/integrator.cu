@@ -1646,6 +1646,7 @@ template <int G, bool FX>
 __global__ void __launch_bounds__(max_threads(G), 1) advance_kernel(const __grid_constant__ AdvanceParams P) {
   extern __shared__ __align__(16) unsigned char smem[];
   if (blockDim.x % G != 0 || blockDim.x < G) return;   // a block of whole groups only
+  if (P.ncells_dev && *P.ncells_dev == 0u) return;     // an empty fallback pass
   stage_mech(Form<FX>::src(P), smem, Form<FX>::bytes(P));
   __syncthreads();
   const typename Form<FX>::View m = Form<FX>::bind(smem, P);

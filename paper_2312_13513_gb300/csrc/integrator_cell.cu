@@ -158,6 +158,7 @@ __global__ void __launch_bounds__(128, 1) cell_advance_kernel(const __grid_const
   using w = Ws<NS>;
   constexpr int N = w::N;
   extern __shared__ __align__(16) unsigned char smem[];
+  if (P.q.ncells_dev && *P.q.ncells_dev == 0u) return;     // an empty fallback pass
   stage(P.fxblob, smem, P.fx.bytes);
   __syncthreads();
   const cell::View m = cell::bind(smem, P.fx, P.blob, &P.lay);
