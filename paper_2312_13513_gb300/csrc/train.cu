@@ -53,45 +53,100 @@ __device__ __forceinline__ float gelu_grad(float v) {
   return 0.5f * (1.0f + erff(v * 0.70710678118654752f)) + v * 0.3989422804014327f * expf(-0.5f * v * v);
 }
 
-__global__ void k_gelu_bwd(const float* dA, const float* Z, float* dZf, __nv_bfloat16* dZb, int64_t n) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const float g = dA[i] * gelu_grad(Z[i]);
-    dZf[i] = g;
-    dZb[i] = __float2bfloat16_rn(g);
-  }
-}
+// Row block of the column sums' partials and of the gradient tiles below
+constexpr int kColRows = 64;
 
-// out, dZ: [B x ld] (ld = 128); target: [B x nout]
-__global__ void k_mse_grad(const float* out, const float* target, float* dZf, __nv_bfloat16* dZb, double* loss,
-                           int B, int nout, int ld) {
-  double part = 0.0;
-  const float scale = 2.0f / ((float)B * (float)nout);
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (int64_t)B * ld;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int b = (int)(i / ld), c = (int)(i % ld);
-    float g = 0.0f;
-    if (c < nout) {
-      const float d = out[i] - target[(int64_t)b * nout + c];
-      part += (double)d * d;
-      g = scale * d;
-    }
-    dZf[i] = g;
-    dZb[i] = __float2bfloat16_rn(g);
+// Pre-activation gradients of one layer from a 64 x 64 tile per block (32 x 8 threads, two
+// neighbouring columns and rows ty, ty + 8, ... each): BF16 row-major, BF16 transposed (batch
+// contiguous, for the weight gradient) and the tile's column sums (FP32 per thread, the eight
+// partials in FP64) into part[row block][column].  One pass over the tile where separate gradient,
+// transpose and column-sum kernels read it three times; these steps are short kernels on a
+// 4096-row batch, so launches and their tails are what they cost.  grad(row, column) returns the
+// pair of gradients.
+template <class F>
+__device__ __forceinline__ void gradient_tile(F grad, __nv_bfloat16* dZb, __nv_bfloat16* dZt, double* part, int R,
+                                              int C) {
+  __shared__ __nv_bfloat162 t[64][33];               // [column][row pair]
+  __shared__ double red[8][66];
+  const int tx = threadIdx.x, ty = threadIdx.y, c = blockIdx.x * 64 + 2 * tx, r0 = blockIdx.y * kColRows;
+  float s0 = 0.0f, s1 = 0.0f;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int rl = ty + 8 * i, r = r0 + rl;
+    float2 g = make_float2(0.0f, 0.0f);
+    if (c < C && r < R) g = grad(r, c);              // C is even
+    s0 += g.x;
+    s1 += g.y;
+    const __nv_bfloat162 h = __floats2bfloat162_rn(g.x, g.y);
+    if (c < C && r < R) *reinterpret_cast<__nv_bfloat162*>(dZb + (int64_t)r * C + c) = h;
+    __nv_bfloat16* t0 = reinterpret_cast<__nv_bfloat16*>(&t[2 * tx][0]);
+    __nv_bfloat16* t1 = reinterpret_cast<__nv_bfloat16*>(&t[2 * tx + 1][0]);
+    t0[rl] = __low2bfloat16(h);
+    t1[rl] = __high2bfloat16(h);
   }
-  // one atomic per block: the warps' sums through shared memory
-  __shared__ double red[32];
-  for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) red[warp] = part;
+  red[ty][2 * tx] = (double)s0;
+  red[ty][2 * tx + 1] = (double)s1;
   __syncthreads();
-  if (warp == 0) {
-    part = lane < (int)(blockDim.x >> 5) ? red[lane] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-    if (lane == 0 && loss) atomicAdd(loss, part / ((double)B * nout));
+  for (int cl = ty; cl < 64; cl += 8) {
+    const int cc = blockIdx.x * 64 + cl, r = r0 + 2 * tx;
+    if (cc < C && r < R) *reinterpret_cast<__nv_bfloat162*>(dZt + (int64_t)cc * R + r) = t[cl][tx];
+  }
+  const int id = ty * 32 + tx;
+  if (id < 64 && blockIdx.x * 64 + id < C) {
+    double v = 0.0;
+    for (int i = 0; i < 8; ++i) v += red[i][id];
+    part[(int64_t)blockIdx.y * C + blockIdx.x * 64 + id] = v;
   }
 }
 
-// several BF16 transposes in one launch: blockIdx.z selects the job (out[c * R + r] = in[r * C + c])
+// dZ = dA GELU'(Z)
+__global__ void __launch_bounds__(256) k_gelu_bwd(const float* dA, const float* Z, __nv_bfloat16* dZb,
+                                                  __nv_bfloat16* dZt, double* part, int R, int C) {
+  gradient_tile(
+      [&](int r, int c) {
+        const float2 a = *reinterpret_cast<const float2*>(dA + (int64_t)r * C + c);
+        const float2 z = *reinterpret_cast<const float2*>(Z + (int64_t)r * C + c);
+        return make_float2(a.x * gelu_grad(z.x), a.y * gelu_grad(z.y));
+      },
+      dZb, dZt, part, R, C);
+}
+
+// dZ = 2 (out - target) / (B nout) of the mean-squared error; out [B x ld], target [B x nout]; the
+// block's share of the loss into loss_part
+__global__ void __launch_bounds__(256) k_mse_grad(const float* out, const float* target, __nv_bfloat16* dZb,
+                                                  __nv_bfloat16* dZt, double* part, double* loss_part, int B, int nout,
+                                                  int ld) {
+  const float scale = 2.0f / ((float)B * (float)nout);
+  double sum = 0.0;
+  gradient_tile(
+      [&](int r, int c) {
+        float2 g = make_float2(0.0f, 0.0f);
+        if (c < nout) {
+          const float d = out[(int64_t)r * ld + c] - target[(int64_t)r * nout + c];
+          sum += (double)d * d;
+          g.x = scale * d;
+        }
+        if (c + 1 < nout) {
+          const float d = out[(int64_t)r * ld + c + 1] - target[(int64_t)r * nout + c + 1];
+          sum += (double)d * d;
+          g.y = scale * d;
+        }
+        return g;
+      },
+      dZb, dZt, part, B, ld);
+  __shared__ double red[8];
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if (threadIdx.x == 0) red[threadIdx.y] = sum;
+  __syncthreads();
+  if (threadIdx.x == 0 && threadIdx.y == 0) {
+    double v = 0.0;
+    for (int i = 0; i < 8; ++i) v += red[i];
+    loss_part[blockIdx.y * gridDim.x + blockIdx.x] = v;
+  }
+}
+
+// several BF16 transposes in one launch: blockIdx.z selects the job (out[c * R + r] = in[r * C + c];
+// R and C even), 64 x 64 tiles with two elements per access on both sides
 struct TransposeJob {
   const __nv_bfloat16* in;
   __nv_bfloat16* out;
@@ -102,77 +157,105 @@ struct TransposeSet {
   int n;
 };
 
-__global__ void k_transpose_set(const __grid_constant__ TransposeSet S) {
+__global__ void __launch_bounds__(256) k_transpose_set(const __grid_constant__ TransposeSet S) {
   if ((int)blockIdx.z >= S.n) return;
   const TransposeJob& J = S.j[blockIdx.z];
-  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
+  const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64, tx = threadIdx.x, ty = threadIdx.y;
   if (r0 >= J.R || c0 >= J.C) return;                // the whole block: before the barrier
-  __shared__ __nv_bfloat16 t[32][33];
-  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-    const int r = r0 + i, c = c0 + threadIdx.x;
-    if (r < J.R && c < J.C) t[i][threadIdx.x] = J.in[(int64_t)r * J.C + c];
+  __shared__ __nv_bfloat162 t[64][33];               // [column][row pair]
+  for (int rl = ty; rl < 64; rl += 8) {
+    const int r = r0 + rl, c = c0 + 2 * tx;
+    if (r < J.R && c < J.C) {
+      const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162*>(J.in + (int64_t)r * J.C + c);
+      reinterpret_cast<__nv_bfloat16*>(&t[2 * tx][0])[rl] = __low2bfloat16(h);
+      reinterpret_cast<__nv_bfloat16*>(&t[2 * tx + 1][0])[rl] = __high2bfloat16(h);
+    }
   }
   __syncthreads();
-  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-    const int c = c0 + i, r = r0 + threadIdx.x;
-    if (r < J.R && c < J.C) J.out[(int64_t)c * J.R + r] = t[threadIdx.x][i];
+  for (int cl = ty; cl < 64; cl += 8) {
+    const int c = c0 + cl, r = r0 + 2 * tx;
+    if (r < J.R && c < J.C) *reinterpret_cast<__nv_bfloat162*>(J.out + (int64_t)c * J.R + r) = t[cl][tx];
   }
 }
 
 void launch_transposes(const TransposeSet& S, cudaStream_t st) {
   int gx = 1, gy = 1;
   for (int k = 0; k < S.n; ++k) {
-    gx = std::max(gx, (S.j[k].C + 31) / 32);
-    gy = std::max(gy, (S.j[k].R + 31) / 32);
+    gx = std::max(gx, (S.j[k].C + 63) / 64);
+    gy = std::max(gy, (S.j[k].R + 63) / 64);
   }
   k_transpose_set<<<dim3(gx, gy, S.n), dim3(32, 8), 0, st>>>(S);
 }
 
-// column sums of a [R x C] FP32 matrix, in two deterministic passes spread over the whole GPU:
-// block (x, y) sums rows [y * kColRows, ...) of 32 columns (8 thread rows, FP32, then the 8
-// partials in FP64) into part[y][c]; k_colsum_finish adds the row-block partials of a column.
-constexpr int kColRows = 64;
-__global__ void k_colsum_part(const float* A, double* part, int R, int C) {
-  __shared__ double red[8][33];
-  const int c = blockIdx.x * 32 + threadIdx.x;
-  const int r0 = blockIdx.y * kColRows;
-  float acc = 0.0f;
-  if (c < C)
-    for (int r = r0 + threadIdx.y; r < min(R, r0 + kColRows); r += 8) acc += A[(int64_t)r * C + c];
-  red[threadIdx.y][threadIdx.x] = (double)acc;
-  __syncthreads();
-  if (threadIdx.y == 0 && c < C) {
-    double t = 0.0;
-    for (int i = 0; i < 8; ++i) t += red[i][threadIdx.x];
-    part[(int64_t)blockIdx.y * C + c] = t;
-  }
-}
+// The end of a backward pass in one launch: every layer's weight gradient as the ordered sum of its
+// split-K partials (the first layer's split blocks folded onto the master's columns), every bias
+// gradient as the column sum of its row-block partials (a warp per column), and the loss (the
+// last block, in a fixed order).  Deterministic.
+struct FinishSeg {
+  const float* parts;       // split-K partials (one: the product itself)
+  float* dW;
+  int64_t n;                // out_pad * in_pad
+  int splits, ld, fold;     // fold > 0: n_in of the first layer
+  const double* colpart;
+  float* db;
+  int cols, block0, wblocks;      // blocks block0 .. + wblocks: dW, then (cols + 7) / 8 blocks: db
+};
+struct FinishSet {
+  FinishSeg s[MAXL];
+  int n, nparts;
+  const double* loss_part;
+  int n_loss;
+  double loss_scale;
+  double *loss, *loss_out;  // loss_out nullable
+};
 
-// out[i] = sum over s of parts[s * stride + i], in the order s = 0, 1, ...: the split-K partial
-// products of a weight gradient added deterministically
-__global__ void k_sum_parts(const float* parts, float* out, int64_t n, int splits, int64_t stride) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    float v = parts[i];
-    for (int s = 1; s < splits; ++s) v += parts[s * stride + i];
-    out[i] = v;
+__global__ void __launch_bounds__(256) k_finish_grads(const __grid_constant__ FinishSet S) {
+  const int lane = threadIdx.x & 31;
+  if (blockIdx.x == gridDim.x - 1) {
+    if (threadIdx.x < 32) {
+      double t = 0.0;
+      for (int i = lane; i < S.n_loss; i += 32) t += S.loss_part[i];
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (lane == 0) {
+        *S.loss = t * S.loss_scale;
+        if (S.loss_out) *S.loss_out = t * S.loss_scale;
+      }
+    }
+    return;
   }
-}
-
-// one warp per column: the lanes sum strided partials, then a shuffle reduction
-__global__ void k_colsum_finish(const double* part, float* s, int nparts, int C) {
-  const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (c >= C) return;                                // whole warps leave together
+  int k = 0;
+  while (k + 1 < S.n && S.s[k + 1].block0 <= (int)blockIdx.x) ++k;
+  const FinishSeg& q = S.s[k];
+  const int blk = blockIdx.x - q.block0;
+  if (blk < q.wblocks) {
+    for (int64_t i = (int64_t)blk * blockDim.x + threadIdx.x; i < q.n; i += (int64_t)q.wblocks * blockDim.x) {
+      float v = 0.0f;
+      const int c = q.fold ? (int)(i % q.ld) : 0;
+      if (!q.fold || c < q.fold) {
+        v = q.parts[i];
+        for (int s = 1; s < q.splits; ++s) v += q.parts[s * q.n + i];
+        if (q.fold) {
+          float u = q.parts[i + q.fold];
+          for (int s = 1; s < q.splits; ++s) u += q.parts[s * q.n + i + q.fold];
+          v += u;
+        }
+      }
+      q.dW[i] = v;
+    }
+    return;
+  }
+  const int c = (blk - q.wblocks) * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (c >= q.cols) return;                           // whole warps leave together
   double t = 0.0;
-  for (int i = lane; i < nparts; i += 32) t += part[(int64_t)i * C + c];
+  for (int i = lane; i < S.nparts; i += 32) t += q.colpart[(int64_t)i * q.cols + c];
   for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  if (lane == 0) s[c] = (float)t;
+  if (lane == 0) q.db[c] = (float)t;
 }
 
-// Adam on a [rows x cols] parameter block (cols = 1 for biases); writes the BF16 copy of W if given
-// (its transpose follows by the tiled k_transpose)
 // Adam over every parameter block of the network in one launch: block b of the grid serves the
 // segment whose first block is the last one <= b; each segment is one weight matrix or bias
-// vector (W, its gradient G, moments m and v; Wb: the BF16 copy of W to write, or null).
+// vector (W, its gradient G, moments m and v; Wb: the BF16 copy of W to write, or null; nin > 0: the
+// first layer, whose copy is the split row [W_hi | W_hi | W_lo | 0] of pitch ld).
 struct AdamSeg {
   float* W;
   const float* G;
@@ -180,7 +263,7 @@ struct AdamSeg {
   float* v;
   __nv_bfloat16* Wb;
   int64_t n;
-  int block0;
+  int block0, nin, ld;
 };
 struct AdamSet {
   AdamSeg s[2 * MAXL];
@@ -202,7 +285,17 @@ __global__ void k_adam_set(const __grid_constant__ AdamSet S, const float* coef,
     q.v[i] = vi;
     const float w = q.W[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
     q.W[i] = w;
-    if (q.Wb) q.Wb[i] = __float2bfloat16_rn(w);
+    if (q.nin > 0) {
+      const int c = (int)(i % q.ld);
+      if (c < q.nin) {
+        const __nv_bfloat16 hi = __float2bfloat16_rn(w);
+        q.Wb[i] = hi;
+        q.Wb[i + q.nin] = hi;
+        q.Wb[i + 2 * q.nin] = __float2bfloat16_rn(w - __bfloat162float(hi));
+      }
+    } else if (q.Wb) {
+      q.Wb[i] = __float2bfloat16_rn(w);
+    }
   }
 }
 
@@ -231,16 +324,6 @@ __global__ void k_split_bf16(const float* W, __nv_bfloat16* Wb, int rows, int ld
   }
 }
 
-// fold the first layer's block gradient into the master's columns: dW[:, c] += dW[:, nin + c]
-// for c < nin, zero elsewhere (one thread per row: the row is read before it is written)
-__global__ void k_fold_split_grad(float* dW, int rows, int ld, int nin) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= rows) return;
-  float* row = dW + (int64_t)r * ld;
-  for (int c = 0; c < nin; ++c) row[c] += row[nin + c];
-  for (int c = nin; c < ld; ++c) row[c] = 0.0f;
-}
-
 __global__ void k_to_bf16(const float* W, __nv_bfloat16* Wb, __nv_bfloat16* Wt, int rows, int cols) {
   const int64_t n = (int64_t)rows * cols;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -251,13 +334,29 @@ __global__ void k_to_bf16(const float* W, __nv_bfloat16* Wb, __nv_bfloat16* Wt, 
   }
 }
 
-// dst[r * ld + c] = scale * src[r * cols + c] for the real block of a padded gradient buffer
-// (the padding of dst keeps its zeros)
-__global__ void k_unpack_scaled(const float* src, float* dst, int rows, int cols, int ld, float scale) {
-  const int64_t n = (int64_t)rows * cols;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int r = (int)(i / cols), c = (int)(i % cols);
-    dst[(int64_t)r * ld + c] = scale * src[i];
+// Every real (unpadded) gradient block between the padded buffers and the flat layout, one launch:
+// segment q covers flat elements [q.flat, q.flat + rows * cols) of a buffer with row pitch ld.
+struct FlatSeg {
+  float* buf;
+  int64_t flat, n;
+  int cols, ld;
+};
+struct FlatSet {
+  FlatSeg s[2 * MAXL];
+  int n;
+  int64_t total;
+};
+
+// unpack: buf = scale * flat (the padding keeps its zeros); otherwise flat = buf
+__global__ void k_flat_grads(const __grid_constant__ FlatSet S, float* flat, const float* src, float scale, int unpack) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < S.total; i += (int64_t)gridDim.x * blockDim.x) {
+    int k = 0;
+    while (k + 1 < S.n && S.s[k + 1].flat <= i) ++k;
+    const FlatSeg& q = S.s[k];
+    const int e = (int)(i - q.flat), r = e / q.cols;
+    float* x = q.buf + (int64_t)r * q.ld + (e - r * q.cols);
+    if (unpack) *x = scale * src[i];
+    else flat[i] = *x;
   }
 }
 
@@ -365,11 +464,12 @@ struct chem_trainer_s {
   __nv_bfloat16 *Wb[MAXL], *Wt[MAXL];
   float* Z[MAXL];                  // pre-activations [B x out_pad]
   __nv_bfloat16* A[MAXL];          // A[0] = caller's input, A[l] = bf16(GELU(Z[l-1]))
-  float *dA, *dZf;
-  float* dWparts;                  // split-K partials of the weight gradients (null: no layer splits)
+  float* dA;
+  float* dWparts[MAXL];            // split-K partials of each layer's weight gradient (splits x W)
   int splitsW[MAXL];               // K splits of each layer's weight-gradient product
-  double* colpart;                 // row-block partial column sums [B / 64 x max width]
-  __nv_bfloat16 *dZb, *dZt, *At;
+  double* colpart[MAXL];           // row-block partial column sums [B / 64 x out_pad]
+  double* loss_part;               // the loss gradient kernel's block sums
+  __nv_bfloat16 *dZb, *dZt, *At[MAXL];
   int* err;
   double* loss;
   int64_t* d_step;                 // Adam steps taken (device: a captured step advances it)
@@ -468,28 +568,32 @@ extern "C" int chem_mlp_trainer_create_layers(int n_in, int n_out, int n_hidden,
   if (!rc) rc = tr_alloc(t, &p, (size_t)batch * maxw * 4), t->dA = (float*)p;
   // weight gradients dW = dZ^T A have few output tiles and K = batch: split K over the SMs (a
   // power of two dividing the 64-wide K steps, splits x tiles at most the SM count) and add the
-  // partials in a fixed order
+  // partials in a fixed order (k_finish_grads)
   if (!rc) {
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int nk = (batch + 63) / 64;
-    size_t parts = 0;
-    for (int l = 0; l < NL; ++l) {
+    for (int l = 0; l < NL && !rc; ++l) {
       const long long tiles = (long long)((t->out_pad[l] + 127) / 128) * ((t->in_pad[l] + 127) / 128);
       int sp = 1;
       while (nk % (2 * sp) == 0 && tiles * 2 * sp <= sms) sp *= 2;
       t->splitsW[l] = sp;
-      if (sp > 1) parts = std::max(parts, (size_t)sp * t->out_pad[l] * t->in_pad[l]);
+      rc = tr_alloc(t, &p, (size_t)sp * t->out_pad[l] * t->in_pad[l] * 4);
+      t->dWparts[l] = (float*)p;
     }
-    t->dWparts = nullptr;
-    if (parts) rc = tr_alloc(t, &p, parts * 4), t->dWparts = (float*)p;
   }
-  if (!rc) rc = tr_alloc(t, &p, (size_t)batch * maxw * 4), t->dZf = (float*)p;
+  const size_t nrb = (batch + kColRows - 1) / kColRows;
+  for (int l = 0; l < NL && !rc; ++l) {
+    rc = tr_alloc(t, &p, (size_t)batch * ins[l] * 2);
+    t->At[l] = (__nv_bfloat16*)p;
+    if (rc) break;
+    rc = tr_alloc(t, &p, nrb * outs[l] * 8);
+    t->colpart[l] = (double*)p;
+  }
   if (!rc) rc = tr_alloc(t, &p, (size_t)batch * maxw * 2), t->dZb = (__nv_bfloat16*)p;
   if (!rc) rc = tr_alloc(t, &p, (size_t)batch * maxw * 2), t->dZt = (__nv_bfloat16*)p;
-  if (!rc) rc = tr_alloc(t, &p, (size_t)batch * maxw * 2), t->At = (__nv_bfloat16*)p;
-  if (!rc) rc = tr_alloc(t, &p, (size_t)((batch + kColRows - 1) / kColRows) * maxw * 8), t->colpart = (double*)p;
+  if (!rc) rc = tr_alloc(t, &p, nrb * ((PADIO + 63) / 64) * 8), t->loss_part = (double*)p;
   if (!rc) rc = tr_alloc(t, &p, 16), t->err = (int*)p;
   if (!rc) rc = tr_alloc(t, &p, 16), t->loss = (double*)p;
   if (!rc) rc = tr_alloc(t, &p, 16), t->d_step = (int64_t*)p;
@@ -528,43 +632,44 @@ extern "C" int chem_mlp_backward(chem_trainer_t t, const float* target, double* 
   if (!t || !target) { set_error("NULL argument"); return CHEM_EINVAL; }
   cudaStream_t st = (cudaStream_t)stream;
   const int B = t->B, NL = t->nl;
-  CHEM_CUDA_TRY(cudaMemsetAsync(t->loss, 0, sizeof(double), st));
-  k_mse_grad<<<std::min(grid_for((int64_t)B * PADIO), 1024u), 256, 0, st>>>(t->Z[NL - 1], target, t->dZf, t->dZb,
-                                                                         t->loss, B, t->nout, PADIO);
+  // A^T of every layer (batch contiguous, for the weight gradients)
+  TransposeSet T{};
+  for (int l = 0; l < NL; ++l) T.j[T.n++] = TransposeJob{t->A[l], t->At[l], B, t->in_pad[l]};
+  launch_transposes(T, st);
+  const int nrb = (B + kColRows - 1) / kColRows;
+  const dim3 mse_grid((PADIO + 63) / 64, nrb);
+  k_mse_grad<<<mse_grid, dim3(32, 8), 0, st>>>(t->Z[NL - 1], target, t->dZb, t->dZt, t->colpart[NL - 1],
+                                               t->loss_part, B, t->nout, PADIO);
   for (int l = NL - 1; l >= 0; --l) {
     const int nout = t->out_pad[l], nin = t->in_pad[l];
-    // dZ^T and A^T (batch contiguous) for the weight gradient
-    {
-      TransposeSet T{};
-      T.j[0] = TransposeJob{t->dZb, t->dZt, B, nout};
-      T.j[1] = TransposeJob{t->A[l], t->At, B, nin};
-      T.n = 2;
-      launch_transposes(T, st);
-    }
     int rc;
-    if (t->splitsW[l] > 1) {
-      const int64_t n = (int64_t)nout * nin;
-      rc = gemm_bf16_splitk(t->dZt, B, t->At, B, t->dWparts, nin, n, t->splitsW[l], nout, nin, B, t->err, st);
-      if (rc) return rc;
-      k_sum_parts<<<grid_for(n), 256, 0, st>>>(t->dWparts, t->dW[l], n, t->splitsW[l], n);
-    } else {
-      rc = gemm_bf16(t->dZt, B, t->At, B, t->dW[l], nin, nullptr, nout, nin, B, t->err, st);
-      if (rc) return rc;
-    }
-    if (l == 0) k_fold_split_grad<<<(nout + 127) / 128, 128, 0, st>>>(t->dW[0], nout, nin, t->nin);
-    {
-      const int nparts = (B + kColRows - 1) / kColRows;
-      k_colsum_part<<<dim3((nout + 31) / 32, nparts), dim3(32, 8), 0, st>>>(t->dZf, t->colpart, B, nout);
-      k_colsum_finish<<<(nout + 7) / 8, 256, 0, st>>>(t->colpart, t->db[l], nparts, nout);
-    }
+    if (t->splitsW[l] > 1)
+      rc = gemm_bf16_splitk(t->dZt, B, t->At[l], B, t->dWparts[l], nin, (int64_t)nout * nin, t->splitsW[l], nout,
+                            nin, B, t->err, st);
+    else
+      rc = gemm_bf16(t->dZt, B, t->At[l], B, t->dWparts[l], nin, nullptr, nout, nin, B, t->err, st);
+    if (rc) return rc;
     if (l > 0) {
       rc = gemm_bf16(t->dZb, nout, t->Wt[l], nout, t->dA, nin, nullptr, B, nin, nout, t->err, st);
       if (rc) return rc;
-      const int64_t n = (int64_t)B * nin;
-      k_gelu_bwd<<<grid_for(n), 256, 0, st>>>(t->dA, t->Z[l - 1], t->dZf, t->dZb, n);
+      k_gelu_bwd<<<dim3((nin + 63) / 64, nrb), dim3(32, 8), 0, st>>>(t->dA, t->Z[l - 1], t->dZb, t->dZt,
+                                                                     t->colpart[l - 1], B, nin);
     }
   }
-  if (loss_out) CHEM_CUDA_TRY(cudaMemcpyAsync(loss_out, t->loss, sizeof(double), cudaMemcpyDeviceToDevice, st));
+  FinishSet F{};
+  int blocks = 0;
+  for (int l = 0; l < NL; ++l) {
+    const int64_t n = (int64_t)t->out_pad[l] * t->in_pad[l];
+    const int wb = (int)std::min<int64_t>((n + 255) / 256, 1024);
+    F.s[F.n++] = FinishSeg{t->dWparts[l], t->dW[l], n, t->splitsW[l], t->in_pad[l], l == 0 ? t->nin : 0,
+                           t->colpart[l], t->db[l], t->out_pad[l], blocks, wb};
+    blocks += wb + (t->out_pad[l] + 7) / 8;
+  }
+  F.nparts = nrb;
+  F.loss_part = t->loss_part; F.n_loss = (int)(mse_grid.x * mse_grid.y);
+  F.loss_scale = 1.0 / ((double)B * t->nout);
+  F.loss = t->loss; F.loss_out = loss_out;
+  k_finish_grads<<<blocks + 1, 256, 0, st>>>(F);
   CHEM_CUDA_TRY(cudaGetLastError());
   return CHEM_OK;
 }
@@ -572,27 +677,24 @@ extern "C" int chem_mlp_backward(chem_trainer_t t, const float* target, double* 
 static int adam_step(chem_trainer_t t, const float* lr_dev, float lr, float beta1, float beta2, float eps,
                      cudaStream_t st) {
   k_adam_prep<<<1, 1, 0, st>>>(t->d_step, t->d_coef, lr_dev, lr, beta1, beta2);
-  // every weight matrix and bias vector in one launch (BF16 copies of the hidden weights written
-  // on the way), then the transposed copies the backward pass multiplies with and the first
-  // layer's split copy
+  // every weight matrix and bias vector in one launch (their BF16 copies written on the way), then
+  // the transposed copies the backward pass multiplies with
   AdamSet A{};
   int blocks = 0;
-  auto add = [&](float* W, const float* G, float* m, float* v, __nv_bfloat16* Wb, int64_t n) {
-    A.s[A.n] = AdamSeg{W, G, m, v, Wb, n, blocks};
+  auto add = [&](float* W, const float* G, float* m, float* v, __nv_bfloat16* Wb, int64_t n, int nin, int ld) {
+    A.s[A.n] = AdamSeg{W, G, m, v, Wb, n, blocks, nin, ld};
     blocks += (int)std::min<int64_t>((n + 255) / 256, 1024);
     ++A.n;
   };
   for (int l = 0; l < t->nl; ++l) {
     const int r = t->out_pad[l], c = t->in_pad[l];
-    add(t->W[l], t->dW[l], t->mW[l], t->vW[l], l == 0 ? nullptr : t->Wb[l], (int64_t)r * c);
-    add(t->b[l], t->db[l], t->mb[l], t->vb[l], nullptr, r);
+    add(t->W[l], t->dW[l], t->mW[l], t->vW[l], t->Wb[l], (int64_t)r * c, l == 0 ? t->nin : 0, c);
+    add(t->b[l], t->db[l], t->mb[l], t->vb[l], nullptr, r, 0, 1);
   }
   k_adam_set<<<blocks, 256, 0, st>>>(A, t->d_coef, beta1, beta2, eps);
   TransposeSet T{};
   for (int l = 1; l < t->nl; ++l) T.j[T.n++] = TransposeJob{t->Wb[l], t->Wt[l], t->out_pad[l], t->in_pad[l]};
   if (T.n) launch_transposes(T, st);
-  k_split_bf16<<<grid_for((int64_t)t->out_pad[0] * t->in_pad[0]), 256, 0, st>>>(t->W[0], t->Wb[0], t->out_pad[0],
-                                                                                 t->in_pad[0], t->nin);
   CHEM_CUDA_TRY(cudaGetLastError());
   return CHEM_OK;
 }
@@ -644,32 +746,32 @@ extern "C" int chem_mlp_grad_count(chem_trainer_t t, int64_t* n) {
   return CHEM_OK;
 }
 
-extern "C" int chem_mlp_grad_pack(chem_trainer_t t, float* flat, chem_stream_t stream) {
-  if (!t || !flat) { set_error("NULL argument"); return CHEM_EINVAL; }
-  cudaStream_t st = (cudaStream_t)stream;
+static FlatSet flat_set(chem_trainer_t t) {
+  FlatSet S{};
   int64_t o = 0;
   for (int l = 0; l < t->nl; ++l) {
-    const int ro = t->real_out[l], ri = t->real_in[l];
-    CHEM_CUDA_TRY(cudaMemcpy2DAsync(flat + o, (size_t)ri * 4, t->dW[l], (size_t)t->in_pad[l] * 4, (size_t)ri * 4, ro,
-                                    cudaMemcpyDeviceToDevice, st));
-    o += (int64_t)ro * ri;
-    CHEM_CUDA_TRY(cudaMemcpyAsync(flat + o, t->db[l], (size_t)ro * 4, cudaMemcpyDeviceToDevice, st));
+    const int64_t ro = t->real_out[l], ri = t->real_in[l];
+    S.s[S.n++] = FlatSeg{t->dW[l], o, ro * ri, (int)ri, t->in_pad[l]};
+    o += ro * ri;
+    S.s[S.n++] = FlatSeg{t->db[l], o, ro, (int)ro, (int)ro};
     o += ro;
   }
+  S.total = o;
+  return S;
+}
+
+extern "C" int chem_mlp_grad_pack(chem_trainer_t t, float* flat, chem_stream_t stream) {
+  if (!t || !flat) { set_error("NULL argument"); return CHEM_EINVAL; }
+  const FlatSet S = flat_set(t);
+  k_flat_grads<<<grid_for(S.total), 256, 0, (cudaStream_t)stream>>>(S, flat, nullptr, 1.0f, 0);
+  CHEM_CUDA_TRY(cudaGetLastError());
   return CHEM_OK;
 }
 
 extern "C" int chem_mlp_grad_unpack(chem_trainer_t t, const float* flat, float scale, chem_stream_t stream) {
   if (!t || !flat || !std::isfinite(scale)) { set_error("bad arguments"); return CHEM_EINVAL; }
-  cudaStream_t st = (cudaStream_t)stream;
-  int64_t o = 0;
-  for (int l = 0; l < t->nl; ++l) {
-    const int ro = t->real_out[l], ri = t->real_in[l];
-    k_unpack_scaled<<<grid_for((int64_t)ro * ri), 256, 0, st>>>(flat + o, t->dW[l], ro, ri, t->in_pad[l], scale);
-    o += (int64_t)ro * ri;
-    k_unpack_scaled<<<grid_for(ro), 256, 0, st>>>(flat + o, t->db[l], ro, 1, 1, scale);
-    o += ro;
-  }
+  const FlatSet S = flat_set(t);
+  k_flat_grads<<<grid_for(S.total), 256, 0, (cudaStream_t)stream>>>(S, nullptr, flat, scale, 1);
   CHEM_CUDA_TRY(cudaGetLastError());
   return CHEM_OK;
 }
