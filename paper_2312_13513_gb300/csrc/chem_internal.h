@@ -20,6 +20,10 @@ constexpr double TMID = 1000.0;
 void set_error(const char* fmt, ...);
 int cuda_fail(cudaError_t e, const char* what);
 
+// stream-ordered temporary of one call (freed with cudaFreeAsync on the same stream), from the
+// library's pool of the current device
+cudaError_t ws_alloc(void** p, size_t bytes, cudaStream_t stream);
+
 #define CHEM_CUDA_TRY(call)                                   \
   do {                                                        \
     cudaError_t e_ = (call);                                  \

@@ -1948,7 +1948,7 @@ int launch_advance(chem_mech_s* m, double* T, const double* p, double* Y, int64_
   int rc = pick_shape(m, opt, &s);
   if (rc) return rc;
   unsigned long long* counter = nullptr;
-  CHEM_CUDA_TRY(cudaMallocAsync((void**)&counter, sizeof(unsigned long long), stream));
+  CHEM_CUDA_TRY(ws_alloc((void**)&counter, sizeof(unsigned long long), stream));
   CHEM_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(unsigned long long), stream));
   AdvanceParams P;
   mech_args(m, s, &P);
@@ -1977,7 +1977,7 @@ int launch_advance_counted(chem_mech_s* m, double* T, const double* p, double* Y
   int rc = pick_shape(m, nullptr, &s);
   if (rc) return rc;
   unsigned long long* counter = nullptr;
-  CHEM_CUDA_TRY(cudaMallocAsync((void**)&counter, sizeof(unsigned long long), stream));
+  CHEM_CUDA_TRY(ws_alloc((void**)&counter, sizeof(unsigned long long), stream));
   CHEM_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(unsigned long long), stream));
   AdvanceParams P;
   mech_args(m, s, &P);
@@ -2028,7 +2028,7 @@ int launch_advance_batch(chem_mech_s* m, const chem_segment* segs, int nseg, cud
     P.ncells_dev = nullptr;
     P.budget_ns = 0;
     unsigned long long* counter = nullptr;
-    CHEM_CUDA_TRY(cudaMallocAsync((void**)&counter, sizeof(unsigned long long), stream));
+    CHEM_CUDA_TRY(ws_alloc((void**)&counter, sizeof(unsigned long long), stream));
     CHEM_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(unsigned long long), stream));
     P.counter = counter;
     rc = dispatch_adv(s, P, nullptr, stream);

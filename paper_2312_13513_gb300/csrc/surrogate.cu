@@ -487,26 +487,44 @@ struct PostParams {
 };
 
 
-// The mixture's NASA-7 polynomials of one temperature range for a register-resident
-// composition (the sums of mixture_nasa, with the species loop unrolled to the array extent).
+// FP32 value near x (truncated) and exact FP64 value of f without the FP64 pipe's conversion
+// instructions (each takes the pipe as long as an FMA): the exponent is rebiased and the mantissa
+// shifted by integer instructions; what leaves the normal range takes the conversion
+__device__ __forceinline__ float f32_of(double x) {
+  const unsigned h = (unsigned)__double2hiint(x), e = h & 0x7ff00000u;
+  if (e - 0x38100000u >= 0x47e00000u - 0x38100000u) return (float)x;
+  const unsigned m = __funnelshift_l((unsigned)__double2loint(x), h, 3);
+  return __uint_as_float((h & 0x80000000u) | ((m - 0xC0000000u) & 0x7fffffffu));
+}
+__device__ __forceinline__ double f64_of(float f) {
+  const unsigned u = __float_as_uint(f), e = u & 0x7f800000u;
+  if (e == 0u || e == 0x7f800000u) return (double)f;
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+
+// The mixture's NASA-7 enthalpy polynomial of one temperature range for a register-resident
+// composition (the sums of mixture_nasa, with the species loop unrolled to the array extent), and
+// its cp polynomial in FP32: cp only scales the Newton steps on T (an error of 1e-7 in it leaves
+// 1e-7 of a step, and the accepted last step is below 1e-9 T).
 template <int AS>
 __device__ __forceinline__ void mixture_poly(const double (&Y)[AS], int ns, int rg, const double* hcoef,
                                              const double* ccoef, const double* invW, double (&Ah)[6],
-                                             double (&Ac)[5]) {
+                                             float (&Ac)[5]) {
 #pragma unroll
   for (int i = 0; i < 6; ++i) Ah[i] = 0.0;
 #pragma unroll
-  for (int i = 0; i < 5; ++i) Ac[i] = 0.0;
+  for (int i = 0; i < 5; ++i) Ac[i] = 0.0f;
 #pragma unroll
   for (int k = 0; k < AS; ++k) {
     if (k < ns) {
       const double yw = Y[k] * __ldg(invW + k);
+      const float yf = f32_of(yw);
       const double* a = hcoef + (rg * ns + k) * 6;
       const double* c = ccoef + (rg * ns + k) * 5;
 #pragma unroll
-      for (int i = 0; i < 6; ++i) Ah[i] = fma(yw, a[i], Ah[i]);
+      for (int i = 0; i < 6; ++i) Ah[i] = fma(yw, __ldg(a + i), Ah[i]);
 #pragma unroll
-      for (int i = 0; i < 5; ++i) Ac[i] = fma(yw, c[i], Ac[i]);
+      for (int i = 0; i < 5; ++i) Ac[i] = fmaf(yf, f32_of(__ldg(c + i)), Ac[i]);
     }
   }
 }
@@ -518,7 +536,7 @@ __device__ __forceinline__ void mixture_poly(const double (&Y)[AS], int ns, int 
 // composition's change (no separate sums of the start state), and reciprocals take three FP64
 // instructions (fx::rcp): about 350 FP64 instructions a cell instead of 540.
 template <int NS_, int NE_>
-__global__ void __launch_bounds__(256) surrogate_post_kernel(const PostParams P) {
+__global__ void __launch_bounds__(64) surrogate_post_kernel(const PostParams P) {
   constexpr int AS = NS_ > 0 ? NS_ : MAXNS;          // array extents
   constexpr int AE = NE_ > 0 ? NE_ : NEMAX;
   const int ns = NS_ > 0 ? NS_ : P.lay.ns;
@@ -535,8 +553,9 @@ __global__ void __launch_bounds__(256) surrogate_post_kernel(const PostParams P)
     for (int k = 0; k < AS; ++k) {
       if (k < ns) {
         Y0[k] = P.Y[(int64_t)k * P.ld + cell];
-        Y1[k] = (double)P.ynet[(int64_t)k * P.ncells + cell];
-        if (!isfinite(Y1[k])) pass = false;
+        const float yn = P.ynet[(int64_t)k * P.ncells + cell];
+        if ((__float_as_uint(yn) & 0x7f800000u) == 0x7f800000u) pass = false;      // infinite or NaN
+        Y1[k] = f64_of(yn);
       }
     }
     double Tn = T0;
@@ -679,21 +698,24 @@ __global__ void __launch_bounds__(256) surrogate_post_kernel(const PostParams P)
             if (k < ns) {
               const double* a = hcoef + (rg0 * ns + k) * 6;
               const double hR = a[5] + T0 * (a[0] + T0 * (a[1] + T0 * (a[2] + T0 * (a[3] + T0 * a[4]))));
-              hs += Y0[k] * hR * __ldg(invW + k);
+              hs = fma(Y0[k] * __ldg(invW + k), hR, hs);
             }
           }
-          h0 = RU * hs;
+          h0 = hs;
         }
-        double Ah[6], Ac[5];
+        // h in units of R: dT = (h / R - h0 / R) / (cp / R)
+        double Ah[6];
+        float Ac[5];
         int rg = Tn < TMID ? 0 : 1;
         mixture_poly<AS>(Y1, ns, rg, hcoef, ccoef, invW, Ah, Ac);
         bool conv = false;
         for (int it = 0; it < 50; ++it) {
           const int r = Tn < TMID ? 0 : 1;
           if (r != rg) { rg = r; mixture_poly<AS>(Y1, ns, rg, hcoef, ccoef, invW, Ah, Ac); }
-          double hh, cp;
-          h_cp_from_mixture(Ah, Ac, Tn, &hh, &cp);
-          const double dT = (hh - h0) * fx::rcp(cp);
+          const double hh = Ah[5] + Tn * (Ah[0] + Tn * (Ah[1] + Tn * (Ah[2] + Tn * (Ah[3] + Tn * Ah[4]))));
+          const float tf = f32_of(Tn);
+          const float cp = fmaf(tf, fmaf(tf, fmaf(tf, fmaf(tf, Ac[4], Ac[3]), Ac[2]), Ac[1]), Ac[0]);
+          const double dT = (hh - h0) * f64_of(1.0f / cp);
           Tn -= dT;
           if (!(Tn >= 200.0 && Tn <= 6000.0)) break;
           if (fabs(dT) < 1e-9 * Tn) { conv = true; break; }
@@ -1247,7 +1269,7 @@ extern "C" int chem_surrogate_forward(chem_model_t md, const double* T, const do
   if (!T || !p || !Y || !ynet || !out_of_box) { set_error("NULL pointer"); return CHEM_EINVAL; }
   cudaStream_t st = (cudaStream_t)stream;
   int* err = nullptr;
-  CHEM_CUDA_TRY(cudaMallocAsync((void**)&err, sizeof(int), st));
+  CHEM_CUDA_TRY(ws_alloc((void**)&err, sizeof(int), st));
   CHEM_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int), st));
   int rc = surrogate_forward(md, T, p, Y, ld, ncells, ynet, zout, out_of_box, err, st);
   int herr = 0;
@@ -1349,7 +1371,7 @@ extern "C" int chem_surrogate_advance_batch(chem_model_t md, chem_mech_t mech, c
     P.nseg = cnt; P.ns = ns; P.n = n;
     unsigned char* ws = nullptr;
     const size_t bT = (size_t)n * 8, bY = (size_t)n * ns * 8, bR = ((size_t)n + 15) & ~(size_t)15;
-    CHEM_CUDA_TRY(cudaMallocAsync((void**)&ws, 2 * bT + bY + bR, st));
+    CHEM_CUDA_TRY(ws_alloc((void**)&ws, 2 * bT + bY + bR, st));
     P.T = (double*)ws; P.p = (double*)(ws + bT); P.Y = (double*)(ws + 2 * bT);
     int8_t* route = (int8_t*)(ws + 2 * bT + bY);
     P.route = route;
@@ -1389,7 +1411,7 @@ extern "C" int chem_surrogate_advance(chem_model_t md, chem_mech_t mech, double*
   const size_t b_ynet = (size_t)ncells * md->ns * 4, b_box = ((size_t)ncells + 15) & ~(size_t)15;
   const size_t b_idx = (size_t)ncells * 4;
   unsigned char* ws = nullptr;
-  CHEM_CUDA_TRY(cudaMallocAsync((void**)&ws, b_ynet + b_box + b_idx + 64, st));
+  CHEM_CUDA_TRY(ws_alloc((void**)&ws, b_ynet + b_box + b_idx + 64, st));
   float* ynet = (float*)ws;
   uint8_t* box = ws + b_ynet;
   int32_t* fb_idx = (int32_t*)(ws + b_ynet + b_box);
@@ -1405,9 +1427,12 @@ extern "C" int chem_surrogate_advance(chem_model_t md, chem_mech_t mech, double*
     int sms = 0, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const long long blocks = std::min<long long>((ncells + 255) / 256, (long long)sms * 16);
-    if (md->ns == 9 && md->ne == 3) surrogate_post_kernel<9, 3><<<(unsigned)blocks, 256, 0, st>>>(Q);
-    else surrogate_post_general<<<(unsigned)blocks, 256, 0, st>>>(Q);
+    // two-warp blocks: a warp's chain of FP64 instructions has a sub-partition to itself while there
+    // are no more than two blocks an SM (10007 cells: 157 blocks on 152 SMs; 256-thread blocks used
+    // 40 SMs and took 35 us)
+    const long long blocks = std::min<long long>((ncells + 63) / 64, (long long)sms * 64);
+    if (md->ns == 9 && md->ne == 3) surrogate_post_kernel<9, 3><<<(unsigned)blocks, 64, 0, st>>>(Q);
+    else surrogate_post_general<<<(unsigned)blocks, 64, 0, st>>>(Q);
     cudaError_t le = cudaGetLastError();
     if (le != cudaSuccess) rc = cuda_fail(le, "surrogate_post_kernel");
   }
