@@ -76,14 +76,14 @@ int make_tmap_bf16(CUtensorMap* map, const void* base, int64_t rows, int64_t col
 
 namespace {
 
-constexpr int BM = 128, BN = 128, BK = 64;      // tile rows, the narrower tile width, K step
+constexpr int BM = 128, BN = 128, BK = 64;      // tile rows, the narrowest tile width, K step
 
 struct GemmArgs {
   float* C;
   __nv_bfloat16* Cb;       // non-null: BF16 output of the activation epilogue instead of C
   float* Cz;               // with Cb (persistent kernel): also the FP32 pre-activation, same pitch
   int gelu;                // activation epilogue: apply GELU before rounding
-  int vec;                 // output base and row pitch allow 16-byte stores
+  int vec;                 // bytes per store that output bases and row pitch allow: 32, 16 or 0
   const float* bias;
   int M, N, K;
   int64_t ldc;
@@ -100,17 +100,20 @@ struct GemmArgs {
 // within a row block, so consecutive tiles share their A rows in L2) with a 128 x BN_ tile and
 // two TMEM accumulators: the epilogue of one tile runs while the MMAs of the next fill the other
 // accumulator.  Warp 0 (one lane): TMA producer over a STAGES_P-stage ring; warp 1 (one lane):
-// MMA issuer; warps 2-17: epilogue (warp w reads TMEM lanes 32 (w % 4) .. + 31 and the columns of
-// quarter (w - 2) / 4 of the tile: four warps per scheduler hide the latency of the bias, GELU and
-// store chain), storing each row's 32-column pieces straight to global memory.
+// MMA issuer; warps 2-17: epilogue (warp w reads TMEM lanes 32 (w % 4) .. + 31 and every fourth
+// 16-column unit of the tile: four warps per scheduler hide the latency of the bias, GELU and store
+// chain), storing each row's 16 columns straight to global memory, 32 bytes a lane and store where
+// the output's alignment allows it (one whole sector).
 // ---------------------------------------------------------------------------------------
 constexpr int kPersistThreads = 576;     // TMA warp, MMA warp, sixteen epilogue warps
 
 template <int BN_>
 struct PersistCfg {
-  static constexpr int STAGES_P = BN_ == 256 ? 4 : 6;
+  static constexpr int STAGES_P = BN_ > 160 ? 4 : (BN_ > 128 ? 5 : 6);
+  static constexpr int ACC = BN_ > 128 ? 256 : 128;        // TMEM columns between the two accumulators
+  static constexpr int TMEM = 2 * ACC;
   static constexpr int TA = BM * BK * 2;                   // 16 KB
-  static constexpr int TB = BN_ * BK * 2;                  // 16 or 32 KB
+  static constexpr int TB = BN_ * BK * 2;                  // 16 to 32 KB, whole 8-row groups
   static constexpr int SMEM = STAGES_P * (TA + TB) + 1024 + 256;
 };
 
@@ -155,7 +158,7 @@ __global__ void __launch_bounds__(kPersistThreads, 1)
     prefetch_tmap(&tmA);
     prefetch_tmap(&tmB);
   }
-  if (warp == 0) tmem_alloc(tmem_slot, 2 * BN_);
+  if (warp == 0) tmem_alloc(tmem_slot, Cfg::TMEM);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -192,7 +195,7 @@ __global__ void __launch_bounds__(kPersistThreads, 1)
         // the epilogue has drained this accumulator (its use two tiles ago)
         if (rd >= 2 && !mbar_wait(&acc_empty[b], (uint32_t)(((rd - 2) >> 1) & 1), a.err)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t d = tmem + (uint32_t)(b * BN_);
+        const uint32_t d = tmem + (uint32_t)(b * Cfg::ACC);
         for (int kb = 0; kb < nk; ++kb, ++it) {
           const int s = (int)(it % NS);
           if (!mbar_wait(&full[s], (uint32_t)((it / NS) & 1), a.err)) { ok = false; break; }
@@ -211,7 +214,7 @@ __global__ void __launch_bounds__(kPersistThreads, 1)
     // epilogue warps 2-17
     const int quarter = warp & 3, part = (warp - 2) >> 2;
     const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16);
-    constexpr int HW = BN_ / 4;                              // columns per epilogue warp
+    constexpr int UNITS = BN_ / 16;
     bool ok = true;
     for (long long rd = 0; rd < rounds && ok; ++rd) {
       int m0, n0, kb0, split;
@@ -221,75 +224,61 @@ __global__ void __launch_bounds__(kPersistThreads, 1)
       tc_fence_after();
       const int row = m0 + quarter * 32 + lane;
       const bool rv = row < a.M;
-      const uint32_t tb = trow + (uint32_t)(b * BN_ + part * HW);
+      const uint32_t tb = trow + (uint32_t)(b * Cfg::ACC);
 #pragma unroll 1
-      for (int cc = 0; cc < HW; cc += 32) {
-        uint32_t r[32];
-        tmem_ld32(tb + cc, r);
-        tmem_ld_wait(r);
-        const int col = n0 + part * HW + cc;
-        if (a.Cb) {
-          if (a.Cz) {
-            // the pre-activation z = acc + bias, kept in r for the activation below
+      for (int u = part; u < UNITS; u += 4) {
+        uint32_t r[16];
+        tmem_ld16(tb + 16 * u, r);
+        tmem_ld_wait16(r);
+        const int col = n0 + 16 * u;
+        const bool full = col + 16 <= a.N;
+        if (a.bias) {
 #pragma unroll
-            for (int j = 0; j < 32; ++j)
-              r[j] = __float_as_uint(__uint_as_float(r[j]) + (a.bias && col + j < a.N ? a.bias[col + j] : 0.0f));
-            if (rv) {
-              float* outz = a.Cz + (int64_t)row * a.ldc + col;
-              if (a.vec && col + 32 <= a.N) {
+          for (int j = 0; j < 16; ++j)
+            r[j] = __float_as_uint(__uint_as_float(r[j]) + (full || col + j < a.N ? __ldg(a.bias + col + j) : 0.0f));
+        }
+        if (!a.Cb || a.Cz) {                                 // FP32: the product, or the pre-activation
+          if (rv) {
+            float* out = (a.Cb ? a.Cz : a.C + (SPLITK_ ? split * a.split_stride : 0)) + (int64_t)row * a.ldc + col;
+            if (full && a.vec == 32) {
+              st_global_32(out, r);
+              st_global_32(out + 8, r + 8);
+            } else if (full && a.vec == 16) {
 #pragma unroll
-                for (int q = 0; q < 8; ++q)
-                  reinterpret_cast<float4*>(outz)[q] =
-                      make_float4(__uint_as_float(r[4 * q]), __uint_as_float(r[4 * q + 1]),
-                                  __uint_as_float(r[4 * q + 2]), __uint_as_float(r[4 * q + 3]));
-              } else {
+              for (int q = 0; q < 4; ++q)
+                reinterpret_cast<uint4*>(out)[q] = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+            } else {
 #pragma unroll
-                for (int j = 0; j < 32; ++j)
-                  if (col + j < a.N) outz[j] = __uint_as_float(r[j]);
-              }
+              for (int j = 0; j < 16; ++j)
+                if (col + j < a.N) out[j] = __uint_as_float(r[j]);
             }
           }
-          const bool add_bias = a.bias && !a.Cz;
-          uint32_t pk[16];
+        }
+        if (a.Cb) {
+          uint32_t pk[8];
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const int cj = col + 2 * j;
-            float v0 = __uint_as_float(r[2 * j]) + (add_bias && cj < a.N ? a.bias[cj] : 0.0f);
-            float v1 = __uint_as_float(r[2 * j + 1]) + (add_bias && cj + 1 < a.N ? a.bias[cj + 1] : 0.0f);
+          for (int j = 0; j < 8; ++j) {
+            float v0 = __uint_as_float(r[2 * j]), v1 = __uint_as_float(r[2 * j + 1]);
             if (a.gelu) gelu2(v0, v1);
             __nv_bfloat162 hv = __floats2bfloat162_rn(v0, v1);
             pk[j] = *reinterpret_cast<uint32_t*>(&hv);
           }
           if (rv) {
             __nv_bfloat16* out = a.Cb + (int64_t)row * a.ldc + col;
-            if (a.vec && col + 32 <= a.N) {
-#pragma unroll
-              for (int q = 0; q < 4; ++q)
-                reinterpret_cast<uint4*>(out)[q] = make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
+            if (full && a.vec == 32) {
+              st_global_32(out, pk);
+            } else if (full && a.vec == 16) {
+              reinterpret_cast<uint4*>(out)[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+              reinterpret_cast<uint4*>(out)[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
             } else {
 #pragma unroll
-              for (int j = 0; j < 32; ++j) {
+              for (int j = 0; j < 16; ++j) {
                 if (col + j < a.N) {
                   const uint32_t w = pk[j >> 1];
                   reinterpret_cast<uint16_t*>(out)[j] = (uint16_t)((j & 1) ? (w >> 16) : (w & 0xffffu));
                 }
               }
             }
-          }
-        } else if (rv) {
-          float* out = a.C + (SPLITK_ ? split * a.split_stride : 0) + (int64_t)row * a.ldc + col;
-          float v[32];
-#pragma unroll
-          for (int j = 0; j < 32; ++j)
-            v[j] = __uint_as_float(r[j]) + (a.bias && col + j < a.N ? a.bias[col + j] : 0.0f);
-          if (a.vec && col + 32 <= a.N) {
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-              reinterpret_cast<float4*>(out)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-          } else {
-#pragma unroll
-            for (int j = 0; j < 32; ++j)
-              if (col + j < a.N) out[j] = v[j];
           }
         }
       }
@@ -299,7 +288,7 @@ __global__ void __launch_bounds__(kPersistThreads, 1)
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) tmem_dealloc(tmem, 2 * BN_);
+  if (warp == 0) tmem_dealloc(tmem, Cfg::TMEM);
 }
 
 }  // namespace
@@ -327,12 +316,13 @@ static int gemm_launch(const void* A, int64_t lda, const void* B, int64_t ldb, f
   CUtensorMap ta, tb;
   int rc = make_tmap_bf16(&ta, A, M, K, lda, BM, BK);
   if (rc) return rc;
-  rc = make_tmap_bf16(&tb, B, N, K, ldb, BN, BK);
-  if (rc) return rc;
-  const uintptr_t obase = C ? (uintptr_t)C : (uintptr_t)Cb;
-  const int64_t opitch = ldc * (C ? 4 : 2);
-  int vec = (obase % 16 == 0 && opitch % 16 == 0) ? 1 : 0;
-  if (Cz && ((uintptr_t)Cz % 16 != 0 || (ldc * 4) % 16 != 0)) vec = 0;
+  // the widest store that every output row's 16-column pieces allow
+  auto width = [&](const void* p, int64_t pitch, int64_t stride) {
+    const uintptr_t m = (uintptr_t)p | (uintptr_t)pitch | (uintptr_t)stride;
+    return m % 32 == 0 ? 32 : (m % 16 == 0 ? 16 : 0);
+  };
+  int vec = C ? width(C, ldc * 4, splits > 1 ? split_stride * 4 : 0) : width(Cb, ldc * 2, 0);
+  if (Cz) vec = std::min(vec, width(Cz, ldc * 4, 0));
   GemmArgs g{C, (__nv_bfloat16*)Cb, Cz, gelu, vec, bias, M, N, K, ldc, err};
   g.splits = splits;
   g.split_stride = split_stride;
@@ -342,22 +332,38 @@ static int gemm_launch(const void* A, int64_t lda, const void* B, int64_t ldb, f
     CHEM_CUDA_TRY(cudaGetDevice(&dev));
     CHEM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   }
-  // persistent kernel, 256-column tiles unless 128-column tiles pad N less, or unless 256-column
-  // tiles would leave SMs without a tile (small products: more, smaller tiles finish sooner)
-  const int pad128 = (N + 127) / 128 * 128 - N, pad256 = (N + 255) / 256 * 256 - N;
-  int bn = (N >= 256 && pad256 <= pad128) ? 256 : 128;
-  if (bn == 256 && (long long)((M + BM - 1) / BM) * ((N + 255) / 256) * splits < sms) bn = 128;
+  // Tile width.  Operand traffic from L2 bounds the large products (65536 x 800 x 1600 on 128-wide
+  // tiles: 10 TB/s at 814 TFLOP/s), and a row block's traffic is its tile count times the rows of A
+  // and B that a tile reads: the width of 256, 208, 160 or 128 that needs the least (800 and 400
+  // columns: 208, four and two tiles).  128 where wider tiles would leave SMs without one (small
+  // products: more, smaller tiles finish sooner).
+  int bn = 256;
+  long long cost = -1;
+  for (int w : {256, 208, 160, 128}) {
+    const long long c = (long long)((N + w - 1) / w) * (BM + w);
+    if (cost < 0 || c < cost) { cost = c; bn = w; }
+  }
+  if (bn > 128 && (long long)((M + BM - 1) / BM) * ((N + bn - 1) / bn) * splits < sms) bn = 128;
   const long long ntiles = (long long)((M + BM - 1) / BM) * ((N + bn - 1) / bn) * splits;
   const unsigned grid = (unsigned)std::min<long long>(ntiles, sms);
-  if (bn == 256) {
-    CUtensorMap tb2;
-    rc = make_tmap_bf16(&tb2, B, N, K, ldb, 256, BK);
-    if (rc) return rc;
-    rc = splits > 1 ? launch_persistent<256, true>(ta, tb2, g, grid, stream)
-                    : launch_persistent<256, false>(ta, tb2, g, grid, stream);
-  } else {
-    rc = splits > 1 ? launch_persistent<128, true>(ta, tb, g, grid, stream)
-                    : launch_persistent<128, false>(ta, tb, g, grid, stream);
+  rc = make_tmap_bf16(&tb, B, N, K, ldb, bn, BK);
+  if (rc) return rc;
+  switch (bn) {
+    case 256:
+      rc = splits > 1 ? launch_persistent<256, true>(ta, tb, g, grid, stream)
+                      : launch_persistent<256, false>(ta, tb, g, grid, stream);
+      break;
+    case 208:
+      rc = splits > 1 ? launch_persistent<208, true>(ta, tb, g, grid, stream)
+                      : launch_persistent<208, false>(ta, tb, g, grid, stream);
+      break;
+    case 160:
+      rc = splits > 1 ? launch_persistent<160, true>(ta, tb, g, grid, stream)
+                      : launch_persistent<160, false>(ta, tb, g, grid, stream);
+      break;
+    default:
+      rc = splits > 1 ? launch_persistent<128, true>(ta, tb, g, grid, stream)
+                      : launch_persistent<128, false>(ta, tb, g, grid, stream);
   }
   if (rc) return rc;
   CHEM_CUDA_TRY(cudaGetLastError());

@@ -4,12 +4,12 @@
 //
 // The widths do not fit the fused single-network kernel (a 128 x 1600 BF16 activation tile alone
 // is 400 KB), so the networks run layer by layer on the tcgen05 GEMM with its activation epilogue
-// (bias, exact-erf GELU and BF16 rounding fused into the accumulator read-back): per chunk of
-// 16384 cells, one feature kernel; one grouped GEMM for the first layers of all networks (they
-// share the input, so their weights stack into one [nnet h1 x 64] operand); then for every species
-// two GEMMs reading its column block of that output and an output dot product; then one
-// inverse-transform kernel.  A species' later activations (26 + 13 MB) stay in the 129 MB L2.  The output layer (400 -> 1) is a warp-per-cell dot
-// product of BF16 values with FP32 accumulation, the precision of the single network's output MMA.
+// (bias, exact-erf GELU and BF16 rounding fused into the accumulator read-back): per pass of about
+// 32768 cells, one feature kernel; for every species three GEMMs and an output dot product; then one
+// inverse-transform kernel.  One species' activations (105 + 52 + 26 MB) turn over in the 129 MB L2;
+// stacking all first layers into one GEMM wrote and re-read 1.7 GB a pass.  The output layer
+// (400 -> 1) is a warp-per-cell dot product of BF16 values with FP32 accumulation, the precision of
+// the single network's output MMA.
 // Everything after the network (projection, Newton on T, fallback) is shared with the single
 // network (surrogate.cu).
 #include <cuda_bf16.h>
@@ -31,10 +31,11 @@ int gemm_bf16_act(const void* A, int64_t lda, const void* B, int64_t ldb, void* 
 
 namespace {
 
-// cells per pass of the layer-by-layer schedule: 65536 rows give the GEMMs enough tiles to fill
-// the GPU several times over; the stacked first-layer output of a pass is 65536 x (networks x h1)
-// BF16 (1.7 GB for eight 1600-wide networks, stream-ordered workspace)
-constexpr int64_t kPsChunk = 65536;
+// Cells per pass of the layer-by-layer schedule, about: 32768 rows give the GEMMs enough tiles to
+// fill the GPU several times over, and a network's first-layer output of a pass (32768 x 1600 BF16,
+// 105 MB) is read back from the 129 MB L2 by its second layer.  Passes are of equal size, so that no
+// short one runs every layer for a few cells.
+constexpr int64_t kPsChunk = 32768;
 
 struct PsFeatParams {
   const double *T, *p, *Y;
@@ -131,14 +132,14 @@ int surrogate_forward_ps(chem_model_s* md, const double* T, const double* p, con
                          int64_t ncells, float* ynet, float* zout, uint8_t* outbox, int* err,
                          cudaStream_t st) {
   const int h1 = md->h[0], h2 = md->h[1], h3 = md->h[2];
-  const int64_t chunk = std::min<int64_t>(ncells, kPsChunk);
+  const int64_t passes = std::max<int64_t>(1, (ncells + kPsChunk / 2) / kPsChunk);
+  const int64_t chunk = std::min<int64_t>(ncells, ((ncells + passes - 1) / passes + 127) / 128 * 128);
   const int64_t Mp = std::max<int64_t>(chunk, 128);           // a GEMM needs at least one 128-row tile
   auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
-  const int nnet = std::max(md->nnet, 1), ld1 = nnet * h1;     // A1 holds every network's first layer
-  const size_t bX = al((size_t)Mp * SUR_KIN * 2), bA1 = al((size_t)Mp * ld1 * 2), bA2 = al((size_t)Mp * h2 * 2);
+  const size_t bX = al((size_t)Mp * SUR_KIN * 2), bA1 = al((size_t)Mp * h1 * 2), bA2 = al((size_t)Mp * h2 * 2);
   const size_t bA3 = al((size_t)Mp * h3 * 2), bz = al((size_t)std::max(md->nnet, 1) * Mp * 4);
   unsigned char* ws = nullptr;
-  CHEM_CUDA_TRY(cudaMallocAsync((void**)&ws, bX + bA1 + bA2 + bA3 + bz, st));
+  CHEM_CUDA_TRY(ws_alloc((void**)&ws, bX + bA1 + bA2 + bA3 + bz, st));
   __nv_bfloat16* X = (__nv_bfloat16*)ws;
   __nv_bfloat16* A1 = (__nv_bfloat16*)(ws + bX);
   __nv_bfloat16* A2 = (__nv_bfloat16*)(ws + bX + bA1);
@@ -157,12 +158,10 @@ int surrogate_forward_ps(chem_model_s* md, const double* T, const double* p, con
     F.ns = md->ns; F.nin = md->nin; F.xmu = md->xmu; F.xsd = md->xsd; F.lo = md->lo; F.hi = md->hi;
     F.X = X; F.outbox = outbox + c0;
     k_ps_features<<<blocks_for(M, 256), 256, 0, st>>>(F);
-    if (md->nnet > 0)   // stacked first layers: net s's weights and biases follow net s - 1's
-      rc = gemm_bf16_act(X, SUR_KIN, md->net[0].W1, SUR_KIN, A1, ld1, md->net[0].b1, 1, M, md->nnet * h1, SUR_KIN,
-                         err, st);
     for (int s = 0; s < md->nnet && !rc; ++s) {
       const PsNet& n = md->net[s];
-      rc = gemm_bf16_act(A1 + (size_t)s * h1, ld1, n.W2, h1, A2, h2, n.b2, 1, M, h2, h1, err, st);
+      rc = gemm_bf16_act(X, SUR_KIN, n.W1, SUR_KIN, A1, h1, n.b1, 1, M, h1, SUR_KIN, err, st);
+      if (!rc) rc = gemm_bf16_act(A1, h1, n.W2, h1, A2, h2, n.b2, 1, M, h2, h1, err, st);
       if (!rc) rc = gemm_bf16_act(A2, h2, n.W3, h2, A3, h3, n.b3, 1, M, h3, h2, err, st);
       if (!rc) k_ps_out<<<blocks_for(nc * 32, 256), 256, 0, st>>>(A3, h3, (const __nv_bfloat16*)n.w4, n.b4, nc,
                                                                   z + (int64_t)s * Mp);

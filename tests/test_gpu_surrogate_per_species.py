@@ -156,3 +156,35 @@ def test_trainer_with_per_species_widths_matches_oracle():
         rel = np.linalg.norm(dW[l] - gW[l]) / np.linalg.norm(gW[l])
         relb = np.linalg.norm(db[l] - gb[l]) / np.linalg.norm(gb[l])
         assert rel < 2e-2 and relb < 2e-2, (l, rel, relb)
+
+
+@pytest.mark.parametrize("M,N,K,ldc", [(128, 128, 64, 128), (300, 160, 64, 160), (385, 208, 128, 208), (257, 400, 192, 400),
+                                       (20000, 400, 64, 400), (20000, 800, 64, 801), (20000, 833, 64, 840),
+                                       (20000, 1600, 64, 1608), (129, 513, 70, 513)])
+def test_gemm_tile_widths_and_store_widths(M, N, K, ldc):
+    """Every tile width the dispatch picks (128 to 256 columns), ragged edges in M, N and K, and
+    outputs whose pitch allows 32-byte, 16-byte and single stores, against FP32 torch."""
+    import ctypes
+    from paper_2312_13513_gb300 import _lib
+    g = torch.Generator(device="cuda").manual_seed(M + N)
+    lda = (K + 7) // 8 * 8
+    A = torch.randn(M, lda, device="cuda", generator=g).bfloat16()
+    B = (torch.randn(N, lda, device="cuda", generator=g) / K ** 0.5).bfloat16()
+    bias = torch.randn(N, device="cuda", generator=g)
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    st = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    p = lambda t: ctypes.c_void_p(t.data_ptr())
+    C = torch.full((M, ldc), 7.0, device="cuda")
+    Cb = torch.full((M, ldc), 7.0, device="cuda", dtype=torch.bfloat16)
+    L = _lib.load()
+    assert L.chem_gemm_bf16(p(A), lda, p(B), lda, p(C), ldc, p(bias), M, N, K, p(err), st) == 0
+    assert L.chem_gemm_bf16_act(p(A), lda, p(B), lda, p(Cb), ldc, p(bias), 1, M, N, K, p(err), st) == 0
+    torch.cuda.synchronize()
+    assert int(err.item()) == 0
+    ref = A[:, :K].double() @ B[:, :K].double().T + bias.double()
+    # FP32 accumulation of K products of size O(1 / sqrt K): K additions at 2^-24 of at most ~6
+    assert torch.allclose(C[:, :N].double(), ref, rtol=0, atol=6 * K * 2.0 ** -24)
+    act = torch.nn.functional.gelu(ref)
+    # one BF16 rounding (2^-9 relative) and the GELU form's 5e-7
+    assert torch.all((Cb[:, :N].double() - act).abs() <= 2.0 ** -8 * act.abs() + 1e-5)
+    assert torch.all(C[:, N:] == 7.0) and torch.all(Cb[:, N:] == 7.0)         # nothing beyond column N
