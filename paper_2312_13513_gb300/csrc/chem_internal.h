@@ -100,6 +100,7 @@ struct chem_mech_s {
   void* d_tab = nullptr;                  // tables of fixed.cuh
   const unsigned long long *d_e2 = nullptr, *d_lg = nullptr;
   const unsigned int* d_rc = nullptr;
+  const chem::FxEnthalpy* d_hk = nullptr; // [2][ns], null where a coefficient does not fit
 };
 
 namespace chem {

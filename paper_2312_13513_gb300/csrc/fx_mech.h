@@ -53,6 +53,16 @@ struct FxSpecies {
   int64_t c[5];               // cp/R
 };
 
+// Enthalpy h/(R W) (K mol/g) and heat capacity cp/(R W) of one species in one temperature range as
+// polynomials in tau = T / 2^r, each scaled by the largest power of two at which the magnitudes of its
+// terms sum to less than 2^62 (2^fh, 2^fc); the leading coefficients h[5] and c[4] are biased.
+// cf: the heat capacity in FP32
+struct FxEnthalpy {
+  int64_t h[6], c[5];
+  int32_t fh, fc;
+  float cf[5], pad[3];
+};
+
 struct FxLayout {
   int ns, ntb, bytes;         // bytes = 0: no fixed-point form
   int o_exp2, o_lg, o_rcp;    // tables of fixed.cuh

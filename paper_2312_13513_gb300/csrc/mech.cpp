@@ -157,6 +157,8 @@ struct FxNumbers {
   std::vector<FxTroe> troe;
   int64_t lpr0 = 0;
   const long double l2 = std::log(2.0L);
+  bool hok = true;                                 // the enthalpy polynomials below fit
+  std::vector<FxEnthalpy> hk;                      // [2][ns]
 
   int64_t q52l(long double v, double lim) {
     if (!(std::fabs((double)v) <= lim)) { ok = false; return 0; }
@@ -208,7 +210,7 @@ struct FxNumbers {
     *Ta_ = fx::biased(fits ? q52l((long double)Ea / (long double)RC / l2 / 128.0L, 1900.0) : 0);
   }
 
-  FxNumbers(const chem_mech_desc* d, const std::vector<std::vector<int>>& nu) {
+  FxNumbers(const chem_mech_desc* d, const std::vector<std::vector<int>>& nu, const std::vector<double>& W) {
     const int ns = d->n_species, nr = d->n_reactions;
     sp.resize(2 * (size_t)ns);
     for (int r = 0; r < 2; ++r)
@@ -238,6 +240,31 @@ struct FxNumbers {
         sg += 12.0 * std::fabs((double)S.gl) / 16.0;
         if (!(std::max(std::max(sg, sh_), sc) <= 2000.0 * 4503599627370496.0)) ok = false;
         for (int64_t* x : {&S.g[4], &S.h[4], &S.c[4], &S.ga6, &S.gl, &S.ha6}) *x = (int64_t)fx::biased(*x);
+      }
+    hk.resize(2 * (size_t)ns);
+    for (int r = 0; r < 2; ++r)
+      for (int k = 0; k < ns; ++k) {
+        const double* a = (r == 0 ? d->nasa_lo : d->nasa_hi) + 7 * k;
+        FxEnthalpy& E = hk[(size_t)r * ns + k];
+        const long double t = std::ldexp(1.0L, r == 0 ? kFxR0 : kFxR1), w = W[k];
+        long double hv[6], cv[5], pw = 1.0L, hs = 0.0L, cs = 0.0L;
+        hv[0] = a[5] / w;
+        for (int i = 0; i < 5; ++i) {
+          cv[i] = a[i] * pw / w;
+          pw *= t;
+          hv[i + 1] = a[i] / (i + 1) * pw / w;
+        }
+        for (int i = 0; i < 6; ++i) hs += std::fabs(hv[i]);
+        for (int i = 0; i < 5; ++i) cs += std::fabs(cv[i]);
+        if (!(hs < 1e12L && cs < 1e12L)) { hok = false; continue; }
+        auto frac = [](long double sum) { return sum > 0.0L ? std::min(60, 61 - (int)std::floor(std::log2(sum))) : 60; };
+        E.fh = frac(hs * 1.0001L);
+        E.fc = frac(cs * 1.0001L);
+        for (int i = 0; i < 6; ++i) E.h[i] = (int64_t)std::nearbyintl(std::ldexp(hv[i], E.fh));
+        for (int i = 0; i < 5; ++i) E.c[i] = (int64_t)std::nearbyintl(std::ldexp(cv[i], E.fc));
+        E.h[5] = (int64_t)fx::biased(E.h[5]);
+        E.c[4] = (int64_t)fx::biased(E.c[4]);
+        for (int i = 0; i < 5; ++i) E.cf[i] = (float)cv[i];
       }
     lpr0 = q52l(std::log((long double)PATM / (long double)RU) / l2, 1000.0);
     lnA.resize(nr); beta.resize(nr); Ta.resize(nr);
@@ -699,21 +726,25 @@ int build(const chem_mech_desc* din, chem_mech_s* m) {
   }
   P.nterm = (int)src.size();
 
+  const FxNumbers fxn(d, nu, m->W);
   {
-    // the tables of fixed.cuh in global memory: step control of every kernel, temperature functions
+    // the tables of fixed.cuh in global memory (step control of every kernel, transport fits) and
+    // the enthalpy polynomials (thermo kernels, surrogate post-processing)
     Builder T;
     const int o0 = T.add(sizeof(kExp2Tab)), o1 = T.add(sizeof(kLog2Tab)), o2 = T.add(sizeof(kRcpTab));
     memcpy(T.at<unsigned char>(o0), kExp2Tab, sizeof(kExp2Tab));
     memcpy(T.at<unsigned char>(o1), kLog2Tab, sizeof(kLog2Tab));
     memcpy(T.at<unsigned char>(o2), kRcpTab, sizeof(kRcpTab));
+    const int o3 = T.add((int)(fxn.hk.size() * sizeof(FxEnthalpy)));
+    put(T, o3, fxn.hk);
     CHEM_CUDA_TRY(cudaMalloc(&m->d_tab, T.buf.size()));
     CHEM_CUDA_TRY(cudaMemcpy(m->d_tab, T.buf.data(), T.buf.size(), cudaMemcpyHostToDevice));
     const unsigned char* t = (const unsigned char*)m->d_tab;
     m->d_e2 = (const unsigned long long*)(t + o0);
     m->d_lg = (const unsigned long long*)(t + o1);
     m->d_rc = (const unsigned int*)(t + o2);
+    m->d_hk = fxn.hok ? (const FxEnthalpy*)(t + o3) : nullptr;
   }
-  const FxNumbers fxn(d, nu);
   const std::vector<unsigned char> fxb = build_fx(d, m, fxn, nu, &m->fx);
   CHEM_CUDA_TRY(cudaGetDevice(&m->device));
   {

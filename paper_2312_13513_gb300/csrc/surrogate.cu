@@ -472,6 +472,7 @@ constexpr int NEMAX = 8;
 struct PostParams {
   const unsigned char* blob;   // mechanism blob (global memory)
   MechLayout lay;
+  const FxEnthalpy* hk;        // fixed-point enthalpies (nullable)
   const double* Aem;           // [ne][ns] element mass fractions a_ek M_e / W_k, then the pair
                                // products A_ek A_fk, e >= f ([ne (ne + 1) / 2][ns])
   int ne;
@@ -487,46 +488,9 @@ struct PostParams {
 };
 
 
-// FP32 value near x (truncated) and exact FP64 value of f without the FP64 pipe's conversion
-// instructions (each takes the pipe as long as an FMA): the exponent is rebiased and the mantissa
-// shifted by integer instructions; what leaves the normal range takes the conversion
-__device__ __forceinline__ float f32_of(double x) {
-  const unsigned h = (unsigned)__double2hiint(x), e = h & 0x7ff00000u;
-  if (e - 0x38100000u >= 0x47e00000u - 0x38100000u) return (float)x;
-  const unsigned m = __funnelshift_l((unsigned)__double2loint(x), h, 3);
-  return __uint_as_float((h & 0x80000000u) | ((m - 0xC0000000u) & 0x7fffffffu));
-}
-__device__ __forceinline__ double f64_of(float f) {
-  const unsigned u = __float_as_uint(f), e = u & 0x7f800000u;
-  if (e == 0u || e == 0x7f800000u) return (double)f;
-  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
-}
-
-// The mixture's NASA-7 enthalpy polynomial of one temperature range for a register-resident
-// composition (the sums of mixture_nasa, with the species loop unrolled to the array extent), and
-// its cp polynomial in FP32: cp only scales the Newton steps on T (an error of 1e-7 in it leaves
-// 1e-7 of a step, and the accepted last step is below 1e-9 T).
-template <int AS>
-__device__ __forceinline__ void mixture_poly(const double (&Y)[AS], int ns, int rg, const double* hcoef,
-                                             const double* ccoef, const double* invW, double (&Ah)[6],
-                                             float (&Ac)[5]) {
-#pragma unroll
-  for (int i = 0; i < 6; ++i) Ah[i] = 0.0;
-#pragma unroll
-  for (int i = 0; i < 5; ++i) Ac[i] = 0.0f;
-#pragma unroll
-  for (int k = 0; k < AS; ++k) {
-    if (k < ns) {
-      const double yw = Y[k] * __ldg(invW + k);
-      const float yf = f32_of(yw);
-      const double* a = hcoef + (rg * ns + k) * 6;
-      const double* c = ccoef + (rg * ns + k) * 5;
-#pragma unroll
-      for (int i = 0; i < 6; ++i) Ah[i] = fma(yw, __ldg(a + i), Ah[i]);
-#pragma unroll
-      for (int i = 0; i < 5; ++i) Ac[i] = fmaf(yf, f32_of(__ldg(c + i)), Ac[i]);
-    }
-  }
+// h/R = a6 + a1 T + ... + a5 T^5 / 5 (K) in FP64, from the h/RT coefficients of one species
+__device__ __forceinline__ double h_over_r64(const double* a, double T) {
+  return a[5] + T * (a[0] + T * (a[1] + T * (a[2] + T * (a[3] + T * a[4]))));
 }
 
 // One cell's post-processing for a mechanism of NS_ species and NE_ elements known at compile
@@ -537,188 +501,183 @@ __device__ __forceinline__ void mixture_poly(const double (&Y)[AS], int ns, int 
 // instructions (fx::rcp): about 350 FP64 instructions a cell instead of 540.
 template <int NS_, int NE_>
 __global__ void __launch_bounds__(64) surrogate_post_kernel(const PostParams P) {
-  constexpr int AS = NS_ > 0 ? NS_ : MAXNS;          // array extents
-  constexpr int AE = NE_ > 0 ? NE_ : NEMAX;
-  const int ns = NS_ > 0 ? NS_ : P.lay.ns;
-  const int ne = NE_ > 0 ? NE_ : P.ne;
+  constexpr int ns = NS_, ne = NE_;
+  // the element matrix, its pair products and the species polynomials, read once per block with one
+  // latency (a warp that has a single cell per thread waited for each of their cache lines in turn)
+  __shared__ double sA[(ne + ne * (ne + 1) / 2) * ns];
+  __shared__ __align__(16) FxEnthalpy sE[2 * ns];
+  for (int i = threadIdx.x; i < (ne + ne * (ne + 1) / 2) * ns; i += blockDim.x) sA[i] = __ldg(P.Aem + i);
+  if (P.hk)
+    for (int i = threadIdx.x; i < 2 * ns * (int)(sizeof(FxEnthalpy) / 16); i += blockDim.x)
+      ((uint4*)sE)[i] = __ldg((const uint4*)P.hk + i);
+  __syncthreads();
   const double* hcoef = (const double*)(P.blob + P.lay.o_hc);
   const double* ccoef = (const double*)(P.blob + P.lay.o_cpc);
   const double* invW = (const double*)(P.blob + P.lay.o_invW);
   for (int64_t cell = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; cell < P.ncells;
        cell += (int64_t)gridDim.x * blockDim.x) {
     bool pass = P.outbox[cell] == 0;
-    double Y0[AS], Y1[AS];
+    double Y0[ns], Y1[ns];
     const double T0 = P.T[cell];
 #pragma unroll
-    for (int k = 0; k < AS; ++k) {
-      if (k < ns) {
-        Y0[k] = P.Y[(int64_t)k * P.ld + cell];
-        const float yn = P.ynet[(int64_t)k * P.ncells + cell];
-        if ((__float_as_uint(yn) & 0x7f800000u) == 0x7f800000u) pass = false;      // infinite or NaN
-        Y1[k] = f64_of(yn);
-      }
+    for (int k = 0; k < ns; ++k) {
+      Y0[k] = P.Y[(int64_t)k * P.ld + cell];
+      const float yn = P.ynet[(int64_t)k * P.ncells + cell];
+      if ((__float_as_uint(yn) & 0x7f800000u) == 0x7f800000u) pass = false;      // infinite or NaN
+      Y1[k] = f64_of(yn);
     }
     double Tn = T0;
     if (pass) {
       // element-conservation projection: Y'' = Y' - D A^T (A D A^T)^-1 (A Y' - b), D = diag(Y' + 1e-12)
-      double lam[AE], G[AE][AE], D[AS];
+      double lam[ne], G[ne][ne], D[ns];
 #pragma unroll
-      for (int e = 0; e < AE; ++e) lam[e] = 0.0;
+      for (int e = 0; e < ne; ++e) lam[e] = 0.0;
 #pragma unroll
-      for (int k = 0; k < AS; ++k) {
-        if (k < ns) {
-          const double d = Y1[k] - Y0[k];
-          D[k] = Y1[k] + 1e-12;
+      for (int k = 0; k < ns; ++k) {
+        const double d = Y1[k] - Y0[k];
+        D[k] = Y1[k] + 1e-12;
 #pragma unroll
-          for (int e = 0; e < AE; ++e)
-            if (e < ne) {
-              const double a = __ldg(P.Aem + e * ns + k);
-              if (__double2hiint(a) != 0) lam[e] = fma(a, d, lam[e]);
-            }
+        for (int e = 0; e < ne; ++e) {
+          const double a = sA[e * ns + k];
+          if (__double2hiint(a) != 0) lam[e] = fma(a, d, lam[e]);
         }
       }
-      const double* AA = P.Aem + ne * ns;
+      const double* AA = sA + ne * ns;
 #pragma unroll
-      for (int e = 0; e < AE; ++e)
+      for (int e = 0; e < ne; ++e)
 #pragma unroll
         for (int f = 0; f <= e; ++f) {
-          if (e < ne) {
-            double sg = 0.0;
+          double sg = 0.0;
 #pragma unroll
-            for (int k = 0; k < AS; ++k)
-              if (k < ns) {
-                const double a = __ldg(AA + k);
-                if (__double2hiint(a) != 0) sg = fma(a, D[k], sg);
-              }
-            AA += ns;
-            G[e][f] = sg;
-            G[f][e] = sg;
+          for (int k = 0; k < ns; ++k) {
+            const double a = AA[k];
+            if (__double2hiint(a) != 0) sg = fma(a, D[k], sg);
           }
+          AA += ns;
+          G[e][f] = sg;
+          G[f][e] = sg;
         }
       // Gaussian elimination with partial pivoting on the small SPD system; one reciprocal per
       // pivot serves the elimination below it and the back substitution
-      double inv_piv[AE];
+      double inv_piv[ne];
 #pragma unroll
-      for (int k = 0; k < AE; ++k) {
-        if (k < ne && pass) {
+      for (int k = 0; k < ne; ++k) {
+        if (pass) {
           // pivot search on values (no runtime index into the register array)
           int pr = k;
-          double gmax = fabs(G[k][k]);
+          double gmax = G[k][k];
 #pragma unroll
-          for (int i = k + 1; i < AE; ++i)
-            if (i < ne && fabs(G[i][k]) > gmax) { pr = i; gmax = fabs(G[i][k]); }
-          if (gmax == 0.0) {
+          for (int i = k + 1; i < ne; ++i)
+            if (less_abs(gmax, G[i][k])) { pr = i; gmax = G[i][k]; }
+          if ((__double_as_longlong(gmax) << 1) == 0) {
             pass = false;
           } else {
             if (pr != k) {
 #pragma unroll
-              for (int j = 0; j < AE; ++j) {
-                if (j < ne) {
-                  double gk = G[k][j], gp = 0.0;
+              for (int j = 0; j < ne; ++j) {
+                double gk = G[k][j], gp = 0.0;
 #pragma unroll
-                  for (int i = k + 1; i < AE; ++i) if (i == pr) gp = G[i][j];
-                  G[k][j] = gp;
+                for (int i = k + 1; i < ne; ++i) if (i == pr) gp = G[i][j];
+                G[k][j] = gp;
 #pragma unroll
-                  for (int i = k + 1; i < AE; ++i) if (i == pr) G[i][j] = gk;
-                }
+                for (int i = k + 1; i < ne; ++i) if (i == pr) G[i][j] = gk;
               }
               double lk = lam[k], lp = 0.0;
 #pragma unroll
-              for (int i = k + 1; i < AE; ++i) if (i == pr) lp = lam[i];
+              for (int i = k + 1; i < ne; ++i) if (i == pr) lp = lam[i];
               lam[k] = lp;
 #pragma unroll
-              for (int i = k + 1; i < AE; ++i) if (i == pr) lam[i] = lk;
+              for (int i = k + 1; i < ne; ++i) if (i == pr) lam[i] = lk;
             }
             inv_piv[k] = fx::rcp(G[k][k]);
 #pragma unroll
-            for (int i = k + 1; i < AE; ++i) {
-              if (i < ne) {
-                const double l = G[i][k] * inv_piv[k];
+            for (int i = k + 1; i < ne; ++i) {
+              const double l = G[i][k] * inv_piv[k];
 #pragma unroll
-                for (int j = k; j < AE; ++j)
-                  if (j < ne) G[i][j] -= l * G[k][j];
-                lam[i] -= l * lam[k];
-              }
+              for (int j = k; j < ne; ++j)
+                G[i][j] -= l * G[k][j];
+              lam[i] -= l * lam[k];
             }
           }
         }
       }
       if (pass) {
 #pragma unroll
-        for (int i = AE - 1; i >= 0; --i) {
-          if (i < ne) {
-            double sl = lam[i];
+        for (int i = ne - 1; i >= 0; --i) {
+          double sl = lam[i];
 #pragma unroll
-            for (int j = i + 1; j < AE; ++j)
-              if (j < ne) sl -= G[i][j] * lam[j];
-            lam[i] = sl * inv_piv[i];
+          for (int j = i + 1; j < ne; ++j)
+            sl -= G[i][j] * lam[j];
+          lam[i] = sl * inv_piv[i];
+        }
+        double ds = 0.0, res[ne];
+#pragma unroll
+        for (int e = 0; e < ne; ++e) res[e] = 0.0;
+#pragma unroll
+        for (int k = 0; k < ns; ++k) {
+          double c = 0.0;
+#pragma unroll
+          for (int e = 0; e < ne; ++e) {
+            const double a = sA[e * ns + k];
+            if (__double2hiint(a) != 0) c = fma(a, lam[e], c);
+          }
+          const double y = fma(-D[k], c, Y1[k]);
+          Y1[k] = __double2hiint(y) < 0 ? 0.0 : y;       // clipped at 0 (NaN stays and fails below)
+          const double d = Y1[k] - Y0[k];
+          ds += d;
+#pragma unroll
+          for (int e = 0; e < ne; ++e) {
+            const double a = sA[e * ns + k];
+            if (__double2hiint(a) != 0) res[e] = fma(a, d, res[e]);
           }
         }
-        double ds = 0.0, res[AE];
+        if (less_abs(1e-9, ds)) pass = false;           // NaN too
 #pragma unroll
-        for (int e = 0; e < AE; ++e) res[e] = 0.0;
-#pragma unroll
-        for (int k = 0; k < AS; ++k) {
-          if (k < ns) {
-            double c = 0.0;
-#pragma unroll
-            for (int e = 0; e < AE; ++e)
-              if (e < ne) {
-                const double a = __ldg(P.Aem + e * ns + k);
-                if (__double2hiint(a) != 0) c = fma(a, lam[e], c);
-              }
-            const double y = fma(-D[k], c, Y1[k]);
-            Y1[k] = __double2hiint(y) < 0 ? 0.0 : y;       // clipped at 0 (NaN stays and fails below)
-            const double d = Y1[k] - Y0[k];
-            ds += d;
-#pragma unroll
-            for (int e = 0; e < AE; ++e)
-              if (e < ne) {
-                const double a = __ldg(P.Aem + e * ns + k);
-                if (__double2hiint(a) != 0) res[e] = fma(a, d, res[e]);
-              }
-          }
-        }
-        if (!(fabs(ds) <= 1e-9)) pass = false;
-#pragma unroll
-        for (int e = 0; e < AE; ++e)
-          if (e < ne && !(fabs(res[e]) <= 1e-9)) pass = false;
+        for (int e = 0; e < ne; ++e)
+          if (less_abs(1e-9, res[e])) pass = false;
       }
       if (pass) {
-        // temperature from enthalpy conservation: h(T, Y'') = h(T0, Y0); the new composition is
-        // fixed during the iteration, so its mixture NASA-7 polynomial is formed once per
-        // temperature range visited
-        double h0;
-        {
-          // h / R = a5 + a0 T + ... + a4 T^5 per species (no division by T)
-          const int rg0 = T0 < TMID ? 0 : 1;
-          double hs = 0.0;
-#pragma unroll
-          for (int k = 0; k < AS; ++k) {
-            if (k < ns) {
-              const double* a = hcoef + (rg0 * ns + k) * 6;
-              const double hR = a[5] + T0 * (a[0] + T0 * (a[1] + T0 * (a[2] + T0 * (a[3] + T0 * a[4]))));
-              hs = fma(Y0[k] * __ldg(invW + k), hR, hs);
-            }
-          }
-          h0 = hs;
-        }
-        // h in units of R: dT = (h / R - h0 / R) / (cp / R)
-        double Ah[6];
-        float Ac[5];
-        int rg = Tn < TMID ? 0 : 1;
-        mixture_poly<AS>(Y1, ns, rg, hcoef, ccoef, invW, Ah, Ac);
+        // temperature from enthalpy conservation: h(T, Y'') = h(T0, Y0), enthalpies in units of R;
+        // the first step's polynomials serve both sides.  cp only scales the steps (FP32: an error
+        // of 1e-5 in it leaves 1e-5 of a step, and the accepted last step is below 1e-9 T)
+        double h0 = 0.0;
         bool conv = false;
         for (int it = 0; it < 50; ++it) {
-          const int r = Tn < TMID ? 0 : 1;
-          if (r != rg) { rg = r; mixture_poly<AS>(Y1, ns, rg, hcoef, ccoef, invW, Ah, Ac); }
-          const double hh = Ah[5] + Tn * (Ah[0] + Tn * (Ah[1] + Tn * (Ah[2] + Tn * (Ah[3] + Tn * Ah[4]))));
-          const float tf = f32_of(Tn);
-          const float cp = fmaf(tf, fmaf(tf, fmaf(tf, fmaf(tf, Ac[4], Ac[3]), Ac[2]), Ac[1]), Ac[0]);
+          double hh = 0.0, hW[ns];
+          float cp = 0.0f;
+          const Tau q = tau_of(Tn);
+          if (P.hk && q.fast) {
+            const FxEnthalpy* E = sE + q.rg * ns;
+#pragma unroll
+            for (int k = 0; k < ns; ++k) {
+              hW[k] = fx_enthalpy<true>(E[k], q);
+              cp = fmaf(f32_of(Y1[k]), cp_f32<true>(E[k], q), cp);
+            }
+          } else {
+#pragma unroll 1
+            for (int k = 0; k < ns; ++k) {
+              const double* c = ccoef + (q.rg * ns + k) * 5;
+              const double iw = __ldg(invW + k);
+              const double h = h_over_r64(hcoef + (q.rg * ns + k) * 6, Tn) * iw;
+              const double cW = (c[0] + Tn * (c[1] + Tn * (c[2] + Tn * (c[3] + Tn * c[4])))) * iw;
+#pragma unroll
+              for (int j = 0; j < ns; ++j)              // no runtime index into register arrays
+                if (j == k) {
+                  hW[j] = h;
+                  cp = fmaf((float)Y1[j], (float)cW, cp);
+                }
+            }
+          }
+#pragma unroll
+          for (int k = 0; k < ns; ++k) hh = fma(Y1[k], hW[k], hh);
+          if (it == 0) {
+#pragma unroll
+            for (int k = 0; k < ns; ++k) h0 = fma(Y0[k], hW[k], h0);
+          }
           const double dT = (hh - h0) * f64_of(1.0f / cp);
           Tn -= dT;
-          if (!(Tn >= 200.0 && Tn <= 6000.0)) break;
-          if (fabs(dT) < 1e-9 * Tn) { conv = true; break; }
+          if (!in_bounds(Tn, 200.0, 6000.0)) break;
+          if (less_abs(dT, 1e-9 * Tn)) { conv = true; break; }
         }
         if (!conv) pass = false;
       }
@@ -726,8 +685,8 @@ __global__ void __launch_bounds__(64) surrogate_post_kernel(const PostParams P) 
     if (pass) {
       P.T[cell] = Tn;
 #pragma unroll
-      for (int k = 0; k < AS; ++k)
-        if (k < ns) P.Y[(int64_t)k * P.ld + cell] = Y1[k];
+      for (int k = 0; k < ns; ++k)
+        P.Y[(int64_t)k * P.ld + cell] = Y1[k];
     } else {
       const unsigned slot = atomicAdd(P.fb_count, 1u);
       P.fb_idx[slot] = (int32_t)cell;
@@ -851,25 +810,34 @@ __global__ void surrogate_post_general(const PostParams P) {
 }
 
 // heat-release rate of a step: q = -rho0 sum_k h_k(T0) (Y1_k - Y0_k) / (W_k dt), h_k molar
-__global__ void heat_release_kernel(const unsigned char* blob, MechLayout L, const double* T0, const double* p,
-                                    const double* Y0, const double* Y1, int64_t ld, int64_t n, double dt,
-                                    double* q) {
+__global__ void __launch_bounds__(128) heat_release_kernel(const unsigned char* blob, MechLayout L,
+                                                           const FxEnthalpy* hk, const double* T0, const double* p,
+                                                           const double* Y0, const double* Y1, int64_t ld, int64_t n,
+                                                           double dt, double* q) {
   const int ns = L.ns;
   const double* hc = (const double*)(blob + L.o_hc);
   const double* invW = (const double*)(blob + L.o_invW);
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (int64_t)gridDim.x * blockDim.x) {
-    const double T = T0[c], invT = 1.0 / T;
-    const int rg = T < TMID ? 0 : 1;
-    double S = 0.0, acc = 0.0;
-    for (int k = 0; k < ns; ++k) {
-      const double* a = hc + (rg * ns + k) * 6;
-      const double hRT = a[0] + T * (a[1] + T * (a[2] + T * (a[3] + T * a[4]))) + a[5] * invT;
-      const double y0 = Y0[(int64_t)k * ld + c];
-      S += y0 * __ldg(invW + k);
-      acc += hRT * (Y1[(int64_t)k * ld + c] - y0) * __ldg(invW + k);
+    const double T = T0[c];
+    const Tau tq = tau_of(T);
+    double S = 0.0, acc = 0.0;                     // acc = sum h dY / (R W)
+    if (hk && tq.fast) {
+      const FxEnthalpy* E = hk + tq.rg * ns;
+#pragma unroll 3
+      for (int k = 0; k < ns; ++k) {
+        const double y0 = Y0[(int64_t)k * ld + c], y1 = Y1[(int64_t)k * ld + c];
+        S = fma(y0, __ldg(invW + k), S);
+        acc = fma(fx_enthalpy(E[k], tq), y1 - y0, acc);
+      }
+    } else {
+      for (int k = 0; k < ns; ++k) {
+        const double y0 = Y0[(int64_t)k * ld + c], iw = __ldg(invW + k);
+        S = fma(y0, iw, S);
+        acc = fma(h_over_r64(hc + (tq.rg * ns + k) * 6, T) * iw, Y1[(int64_t)k * ld + c] - y0, acc);
+      }
     }
-    const double rho = p[c] / (RU * T * S);
-    q[c] = -rho * RU * T * acc / dt;
+    // -rho RU acc / dt with rho = p / (RU T S)
+    q[c] = -p[c] * acc * fx::rcp(T * S * dt);
   }
 }
 
@@ -884,9 +852,9 @@ extern "C" int chem_heat_release(chem_mech_t m, const double* T0, const double* 
     return CHEM_EINVAL;
   }
   if (ncells == 0) return CHEM_OK;
-  const unsigned blocks = (unsigned)std::min<int64_t>((ncells + 255) / 256, 8192);
-  heat_release_kernel<<<blocks, 256, 0, (cudaStream_t)stream>>>((const unsigned char*)m->d_blob, m->lay, T0, p,
-                                                                  Y0, Y1, ld, ncells, dt, q);
+  const unsigned blocks = (unsigned)std::min<int64_t>((ncells + 127) / 128, 16384);
+  heat_release_kernel<<<blocks, 128, 0, (cudaStream_t)stream>>>((const unsigned char*)m->d_blob, m->lay, m->d_hk, T0,
+                                                                  p, Y0, Y1, ld, ncells, dt, q);
   CHEM_CUDA_TRY(cudaGetLastError());
   return CHEM_OK;
 }
@@ -1421,7 +1389,7 @@ extern "C" int chem_surrogate_advance(chem_model_t md, chem_mech_t mech, double*
   int rc = surrogate_forward(md, T, p, Y, ld, ncells, ynet, nullptr, box, err, st);
   if (!rc) {
     PostParams Q;
-    Q.blob = (const unsigned char*)mech->d_blob; Q.lay = mech->lay; Q.Aem = md->d_A; Q.ne = md->ne;
+    Q.blob = (const unsigned char*)mech->d_blob; Q.lay = mech->lay; Q.hk = mech->d_hk; Q.Aem = md->d_A; Q.ne = md->ne;
     Q.T = T; Q.p = p; Q.Y = Y; Q.ld = ld; Q.ncells = ncells; Q.ynet = ynet; Q.outbox = box;
     Q.route = route_out; Q.fb_idx = fb_idx; Q.fb_count = fb_count;
     int sms = 0, dev = 0;

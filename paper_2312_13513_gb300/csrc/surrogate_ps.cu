@@ -83,15 +83,25 @@ __global__ void k_ps_features(const PsFeatParams P) {
   }
 }
 
-// output layer: z[c] = sum_i A3[c, i] w4[i] + b4 (BF16 products, FP32 sums), one warp per cell
+// output layer: z[c] = sum_i A3[c, i] w4[i] + b4 (BF16 products, FP32 sums), one warp per cell, eight
+// values a load (h3 is a multiple of 8)
 __global__ void k_ps_out(const __nv_bfloat16* A3, int h3, const __nv_bfloat16* w4, const float* b4, int64_t nc,
                          float* z) {
   const int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (c >= nc) return;
-  const __nv_bfloat16* a = A3 + c * h3;
+  const uint4* a = reinterpret_cast<const uint4*>(A3 + c * h3);
+  const uint4* w = reinterpret_cast<const uint4*>(w4);
   float acc = 0.0f;
-  for (int i = lane; i < h3; i += 32) acc = fmaf(__bfloat162float(a[i]), __bfloat162float(w4[i]), acc);
+  for (int i = lane; i < h3 / 8; i += 32) {
+    const uint4 av = a[i], wv = __ldg(w + i);
+    const uint32_t ax[4] = {av.x, av.y, av.z, av.w}, wx[4] = {wv.x, wv.y, wv.z, wv.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {                // a BF16 value is the high half of its FP32 value
+      acc = fmaf(__uint_as_float(ax[j] << 16), __uint_as_float(wx[j] << 16), acc);
+      acc = fmaf(__uint_as_float(ax[j] & 0xffff0000u), __uint_as_float(wx[j] & 0xffff0000u), acc);
+    }
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if (lane == 0) z[c] = acc + b4[0];

@@ -53,36 +53,69 @@ namespace {
 
 constexpr double kPatm = 1.01325e6;
 
-__global__ void mixture_thermo_kernel(const unsigned char* blob, MechLayout L, const double* T, const double* Y,
-                                      int64_t ld, int64_t n, double* h, double* cp) {
+// The FP64 pipe bounds these kernels (100003 H2 cells: 28 us at about 130 FP64 instructions a cell);
+// with the species polynomials in fixed point two FP64 instructions a species are left.
+__global__ void __launch_bounds__(128) mixture_thermo_kernel(const unsigned char* blob, MechLayout L,
+                                                             const FxEnthalpy* hk, const double* T, const double* Y,
+                                                             int64_t ld, int64_t n, double* h, double* cp) {
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (int64_t)gridDim.x * blockDim.x) {
     double hh, cc;
-    h_cp_mass(blob, L, T[c], Y, ld, c, nullptr, &hh, &cc);
+    const Tau q = tau_of(T[c]);
+    if (hk && q.fast) {
+      hh = 0.0;
+      cc = 0.0;
+      const FxEnthalpy* E = hk + q.rg * L.ns;
+#pragma unroll 3
+      for (int k = 0; k < L.ns; ++k) {
+        const double y = Y[(int64_t)k * ld + c];
+        hh = fma(y, fx_enthalpy(E[k], q), hh);
+        cc = fma(y, fx_cp(E[k], q), cc);
+      }
+      hh *= RU;
+      cc *= RU;
+    } else {
+      h_cp_mass(blob, L, T[c], Y, ld, c, nullptr, &hh, &cc);
+    }
     if (h) h[c] = hh;
     if (cp) cp[c] = cc;
   }
 }
 
-__global__ void temperature_from_h_kernel(const unsigned char* blob, MechLayout L, const double* h0,
-                                          const double* Y, int64_t ld, int64_t n, double* T, int8_t* status) {
+__global__ void __launch_bounds__(128) temperature_from_h_kernel(const unsigned char* blob, MechLayout L,
+                                                                 const FxEnthalpy* hk, const double* h0,
+                                                                 const double* Y, int64_t ld, int64_t n, double* T,
+                                                                 int8_t* status) {
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (int64_t)gridDim.x * blockDim.x) {
     const double target = h0[c];
     double Tn = T[c];
     bool conv = false;
     if (isfinite(target) && Tn >= 200.0 && Tn <= 6000.0) {
-      // the composition is fixed during the iteration: its mixture polynomial once per temperature
-      // range visited (11 FP64 instructions a species), then 9 an iteration instead of 13 a species
-      double Ah[6], Ac[5];
-      int rg = -1;
+      const double tr = target * (1.0 / RU);
       for (int it = 0; it < 50; ++it) {
-        const int r = Tn < TMID ? 0 : 1;
-        if (r != rg) { rg = r; mixture_nasa_cell(blob, L, rg, Y, ld, c, Ah, Ac); }
-        double hh, cp;
-        h_cp_from_mixture(Ah, Ac, Tn, &hh, &cp);
-        const double dT = (hh - target) * fx::rcp(cp);
+        double dT;
+        const Tau q = tau_of(Tn);
+        // cp only scales the step: FP32, where its magnitude allows
+        double hs = 0.0;
+        float cs = 0.0f;
+        if (hk && q.fast) {
+          const FxEnthalpy* E = hk + q.rg * L.ns;
+#pragma unroll 3
+          for (int k = 0; k < L.ns; ++k) {
+            const double y = Y[(int64_t)k * ld + c];
+            hs = fma(y, fx_enthalpy(E[k], q), hs);
+            cs = fmaf(f32_of(y), cp_f32(E[k], q), cs);
+          }
+        }
+        if (cs > 1e-30f && cs < 1e30f) {
+          dT = (hs - tr) * f64_of(1.0f / cs);
+        } else {
+          double hh, cp;
+          h_cp_mass(blob, L, Tn, Y, ld, c, nullptr, &hh, &cp);
+          dT = (hh - target) / cp;
+        }
         Tn -= dT;
-        if (!(Tn >= 200.0 && Tn <= 6000.0)) break;
-        if (fabs(dT) < 1e-9 * Tn) { conv = true; break; }
+        if (!in_bounds(Tn, 200.0, 6000.0)) break;
+        if (less_abs(dT, 1e-9 * Tn)) { conv = true; break; }
       }
     }
     if (conv) T[c] = Tn;
@@ -356,8 +389,8 @@ extern "C" int chem_mixture_thermo(chem_mech_t m, const double* T, const double*
   if (!m || ncells < 0 || ld < ncells) { set_error("bad arguments"); return CHEM_EINVAL; }
   if (ncells == 0) return CHEM_OK;
   if (!T || !Y || (!h && !cp)) { set_error("NULL pointer"); return CHEM_EINVAL; }
-  mixture_thermo_kernel<<<grid_cells(ncells, 256), 256, 0, (cudaStream_t)stream>>>(
-      (const unsigned char*)m->d_blob, m->lay, T, Y, ld, ncells, h, cp);
+  mixture_thermo_kernel<<<grid_cells(ncells, 128), 128, 0, (cudaStream_t)stream>>>(
+      (const unsigned char*)m->d_blob, m->lay, m->d_hk, T, Y, ld, ncells, h, cp);
   CHEM_CUDA_TRY(cudaGetLastError());
   return CHEM_OK;
 }
@@ -367,8 +400,8 @@ extern "C" int chem_temperature_from_enthalpy(chem_mech_t m, const double* h, co
   if (!m || ncells < 0 || ld < ncells) { set_error("bad arguments"); return CHEM_EINVAL; }
   if (ncells == 0) return CHEM_OK;
   if (!h || !Y || !T) { set_error("NULL pointer"); return CHEM_EINVAL; }
-  temperature_from_h_kernel<<<grid_cells(ncells, 256), 256, 0, (cudaStream_t)stream>>>(
-      (const unsigned char*)m->d_blob, m->lay, h, Y, ld, ncells, T, status);
+  temperature_from_h_kernel<<<grid_cells(ncells, 128), 128, 0, (cudaStream_t)stream>>>(
+      (const unsigned char*)m->d_blob, m->lay, m->d_hk, h, Y, ld, ncells, T, status);
   CHEM_CUDA_TRY(cudaGetLastError());
   return CHEM_OK;
 }

@@ -10,7 +10,7 @@ from synth.states import les_field, load_table, quasi_dns_field  # noqa: E402
 from synth.transport import generate_transport  # noqa: E402
 
 from gpu_common import to_dev  # noqa: E402
-from helpers import random_states  # noqa: E402
+from helpers import random_states, with_inert_species  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
@@ -98,3 +98,58 @@ def test_temperature_from_enthalpy_flags_failures(h2):
     s = st.cpu().numpy()
     assert s[0] == 1 and s[1] == 1 and s[2] == 1
     assert torch.equal(Td[:3], before[:3])             # unconverged cells keep their temperature
+
+
+@pytest.mark.parametrize("ns", [9, 15, 16])
+def test_transport_at_the_edges_of_its_ranges(h2, ns):
+    """Both kernels (one thread per cell up to 15 species, a warp per cell beyond) inside, at and
+    outside the temperatures of the fixed-point fits, [1, 65536), in odd numbers of cells."""
+    mech = with_inert_species(h2, ns - h2.ns) if ns > h2.ns else h2
+    tr = generate_transport(mech)
+    T = np.array([0.5, np.nextafter(1.0, 0.0), 1.0, 250.0, 1000.0, 3500.0, np.nextafter(65536.0, 0.0), 65536.0, 2e5] * 5)[:41]
+    rng = np.random.default_rng(47)
+    Y = rng.dirichlet(np.full(mech.ns, 0.4), T.size).T.copy()
+    Y[:, 40] = 0.0; Y[0, 40] = 1.0                      # one species alone
+    p = np.full(T.size, 1.01325e6)
+    dm = cg.Mechanism(mech)
+    gt = cg.Transport(dm, tr)
+    Td, pd, Yd = to_dev(T, p, Y)
+    mu = torch.empty_like(Td); lam = torch.empty_like(Td); D = torch.empty_like(Yd)
+    gt(Td, pd, Yd, mu, lam, D)
+    torch.cuda.synchronize()
+    mu_r, lam_r, D_r = ot.mixture_cells(tr, mech.W, T, p, Y)
+    for got, ref in ((mu, mu_r), (lam, lam_r), (D, D_r)):
+        assert np.allclose(got.cpu().numpy(), ref, rtol=1e-11, atol=0)
+
+
+@pytest.mark.parametrize("kind", ["h2", "ch4"])
+def test_enthalpies_at_the_edges_of_the_fixed_point_range(kind, h2, ch4):
+    """Mixture h, cp and heat release at the ends of both polynomial ranges and of the fixed-point
+    range [128, 4096), and outside it, against the NASA polynomials in extended precision."""
+    mech = h2 if kind == "h2" else ch4
+    T = np.array([90.0, np.nextafter(128.0, 0), 128.0, 298.15, np.nextafter(1000.0, 0), 1000.0, 1023.5, 1024.0, 2900.0,
+                  np.nextafter(4096.0, 0), 4096.0, 5500.0] * 3)[:35]
+    rng = np.random.default_rng(48)
+    Y = rng.dirichlet(np.full(mech.ns, 0.4), T.size).T.copy()
+    Y1 = rng.dirichlet(np.full(mech.ns, 0.4), T.size).T.copy()
+    p = np.full(T.size, 1.01325e6)
+    dm = cg.Mechanism(mech)
+    Td, pd, Yd = to_dev(T, p, Y)
+    h = torch.empty_like(Td); cp = torch.empty_like(Td)
+    cg.mixture_thermo(dm, Td, Yd, h, cp)
+    q = cg.heat_release(dm, Td, pd, Yd, to_dev(T, p, Y1)[2], 1e-6)
+    torch.cuda.synchronize()
+    L = np.longdouble
+    a = np.where((T < 1000.0)[None, None], mech.nasa_lo[:, :, None], mech.nasa_hi[:, :, None]).astype(L)   # [ns, 7, n]
+    t = T.astype(L)
+    terms = np.stack([a[:, 5]] + [a[:, i] * t ** (i + 1) / (i + 1) for i in range(5)])
+    cterms = np.stack([a[:, i] * t ** i for i in range(5)])
+    w = 1.0 / mech.W.astype(L)[:, None]
+    ru = L(8.314462618e7)
+    # 1e-13 of the magnitudes that are summed: 2^-42 K times a dozen units in fixed point (about
+    # 3e-12 K against hundreds), about ten roundings of 1.1e-16 in FP64
+    for got, ref, mag in ((h, ru * (terms.sum(0) * Y * w).sum(0), ru * (np.abs(terms).sum(0) * Y * w).sum(0)),
+                          (cp, ru * (cterms.sum(0) * Y * w).sum(0), ru * (np.abs(cterms).sum(0) * Y * w).sum(0)),
+                          (q, -(p / (t * (Y * w).sum(0))) * (terms.sum(0) * (Y1.astype(L) - Y) * w).sum(0) / L(1e-6),
+                           p / (t * (Y * w).sum(0)) * (np.abs(terms).sum(0) * (Y1 + Y) * w).sum(0) / L(1e-6))):
+        assert np.all(np.abs(got.cpu().numpy() - ref) <= 1e-13 * mag)
