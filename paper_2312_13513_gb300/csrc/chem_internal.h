@@ -94,6 +94,8 @@ struct chem_mech_s {
   chem::JacProgram jac{};
   chem::FxLayout fx{};                    // fixed-point form (integrator_cell.cu), bytes = 0: none
   void* d_fx = nullptr;
+  chem::CoLayout co{};                  // its gather programs, for several lanes per cell
+  void* d_co = nullptr;
   chem::GxLayout gx{};                    // the group kernels' fixed-point form, bytes = 0: none
   chem::GxJac gxj{};
   void *d_gx = nullptr, *d_gxj = nullptr; // blob; Jacobian program

@@ -76,6 +76,22 @@ struct FxLayout {
   int64_t lpr0;               // log2(p_atm / R), Q11.52
 };
 
+// Gather form of a cell's sums for several lanes per cell (integrator_coop.cu), where one thread
+// scatters: per species the terms of its production rate (reaction << 4 | (coefficient + 8)), per
+// entry of d(wdot)/dC (negated) the terms coef * value, both in the order in which the one thread
+// adds them.  Values: 4 j + slot the derivative of reaction j by its slot's species, 4 n + j - n_plain
+// the collision partners' factor of reaction j.  Entries by falling term count.
+struct CoTerm {
+  double coef;
+  int src, pad;
+};
+struct CoLayout {
+  int bytes;                  // 0: none (a reaction outside FxRate)
+  int n, nent, nval;          // FxRate records, entries, values
+  int o_woff, o_wterm;        // int [ns + 1], [..]
+  int o_eoff, o_epos, o_term; // int [nent + 1], row * N + column [nent], CoTerm [..]
+};
+
 // The same for the group kernels (integrator.cu): one lane per reaction, so the records are arrays;
 // species slots are indices, ns in an empty one.
 struct GxLayout {

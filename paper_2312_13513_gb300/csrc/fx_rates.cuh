@@ -173,7 +173,7 @@ __device__ __forceinline__ bool troe_fast(const Ctx& m, const FxTroe& t, const T
     Fc += e2;
   }
   if (!positive_normal(Fc)) return false;
-  const double Prr = exp2_q52(Xk, m.e2) * Mc;
+  const double Prr = __dmul_rn(exp2_q52(Xk, m.e2), Mc);
   const double l2F = to_double(log2_q52(Fc, m.rc, m.lg), 52);
   // log2 k0/kinf + log2 [M] stays below 2046 in magnitude
   const double l2P = to_double(Xk + log2_q52(Mc, m.rc, m.lg), 52);
@@ -195,11 +195,11 @@ __device__ __forceinline__ bool troe_fast(const Ctx& m, const FxTroe& t, const T
     const double dGdlogPr = g2 * (n * rd2);
     const double df1dL = fma(-0.67, d, u * (1.27 - 0.14 * 0.67)) * rd2;
     const double dGdL = fma(g2, df1dL, rden);
-    double dFc = -(1.0 - t.a) * t.iT3 * e3 - t.a * t.iT1 * e1;
-    if (t.has_t2 != 0.0) dFc += t.T2 * invT * invT * e2;
+    double dFc = fma(-(1.0 - t.a) * t.iT3, e3, -(t.a * t.iT1 * e1));
+    if (t.has_t2 != 0.0) dFc = fma(t.T2 * invT * invT, e2, dFc);
     const double s = opr + dGdlogPr;
     const double dlnPr = fma(t.Ta0K * q.invT, q.invT, t.b0d * q.invT) - dlnkinf;
-    *dln = dlnkinf + dlnPr * s + dGdL * dFc * rcp(Fc);
+    *dln = fma(dGdL * dFc, rcp(Fc), fma(dlnPr, s, dlnkinf));
     *dM = s * rcp(Mc);
   }
   return true;

@@ -6,8 +6,10 @@
 // dense LU with partial pivoting, six stages, embedded error estimate, adaptive sub-steps.
 //
 // Work decomposition ("group per cell"): a group of G threads owns one cell at a time.
-//   G = 2   (sixteen cells per warp, sub-warp groups) for small mechanisms (N = ns + 1 <= 16,
-//           H2-sized): FP64 instructions issue warp-wide whatever the active mask, so a warp per
+//   G = 1   (one thread per cell, integrator_cell.cu; 8 or 16 lanes with the same operations for
+//           launches of few cells, integrator_coop.cu) for 8 to 11 species in fixed point;
+//   G = 2   (sixteen cells per warp, sub-warp groups) for the other small mechanisms (N = ns + 1
+//           <= 16): FP64 instructions issue warp-wide whatever the active mask, so a warp per
 //           10-unknown cell would leave most FP64 lanes idle; two lanes split a 10-long loop
 //           into 5 full rounds (four lanes would idle half a round) and halve the lanes that
 //           sit out per-cell scalar work;
@@ -16,9 +18,9 @@
 // trailing updates and the triangular solves; sums use warp shuffles.  The mechanism (NASA-7
 // coefficients, Arrhenius, fall-off, efficiency lists) is staged once per CTA into shared memory
 // and shared by all groups of the CTA (§3.2 keeps constant coefficients in fast on-chip memory).
-// The kernel is persistent: groups claim chunks of consecutive cells from a device work queue
-// (one atomicAdd), load them species-row by species-row (coalesced 64-byte rows of the SoA
-// state, §3.2), integrate them one after another and store them back, so cells needing many
+// The kernel is persistent: groups claim chunks of one or two consecutive cells from a device work
+// queue (one atomicAdd), load them species-row by species-row (SoA state, §3.2), integrate them one
+// after another and store them back, so cells needing many
 // sub-steps do not stall the rest of the grid.
 #include <cuda_runtime.h>
 #include <math.h>

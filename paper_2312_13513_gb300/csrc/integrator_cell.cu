@@ -13,6 +13,12 @@
 #include "integrator_cell.cuh"
 
 namespace chem {
+
+// several lanes per cell (integrator_coop.cu)
+int cell_lanes(const chem_mech_s* m, int64_t ncells, int ctas, int smem_max);
+int launch_coop_advance(const chem_mech_s* m, const QueueParams& Q, int lanes, int sms, int smem_max, int max_ctas,
+                        cudaStream_t stream);
+
 namespace {
 
 using cell::Ws;
@@ -387,6 +393,14 @@ bool cell_kernel_fits(const chem_mech_s* m) {
 }
 
 int launch_cell_advance(const chem_mech_s* m, const QueueParams& Q, const chem_options* opt, cudaStream_t stream) {
+  int dev = 0, sms = 0, smem_max = 0;
+  CHEM_CUDA_TRY(cudaGetDevice(&dev));
+  CHEM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  CHEM_CUDA_TRY(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  const int max_ctas = opt ? opt->max_ctas : 0;
+  const bool shaped = opt && opt->groups_per_cta > 0;
+  const int lanes = shaped ? 1 : cell_lanes(m, Q.total_chunks, max_ctas > 0 ? std::min(sms, max_ctas) : sms, smem_max);
+  if (lanes > 1) return launch_coop_advance(m, Q, lanes, sms, smem_max, max_ctas, stream);
   switch (m->ns) {
     case 8: return advance_t<8>(m, Q, opt, stream);
     case 9: return advance_t<9>(m, Q, opt, stream);

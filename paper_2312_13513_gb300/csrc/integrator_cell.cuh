@@ -10,6 +10,10 @@
 // fixed point (log2 kr = log2 kf + Delta G / (RT ln 2): integer adds), so exponentials, logarithms,
 // NASA-7 polynomials and reciprocals of T leave the FP64 pipe.
 //
+// Sums that a compiler could contract in more than one way are written as explicit FMAs: the kernel
+// for few cells (integrator_coop.cu) does the same operations in the same order, so that a cell's
+// result does not depend on the launch it is part of.
+//
 // Layout: a warp owns 32 cells; element e of a lane's workspace is at e * 32 + lane (doubles), so
 // every access, also by a lane-dependent row after pivoting, is free of bank conflicts.
 #pragma once
@@ -77,30 +81,40 @@ __device__ __forceinline__ View bind(const unsigned char* s, const FxLayout& L, 
   return v;
 }
 
-// Species thermo in FP64 (temperatures outside the fixed-point range): g/RT and h/RT (cp/R with
-// jac) into the workspace; sum c cp/R and its temperature derivative, c = Y / W in the workspace
+// Species k in FP64 (temperatures outside the fixed-point range): g/RT, h/RT, cp/R, d(cp/R)/dT
+struct Species64 {
+  double g, h, cp, dcp;
+};
+static __device__ __noinline__ Species64 species64(const View& m, int ns, int k, double T) {
+  const MechLayout& L = *m.lay;
+  const int rg = T < TMID ? 0 : 1;
+  const double lnT = log(T), invT = 1.0 / T;
+  const double* hc = (const double*)(m.blob + L.o_hc) + (rg * ns + k) * 6;
+  const double* sc = (const double*)(m.blob + L.o_sc) + (rg * ns + k) * 6;
+  const double* cc = (const double*)(m.blob + L.o_cpc) + (rg * ns + k) * 5;
+  Species64 r;
+  r.h = hc[0] + T * (hc[1] + T * (hc[2] + T * (hc[3] + T * hc[4]))) + hc[5] * invT;
+  r.g = r.h - (sc[0] * lnT + T * (sc[1] + T * (sc[2] + T * (sc[3] + T * sc[4]))) + sc[5]);
+  r.cp = cc[0] + T * (cc[1] + T * (cc[2] + T * (cc[3] + T * cc[4])));
+  r.dcp = cc[1] + T * (2.0 * cc[2] + T * (3.0 * cc[3] + T * (4.0 * cc[4])));
+  return r;
+}
+// all species of a cell into its workspace (cp/R with jac); sum c cp/R and its temperature
+// derivative, c = Y / W in the workspace
 template <int NS>
 __device__ __noinline__ void slow_species(const View& m, double* col, double T, double* cp_out, double* dcp_out,
                                           bool jac) {
   using w = Ws<NS>;
-  const MechLayout& L = *m.lay;
-  const int rg = T < TMID ? 0 : 1;
-  const double lnT = log(T), invT = 1.0 / T;
   double cps = 0.0, dcps = 0.0;
   for (int k = 0; k < NS; ++k) {
-    const double* hc = (const double*)(m.blob + L.o_hc) + (rg * NS + k) * 6;
-    const double* sc = (const double*)(m.blob + L.o_sc) + (rg * NS + k) * 6;
-    const double* cc = (const double*)(m.blob + L.o_cpc) + (rg * NS + k) * 5;
-    const double h = hc[0] + T * (hc[1] + T * (hc[2] + T * (hc[3] + T * hc[4]))) + hc[5] * invT;
-    const double s = sc[0] * lnT + T * (sc[1] + T * (sc[2] + T * (sc[3] + T * sc[4]))) + sc[5];
-    const double cp = cc[0] + T * (cc[1] + T * (cc[2] + T * (cc[3] + T * cc[4])));
-    col[(w::G + k) * 32] = h - s;
-    col[(w::H + k) * 32] = h;
+    const Species64 r = species64(m, NS, k, T);
+    col[(w::G + k) * 32] = r.g;
+    col[(w::H + k) * 32] = r.h;
     const double c = col[(w::C + k) * 32];
-    cps = fma(c, cp, cps);
+    cps = fma(c, r.cp, cps);
     if (jac) {
-      dcps += c * (cc[1] + T * (2.0 * cc[2] + T * (3.0 * cc[3] + T * (4.0 * cc[4]))));
-      col[(w::CP + k) * 32] = cp;
+      dcps = fma(c, r.dcp, dcps);
+      col[(w::CP + k) * 32] = r.cp;
     }
   }
   *cp_out = cps;
@@ -209,7 +223,7 @@ __device__ __forceinline__ void rhs(const View& m, double* col, double T, YF Yk,
   double c[NS];
 #pragma unroll
   for (int k = 0; k < NS; ++k) {
-    c[k] = Yk(k) * m.invW[k];
+    c[k] = __dmul_rn(Yk(k), m.invW[k]);
     S += c[k];
     col[(w::C + k) * 32] = c[k];
   }
@@ -387,13 +401,13 @@ __device__ __forceinline__ void rhs(const View& m, double* col, double T, YF Yk,
       if (third) q *= Mc;
       scatter(*R, q);
     } else {
-      const double fwd = kf * (a0 * a1), rev = kr * (b0 * b1), net = fwd - rev;
+      const double rev = kr * (b0 * b1), net = fma(kf, a0 * a1, -rev);
       double dqdT = fma(net, dlnkf, rev * dlnKc_of(s, R->dnu));
       double q = net, ka = kf, kb = kr;
       if (third) { q *= Mc; dqdT *= Mc; ka *= Mc; kb *= Mc; }
       derivatives(*R, s, ka, kb, a0, a1, b0, b1, q, dqdT);
       if (third) partner_rows(*R, net);
-      else if (j >= n2) partner_rows(*R, fastk ? dMr * net : dkfdM * (a0 * a1 - b0 * b1 * invKc));
+      else if (j >= n2) partner_rows(*R, fastk ? dMr * net : dkfdM * fma(a0, a1, -(b0 * b1 * invKc)));
     }
   }
   // ---- reactions with three species on a side or more than four net species ----
@@ -431,19 +445,19 @@ __device__ __forceinline__ void rhs(const View& m, double* col, double T, YF Yk,
     Rh = fma(-col[(w::H + k) * 32], s, Rh);
     const double dk = -s - col[(w::WK + k) * 32];
     col[(w::RK + k) * 32] = dk * rS;
-    Jm[(k * N - 1) * 32] = -(m.W[k] * invrho * (col[(w::DWDT + k) * 32] - dk * t.invT));
+    Jm[(k * N - 1) * 32] = -(m.W[k] * invrho * fma(-dk, t.invT, col[(w::DWDT + k) * 32]));
   }
   const double TQ = T * Q, TRh = T * Rh;
   const double Qr = TQ * ircp;                 // -f_0
-  col[w::M * 32] = (r31 + T * r32 - Rh) * ircp + Qr * (cps * t.invT - dcps) * (rho * ircp);
-  const double RhS = TRh * iS, cpS = cps * iS, Qrr = Qr * rho;
+  col[w::M * 32] = fma(fma(T, r32, r31) - Rh, ircp, Qr * fma(cps, t.invT, -dcps) * (rho * ircp));
+  const double RhS = TRh * iS, cpS = __dmul_rn(cps, iS), Qrr = Qr * rho;
 #pragma unroll 2
   for (int mm = 0; mm < NS; ++mm) {
     double s = 0.0;
 #pragma unroll
     for (int k = 0; k < NS; ++k) s = fma(-col[(w::H + k) * 32], Jm[(k * N + mm) * 32], s);
     const double Hm = T * s;
-    Jm[(mm - N) * 32] = m.invW[mm] * ircp * ((rho * Hm - RhS) - Qrr * (col[(w::CP + mm) * 32] - cpS));
+    Jm[(mm - N) * 32] = m.invW[mm] * ircp * fma(-Qrr, col[(w::CP + mm) * 32] - cpS, fma(rho, Hm, -RhS));
   }
 #pragma unroll 2
   for (int k = 0; k < NS; ++k) {

@@ -397,6 +397,53 @@ std::vector<unsigned char> build_fx(const chem_mech_desc* d, const chem_mech_s* 
   return B.buf;
 }
 
+// gather programs of the blob that build_fx made (CoLayout)
+std::vector<unsigned char> build_co(const std::vector<unsigned char>& fxb, const FxLayout& F, CoLayout* L) {
+  *L = CoLayout{};
+  if (!F.bytes || F.n_gen) return {};
+  const int ns = F.ns, N = ns + 1, n = F.n_plain + F.n_tb + F.n_fo;
+  const FxRate* R = (const FxRate*)(fxb.data() + F.o_rate);
+  const double* eff = (const double*)(fxb.data() + F.o_eff);
+  std::vector<std::vector<int>> wt(ns);
+  std::vector<std::vector<CoTerm>> en((size_t)ns * ns);
+  for (int j = 0; j < n; ++j) {
+    for (int i = 0; i < 4; ++i)
+      if (R[j].nu[i] != 0.0) wt[R[j].w[i] / 256].push_back(j << 4 | ((int)R[j].nu[i] + 8));
+    for (int s = 0; s < 4; ++s) {
+      if (R[j].c[s] / 256 == ns) continue;
+      for (int i = 0; i < 4; ++i)
+        if (R[j].nu[i] != 0.0) en[(size_t)(R[j].w[i] / 256) * ns + R[j].c[s] / 256].push_back({-R[j].nu[i], 4 * j + s, 0});
+    }
+    if (j < F.n_plain) continue;
+    for (int i = 0; i < 4; ++i)
+      if (R[j].nu[i] != 0.0)
+        for (int k = 0; k < ns; ++k)
+          en[(size_t)(R[j].w[i] / 256) * ns + k].push_back({-R[j].nu[i] * eff[R[j].tb * ns + k], 4 * n + j - F.n_plain, 0});
+  }
+  std::vector<int> order, woff(1, 0), wterm, eoff(1, 0), epos;
+  std::vector<CoTerm> term;
+  for (int k = 0; k < ns; ++k) { wterm.insert(wterm.end(), wt[k].begin(), wt[k].end()); woff.push_back((int)wterm.size()); }
+  for (int e = 0; e < ns * ns; ++e)
+    if (!en[e].empty()) order.push_back(e);
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return en[a].size() > en[b].size(); });
+  for (int e : order) {
+    term.insert(term.end(), en[e].begin(), en[e].end());
+    eoff.push_back((int)term.size());
+    epos.push_back((1 + e / ns) * N + 1 + e % ns);
+  }
+  Builder B;
+  L->n = n; L->nent = (int)order.size(); L->nval = 4 * n + F.n_tb + F.n_fo;
+  L->o_woff = B.add(4 * (int)woff.size());
+  L->o_wterm = B.add(4 * (int)wterm.size());
+  L->o_eoff = B.add(4 * (int)eoff.size());
+  L->o_epos = B.add(4 * (int)epos.size());
+  L->o_term = B.add((int)(sizeof(CoTerm) * term.size()));
+  put(B, L->o_woff, woff); put(B, L->o_wterm, wterm); put(B, L->o_eoff, eoff); put(B, L->o_epos, epos);
+  put(B, L->o_term, term);
+  L->bytes = (int)B.buf.size();
+  return B.buf;
+}
+
 // Blob of the group kernels' fixed-point form, and their Jacobian program (one global allocation
 // each, uploaded here).
 int build_gx(const chem_mech_desc* d, chem_mech_s* m, const FxNumbers& F, const std::vector<std::vector<int>>& nu,
@@ -754,6 +801,11 @@ int build(const chem_mech_desc* din, chem_mech_s* m) {
   if (m->fx.bytes) {
     CHEM_CUDA_TRY(cudaMalloc(&m->d_fx, m->fx.bytes));
     CHEM_CUDA_TRY(cudaMemcpy(m->d_fx, fxb.data(), m->fx.bytes, cudaMemcpyHostToDevice));
+    const std::vector<unsigned char> cob = build_co(fxb, m->fx, &m->co);
+    if (m->co.bytes) {
+      CHEM_CUDA_TRY(cudaMalloc(&m->d_co, m->co.bytes));
+      CHEM_CUDA_TRY(cudaMemcpy(m->d_co, cob.data(), m->co.bytes, cudaMemcpyHostToDevice));
+    }
   }
   CHEM_CUDA_TRY(cudaMalloc(&m->d_blob, L.bytes));
   CHEM_CUDA_TRY(cudaMemcpy(m->d_blob, B.buf.data(), L.bytes, cudaMemcpyHostToDevice));
@@ -960,6 +1012,7 @@ extern "C" int chem_free_mechanism(chem_mech_t m) {
   if (m->d_blob) cudaFree(m->d_blob);
   if (m->d_jac) cudaFree(m->d_jac);
   if (m->d_fx) cudaFree(m->d_fx);
+  if (m->d_co) cudaFree(m->d_co);
   if (m->d_tab) cudaFree(m->d_tab);
   if (m->d_gx) cudaFree(m->d_gx);
   if (m->d_gxj) cudaFree(m->d_gxj);

@@ -137,3 +137,31 @@ def test_advance_agrees_with_the_group_kernel(h2, which, n):
     # (two cells of "slow" end in H_UNDERFLOW, in the oracle too: a rate with T^40)
     assert np.array_equal(got[0][2], got[1][2]) and np.mean(got[0][2] == 0) > 0.99 - 1.0 / n
     assert np.all(within(got[1][0], got[1][1], got[0][0], got[0][1]))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("which,per_sm,extra", [("8", 0, 1), ("9", 0, 5), ("9", 28, 0), ("9", 28, 1), ("9", 104, 0),
+                                                ("10", 28, 3), ("11", 0, 129), ("11", 30, 0), ("slow", 0, 65),
+                                                ("slow", 29, 0)])
+def test_few_cells_take_several_lanes(h2, which, per_sm, extra):
+    """Launches of few cells (16 or 8 lanes a cell, lines at 28 and 104 cells per SM) against the same
+    cells inside a launch beyond both lines (one thread per cell): the same operations, so the same
+    bits."""
+    import torch
+    import paper_2312_13513_gb300 as cg
+    from gpu_common import to_dev
+    from helpers import random_states
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n, big = per_sm * sms + extra, 104 * sms + 33
+    m = _mechs(h2)[which]
+    dm = cg.Mechanism(m)
+    T, p, Y = random_states(h2, big, 60 + n, "H2", Tlo=300.0, Thi=2600.0)
+    Y = np.vstack([Y, np.full((max(0, m.ns - h2.ns), big), 1e-3)])[:m.ns]
+    Tb, pb, Yb = to_dev(T, p, Y)
+    sb = torch.full((big,), -1, dtype=torch.int8, device="cuda"); kb = torch.zeros(big, dtype=torch.int32, device="cuda")
+    cg.advance(dm, Tb, pb, Yb, 5e-7, status=sb, nsub=kb)
+    Ts, ps, Ys = to_dev(T[:n].copy(), p[:n].copy(), Y[:, :n].copy())
+    ss = torch.full((n,), -1, dtype=torch.int8, device="cuda"); ks = torch.zeros(n, dtype=torch.int32, device="cuda")
+    cg.advance(dm, Ts, ps, Ys, 5e-7, status=ss, nsub=ks)
+    assert torch.equal(ss, sb[:n]) and torch.equal(ks, kb[:n])
+    assert torch.equal(Ts, Tb[:n]) and torch.equal(Ys, Yb[:, :n])
