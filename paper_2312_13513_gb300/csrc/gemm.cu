@@ -25,6 +25,7 @@
 
 #include "chem_internal.h"
 #include "gelu.cuh"
+#include "pdl.cuh"
 #include "sm100.h"
 
 namespace chem {
@@ -163,6 +164,8 @@ __global__ void __launch_bounds__(kPersistThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_wait();
+  pdl_trigger();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -302,7 +305,8 @@ static int launch_persistent(const CUtensorMap& ta, const CUtensorMap& tb, const
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, PersistCfg<BN_>::SMEM));
     attr = true;
   }
-  gemm_bf16_persistent<BN_, SPLITK_><<<grid, kPersistThreads, PersistCfg<BN_>::SMEM, stream>>>(ta, tb, g);
+  CHEM_CUDA_TRY(launch_pdl(gemm_bf16_persistent<BN_, SPLITK_>, grid, kPersistThreads, PersistCfg<BN_>::SMEM, stream, ta,
+                           tb, g));
   return CHEM_OK;
 }
 

@@ -1969,18 +1969,16 @@ int launch_advance(chem_mech_s* m, double* T, const double* p, double* Y, int64_
 }
 
 // Indexed integrator launch whose cell count (<= capacity) is read from device memory by the
-// kernel: the surrogate's fallback pass runs without a host round trip.
+// kernel: the surrogate's fallback pass runs without a host round trip.  counter: the launch's
+// work-queue counter, zeroed by the caller.
 int launch_advance_counted(chem_mech_s* m, double* T, const double* p, double* Y, int64_t ld,
-                           double dt, int64_t capacity, const unsigned int* count_dev, double rtol,
-                           double atol, const int32_t* idx, cudaStream_t stream) {
-  if (!m || !count_dev || !idx) { set_error("NULL argument"); return CHEM_EINVAL; }
+                           double dt, int64_t capacity, const unsigned int* count_dev, unsigned long long* counter,
+                           double rtol, double atol, const int32_t* idx, cudaStream_t stream) {
+  if (!m || !count_dev || !counter || !idx) { set_error("NULL argument"); return CHEM_EINVAL; }
   if (capacity <= 0) return CHEM_OK;
   LaunchShape s;
   int rc = pick_shape(m, nullptr, &s);
   if (rc) return rc;
-  unsigned long long* counter = nullptr;
-  CHEM_CUDA_TRY(ws_alloc((void**)&counter, sizeof(unsigned long long), stream));
-  CHEM_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(unsigned long long), stream));
   AdvanceParams P;
   mech_args(m, s, &P);
   P.segs[0] = Segment{T, p, Y, ld, capacity, idx, nullptr, nullptr, nullptr, dt, rtol, atol, 0};
@@ -1990,11 +1988,7 @@ int launch_advance_counted(chem_mech_s* m, double* T, const double* p, double* Y
   P.counter = counter;
   P.ncells_dev = count_dev;
   P.budget_ns = 0;
-  rc = dispatch_adv(s, P, nullptr, stream);
-  cudaError_t fe = cudaFreeAsync(counter, stream);
-  if (rc) return rc;
-  CHEM_CUDA_TRY(fe);
-  return CHEM_OK;
+  return dispatch_adv(s, P, nullptr, stream);
 }
 
 // Batched launch: the chunks of all segments go through one work queue of one persistent

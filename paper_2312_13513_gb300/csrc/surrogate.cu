@@ -42,6 +42,7 @@
 #include "fx_rates.cuh"
 #include "sm100.h"
 #include "gelu.cuh"
+#include "pdl.cuh"
 #include "surrogate_model.h"
 #include "thermo.cuh"
 
@@ -242,6 +243,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_wait();
+  pdl_trigger();
 
   if (warp == kTmaWarp) {
     if (lane == 0) {
@@ -502,6 +505,8 @@ __device__ __forceinline__ double h_over_r64(const double* a, double T) {
 template <int NS_, int NE_>
 __global__ void __launch_bounds__(64) surrogate_post_kernel(const PostParams P) {
   constexpr int ns = NS_, ne = NE_;
+  pdl_wait();
+  pdl_trigger();
   // the element matrix, its pair products and the species polynomials, read once per block with one
   // latency (a warp that has a single cell per thread waited for each of their cache lines in turn)
   __shared__ double sA[(ne + ne * (ne + 1) / 2) * ns];
@@ -698,6 +703,8 @@ __global__ void __launch_bounds__(64) surrogate_post_kernel(const PostParams P) 
 // The same post-processing for any species and element counts (runtime loops; per-cell arrays
 // sized for the maxima, in local memory).
 __global__ void surrogate_post_general(const PostParams P) {
+  pdl_wait();
+  pdl_trigger();
   const int ns = P.lay.ns;
   for (int64_t cell = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; cell < P.ncells;
        cell += (int64_t)gridDim.x * blockDim.x) {
@@ -906,19 +913,14 @@ int surrogate_forward(chem_model_s* md, const double* T, const double* p, const 
   if (ncells < 1) return CHEM_OK;
   const long long ntiles = (ncells + TM - 1) / TM;
   const long long grid = std::min<long long>(ntiles, max_ctas);
-  if (md->ns == 9)
-    surrogate_forward_kernel<9><<<(unsigned)grid, kFwdThreads, FWD_SMEM, stream>>>(md->tw[0], md->tw[1], md->tw[2],
-                                                                                  md->tw[3], md->tw[4], P);
-  else
-    surrogate_forward_kernel<0><<<(unsigned)grid, kFwdThreads, FWD_SMEM, stream>>>(md->tw[0], md->tw[1], md->tw[2],
-                                                                                  md->tw[3], md->tw[4], P);
-  CHEM_CUDA_TRY(cudaGetLastError());
+  CHEM_CUDA_TRY(launch_pdl(md->ns == 9 ? surrogate_forward_kernel<9> : surrogate_forward_kernel<0>, (unsigned)grid,
+                           kFwdThreads, FWD_SMEM, stream, md->tw[0], md->tw[1], md->tw[2], md->tw[3], md->tw[4], P));
   return CHEM_OK;
 }
 
 int launch_advance_counted(chem_mech_s* m, double* T, const double* p, double* Y, int64_t ld,
-                           double dt, int64_t capacity, const unsigned int* count_dev, double rtol,
-                           double atol, const int32_t* idx, cudaStream_t stream);
+                           double dt, int64_t capacity, const unsigned int* count_dev, unsigned long long* counter,
+                           double rtol, double atol, const int32_t* idx, cudaStream_t stream);
 
 }  // namespace chem
 
@@ -1375,9 +1377,9 @@ extern "C" int chem_surrogate_advance(chem_model_t md, chem_mech_t mech, double*
   if (ncells == 0) return CHEM_OK;
   if (!T || !p || !Y) { set_error("NULL state pointer"); return CHEM_EINVAL; }
   cudaStream_t st = (cudaStream_t)stream;
-  // per-call temporaries from the stream-ordered allocator: net output, box flags, fallback list
-  const size_t b_ynet = (size_t)ncells * md->ns * 4, b_box = ((size_t)ncells + 15) & ~(size_t)15;
-  const size_t b_idx = (size_t)ncells * 4;
+  // per-call temporaries from the library's pool: net output, box flags, fallback list, counters
+  auto al = [](size_t b) { return (b + 15) & ~(size_t)15; };
+  const size_t b_ynet = al((size_t)ncells * md->ns * 4), b_box = al((size_t)ncells), b_idx = al((size_t)ncells * 4);
   unsigned char* ws = nullptr;
   CHEM_CUDA_TRY(ws_alloc((void**)&ws, b_ynet + b_box + b_idx + 64, st));
   float* ynet = (float*)ws;
@@ -1385,6 +1387,7 @@ extern "C" int chem_surrogate_advance(chem_model_t md, chem_mech_t mech, double*
   int32_t* fb_idx = (int32_t*)(ws + b_ynet + b_box);
   unsigned int* fb_count = (unsigned int*)(ws + b_ynet + b_box + b_idx);
   int* err = (int*)(fb_count + 4);
+  unsigned long long* queue = (unsigned long long*)(fb_count + 8);   // the fallback launch's work queue
   CHEM_CUDA_TRY(cudaMemsetAsync(fb_count, 0, 64, st));
   int rc = surrogate_forward(md, T, p, Y, ld, ncells, ynet, nullptr, box, err, st);
   if (!rc) {
@@ -1399,13 +1402,12 @@ extern "C" int chem_surrogate_advance(chem_model_t md, chem_mech_t mech, double*
     // are no more than two blocks an SM (10007 cells: 157 blocks on 152 SMs; 256-thread blocks used
     // 40 SMs and took 35 us)
     const long long blocks = std::min<long long>((ncells + 63) / 64, (long long)sms * 64);
-    if (md->ns == 9 && md->ne == 3) surrogate_post_kernel<9, 3><<<(unsigned)blocks, 64, 0, st>>>(Q);
-    else surrogate_post_general<<<(unsigned)blocks, 64, 0, st>>>(Q);
-    cudaError_t le = cudaGetLastError();
+    const cudaError_t le = launch_pdl(md->ns == 9 && md->ne == 3 ? surrogate_post_kernel<9, 3> : surrogate_post_general,
+                                      (unsigned)blocks, 64, 0, st, Q);
     if (le != cudaSuccess) rc = cuda_fail(le, "surrogate_post_kernel");
   }
   if (!rc)
-    rc = launch_advance_counted(mech, T, p, Y, ld, dt, ncells, fb_count, rtol, atol, fb_idx, st);
+    rc = launch_advance_counted(mech, T, p, Y, ld, dt, ncells, fb_count, queue, rtol, atol, fb_idx, st);
   cudaError_t fe = cudaFreeAsync(ws, st);
   if (rc) return rc;
   CHEM_CUDA_TRY(fe);

@@ -22,6 +22,7 @@
 #include <vector>
 
 #include "chem_internal.h"
+#include "pdl.cuh"
 #include "surrogate_model.h"
 
 namespace chem {
@@ -49,6 +50,8 @@ struct PsFeatParams {
 // features of one cell, exactly as the single network's feature warps form them: T, ln p and the
 // Box-Cox transformed mass fractions in FP32, z-scored, split into [x_hi | x_lo | x_hi | 0]
 __global__ void k_ps_features(const PsFeatParams P) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= P.M) return;
   float x[SUR_KIN];
@@ -87,6 +90,8 @@ __global__ void k_ps_features(const PsFeatParams P) {
 // values a load (h3 is a multiple of 8)
 __global__ void k_ps_out(const __nv_bfloat16* A3, int h3, const __nv_bfloat16* w4, const float* b4, int64_t nc,
                          float* z) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (c >= nc) return;
@@ -120,6 +125,8 @@ struct PsInvParams {
 
 // inverse transform: Y' = BC^-1(BC(Y0) + z sd + mu), as the single network's epilogue
 __global__ void k_ps_inverse(const PsInvParams P) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= P.nc) return;
   for (int k = 0; k < P.ns; ++k) {
@@ -167,20 +174,23 @@ int surrogate_forward_ps(chem_model_s* md, const double* T, const double* p, con
     F.T = T + c0; F.p = p + c0; F.Y = Y + c0; F.ld = ld; F.nc = nc; F.M = M;
     F.ns = md->ns; F.nin = md->nin; F.xmu = md->xmu; F.xsd = md->xsd; F.lo = md->lo; F.hi = md->hi;
     F.X = X; F.outbox = outbox + c0;
-    k_ps_features<<<blocks_for(M, 256), 256, 0, st>>>(F);
+    cudaError_t le = launch_pdl(k_ps_features, blocks_for(M, 256), 256, 0, st, F);
+    if (le != cudaSuccess) rc = cuda_fail(le, "per-species feature kernel");
     for (int s = 0; s < md->nnet && !rc; ++s) {
       const PsNet& n = md->net[s];
       rc = gemm_bf16_act(X, SUR_KIN, n.W1, SUR_KIN, A1, h1, n.b1, 1, M, h1, SUR_KIN, err, st);
       if (!rc) rc = gemm_bf16_act(A1, h1, n.W2, h1, A2, h2, n.b2, 1, M, h2, h1, err, st);
       if (!rc) rc = gemm_bf16_act(A2, h2, n.W3, h2, A3, h3, n.b3, 1, M, h3, h2, err, st);
-      if (!rc) k_ps_out<<<blocks_for(nc * 32, 256), 256, 0, st>>>(A3, h3, (const __nv_bfloat16*)n.w4, n.b4, nc,
-                                                                  z + (int64_t)s * Mp);
+      if (!rc) {
+        le = launch_pdl(k_ps_out, blocks_for(nc * 32, 256), 256, 0, st, A3, h3, (const __nv_bfloat16*)n.w4, n.b4, nc,
+                        z + (int64_t)s * Mp);
+        if (le != cudaSuccess) rc = cuda_fail(le, "per-species output kernel");
+      }
     }
     if (rc) break;
     Q.Y = Y + c0; Q.nc = nc; Q.ynet = ynet + c0; Q.zout = zout ? zout + c0 : nullptr;
-    k_ps_inverse<<<blocks_for(nc, 256), 256, 0, st>>>(Q);
-    cudaError_t le = cudaGetLastError();
-    if (le != cudaSuccess) rc = cuda_fail(le, "per-species surrogate kernels");
+    le = launch_pdl(k_ps_inverse, blocks_for(nc, 256), 256, 0, st, Q);
+    if (le != cudaSuccess) rc = cuda_fail(le, "per-species inverse kernel");
   }
   cudaError_t fe = cudaFreeAsync(ws, st);
   if (rc) return rc;

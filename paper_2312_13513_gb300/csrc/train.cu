@@ -31,6 +31,7 @@
 #include <vector>
 
 #include "chem_internal.h"
+#include "pdl.cuh"
 
 namespace chem {
 int gemm_bf16(const void* A, int64_t lda, const void* B, int64_t ldb, float* C, int64_t ldc,
@@ -102,6 +103,8 @@ __device__ __forceinline__ void gradient_tile(F grad, __nv_bfloat16* dZb, __nv_b
 // dZ = dA GELU'(Z)
 __global__ void __launch_bounds__(256) k_gelu_bwd(const float* dA, const float* Z, __nv_bfloat16* dZb,
                                                   __nv_bfloat16* dZt, double* part, int R, int C) {
+  pdl_wait();
+  pdl_trigger();
   gradient_tile(
       [&](int r, int c) {
         const float2 a = *reinterpret_cast<const float2*>(dA + (int64_t)r * C + c);
@@ -116,6 +119,8 @@ __global__ void __launch_bounds__(256) k_gelu_bwd(const float* dA, const float* 
 __global__ void __launch_bounds__(256) k_mse_grad(const float* out, const float* target, __nv_bfloat16* dZb,
                                                   __nv_bfloat16* dZt, double* part, double* loss_part, int B, int nout,
                                                   int ld) {
+  pdl_wait();
+  pdl_trigger();
   const float scale = 2.0f / ((float)B * (float)nout);
   double sum = 0.0;
   gradient_tile(
@@ -158,6 +163,8 @@ struct TransposeSet {
 };
 
 __global__ void __launch_bounds__(256) k_transpose_set(const __grid_constant__ TransposeSet S) {
+  pdl_wait();
+  pdl_trigger();
   if ((int)blockIdx.z >= S.n) return;
   const TransposeJob& J = S.j[blockIdx.z];
   const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64, tx = threadIdx.x, ty = threadIdx.y;
@@ -178,13 +185,14 @@ __global__ void __launch_bounds__(256) k_transpose_set(const __grid_constant__ T
   }
 }
 
-void launch_transposes(const TransposeSet& S, cudaStream_t st) {
+int launch_transposes(const TransposeSet& S, cudaStream_t st) {
   int gx = 1, gy = 1;
   for (int k = 0; k < S.n; ++k) {
     gx = std::max(gx, (S.j[k].C + 63) / 64);
     gy = std::max(gy, (S.j[k].R + 63) / 64);
   }
-  k_transpose_set<<<dim3(gx, gy, S.n), dim3(32, 8), 0, st>>>(S);
+  CHEM_CUDA_TRY(launch_pdl(k_transpose_set, dim3(gx, gy, S.n), dim3(32, 8), 0, st, S));
+  return CHEM_OK;
 }
 
 // The end of a backward pass in one launch: every layer's weight gradient as the ordered sum of its
@@ -210,6 +218,8 @@ struct FinishSet {
 };
 
 __global__ void __launch_bounds__(256) k_finish_grads(const __grid_constant__ FinishSet S) {
+  pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
   if (blockIdx.x == gridDim.x - 1) {
     if (threadIdx.x < 32) {
@@ -271,6 +281,8 @@ struct AdamSet {
 };
 
 __global__ void k_adam_set(const __grid_constant__ AdamSet S, const float* coef, float b1, float b2, float eps) {
+  pdl_wait();
+  pdl_trigger();
   int k = 0;
   while (k + 1 < S.n && S.s[k + 1].block0 <= (int)blockIdx.x) ++k;
   const AdamSeg& q = S.s[k];
@@ -302,6 +314,8 @@ __global__ void k_adam_set(const __grid_constant__ AdamSet S, const float* coef,
 // One Adam step's scalars on the device: step += 1, coef = {lr, 1 - b1^step, 1 - b2^step}, with lr
 // from lr_dev when given (a captured training step reads its learning rate from device memory)
 __global__ void k_adam_prep(int64_t* step, float* coef, const float* lr_dev, float lr, float b1, float b2) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t s = *step + 1;
   *step = s;
   coef[0] = lr_dev ? *lr_dev : lr;
@@ -349,6 +363,8 @@ struct FlatSet {
 
 // unpack: buf = scale * flat (the padding keeps its zeros); otherwise flat = buf
 __global__ void k_flat_grads(const __grid_constant__ FlatSet S, float* flat, const float* src, float scale, int unpack) {
+  pdl_wait();
+  pdl_trigger();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < S.total; i += (int64_t)gridDim.x * blockDim.x) {
     int k = 0;
     while (k + 1 < S.n && S.s[k + 1].flat <= i) ++k;
@@ -635,11 +651,12 @@ extern "C" int chem_mlp_backward(chem_trainer_t t, const float* target, double* 
   // A^T of every layer (batch contiguous, for the weight gradients)
   TransposeSet T{};
   for (int l = 0; l < NL; ++l) T.j[T.n++] = TransposeJob{t->A[l], t->At[l], B, t->in_pad[l]};
-  launch_transposes(T, st);
+  const int trc = launch_transposes(T, st);
+  if (trc) return trc;
   const int nrb = (B + kColRows - 1) / kColRows;
   const dim3 mse_grid((PADIO + 63) / 64, nrb);
-  k_mse_grad<<<mse_grid, dim3(32, 8), 0, st>>>(t->Z[NL - 1], target, t->dZb, t->dZt, t->colpart[NL - 1],
-                                               t->loss_part, B, t->nout, PADIO);
+  CHEM_CUDA_TRY(launch_pdl(k_mse_grad, mse_grid, dim3(32, 8), 0, st, t->Z[NL - 1], target, t->dZb, t->dZt,
+                           t->colpart[NL - 1], t->loss_part, B, t->nout, PADIO));
   for (int l = NL - 1; l >= 0; --l) {
     const int nout = t->out_pad[l], nin = t->in_pad[l];
     int rc;
@@ -652,8 +669,8 @@ extern "C" int chem_mlp_backward(chem_trainer_t t, const float* target, double* 
     if (l > 0) {
       rc = gemm_bf16(t->dZb, nout, t->Wt[l], nout, t->dA, nin, nullptr, B, nin, nout, t->err, st);
       if (rc) return rc;
-      k_gelu_bwd<<<dim3((nin + 63) / 64, nrb), dim3(32, 8), 0, st>>>(t->dA, t->Z[l - 1], t->dZb, t->dZt,
-                                                                     t->colpart[l - 1], B, nin);
+      CHEM_CUDA_TRY(launch_pdl(k_gelu_bwd, dim3((nin + 63) / 64, nrb), dim3(32, 8), 0, st, t->dA, t->Z[l - 1],
+                               t->dZb, t->dZt, t->colpart[l - 1], B, nin));
     }
   }
   FinishSet F{};
@@ -669,14 +686,14 @@ extern "C" int chem_mlp_backward(chem_trainer_t t, const float* target, double* 
   F.loss_part = t->loss_part; F.n_loss = (int)(mse_grid.x * mse_grid.y);
   F.loss_scale = 1.0 / ((double)B * t->nout);
   F.loss = t->loss; F.loss_out = loss_out;
-  k_finish_grads<<<blocks + 1, 256, 0, st>>>(F);
+  CHEM_CUDA_TRY(launch_pdl(k_finish_grads, blocks + 1, 256, 0, st, F));
   CHEM_CUDA_TRY(cudaGetLastError());
   return CHEM_OK;
 }
 
 static int adam_step(chem_trainer_t t, const float* lr_dev, float lr, float beta1, float beta2, float eps,
                      cudaStream_t st) {
-  k_adam_prep<<<1, 1, 0, st>>>(t->d_step, t->d_coef, lr_dev, lr, beta1, beta2);
+  CHEM_CUDA_TRY(launch_pdl(k_adam_prep, 1, 1, 0, st, t->d_step, t->d_coef, lr_dev, lr, beta1, beta2));
   // every weight matrix and bias vector in one launch (their BF16 copies written on the way), then
   // the transposed copies the backward pass multiplies with
   AdamSet A{};
@@ -691,12 +708,10 @@ static int adam_step(chem_trainer_t t, const float* lr_dev, float lr, float beta
     add(t->W[l], t->dW[l], t->mW[l], t->vW[l], t->Wb[l], (int64_t)r * c, l == 0 ? t->nin : 0, c);
     add(t->b[l], t->db[l], t->mb[l], t->vb[l], nullptr, r, 0, 1);
   }
-  k_adam_set<<<blocks, 256, 0, st>>>(A, t->d_coef, beta1, beta2, eps);
+  CHEM_CUDA_TRY(launch_pdl(k_adam_set, blocks, 256, 0, st, A, t->d_coef, beta1, beta2, eps));
   TransposeSet T{};
   for (int l = 1; l < t->nl; ++l) T.j[T.n++] = TransposeJob{t->Wb[l], t->Wt[l], t->out_pad[l], t->in_pad[l]};
-  if (T.n) launch_transposes(T, st);
-  CHEM_CUDA_TRY(cudaGetLastError());
-  return CHEM_OK;
+  return T.n ? launch_transposes(T, st) : CHEM_OK;
 }
 
 extern "C" int chem_mlp_adam_step(chem_trainer_t t, float lr, float beta1, float beta2, float eps,
@@ -763,7 +778,7 @@ static FlatSet flat_set(chem_trainer_t t) {
 extern "C" int chem_mlp_grad_pack(chem_trainer_t t, float* flat, chem_stream_t stream) {
   if (!t || !flat) { set_error("NULL argument"); return CHEM_EINVAL; }
   const FlatSet S = flat_set(t);
-  k_flat_grads<<<grid_for(S.total), 256, 0, (cudaStream_t)stream>>>(S, flat, nullptr, 1.0f, 0);
+  CHEM_CUDA_TRY(launch_pdl(k_flat_grads, grid_for(S.total), 256, 0, (cudaStream_t)stream, S, flat, nullptr, 1.0f, 0));
   CHEM_CUDA_TRY(cudaGetLastError());
   return CHEM_OK;
 }
@@ -771,7 +786,7 @@ extern "C" int chem_mlp_grad_pack(chem_trainer_t t, float* flat, chem_stream_t s
 extern "C" int chem_mlp_grad_unpack(chem_trainer_t t, const float* flat, float scale, chem_stream_t stream) {
   if (!t || !flat || !std::isfinite(scale)) { set_error("bad arguments"); return CHEM_EINVAL; }
   const FlatSet S = flat_set(t);
-  k_flat_grads<<<grid_for(S.total), 256, 0, (cudaStream_t)stream>>>(S, nullptr, flat, scale, 1);
+  CHEM_CUDA_TRY(launch_pdl(k_flat_grads, grid_for(S.total), 256, 0, (cudaStream_t)stream, S, nullptr, flat, scale, 1));
   CHEM_CUDA_TRY(cudaGetLastError());
   return CHEM_OK;
 }
