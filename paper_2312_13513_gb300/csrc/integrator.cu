@@ -41,7 +41,8 @@ namespace chem {
 
 // one thread per cell (integrator_cell.cu)
 bool cell_kernel_fits(const chem_mech_s* m);
-int launch_cell_advance(const chem_mech_s* m, const QueueParams& Q, const chem_options* opt, cudaStream_t stream);
+int launch_cell_advance(const chem_mech_s* m, const QueueParams& Q, bool scratch, const chem_options* opt,
+                        cudaStream_t stream);
 int launch_cell_eval(const chem_mech_s* m, const double* T, const double* p, const double* Y, int64_t ld, int64_t n,
                      double* f, double* J, cudaStream_t stream);
 
@@ -1896,10 +1897,11 @@ int launch_eval_t(const LaunchShape& s, const EvalParams& P, cudaStream_t stream
   return CHEM_OK;
 }
 
+// scratch: whether the launch may take device memory beyond the counter
 int dispatch_adv(const LaunchShape& s, const AdvanceParams& P, const chem_options* opt,
-                 cudaStream_t stream) {
+                 cudaStream_t stream, bool scratch = true) {
   switch (s.G) {
-    case 1: return launch_cell_advance(s.m, P, opt, stream);
+    case 1: return launch_cell_advance(s.m, P, scratch, opt, stream);
     case 2: return launch_adv_t<2>(s, P, opt, stream);
     case 4: return launch_adv_t<4>(s, P, opt, stream);
     case 8: return launch_adv_t<8>(s, P, opt, stream);
@@ -1988,7 +1990,7 @@ int launch_advance_counted(chem_mech_s* m, double* T, const double* p, double* Y
   P.counter = counter;
   P.ncells_dev = count_dev;
   P.budget_ns = 0;
-  return dispatch_adv(s, P, nullptr, stream);
+  return dispatch_adv(s, P, nullptr, stream, false);    // of `capacity` cells usually few are left
 }
 
 // Batched launch: the chunks of all segments go through one work queue of one persistent
@@ -2215,7 +2217,7 @@ int launch_advance_noalloc(chem_mech_s* m, double* T, const double* p, double* Y
   P.counter = counter;
   P.ncells_dev = nullptr;
   P.budget_ns = 0;
-  return dispatch_adv(s, P, nullptr, stream);
+  return dispatch_adv(s, P, nullptr, stream, false);
 }
 
 }  // namespace chem

@@ -28,6 +28,7 @@ struct CellParams {
   MechLayout lay;
   const unsigned char *fxblob, *blob;
   QueueParams q;
+  double* mx;                  // WIDE: the matrices, a warp's N x N x 32 after the other's
 };
 
 struct CellEvalParams {
@@ -49,13 +50,12 @@ __device__ __forceinline__ void stage(const unsigned char* src, unsigned char* d
 // matrix; otherwise e2 = the squared weighted RMS error and the new state left in U_5's place
 // (elements U + 5 N ..: y_new), which the caller copies on acceptance.
 template <int NS>
-__device__ __forceinline__ bool attempt(const cell::View& m, double* col, double p, double invp, double h, double rtol,
+__device__ __forceinline__ bool attempt(const cell::View& m, double* col, double* M, double p, double invp, double h, double rtol,
                                         double atol, double* e2) {
   using w = Ws<NS>;
   constexpr int N = w::N;
   const double invh = fx::rcp(h), ig = invh * (1.0 / kGamma);
-  cell::rhs<NS, true>(m, col, col[w::Y * 32], [&](int k) { return col[(w::Y + 1 + k) * 32]; }, p, invp, w::U);
-  double* M = col + w::M * 32;
+  cell::rhs<NS, true>(m, col, M, col[w::Y * 32], [&](int k) { return col[(w::Y + 1 + k) * 32]; }, p, invp, w::U);
 #pragma unroll
   for (int i = 0; i < N; ++i) M[i * (N + 1) * 32] += ig;
 
@@ -112,7 +112,7 @@ __device__ __forceinline__ bool attempt(const cell::View& m, double* col, double
         for (int j = 0; j < s; ++j) v = fma(ra[j], col[(w::U + j * N + i) * 32], v);
         return v;
       };
-      cell::rhs<NS, false>(m, col, stage_value(0), [&](int k) { return stage_value(1 + k); }, p, invp, us);
+      cell::rhs<NS, false>(m, col, M, stage_value(0), [&](int k) { return stage_value(1 + k); }, p, invp, us);
     }
     // right-hand side f + sum_j (C_sj / h) u_j, then both triangular sweeps in registers
     double b[N], t[N];
@@ -159,8 +159,13 @@ __device__ __forceinline__ bool attempt(const cell::View& m, double* col, double
   return !singular;
 }
 
-template <int NS>
-__global__ void __launch_bounds__(128, 1) cell_advance_kernel(const __grid_constant__ CellParams P) {
+// WIDE: eight warps an SM instead of four.  Four hold their whole workspace in shared memory (51 KB a
+// warp for 9 species) and keep the FP64 pipe 64 % busy: a sub-partition's one warp cannot overlap its
+// integer work with its own FP64 instructions.  With the matrix (half of the workspace) in an
+// L2-resident array of global memory (25 KB a warp, 31 MB in all) two warps share a sub-partition:
+// 2^20 flame cells 108 -> 80.2 ms.  (The vectors in global memory and the matrix in shared memory: 92.9.)
+template <int NS, bool WIDE>
+__global__ void __launch_bounds__(WIDE ? 256 : 128, 1) cell_advance_kernel(const __grid_constant__ CellParams P) {
   using w = Ws<NS>;
   constexpr int N = w::N;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -169,7 +174,11 @@ __global__ void __launch_bounds__(128, 1) cell_advance_kernel(const __grid_const
   __syncthreads();
   const cell::View m = cell::bind(smem, P.fx, P.blob, &P.lay);
   const int lane = threadIdx.x & 31;
-  double* col = (double*)(smem + P.fx.bytes) + (size_t)(threadIdx.x >> 5) * w::TOTAL * 32 + lane;
+  const int wib = threadIdx.x >> 5;
+  double* const sh = (double*)(smem + P.fx.bytes);
+  double* const col = sh + (size_t)wib * (WIDE ? w::VEC : w::TOTAL) * 32 + lane;
+  double* const Mx = WIDE ? P.mx + ((size_t)blockIdx.x * (blockDim.x >> 5) + wib) * N * N * 32 + lane
+                          : col + w::VEC * 32;
   auto dummy = [&] {
 #pragma unroll
     for (int i = 0; i < N; ++i) col[(w::Y + i) * 32] = i == 0 ? 1000.0 : 1.0 / NS;
@@ -251,7 +260,7 @@ __global__ void __launch_bounds__(128, 1) cell_advance_kernel(const __grid_const
     }
     const bool run = active && !stop;
     double e2 = 0.0;
-    const bool ok = attempt<NS>(m, col, p, invp, run ? h : dt, rtol, atol, &e2);
+    const bool ok = attempt<NS>(m, col, Mx, p, invp, run ? h : dt, rtol, atol, &e2);
     if (run) {
       if (!ok) {
         stop = true; status = CHEM_CELL_SINGULAR_LU;
@@ -305,21 +314,21 @@ __global__ void __launch_bounds__(128, 1) cell_eval_kernel(const __grid_constant
     for (int i = 0; i < N; ++i) col[(w::Y + i) * 32] = i == 0 ? P.T[c] : P.Y[(int64_t)(i - 1) * P.ld + c];
     const double p = P.p[c];
     auto Yk = [&](int k) { return col[(w::Y + 1 + k) * 32]; };
-    if (P.J) cell::rhs<NS, true>(m, col, col[w::Y * 32], Yk, p, 1.0 / p, w::U);
-    else cell::rhs<NS, false>(m, col, col[w::Y * 32], Yk, p, 1.0 / p, w::U);
+    if (P.J) cell::rhs<NS, true>(m, col, col + w::VEC * 32, col[w::Y * 32], Yk, p, 1.0 / p, w::U);
+    else cell::rhs<NS, false>(m, col, col + w::VEC * 32, col[w::Y * 32], Yk, p, 1.0 / p, w::U);
     for (int i = 0; i < N; ++i) P.f[(int64_t)i * P.ld + c] = col[(w::U + i) * 32];
     if (P.J)
-      for (int e = 0; e < N * N; ++e) P.J[(int64_t)e * P.ld + c] = -col[(w::M + e) * 32];
+      for (int e = 0; e < N * N; ++e) P.J[(int64_t)e * P.ld + c] = -col[(w::VEC + e) * 32];
   }
 }
 
 struct Shape {
-  int warps, sms;
+  int warps, sms, smem_max;
   size_t smem;          // of `warps` warps
 };
 
-// Warps of 32 cells that fit in an SM's shared memory, at most four: one per sub-partition keeps
-// each FP64 pipe busy (the instruction latency equals the pipe's occupancy), a fifth shares one.
+// Warps of 32 cells whose whole workspace fits in an SM's shared memory, at most four: one per
+// sub-partition (an FP64 instruction's latency equals its occupancy of the pipe), a fifth shares one.
 // Three warps still issue at 89 % of four's FP64 rate (21.4 SM cycles an instruction against 19.0);
 // two would leave half of the sub-partitions idle, so such mechanisms keep the group kernels.
 template <int NS>
@@ -329,6 +338,7 @@ int shape_of(const chem_mech_s* m, Shape* s) {
   CHEM_CUDA_TRY(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   CHEM_CUDA_TRY(cudaDeviceGetAttribute(&s->sms, cudaDevAttrMultiProcessorCount, dev));
   const size_t per = (size_t)Ws<NS>::TOTAL * 256;
+  s->smem_max = smem_max;
   const long long room = (long long)smem_max - m->fx.bytes;
   s->warps = (int)std::min<long long>(4, room / (long long)per);
   s->smem = (size_t)m->fx.bytes + per * std::max(s->warps, 0);
@@ -336,12 +346,12 @@ int shape_of(const chem_mech_s* m, Shape* s) {
 }
 
 template <int NS>
-int advance_t(const chem_mech_s* m, const QueueParams& Q, const chem_options* opt, cudaStream_t stream) {
+int advance_t(const chem_mech_s* m, const QueueParams& Q, bool scratch, const chem_options* opt, cudaStream_t stream) {
   Shape s;
   int rc = shape_of<NS>(m, &s);
   if (rc) return rc;
   if (s.warps < 1) { set_error("mechanism too large for shared memory"); return CHEM_EINVAL; }
-  CHEM_CUDA_TRY(cudaFuncSetAttribute(cell_advance_kernel<NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem));
+  CHEM_CUDA_TRY(cudaFuncSetAttribute((cell_advance_kernel<NS, false>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem));
   const size_t per = (size_t)Ws<NS>::TOTAL * 256;
   int warps = s.warps;
   if (opt && opt->groups_per_cta > 0) warps = std::min(warps, (opt->groups_per_cta + 31) / 32);
@@ -353,7 +363,29 @@ int advance_t(const chem_mech_s* m, const QueueParams& Q, const chem_options* op
   CellParams P;
   P.fx = m->fx; P.lay = m->lay; P.fxblob = (const unsigned char*)m->d_fx; P.blob = (const unsigned char*)m->d_blob;
   P.q = Q;
-  cell_advance_kernel<NS><<<(unsigned)grid, 32 * warps, (size_t)m->fx.bytes + per * warps, stream>>>(P);
+  // eight warps an SM (seven for 10 and 11 species) from 13 warps of cells an SM on (63 k cells on 152 SMs): below, the stiffest cells
+  // of the last warps count for more than the rate (H2 flame, four / eight warps: 40009 cells 9.7 /
+  // 12.6 ms, 80021 16.7 / 14.4, 2^20 108 / 80.2).  Without room for the matrices: four.
+  constexpr size_t kMat = (size_t)Ws<NS>::N * Ws<NS>::N * 256, kVec = (size_t)Ws<NS>::VEC * 256;
+  const int ww = (int)std::min<long long>(8, ((long long)s.smem_max - m->fx.bytes) / (long long)kVec);
+  P.mx = nullptr;
+  if (scratch && warps == s.warps && ww > warps && need >= 13 * grid) {
+    const size_t wide = (size_t)m->fx.bytes + kVec * (size_t)ww;
+    if (ws_alloc((void**)&P.mx, kMat * (size_t)ww * (size_t)grid, stream) == cudaSuccess) {
+      cudaError_t e = cudaFuncSetAttribute((cell_advance_kernel<NS, true>), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)wide);
+      if (e == cudaSuccess) {
+        cell_advance_kernel<NS, true><<<(unsigned)grid, 32 * ww, wide, stream>>>(P);
+        e = cudaGetLastError();
+      }
+      const cudaError_t fe = cudaFreeAsync(P.mx, stream);
+      CHEM_CUDA_TRY(e);
+      CHEM_CUDA_TRY(fe);
+      return CHEM_OK;
+    }
+    (void)cudaGetLastError();
+  }
+  cell_advance_kernel<NS, false><<<(unsigned)grid, 32 * warps, (size_t)m->fx.bytes + per * warps, stream>>>(P);
   CHEM_CUDA_TRY(cudaGetLastError());
   return CHEM_OK;
 }
@@ -380,7 +412,7 @@ int eval_t(const chem_mech_s* m, const double* T, const double* p, const double*
 // has an instance, and at least three warps of cells fit on an SM (see shape_of).
 bool cell_kernel_fits(const chem_mech_s* m) {
   if (!m->fx.bytes) return false;
-  Shape s{0, 0, 0};
+  Shape s{0, 0, 0, 0};
   int rc = CHEM_EINVAL;
   switch (m->ns) {
     case 8: rc = shape_of<8>(m, &s); break;
@@ -392,7 +424,9 @@ bool cell_kernel_fits(const chem_mech_s* m) {
   return rc == CHEM_OK && s.warps >= 3;
 }
 
-int launch_cell_advance(const chem_mech_s* m, const QueueParams& Q, const chem_options* opt, cudaStream_t stream) {
+// scratch: whether the launch may take device memory from the pool
+int launch_cell_advance(const chem_mech_s* m, const QueueParams& Q, bool scratch, const chem_options* opt,
+                        cudaStream_t stream) {
   int dev = 0, sms = 0, smem_max = 0;
   CHEM_CUDA_TRY(cudaGetDevice(&dev));
   CHEM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -402,10 +436,10 @@ int launch_cell_advance(const chem_mech_s* m, const QueueParams& Q, const chem_o
   const int lanes = shaped ? 1 : cell_lanes(m, Q.total_chunks, max_ctas > 0 ? std::min(sms, max_ctas) : sms, smem_max);
   if (lanes > 1) return launch_coop_advance(m, Q, lanes, sms, smem_max, max_ctas, stream);
   switch (m->ns) {
-    case 8: return advance_t<8>(m, Q, opt, stream);
-    case 9: return advance_t<9>(m, Q, opt, stream);
-    case 10: return advance_t<10>(m, Q, opt, stream);
-    case 11: return advance_t<11>(m, Q, opt, stream);
+    case 8: return advance_t<8>(m, Q, scratch, opt, stream);
+    case 9: return advance_t<9>(m, Q, scratch, opt, stream);
+    case 10: return advance_t<10>(m, Q, scratch, opt, stream);
+    case 11: return advance_t<11>(m, Q, scratch, opt, stream);
     default: set_error("no cell kernel for %d species", m->ns); return CHEM_EINVAL;
   }
 }

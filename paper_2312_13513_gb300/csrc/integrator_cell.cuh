@@ -15,7 +15,9 @@
 // result does not depend on the launch it is part of.
 //
 // Layout: a warp owns 32 cells; element e of a lane's workspace is at e * 32 + lane (doubles), so
-// every access, also by a lane-dependent row after pivoting, is free of bank conflicts.
+// every access, also by a lane-dependent row after pivoting, is free of bank conflicts.  The matrix
+// is a second array of the same form: in shared memory, or for large launches in global memory
+// (integrator_cell.cu).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -35,12 +37,13 @@ using fx::Temp;
 using fx::temp_of;
 using fx::troe_fast;
 
-// workspace elements of one cell (doubles): state, six stage vectors, the iteration matrix,
-// concentrations and Gibbs energies (each with the empty slot's 1 and 0 at the end), enthalpies
+// workspace elements of one cell (doubles): state, six stage vectors, concentrations and Gibbs
+// energies (each with the empty slot's 1 and 0 at the end), enthalpies: VEC of them, and the
+// iteration matrix
 template <int NS>
 struct Ws {
   static constexpr int N = NS + 1;
-  static constexpr int Y = 0, U = N, M = 7 * N, C = M + N * N, G = C + N, H = G + N, TOTAL = H + NS;
+  static constexpr int Y = 0, U = N, C = 7 * N, G = C + N, H = G + N, VEC = H + NS, TOTAL = VEC + N * N;
   // scratch inside the stage vectors while the Jacobian is formed (u_0 holds the rates)
   static constexpr int DWDT = U + N, CP = U + 2 * N, RK = U + 3 * N, WK = U + 4 * N;
 };
@@ -145,7 +148,7 @@ __device__ __forceinline__ double partners(const View& m, const double* col, int
 // Any reaction (FxReac): three species on a side, up to six net species.  Adds its production rates
 // and, with JAC, its derivatives.
 template <int NS, bool JAC>
-__device__ __noinline__ void general_reaction(const View& m, double* col, const FxReac& R, const Temp& t, double T,
+__device__ __noinline__ void general_reaction(const View& m, double* col, double* Mx, const FxReac& R, const Temp& t, double T,
                                               fx::i64 shift, fx::i64 D, double Ctot, int uoff) {
   using w = Ws<NS>;
   constexpr int N = w::N;
@@ -189,7 +192,7 @@ __device__ __noinline__ void general_reaction(const View& m, double* col, const 
     for (int i = 0; i < npr; ++i) dH += col[(w::H + R.pr[i]) * 32];
     dqdT = mult * fma(net, dlnkf, rev * (dH * t.invT));
   }
-  double* Jm = col + (w::M + N + 1) * 32;
+  double* Jm = Mx + (N + 1) * 32;
   for (int i = 0; i < nn; ++i) {
     const double nu = m.nu[R.nu[i] + 8];
     double* x = col + (uoff + 1 + R.sp[i]) * 32;
@@ -212,10 +215,10 @@ __device__ __noinline__ void general_reaction(const View& m, double* col, const 
 }
 
 // Right-hand side f(T, Y) into workspace elements uoff .., and with JAC the NEGATED analytic
-// Jacobian -df/dy into the matrix.  Yk(k) returns the mass fraction of species k; p and 1 / p of
+// Jacobian -df/dy into the matrix Mx.  Yk(k) returns the mass fraction of species k; p and 1 / p of
 // the cell.  Writes the concentrations, Gibbs energies and enthalpies of the workspace.
 template <int NS, bool JAC, class YF>
-__device__ __forceinline__ void rhs(const View& m, double* col, double T, YF Yk, double p, double invp, int uoff) {
+__device__ __forceinline__ void rhs(const View& m, double* col, double* Mx, double T, YF Yk, double p, double invp, int uoff) {
   using w = Ws<NS>;
   constexpr int N = w::N;
   const Temp t = temp_of(T, m, JAC);
@@ -274,7 +277,7 @@ __device__ __forceinline__ void rhs(const View& m, double* col, double T, YF Yk,
   col[(w::G + NS) * 32] = 0.0;
   if (JAC) {
 #pragma unroll
-    for (int e = 0; e < NS * NS; ++e) col[(w::M + (1 + e / NS) * N + 1 + e % NS) * 32] = 0.0;
+    for (int e = 0; e < NS * NS; ++e) Mx[((1 + e / NS) * N + 1 + e % NS) * 32] = 0.0;
   }
   const double Ctot = rho * S;
   const fx::i64 D = (fx::i64)((t.L + 128ull) >> 8) - m.lpr0;
@@ -282,7 +285,7 @@ __device__ __forceinline__ void rhs(const View& m, double* col, double T, YF Yk,
   double* const Cc = col + w::C * 32;
   double* const Gc = col + w::G * 32;
   double* const wd = col + (uoff + 1) * 32;
-  double* const Jm = col + (w::M + N + 1) * 32;      // row 1 (species 0), column 1
+  double* const Jm = Mx + (N + 1) * 32;              // row 1 (species 0), column 1
 
   // exponents and concentration products of an FxRate
   auto prepare = [&](const FxRate& R, const Slots& s, fx::i64& Xf, fx::i64& Xr) {
@@ -411,7 +414,7 @@ __device__ __forceinline__ void rhs(const View& m, double* col, double T, YF Yk,
     }
   }
   // ---- reactions with three species on a side or more than four net species ----
-  for (int i = 0; i < m.n_gen; ++i) general_reaction<NS, JAC>(m, col, m.reac[i], t, T, shift, D, Ctot, uoff);
+  for (int i = 0; i < m.n_gen; ++i) general_reaction<NS, JAC>(m, col, Mx, m.reac[i], t, T, shift, D, Ctot, uoff);
 
   // species and temperature rows: f_k = W_k w_k / rho, f_0 = -T sum h/RT w / (rho cp/R)
   double Q = 0.0, r31 = 0.0, r32 = 0.0;
@@ -449,7 +452,7 @@ __device__ __forceinline__ void rhs(const View& m, double* col, double T, YF Yk,
   }
   const double TQ = T * Q, TRh = T * Rh;
   const double Qr = TQ * ircp;                 // -f_0
-  col[w::M * 32] = fma(fma(T, r32, r31) - Rh, ircp, Qr * fma(cps, t.invT, -dcps) * (rho * ircp));
+  Mx[0] = fma(fma(T, r32, r31) - Rh, ircp, Qr * fma(cps, t.invT, -dcps) * (rho * ircp));
   const double RhS = TRh * iS, cpS = __dmul_rn(cps, iS), Qrr = Qr * rho;
 #pragma unroll 2
   for (int mm = 0; mm < NS; ++mm) {

@@ -140,19 +140,21 @@ def test_advance_agrees_with_the_group_kernel(h2, which, n):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("which,per_sm,extra", [("8", 0, 1), ("9", 0, 5), ("9", 28, 0), ("9", 28, 1), ("9", 104, 0),
-                                                ("10", 28, 3), ("11", 0, 129), ("11", 30, 0), ("slow", 0, 65),
-                                                ("slow", 29, 0)])
-def test_few_cells_take_several_lanes(h2, which, per_sm, extra):
-    """Launches of few cells (16 or 8 lanes a cell, lines at 28 and 104 cells per SM) against the same
-    cells inside a launch beyond both lines (one thread per cell): the same operations, so the same
-    bits."""
+@pytest.mark.parametrize("which,per_sm,extra,big_sm", [("8", 0, 1, 104), ("9", 0, 5, 104), ("9", 28, 0, 104),
+                                                       ("9", 28, 1, 104), ("9", 104, 0, 104), ("10", 28, 3, 104),
+                                                       ("11", 0, 129, 104), ("11", 30, 0, 104), ("slow", 0, 65, 104),
+                                                       ("slow", 29, 0, 104), ("9", 120, 7, 420), ("8", 28, 0, 420),
+                                                       ("11", 104, 1, 420), ("slow", 110, 0, 420)])
+def test_launch_size_does_not_change_a_cell(h2, which, per_sm, extra, big_sm):
+    """Launches of few cells (16 or 8 lanes a cell up to 28 and 104 cells per SM) and of many (eight
+    warps an SM from 416 cells per SM on) against one thread per cell in between: the same
+    operations, so the same bits."""
     import torch
     import paper_2312_13513_gb300 as cg
     from gpu_common import to_dev
     from helpers import random_states
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    n, big = per_sm * sms + extra, 104 * sms + 33
+    n, big = per_sm * sms + extra, big_sm * sms + 33
     m = _mechs(h2)[which]
     dm = cg.Mechanism(m)
     T, p, Y = random_states(h2, big, 60 + n, "H2", Tlo=300.0, Thi=2600.0)
