@@ -443,11 +443,9 @@ def small_h2_states(n=4096, seed=12345):
 
 def extra_h2_small(fp64_peak, n=4096, reps=10, group=0):
     """Config 0: the small H2 case (4096 cells, dt = 1e-6 s).  Too few cells to fill the GPU (the
-    bench launch holds 80 two-thread groups = 80 cells per SM): the time is the sequential
-    attempts of the stiffest cells, each attempt's FP64 instructions issued by one warp.  Reported
-    with the library's default group (two threads per cell) and, with the default, also with one
-    warp per cell (group_threads = 32, a caller's option: fewer instructions per attempt for each
-    cell, fewer cells per warp)."""
+    bench launch holds 256 cells per SM, one per thread): the time is the sequential attempts of the
+    stiffest cells.  Reported with the library's default (16 lanes per cell at this size) and, with
+    the default, also with one warp per cell in FP64 (group_threads = 32, a caller's option)."""
     import torch
     from paper_2312_13513_gb300 import flops as fl
     import paper_2312_13513_gb300 as cg
@@ -471,10 +469,10 @@ def extra_h2_small(fp64_peak, n=4096, reps=10, group=0):
     t = timed(group)
     acc = int(ns_.sum()); att = acc + int(nr_.sum())
     _, _, folded = fl.launch_flops(mech, acc, att)
-    slots = torch.cuda.get_device_properties(0).multi_processor_count * 80
+    slots = torch.cuda.get_device_properties(0).multi_processor_count * 256
     out = {"workload": f"FP64 Rodas4, {n} H2/air mixing states (half pre-reacted by this integrator), "
                        "dt=1e-6 s",
-           "group_threads": group or 2, "ms": t * 1e3, "cell_updates_per_s": n / t,
+           "group_threads": group or "default (16 lanes)", "ms": t * 1e3, "cell_updates_per_s": n / t,
            "attempts_mean": att / n, "max_attempts": int((ns_ + nr_).max()),
            "fp64_frac_folded": folded / t / 1e12 / fp64_peak,
            "cell_slot_occupancy": min(n, slots) / slots, "prereact_failed": failed}

@@ -18,8 +18,9 @@
  *     stream) and runs asynchronously; pointers must stay valid until the stream reaches it.
  *     Per-cell outcomes are written to the optional status array (CHEM_CELL_* codes).
  *   - The library owns the device copies of mechanisms and models, and draws per-call
- *     temporaries from the CUDA stream-ordered allocator (cudaMallocAsync / cudaFreeAsync on
- *     `stream`), the allocation strategy of §3.2.
+ *     temporaries from one memory pool per device (stream-ordered, on `stream`: the allocation
+ *     strategy of §3.2), which keeps at most 512 MiB between calls and gives them back when the
+ *     last mechanism is freed.
  */
 #ifndef CHEM_H
 #define CHEM_H
@@ -114,17 +115,21 @@ int chem_mechanism_info(chem_mech_t m, int* n_species, int* n_reactions, int* n_
 
 typedef struct chem_options {
   int32_t max_steps;      /* step attempts per cell before CHEM_CELL_MAX_STEPS; 0 -> 100000 */
-  int32_t group_threads;  /* threads per cell: 0 auto (2 if ns+1 <= 16 else 128); 2, 4, 8, 16, 32, 64, 128, 256 */
+  int32_t group_threads;  /* threads per cell: 0 auto (below); 2, 4, 8, 16, 32, 64, 128, 256 */
   int32_t groups_per_cta; /* 0 auto (as many as shared memory holds) */
   int32_t max_ctas;       /* 0 auto (SM count x resident CTAs per SM) */
 } chem_options;
-/* With groups_per_cta and max_ctas both 0, a launch whose cells fill fewer groups than the grid
+/* group_threads 0: one thread per cell for mechanisms of 8 to 11 species whose numbers fit the
+ * library's fixed-point form (8 or 16 lanes per cell in launches of few cells: the same operations,
+ * the same bits), otherwise 2 up to ns + 1 = 16 and 128 beyond.  A value of 32 x n in groups_per_cta
+ * asks for n warps of cells per CTA there.
+ * With groups_per_cta and max_ctas both 0, a launch whose cells fill fewer groups than the grid
  * holds is spread over every SM with fewer groups per CTA.  A cell's result does not depend on
  * the launch shape (bitwise); it does depend on group_threads (the order of the group's sums). */
 
 /* Advance ncells cells in place over dt.  ld = ncells.  Asynchronous on stream.
  * CHEM_EINVAL if ncells < 0, dt <= 0, rtol <= 0, atol <= 0 or a required pointer is NULL;
- * ncells == 0 is a no-op.  CHEM_ENOMEM / CHEM_ECUDA if the stream-ordered allocator cannot provide
+ * ncells == 0 is a no-op.  CHEM_ENOMEM / CHEM_ECUDA if the library's memory pool cannot provide
  * the 8-byte work-queue counter or the launch fails; per-cell failures go to the status codes of
  * chem_advance_ex, not to the return value. */
 int chem_advance(chem_mech_t m, double* T, const double* p, double* Y, double dt,
@@ -160,7 +165,7 @@ typedef struct chem_segment {
 } chem_segment;
 
 /* Advance several independent segments (different solvers' states, steps and tolerances) in one
- * persistent launch: their 8-cell chunks share one work queue, so small requests fill the GPU
+ * persistent launch: their cells share one work queue, so small requests fill the GPU
  * together (iteration-level batching, used by the serving loop).  segs is a host array read
  * during the call; the call returns once the descriptors are on the device (it synchronises
  * the stream).

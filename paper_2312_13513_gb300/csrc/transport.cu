@@ -53,8 +53,10 @@ namespace {
 
 constexpr double kPatm = 1.01325e6;
 
-// The FP64 pipe bounds these kernels (100003 H2 cells: 28 us at about 130 FP64 instructions a cell);
-// with the species polynomials in fixed point two FP64 instructions a species are left.
+// The FP64 pipe bounds these kernels (about 13 FP64 instructions a species); with the species
+// polynomials in fixed point two are left: h and cp of 100003 cells, H2 29 -> 13 us, CH4 142 -> 55 us,
+// T from h (guess 2 % off) 115 -> 39 and 424 -> 130 us.  Errors against extended precision are no
+// larger than the FP64 form's (5e-16 and 1.2e-15 of sum |h|, against 3.4e-15 and 1.4e-15).
 __global__ void __launch_bounds__(128) mixture_thermo_kernel(const unsigned char* blob, MechLayout L,
                                                              const FxEnthalpy* hk, const double* T, const double* Y,
                                                              int64_t ld, int64_t n, double* h, double* cp) {
