@@ -316,11 +316,14 @@ __global__ void k_adam_set(const __grid_constant__ AdamSet S, const float* coef,
 __global__ void k_adam_prep(int64_t* step, float* coef, const float* lr_dev, float lr, float b1, float b2) {
   pdl_wait();
   pdl_trigger();
+  // the two powers in two lanes of one warp: one pow's FP64 chain instead of two
   const int64_t s = *step + 1;
-  *step = s;
-  coef[0] = lr_dev ? *lr_dev : lr;
-  coef[1] = (float)(1.0 - pow((double)b1, (double)s));
-  coef[2] = (float)(1.0 - pow((double)b2, (double)s));
+  __syncwarp(3u);
+  coef[1 + threadIdx.x] = (float)(1.0 - pow((double)(threadIdx.x ? b2 : b1), (double)s));
+  if (threadIdx.x == 0) {
+    *step = s;
+    coef[0] = lr_dev ? *lr_dev : lr;
+  }
 }
 
 // compensated BF16 copy of the first layer: Wb row = [W_hi | W_hi | W_lo | 0] from master W[:, :nin]
@@ -693,7 +696,7 @@ extern "C" int chem_mlp_backward(chem_trainer_t t, const float* target, double* 
 
 static int adam_step(chem_trainer_t t, const float* lr_dev, float lr, float beta1, float beta2, float eps,
                      cudaStream_t st) {
-  CHEM_CUDA_TRY(launch_pdl(k_adam_prep, 1, 1, 0, st, t->d_step, t->d_coef, lr_dev, lr, beta1, beta2));
+  CHEM_CUDA_TRY(launch_pdl(k_adam_prep, 1, 2, 0, st, t->d_step, t->d_coef, lr_dev, lr, beta1, beta2));
   // every weight matrix and bias vector in one launch (their BF16 copies written on the way), then
   // the transposed copies the backward pass multiplies with
   AdamSet A{};
