@@ -794,6 +794,7 @@ int build(const chem_mech_desc* din, chem_mech_s* m) {
   }
   const std::vector<unsigned char> fxb = build_fx(d, m, fxn, nu, &m->fx);
   CHEM_CUDA_TRY(cudaGetDevice(&m->device));
+  device_pool();                       // made here: the first call may be under stream capture
   {
     const int rc = build_gx(d, m, fxn, nu, L, B);
     if (rc) return rc;

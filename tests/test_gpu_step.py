@@ -94,3 +94,25 @@ def test_step_rejects_bad_descriptions(h2):
     tr = cg.Transport(dm, generate_transport(h2))
     with pytest.raises(cg.ChemError):
         cg.Step(dm, T, p, Y, DT, h0=h0, transport=tr)    # transport without an output
+
+
+def test_first_call_of_a_process_may_be_a_capture():
+    """A step captured before any other call of the process (nothing is set up lazily inside the
+    capture that a capture does not allow)."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    code = """
+import torch, paper_2312_13513_gb300 as cg
+from synth.mechanism import h2_mechanism
+from synth.states import load_table, quasi_dns_field
+f = quasi_dns_field(load_table("h2_flamelet.npz"), n=3001, seed=3)
+m = cg.Mechanism(h2_mechanism())
+d = lambda a: torch.tensor(a, dtype=torch.float64, device="cuda")
+T, p, Y = d(f["T"]), d(f["p"]), d(f["Y"])
+cg.Step(m, T, p, Y, 5e-7).run(graph=True)
+torch.cuda.synchronize()
+"""
+    r = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
