@@ -15,14 +15,17 @@
 //     matrix-vector products with constant matrices: 3 FP64 instructions a pair instead of 5 (all
 //     terms have one sign for non-negative X, nothing cancels);
 //   - small mechanisms (ns <= 15) take one thread per cell, with the cell's vectors in a warp's
-//     interleaved shared memory (conflict-free, no shuffles, no idle lanes); larger ones a warp per
-//     cell, lanes over species and pairs.
+//     interleaved shared memory (conflict-free, no shuffles, no idle lanes); a binary coefficient
+//     joins both species' sums when it is made, so that 45 values a cell are stored instead of 72
+//     and up to sixteen warps share an SM (100003 H2 cells 170 -> 131 us, 2^20 1395 -> 1122 us);
+//     larger mechanisms take a warp per cell, lanes over species and pairs.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
 
 #include <algorithm>
 #include <cmath>
+#include <limits>
 #include <vector>
 
 #include "chem_internal.h"
@@ -199,7 +202,7 @@ __device__ __forceinline__ double mixture_d(const TrParams& P, double dsum, doub
 
 // One thread per cell (ns <= 15).  Shared memory: exp2 table, the fits and Wilke's constants (read
 // by warp-uniform addresses), then per warp the cells' vectors, element e of a lane at e * 32.
-__global__ void __launch_bounds__(256, 1) transport_cell_kernel(const TrParams P) {
+__global__ void __launch_bounds__(512, 1) transport_cell_kernel(const TrParams P) {
   extern __shared__ __align__(16) double tsm[];
   const int ns = P.ns, npair = ns * (ns - 1) / 2;
   fx::u64* e2 = (fx::u64*)tsm;
@@ -215,11 +218,11 @@ __global__ void __launch_bounds__(256, 1) transport_cell_kernel(const TrParams P
   for (int i = threadIdx.x; i < ns; i += blockDim.x) invW[i] = P.invW[i];
   __syncthreads();
   const int lane = threadIdx.x & 31;
-  double* X = invW + ns + (ns & 1) + (size_t)(threadIdx.x >> 5) * (4 * ns + npair) * 32 + lane;   // mole fractions
+  double* X = invW + ns + (ns & 1) + (size_t)(threadIdx.x >> 5) * 5 * ns * 32 + lane;   // mole fractions
   double* X1 = X + ns * 32;                  // X / s
   double* X2 = X1 + ns * 32;                 // X / s^2
   double* s = X2 + ns * 32;                  // mu_k^(1/2)
-  double* E = s + ns * 32;                   // 1 / D_jk(p_atm) per unordered pair
+  double* Ds = s + ns * 32;                  // sum_j X_j / D_jk(p_atm)
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < P.n; c += (int64_t)gridDim.x * blockDim.x) {
     const double T = P.T[c];
     const FitT t = fit_t(T, P);
@@ -246,14 +249,28 @@ __global__ void __launch_bounds__(256, 1) transport_cell_kernel(const TrParams P
       lxi = fma(x, il, lxi);
     }
     if (P.Dm) {
-      if (t.fast) {
+      // the unordered pairs row by row: a coefficient joins both species' sums at once, so that a sum
+      // per species is stored instead of a coefficient per pair
+      for (int k = 0; k < ns; ++k) Ds[k * 32] = 0.0;
+      int q = 0;
+      for (int j = 0; j < ns; ++j) {
+        const double xj = X[j * 32];
+        double sum = Ds[j * 32];
+        if (t.fast) {
 #pragma unroll 4
-        for (int q = 0; q < npair; ++q) E[q * 32] = exp2_any(fit_x(diff_fx + 4 * q, t), e2);
-      } else {
-        for (int q = 0; q < npair; ++q) {
-          const int jk = __ldg(P.pairs + q);
-          E[q * 32] = exp(-poly3(P.diff_poly + 4 * ((jk & 0xffff) * ns + (jk >> 16)), t.lnT));
+          for (int k = j + 1; k < ns; ++k, ++q) {
+            const double e = exp2_any(fit_x(diff_fx + 4 * q, t), e2);       // 1 / D_jk(p_atm)
+            sum = fma(X[k * 32], e, sum);
+            Ds[k * 32] = fma(xj, e, Ds[k * 32]);
+          }
+        } else {
+          for (int k = j + 1; k < ns; ++k) {
+            const double e = exp(-poly3(P.diff_poly + 4 * (j * ns + k), t.lnT));
+            sum = fma(X[k * 32], e, sum);
+            Ds[k * 32] = fma(xj, e, Ds[k * 32]);
+          }
         }
+        P.Dm[(int64_t)j * P.ld + c] = mixture_d(P, sum, P.Y[(int64_t)j * P.ld + c], pr, T, j);
       }
     }
     double num = 0.0;
@@ -269,13 +286,6 @@ __global__ void __launch_bounds__(256, 1) transport_cell_kernel(const TrParams P
         const double sk = s[k * 32];
         const double den = fma(sk, fma(sk, d, b + b), a);
         num = fma(X[k * 32] * sk, sk * fx::rcp(den), num);
-      }
-      if (P.Dm) {
-        double dsum = 0.0;
-        for (int j = 0; j < k; ++j) dsum = fma(X[j * 32], E[pair_index(j, k, ns) * 32], dsum);
-#pragma unroll 3
-        for (int j = k + 1; j < ns; ++j) dsum = fma(X[j * 32], E[pair_index(k, j, ns) * 32], dsum);
-        P.Dm[(int64_t)k * P.ld + c] = mixture_d(P, dsum, P.Y[(int64_t)k * P.ld + c], pr, T, k);
       }
     }
     if (P.mu) P.mu[c] = num;
@@ -514,12 +524,21 @@ extern "C" int chem_transport_eval(chem_transport_t t, const double* T, const do
   CHEM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   constexpr size_t kSmem = 200 * 1024;
   if (ns <= 15) {
-    // as many warps as an SM's shared memory holds, up to eight (two per sub-partition: one warp's
-    // integer work runs beside the other's FP64); fewer where that leaves SMs without a warp
+    // Whole warps per sub-partition, 4 to 16 an SM as far as shared memory goes, more of them overlap one
+    // warp's integer work with the others' FP64 (100003 H2 cells: a pass of the grid takes 43, 49 and
+    // 80 us with up to 4, 8 and 16), but the last pass may be nearly empty: the number with the least
+    // passes times their length, max(11, warps + 4) units of 4 us.
     const size_t fixed = (256 + 8 * (size_t)ns + 4 * npair + 3 * (size_t)ns * ns + ns + (ns & 1)) * 8;
-    const size_t per = (size_t)(4 * ns + npair) * 256;
+    const size_t per = (size_t)5 * ns * 256;
     const int64_t need = (ncells + 31) / 32;
-    const int warps = (int)std::max<int64_t>(1, std::min<int64_t>({8, (int64_t)((kSmem - fixed) / per), (need + sms - 1) / sms}));
+    const int64_t fit = std::max<int64_t>(1, (int64_t)((kSmem - fixed) / per));
+    int64_t best = std::numeric_limits<int64_t>::max();
+    int warps = 1;
+    for (int64_t w : {16, 12, 8, 4}) {
+      w = std::min<int64_t>({w, fit, (need + sms - 1) / sms});
+      const int64_t cost = ((need + sms * w - 1) / (sms * w)) * std::max<int64_t>(11, w + 4);
+      if (cost < best) { best = cost; warps = (int)w; }
+    }
     const size_t smem = fixed + per * warps;
     CHEM_CUDA_TRY(cudaFuncSetAttribute(transport_cell_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const unsigned grid = (unsigned)std::min<int64_t>((need + warps - 1) / warps, sms);

@@ -111,7 +111,7 @@ f = quasi_dns_field(load_table("h2_flamelet.npz"), n=3001, seed=3)
 m = cg.Mechanism(h2_mechanism())
 d = lambda a: torch.tensor(a, dtype=torch.float64, device="cuda")
 T, p, Y = d(f["T"]), d(f["p"]), d(f["Y"])
-cg.Step(m, T, p, Y, 5e-7).run(graph=True)
+cg.Step(m, T, p, Y, 5e-7, h0=torch.empty_like(T)).run(graph=True)
 torch.cuda.synchronize()
 """
     r = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
