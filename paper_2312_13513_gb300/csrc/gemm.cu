@@ -337,10 +337,10 @@ static int gemm_launch(const void* A, int64_t lda, const void* B, int64_t ldb, f
     CHEM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   }
   // Tile width.  Operand traffic from L2 bounds the large products (65536 x 800 x 1600 on 128-wide
-  // tiles: 10 TB/s, 203 us = 826 TFLOP/s; on 208-wide ones 136 us = 1234 TFLOP/s), and a row block's traffic is its tile count times the rows of A
-  // and B that a tile reads: the width of 256, 208, 160 or 128 that needs the least (800 and 400
-  // columns: 208, four and two tiles).  128 where wider tiles would leave SMs without one (small
-  // products: more, smaller tiles finish sooner).
+  // tiles: 10 TB/s, 203 us = 826 TFLOP/s; on 208-wide ones 136 us = 1234 TFLOP/s), and a row block's
+  // traffic is its tile count times the rows of A and B that a tile reads: the width of 256, 208, 160
+  // or 128 that needs the least (800 and 400 columns: 208, four and two tiles).  128 where wider tiles
+  // would leave SMs without one (small products: more, smaller tiles finish sooner).
   int bn = 256;
   long long cost = -1;
   for (int w : {256, 208, 160, 128}) {
