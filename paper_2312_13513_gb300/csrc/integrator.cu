@@ -166,7 +166,8 @@ inline WsLayout make_ws(int ns, int nr, int npieces, int G, bool fx, int ntb) {
   // solve's scratch and the new state share its storage
   w.y = take(N); w.f0 = take(N); w.ys = take(N); w.ynew = w.ys; w.tmp = w.ys; w.fs = take(N);
   w.u = take(6 * N); w.M = take(N * w.LD); w.invd = take(N);
-  w.C = take(ns + 1); w.hRT = take(ns); w.gRT = take(ns + 1); w.cpR = take(ns);
+  // the fixed-point form's empty slot is species ns: concentration 1, no Gibbs energy, no enthalpy
+  w.C = take(ns + 1); w.hRT = take(fx ? ns + 1 : ns); w.gRT = take(ns + 1); w.cpR = take(ns);
   w.wdot = take(ns); w.dwdT = take(ns); w.rk = take(ns); w.Hm = take(ns);
   // dq/dT per reaction is only needed inside a Jacobian evaluation, before the assembly writes the
   // matrix buffer (whose previous content, the last LU, is dead by then): it borrows that buffer
@@ -786,8 +787,9 @@ __device__ __forceinline__ void eval_fx(const Grp<G>& g, const GxView& m, const 
     invrho = fx::rcp(rho);
     if (g.tid == 0) {
       w.sc[S_S] = S; w.sc[S_CP] = cp; w.sc[S_DCP] = dcp; w.sc[S_RHO] = rho; w.sc[S_INVRHO] = invrho;
-      w.C[ns] = 1.0;                                        // the empty slot
+      w.C[ns] = 1.0;                                        // the empty slot, which any place may hold
       w.gRT[ns] = 0.0;
+      w.hRT[ns] = 0.0;
     }
   }
   g.sync();
@@ -848,7 +850,7 @@ __device__ __forceinline__ void eval_fx(const Grp<G>& g, const GxView& m, const 
     }
     const double fwd = kf * Pf, rev = kr * Pr, net = fwd - rev;
     const double mult = ri.x == 1 ? Mc : 1.0;
-    double dH = (w.hRT[pr.x] - w.hRT[re.x]) - (double)ri.y;
+    double dH = (w.hRT[pr.x] - w.hRT[re.x]) - (double)ri.y;      // slot x alone reads an empty slot's 0
     if (pr.y != ns) dH += w.hRT[pr.y];
     if (pr.z != ns) dH += w.hRT[pr.z];
     if (re.y != ns) dH -= w.hRT[re.y];

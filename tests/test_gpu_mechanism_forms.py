@@ -1,0 +1,62 @@
+"""Forms of mechanism that the loader accepts and that the synthetic mechanisms do not have, in every
+integrator kernel, against the oracle."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle  # noqa: E402
+import paper_2312_13513_gb300 as cg  # noqa: E402
+
+from gpu_common import assert_parity, to_dev  # noqa: E402
+from helpers import random_states, with_inert_species  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+def _states(base, m, n, seed, fuel):
+    """Seeded states of the base mechanism, with a little of every species appended to it."""
+    T, p, Y = random_states(base, n, seed, fuel, Tlo=300.0, Thi=2600.0)
+    Y = np.vstack([Y, np.full((m.ns - base.ns, n), 1e-3)])
+    return T, p, Y / Y.sum(axis=0)
+
+
+def _assert_rhs_jac(m, T, p, Y):
+    """f and the Jacobian against the oracle: 1e-10 of each rate and of each column's largest entry (the
+    sums of up to a few hundred terms, each good to about 1e-13), as in test_rhs_and_jacobian_parity."""
+    om, N = oracle.OracleMech(m), m.ns + 1
+    f, J = (a.cpu().numpy() for a in cg.eval_rhs_jac(cg.Mechanism(m), *to_dev(T, p, Y)))
+    for c in range(T.size):
+        y = np.r_[T[c], Y[:, c]]
+        fr, Jr = om.rhs(p[c], y), om.jacobian(p[c], y)
+        assert np.all(np.abs(f[:, c] - fr) <= 1e-10 * (np.abs(fr) + 1e-12 * np.max(np.abs(fr))) + 1e-300), (c, T[c])
+        sc = np.max(np.abs(Jr), axis=0) + 1e-300
+        assert np.all(np.abs(J[:, c].reshape(N, N) - Jr) <= 1e-10 * sc), (c, T[c])
+
+
+def _assert_advance(m, T, p, Y, dt, group):
+    Td, pd, Yd = to_dev(T, p, Y)
+    st = torch.full((T.size,), -1, dtype=torch.int8, device="cuda")
+    cg.advance(cg.Mechanism(m), Td, pd, Yd, dt, status=st, opts=cg.options(group_threads=group) if group else None)
+    assert torch.all(st == 0)
+    assert_parity(oracle.OracleMech(m), T, p, Y, Td.cpu().numpy(), Yd.cpu().numpy(), dt, 1e-6, 1e-10)
+
+
+def _shuffled_slots(m, seed):
+    """The same reactions with the species of each side in any of its three places."""
+    m = m.copy()
+    rng = np.random.default_rng(seed)
+    m.reac, m.prod = rng.permuted(m.reac, axis=1), rng.permuted(m.prod, axis=1)
+    return m
+
+
+@pytest.mark.parametrize("base,inert", [("h2", 0), ("h2", 7), ("ch4", 0), ("ch4", 1), ("ch4", 12)])
+def test_empty_slots_in_any_place(base, inert, request):
+    """An empty slot before a species: odd and even species counts, each integrator kernel."""
+    b = request.getfixturevalue(base)
+    m = _shuffled_slots(with_inert_species(b, inert) if inert else b, 70 + inert)
+    assert np.any(m.reac[:, 0] < 0) and np.any(m.prod[:, 0] < 0)
+    T, p, Y = _states(b, m, 37, 71 + inert, base.upper())
+    _assert_rhs_jac(m, T, p, Y)
+    for group in (0, 64):
+        _assert_advance(m, T, p, Y, 5e-7, group)
