@@ -120,7 +120,7 @@ struct GxLayout {
 constexpr int kGxLanes = 128;
 constexpr int kGxUnroll = 4;                               // term rows are a multiple of this
 struct GxJac {
-  int nslot = 0, npart = 0;                                // term rows
+  int nslot = 0, npart = 0;                                // term rows; of the first kind kGxUnroll at least
   const int4* slot = nullptr;
   const int2* part = nullptr;
   const double* part_coef = nullptr;

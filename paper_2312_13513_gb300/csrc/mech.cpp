@@ -555,8 +555,10 @@ int build_gx(const chem_mech_desc* d, chem_mech_s* m, const FxNumbers& F, const 
       if (npt && !E.part.empty()) pt[p0 + (npt - 1) * kGxLanes + (e - e0)].y = pos;
     }
   }
+  // whole units of rows, and at least one of slots, which the kernel reads ahead unconditionally (no
+  // entries: no reactions, or none with a net production)
   const size_t unit = (size_t)kGxLanes * kGxUnroll;
-  ss.resize((ss.size() + unit - 1) / unit * unit, int4{(2 * nr) << 1, ns | (ns << 16), -1, 0});
+  ss.resize(std::max<size_t>(1, (ss.size() + unit - 1) / unit) * unit, int4{(2 * nr) << 1, ns | (ns << 16), -1, 0});
   pt.resize((pt.size() + unit - 1) / unit * unit, int2{0, -1});
   pc.resize(pt.size(), 0.0);
   for (int k = 0; k < ns; ++k) { rs.insert(rs.end(), rows[k].begin(), rows[k].end()); ro.push_back((int)rs.size()); }

@@ -60,3 +60,33 @@ def test_empty_slots_in_any_place(base, inert, request):
     _assert_rhs_jac(m, T, p, Y)
     for group in (0, 64):
         _assert_advance(m, T, p, Y, 5e-7, group)
+
+
+def _without_reactions(m):
+    m = m.copy()
+    for a in ("rtype", "reac", "prod", "A", "b", "Ea", "troe", "has_t2", "eff"):
+        setattr(m, a, getattr(m, a)[:0].copy())
+    return m
+
+
+@pytest.mark.parametrize("form", ["none", "no net production"])
+@pytest.mark.parametrize("base,inert", [("h2", 0), ("h2", 7), ("ch4", 0)])
+def test_mechanism_that_changes_nothing(base, inert, form, request):
+    """No reactions at all, or none with a net production: no entry in the Jacobian's programs.  Every
+    rate is an exact zero, so the state comes back as it was."""
+    b = request.getfixturevalue(base)
+    m = with_inert_species(b, inert) if inert else b.copy()
+    if form == "none":
+        m = _without_reactions(m)
+    else:
+        m.prod = m.reac.copy()
+    T, p, Y = _states(b, m, 19, 72, base.upper())
+    dm = cg.Mechanism(m)
+    f, J = cg.eval_rhs_jac(dm, *to_dev(T, p, Y))
+    assert torch.all(f == 0.0) and torch.all(J == 0.0)
+    for group in (0, 64):
+        Td, pd, Yd = to_dev(T, p, Y)
+        st = torch.full((T.size,), -1, dtype=torch.int8, device="cuda")
+        cg.advance(dm, Td, pd, Yd, 1e-6, status=st, opts=cg.options(group_threads=group) if group else None)
+        assert torch.all(st == 0)
+        assert np.array_equal(Td.cpu().numpy(), T) and np.array_equal(Yd.cpu().numpy(), Y)
