@@ -1809,6 +1809,8 @@ struct LaunchShape {
   int G, groups, threads;    // G = 1: one thread per cell (integrator_cell.cu)
   bool fx;                   // the fixed-point form
   size_t smem;
+  int smem_max;              // what a block may have: the kernels' attribute (state of the function, so
+                             // a size of one call could fall under another thread's launch)
   WsLayout ws;
 };
 
@@ -1850,6 +1852,7 @@ int pick_shape(const chem_mech_s* m, const chem_options* opt, LaunchShape* s) {
   s->groups = groups;
   s->threads = G * groups;
   s->smem = fixed + per_group * groups;
+  s->smem_max = smem_max;
   return CHEM_OK;
 }
 
@@ -1857,7 +1860,7 @@ template <int G, bool FX = false>
 int launch_adv_t(const LaunchShape& s, const AdvanceParams& P, const chem_options* opt,
                  cudaStream_t stream) {
   CHEM_CUDA_TRY(cudaFuncSetAttribute((advance_kernel<G, FX>), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)s.smem));
+                                     s.smem_max));
   int dev = 0, sms = 0, per_sm = 0;
   CHEM_CUDA_TRY(cudaGetDevice(&dev));
   CHEM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -1891,7 +1894,7 @@ int launch_adv_t(const LaunchShape& s, const AdvanceParams& P, const chem_option
 template <int G, bool FX = false>
 int launch_eval_t(const LaunchShape& s, const EvalParams& P, cudaStream_t stream) {
   CHEM_CUDA_TRY(cudaFuncSetAttribute((eval_kernel<G, FX>), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)s.smem));
+                                     s.smem_max));
   int64_t grid = (P.ncells + s.groups - 1) / s.groups;
   grid = std::min<int64_t>(grid, 65535);
   eval_kernel<G, FX><<<(unsigned)grid, s.threads, s.smem, stream>>>(P);

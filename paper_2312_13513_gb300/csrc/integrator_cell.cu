@@ -323,7 +323,9 @@ __global__ void __launch_bounds__(128, 1) cell_eval_kernel(const __grid_constant
 }
 
 struct Shape {
-  int warps, sms, smem_max;
+  int warps, sms;
+  int smem_max;         // of a block, and the kernels' attribute whatever a launch takes: it is state of the
+                        // function, and another thread may launch one of another size meanwhile
   size_t smem;          // of `warps` warps
 };
 
@@ -351,7 +353,7 @@ int advance_t(const chem_mech_s* m, const QueueParams& Q, bool scratch, const ch
   int rc = shape_of<NS>(m, &s);
   if (rc) return rc;
   if (s.warps < 1) { set_error("mechanism too large for shared memory"); return CHEM_EINVAL; }
-  CHEM_CUDA_TRY(cudaFuncSetAttribute((cell_advance_kernel<NS, false>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem));
+  CHEM_CUDA_TRY(cudaFuncSetAttribute((cell_advance_kernel<NS, false>), cudaFuncAttributeMaxDynamicSharedMemorySize, s.smem_max));
   const size_t per = (size_t)Ws<NS>::TOTAL * 256;
   int warps = s.warps;
   if (opt && opt->groups_per_cta > 0) warps = std::min(warps, (opt->groups_per_cta + 31) / 32);
@@ -373,7 +375,7 @@ int advance_t(const chem_mech_s* m, const QueueParams& Q, bool scratch, const ch
     const size_t wide = (size_t)m->fx.bytes + kVec * (size_t)ww;
     if (ws_alloc((void**)&P.mx, kMat * (size_t)ww * (size_t)grid, stream) == cudaSuccess) {
       cudaError_t e = cudaFuncSetAttribute((cell_advance_kernel<NS, true>), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)wide);
+                                           s.smem_max);
       if (e == cudaSuccess) {
         cell_advance_kernel<NS, true><<<(unsigned)grid, 32 * ww, wide, stream>>>(P);
         e = cudaGetLastError();
@@ -396,7 +398,7 @@ int eval_t(const chem_mech_s* m, const double* T, const double* p, const double*
   Shape s;
   int rc = shape_of<NS>(m, &s);
   if (rc) return rc;
-  CHEM_CUDA_TRY(cudaFuncSetAttribute(cell_eval_kernel<NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem));
+  CHEM_CUDA_TRY(cudaFuncSetAttribute(cell_eval_kernel<NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, s.smem_max));
   CellEvalParams P;
   P.fx = m->fx; P.lay = m->lay; P.fxblob = (const unsigned char*)m->d_fx; P.blob = (const unsigned char*)m->d_blob;
   P.T = T; P.p = p; P.Y = Y; P.ld = ld; P.ncells = n; P.f = f; P.J = J;

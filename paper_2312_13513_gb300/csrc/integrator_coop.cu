@@ -593,8 +593,7 @@ int advance_t(const chem_mech_s* m, const QueueParams& Q, int sms, int smem_max,
   const int64_t need = std::max<int64_t>(1, (Q.total_chunks + 32 / L - 1) / (32 / L));
   warps = std::min<int64_t>(warps, (need + ctas - 1) / ctas);
   const int64_t grid = std::min<int64_t>(ctas, (need + warps - 1) / warps);
-  CHEM_CUDA_TRY(cudaFuncSetAttribute((co_advance_kernel<NS, L>), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(fixed + per * 8 <= (size_t)smem_max ? fixed + per * 8 : smem_max)));
+  CHEM_CUDA_TRY(cudaFuncSetAttribute((co_advance_kernel<NS, L>), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
   co_advance_kernel<NS, L><<<(unsigned)grid, 32 * (unsigned)warps, fixed + per * (size_t)warps, stream>>>(P);
   CHEM_CUDA_TRY(cudaGetLastError());
   return CHEM_OK;

@@ -522,6 +522,8 @@ extern "C" int chem_transport_eval(chem_transport_t t, const double* T, const do
   int dev = 0, sms = 0;
   CHEM_CUDA_TRY(cudaGetDevice(&dev));
   CHEM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  // the kernels' limit, and their attribute whatever a launch takes: it is state of the function, and
+  // another thread may launch one of another size meanwhile
   constexpr size_t kSmem = 200 * 1024;
   if (ns <= 15) {
     // Whole warps per sub-partition, 4 to 16 an SM as far as shared memory goes, more of them overlap one
@@ -540,13 +542,13 @@ extern "C" int chem_transport_eval(chem_transport_t t, const double* T, const do
       if (cost < best) { best = cost; warps = (int)w; }
     }
     const size_t smem = fixed + per * warps;
-    CHEM_CUDA_TRY(cudaFuncSetAttribute(transport_cell_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CHEM_CUDA_TRY(cudaFuncSetAttribute(transport_cell_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem));
     const unsigned grid = (unsigned)std::min<int64_t>((need + warps - 1) / warps, sms);
     transport_cell_kernel<<<grid, 32 * warps, smem, (cudaStream_t)stream>>>(P);
   } else {
     const size_t smem = (256 + 8 * (size_t)(4 * ns + npair)) * sizeof(double);
     if (smem > kSmem) { set_error("mechanism too large for the transport kernel"); return CHEM_EINVAL; }
-    CHEM_CUDA_TRY(cudaFuncSetAttribute(transport_warp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CHEM_CUDA_TRY(cudaFuncSetAttribute(transport_warp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem));
     transport_warp_kernel<<<grid_cells(ncells, 8), 256, smem, (cudaStream_t)stream>>>(P);
   }
   CHEM_CUDA_TRY(cudaGetLastError());
