@@ -138,7 +138,8 @@ __device__ __forceinline__ GxView bind_gx(const unsigned char* s, const GxLayout
 // the workspace (slot indices into w.sc).
 enum : int {
   S_LNT, S_INVT, S_RHO, S_INVRHO, S_GSHIFT, S_EP1, S_IEP1, S_S, S_CP, S_DCP, S_Q, S_IRCP,
-  S_RS, S_QOR2R, S_RHS, S_CPS, S_J00, S_IG, S_INVH, S_EN, S_FAC, S_HR, S_L, S_IT, S_TAU, S_NSC
+  S_RS, S_QOR2R, S_RHS, S_CPS, S_J00, S_IG, S_INVH, S_EN, S_FAC, S_NSC,
+  S_HR = S_NSC, S_L, S_IT, S_TAU, S_NSC_FX        // of the fixed-point form alone
 };
 
 // per-group workspace layout (doubles unless noted); offsets in doubles.  The Jacobian is
@@ -167,7 +168,7 @@ inline WsLayout make_ws(int ns, int nr, int npieces, int G, bool fx, int ntb) {
   w.y = take(N); w.f0 = take(N); w.ys = take(N); w.ynew = w.ys; w.tmp = w.ys; w.fs = take(N);
   w.u = take(6 * N); w.M = take(N * w.LD); w.invd = take(N);
   // the fixed-point form's empty slot is species ns: concentration 1, no Gibbs energy, no enthalpy
-  w.C = take(ns + 1); w.hRT = take(fx ? ns + 1 : ns); w.gRT = take(ns + 1); w.cpR = take(ns);
+  w.C = take(ns + 1); w.hRT = take(fx ? ns + 1 : ns); w.gRT = take(fx ? ns + 1 : ns); w.cpR = take(ns);
   w.wdot = take(ns); w.dwdT = take(ns); w.rk = take(ns); w.Hm = take(ns);
   // dq/dT per reaction is only needed inside a Jacobian evaluation, before the assembly writes the
   // matrix buffer (whose previous content, the last LU, is dead by then): it borrows that buffer
@@ -183,7 +184,7 @@ inline WsLayout make_ws(int ns, int nr, int npieces, int G, bool fx, int ntb) {
   w.wpart = take(G > 32 ? npieces : 0); w.dwpart = take(G > 32 ? npieces : 0);
   // cross-warp reductions and shared scalars exist only for groups wider than a warp
   w.red = take(G > 32 ? 8 * (G / 32) + 8 : 0);
-  w.sc = take(G > 32 ? S_NSC : 0);
+  w.sc = take(G > 32 ? (fx ? S_NSC_FX : S_NSC) : 0);
   w.stage = take(chunk_cells(G) * (N + 1));
   w.ctl = take(2);
   w.perm = take((N + 1) / 2);      // ints
@@ -1828,17 +1829,22 @@ int pick_shape(const chem_mech_s* m, const chem_options* opt, LaunchShape* s) {
     return CHEM_EINVAL;
   }
   s->G = G;
-  // the fixed-point form has an instance for 128-thread groups, the large mechanisms' default; the
-  // other group sizes are a caller's option and keep the FP64 form
-  s->fx = G == 128 && m->gx.bytes > 0;
-  s->ws = make_ws(m->ns, m->nr, m->lay.npieces, G, s->fx, s->fx ? m->gx.ntb : 0);
   int dev = 0;
   CHEM_CUDA_TRY(cudaGetDevice(&dev));
   int smem_max = 0;
   CHEM_CUDA_TRY(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  const size_t per_group = (size_t)s->ws.total * 8;
-  const size_t fixed = (size_t)(s->fx ? m->gx.bytes : m->lay.bytes);
   const int unit = G < 32 ? 32 / G : 1;          // groups per warp: whole warps only
+  // The fixed-point form has an instance for 128-thread groups, the large mechanisms' default; the
+  // other group sizes are a caller's option and keep the FP64 form.  So does a mechanism of which not
+  // one group fits: its tables, its records and its workspace are up to a few KB larger.
+  size_t per_group = 0, fixed = 0;
+  for (int fx = G == 128 && m->gx.bytes > 0 ? 1 : 0; fx >= 0; --fx) {
+    s->fx = fx != 0;
+    s->ws = make_ws(m->ns, m->nr, m->lay.npieces, G, s->fx, s->fx ? m->gx.ntb : 0);
+    per_group = (size_t)s->ws.total * 8;
+    fixed = (size_t)(s->fx ? m->gx.bytes : m->lay.bytes);
+    if (fixed + per_group * unit <= (size_t)smem_max) break;
+  }
   int groups = (opt && opt->groups_per_cta) ? opt->groups_per_cta : max_threads(G) / G;
   groups = std::min(groups, max_threads(G) / G);
   if (G > 32) groups = std::min(groups, 15);     // named barriers 1..15

@@ -90,3 +90,17 @@ def test_mechanism_that_changes_nothing(base, inert, form, request):
         cg.advance(dm, Td, pd, Yd, 1e-6, status=st, opts=cg.options(group_threads=group) if group else None)
         assert torch.all(st == 0)
         assert np.array_equal(Td.cpu().numpy(), T) and np.array_equal(Yd.cpu().numpy(), Y)
+
+
+@pytest.mark.parametrize("ns", [139, 140, 141])
+def test_largest_mechanisms(h2, ns):
+    """Where one cell's workspace is all the shared memory of a block (227 KB): 139 species are the last
+    that fit in fixed point (16 bytes short), 140 the last that fit in FP64, 141 are refused."""
+    m = with_inert_species(h2, ns - h2.ns)
+    T, p, Y = _states(h2, m, 9, 73, "H2")
+    if ns > 140:
+        with pytest.raises(cg.ChemError):
+            cg.eval_rhs_jac(cg.Mechanism(m), *to_dev(T, p, Y))
+        return
+    _assert_rhs_jac(m, T, p, Y)
+    _assert_advance(m, T, p, Y, 5e-7, 0)
