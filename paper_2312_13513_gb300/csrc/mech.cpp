@@ -146,9 +146,9 @@ const uint32_t kRcpTab[128] = {CHEM_FX_RCP_VALUES};
 // The numbers of a mechanism in the fixed-point formats (fixed.cuh, fx_mech.h).  ok = false where a
 // species' polynomials leave them.  No polynomial can leave Q11.52 (its coefficients' magnitudes
 // sum to at most 2000), and every base-2 exponent that a kernel forms stays below 3074 in magnitude
-// (|log2 kf| <= 600 + 32 * 12 + 1900; |log2 kr| <= 1023 + 2000 by the bound on Delta G), so that a
-// wrapped sum is always recognised as out of range (exp2_in_range) and never mistaken for a small
-// one.
+// (|log2 kf| <= 600 + 32 * 12 + 1900; |log2 kr| <= 1023 + 2000 by the bound on Delta G;
+// |log2 k0 / kinf| <= 2050 + 1023, of a kinf in range, by a bound on k0 of its own), so that a wrapped
+// sum is always recognised as out of range (exp2_in_range) and never mistaken for a small one.
 struct FxNumbers {
   bool ok = true;
   std::vector<FxSpecies> sp;                       // [2][ns]
@@ -274,7 +274,8 @@ struct FxNumbers {
       bool fits = worst_dG(d, nu[j], dnu) <= 2000.0;
       if (d->rtype[j] == 2) {
         const double* t = d->troe + 7 * j;
-        fits = fits && in_formats(t[0], t[1], t[2]);
+        fits = fits && in_formats(t[0], t[1], t[2]) &&
+               std::fabs(std::log2(t[0])) + 12.0 * std::fabs(t[1]) + std::fabs(t[2]) / (RC * std::log(2.0) * fx::kTlo) <= 2050.0;
         FxTroe F{};
         rate(t[0], t[1], t[2], fits, &F.lnA0, &F.b0, &F.Ta0);
         F.b0d = t[1]; F.Ta0K = t[2] / RC;

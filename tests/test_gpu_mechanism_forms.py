@@ -104,3 +104,16 @@ def test_largest_mechanisms(h2, ns):
         return
     _assert_rhs_jac(m, T, p, Y)
     _assert_advance(m, T, p, Y, 5e-7, 0)
+
+
+@pytest.mark.parametrize("base", ["h2", "ch4"])
+def test_low_pressure_limit_far_below_the_other(base, request):
+    """k0 = 2^-2296 and kinf = 2^989 at 130 K: their ratio is beyond the range of a fixed-point exponent
+    by more than its width.  k0 is 0 in FP64, and so is the rate."""
+    b = request.getfixturevalue(base)
+    m = b.copy()
+    j = int(np.nonzero(m.rtype == 2)[0][0])
+    m.A[j], m.b[j], m.Ea[j] = 1e150, 0.0, -8.8e4
+    m.troe[j, :3] = 1e-170, 0.0, 3.1e5
+    T, p, Y = _states(b, m, 12, 74, base.upper())
+    _assert_rhs_jac(m, np.linspace(129.0, 133.0, T.size), p, Y)
