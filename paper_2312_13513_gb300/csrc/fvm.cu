@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(256) fvm_to_csr_kernel(int64_t nnz, const int3
 // square root take about 17
 __device__ __forceinline__ double sqrt_ratio(double a, double b) {
   const double x = a * b;
-  if (!((unsigned)__double2hiint(x) - 0x08000000u < 0x70000000u)) return sqrt(a / b);
+  if (!((unsigned)__double2hiint(x) - 0x08000000u < 0x70000000u) || __double2hiint(a) < 0) return sqrt(a / b);
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   const double e = fma(-x * y, y, 1.0);

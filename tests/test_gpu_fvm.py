@@ -140,3 +140,26 @@ def test_odd_array_offsets_change_nothing(shape):
     torch.cuda.synchronize()
     for a, b in zip(got, ref):
         assert torch.equal(a, b)
+
+
+def test_pasr_kappa_of_a_negative_density():
+    """A density that a solver undershot below zero makes both arguments of the mixing time's root
+    negative: the root is the positive one, as the definition (and numpy) has it."""
+    rng = np.random.default_rng(23)
+    n = 4097
+    tau_c = 10.0 ** rng.uniform(-7, -2, n)
+    rho = -rng.uniform(0.2, 1.5, n)
+    mu = rng.uniform(1e-5, 6e-5, n)
+    strain = 10.0 ** rng.uniform(1, 5, n)
+    delta = rng.uniform(2e-4, 2e-3, n)
+    with np.errstate(invalid="ignore"):
+        ref = fvm.pasr_kappa(tau_c, rho, mu, strain, delta, 0.17, 0.5)
+    assert np.any(np.isnan(ref)) and np.any(np.isfinite(ref))
+    k = cg.pasr_kappa(*(torch.tensor(a, device="cuda") for a in (tau_c, rho, mu, strain, delta)), c_s=0.17, c_mix=0.5)
+    # mu + rho nu cancels: a rounding of either term over the difference, halved by the root
+    nu = (0.17 * delta) ** 2 * strain
+    tol = 1e-14 + 2.3e-16 * (mu + np.abs(rho) * nu) / np.abs(mu + rho * nu)
+    got = k.cpu().numpy()
+    assert np.array_equal(np.isnan(got), np.isnan(ref))
+    f = np.isfinite(ref)
+    assert np.all(np.abs(got[f] - ref[f]) <= tol[f])
