@@ -163,3 +163,19 @@ def test_pasr_kappa_of_a_negative_density():
     assert np.array_equal(np.isnan(got), np.isnan(ref))
     f = np.isfinite(ref)
     assert np.all(np.abs(got[f] - ref[f]) <= tol[f])
+
+
+def test_pasr_kappa_is_never_above_one():
+    """Chemical times beside which the mixing time is nothing: kappa is 1, not a unit above it, whatever
+    the time's mantissa (those just below a power of two have the reciprocals with the largest errors)."""
+    rng = np.random.default_rng(24)
+    n = 1 << 20
+    m = 2.0 - np.where(np.arange(n) % 2 == 0, 2.0 ** -8, 1.0) * rng.uniform(0.0, 1.0, n)
+    tau_c = m * 2.0 ** rng.integers(60, 80, n)
+    tau_c[:4] = [1.7e308, 5e-324, np.inf, 1e300]
+    one = np.ones(n)
+    k = cg.pasr_kappa(*(torch.tensor(a, device="cuda") for a in (tau_c, one, 1e-5 * one, 1e3 * one, 1e-3 * one)))
+    got = k.cpu().numpy()
+    ref = fvm.pasr_kappa(tau_c[:4], one[:4], 1e-5 * one[:4], 1e3 * one[:4], 1e-3 * one[:4], 0.17, 1.0)
+    assert np.array_equal(np.isnan(got[:4]), np.isnan(ref)) and np.allclose(got[[0, 1, 3]], ref[[0, 1, 3]], rtol=1e-14, atol=1e-320)
+    assert np.all(got[4:] <= 1.0) and np.all(got[4:] >= 1.0 - 2.3e-16)
