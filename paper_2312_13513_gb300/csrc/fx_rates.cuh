@@ -65,7 +65,8 @@ __device__ __forceinline__ double step_factor(double en2, const u64* e2, const u
 // thermo state of a right-hand side at one temperature
 struct Temp {
   double T, invT;
-  u64 L, iT, tau;    // log2 T (Q4.60), 128 / T and T / 2^r (Q0.64)
+  u64 L, iT, tau;    // log2 T (Q4.60), 128 / T and T / 2^r (Q0.64); L and iT after slow_temp: the words of
+                     // the doubles ln T and 1 / T
   i64 L2, iT2, tau2; // halves of the three (biased products)
   int rg;
   bool fast;             // T in [kTlo, kThi): fixed point
@@ -89,6 +90,19 @@ __device__ __forceinline__ Temp temp_of(double T, const Ctx& m, bool need_inv) {
   return t;
 }
 
+// ln T and 1 / T for the FP64 forms of species and reactions.  slow_temp forms them once per right-hand
+// side for a temperature outside the range; the kernel of several lanes per cell, whose lanes have one
+// or two species and three reactions each, forms them there.
+static __device__ __noinline__ double2 ln_inv(double T) { return make_double2(log(T), 1.0 / T); }
+__device__ __forceinline__ void slow_temp(Temp& t) {
+  const double2 s = ln_inv(t.T);
+  t.L = (u64)__double_as_longlong(s.x);
+  t.iT = (u64)__double_as_longlong(s.y);
+}
+__device__ __forceinline__ double2 ln_inv_of(const Temp& t) {
+  return t.fast ? ln_inv(t.T) : make_double2(__longlong_as_double((i64)t.L), __longlong_as_double((i64)t.iT));
+}
+
 // g/RT of species k as a double (the G array holds Q11.52 / ln 2 in fast cells, doubles in others)
 __device__ __forceinline__ double g_of(double raw, bool fast) {
   return fast ? to_double(__double_as_longlong(raw), 52) * kLn2 : raw;
@@ -97,39 +111,48 @@ __device__ __forceinline__ double g_of(double raw, bool fast) {
 // Rate constants in FP64 for what the fixed-point path leaves out: cells whose temperature is
 // outside its range, reactions whose exponents are.  Reaction id of the FP64 form; G: the cell's
 // Gibbs energies, element k at k * stride.  kf (the high-pressure limit of a fall-off reaction),
-// 1 / Kc, and k0 of a fall-off reaction.
-static __device__ __noinline__ void slow_k(const Ctx& m, const double* G, int stride, int id, double T, bool fast, double* kf,
-                                    double* invKc, double* k0) {
+// 1 / Kc, and k0 of a fall-off reaction; li = ln T and 1 / T.  The exponentials run on the integer pipe
+// here too: 100003 H2 cells of 4100 to 5500 K take 718 ms (two lanes a cell: 745); with the library's,
+// and ln T and 1 / T formed for each reaction, 1016.
+static __device__ __noinline__ void slow_k(const Ctx& m, const double* G, int stride, int id, double2 li, bool fast,
+                                           double* kf, double* invKc, double* k0) {
   const MechLayout& L = *m.lay;
-  const double lnT = log(T), invT = 1.0 / T;
+  const double lnT = li.x, invT = li.y;
   const double* lnA = (const double*)(m.blob + L.o_lnA);
   const double* beta = (const double*)(m.blob + L.o_beta);
   const double* Ta = (const double*)(m.blob + L.o_Ta);
   const short4 re = ((const short4*)(m.blob + L.o_reac))[id], pr = ((const short4*)(m.blob + L.o_prod))[id];
   const short4 ri = ((const short4*)(m.blob + L.o_rinfo))[id];
-  *kf = exp(lnA[id] + beta[id] * lnT - Ta[id] * invT);
+  *kf = exp_any(lnA[id] + beta[id] * lnT - Ta[id] * invT, m.e2);
   if (ri.x == 2) {
     const double* tr = (const double*)(m.blob + L.o_troe) + 8 * ri.w;
-    *k0 = exp(tr[0] + tr[1] * lnT - tr[2] * invT);
+    *k0 = exp_any(tr[0] + tr[1] * lnT - tr[2] * invT, m.e2);
   }
-  auto g = [&](int k) { return k >= 0 ? g_of(G[k * stride], fast) : 0.0; };
-  const double dG = g(pr.x) + g(pr.y) + g(pr.z) - g(re.x) - g(re.y) - g(re.z);
-  const double* cst = (const double*)(m.blob + L.o_const);
-  *invKc = exp(dG - (double)ri.y * (cst[kC_LNPR0] - lnT));
+  double x = 0.0;                                   // Delta G / RT, empty slots skipped
+  if (pr.x >= 0) x = g_of(G[pr.x * stride], fast);
+  if (pr.y >= 0) x += g_of(G[pr.y * stride], fast);
+  if (pr.z >= 0) x += g_of(G[pr.z * stride], fast);
+  if (re.x >= 0) x -= g_of(G[re.x * stride], fast);
+  if (re.y >= 0) x -= g_of(G[re.y * stride], fast);
+  if (re.z >= 0) x -= g_of(G[re.z * stride], fast);
+  if (ri.y != 0) {
+    const double* cst = (const double*)(m.blob + L.o_const);
+    x = fma(cst[kC_NU + 8 + ri.y], lnT - cst[kC_LNPR0], x);
+  }
+  *invKc = exp_any(x, m.e2);
 }
 
 // Troe blending in FP64 from kinf, k0 and the collision-partner sum (the general form: any value
 // of the arguments): kf, d ln kf/dT and d kf/d[M]
-static __device__ __noinline__ void slow_troe(const FxTroe& t, double T, double kinf, double k0, double Mc, double dlnkinf,
-                                       double* kf, double* dlnkf, double* dkfdM) {
-  const double invT = 1.0 / T;
+static __device__ __noinline__ void slow_troe(const Ctx& m, const FxTroe& t, double T, double invT, double kinf, double k0,
+                                              double Mc, double dlnkinf, double* kf, double* dlnkf, double* dkfdM) {
   *kf = 0.0; *dlnkf = 0.0; *dkfdM = 0.0;
   if (kinf == 0.0 || k0 == 0.0) return;
-  const double e3 = exp(-T * t.iT3), e1 = exp(-T * t.iT1);
+  const double e3 = exp_any(-T * t.iT3, m.e2), e1 = exp_any(-T * t.iT1, m.e2);
   double Fc = (1.0 - t.a) * e3 + t.a * e1;
   double dFc = -(1.0 - t.a) * t.iT3 * e3 - t.a * t.iT1 * e1;
   if (t.has_t2 != 0.0) {
-    const double e2 = exp(-t.T2 * invT);
+    const double e2 = exp_any(-t.T2 * invT, m.e2);
     Fc += e2;
     dFc += t.T2 * invT * invT * e2;
   }
@@ -144,7 +167,7 @@ static __device__ __noinline__ void slow_troe(const FxTroe& t, double T, double 
   const double d = n - 0.14 * u;
   const double f1 = u / d;
   const double den = 1.0 + f1 * f1;
-  const double F = exp(2.302585092994046 * (L / den));
+  const double F = exp_any(2.302585092994046 * (L / den), m.e2);
   const double opr = 1.0 / (1.0 + Prr);
   *kf = kinf * (Prr * opr) * F;
   const double dGdlogPr = -2.0 * L * f1 / (den * den) * (n / (d * d));
@@ -213,18 +236,23 @@ __device__ __forceinline__ i64 exponent_f(const R& r, const Temp& t, i64 shift) 
   return r.lnA + (i64)(umulhi3(r.beta, t.L) - umulhi3(r.Ta, t.iT)) + shift;
 }
 
-// FP64 rate constants of a reaction that (or whose cell) is outside the fixed-point range; kf and kr
-// with the fall-off blending of Troe record t (nullable), d ln kf/dT, d kf/d[M] and 1 / Kc
+// FP64 rate constants of a reaction that (or whose cell) is outside the fixed-point range, li = ln T and
+// 1 / T; kf and kr with the fall-off blending of Troe record t (nullable), d ln kf/dT, d kf/d[M] and 1 / Kc
 static __device__ __noinline__ void slow_rate(const Ctx& m, const double* G, int stride, int id, const FxTroe* t, double T,
-                                       bool fast, double Mc, double* kf, double* kr, double* dlnkf, double* dkfdM,
-                                       double* invKc) {
+                                              double2 li, bool fast, double Mc, double* kf, double* kr, double* dlnkf,
+                                              double* dkfdM, double* invKc) {
   double k0 = 0.0;
-  slow_k(m, G, stride, id, T, fast, kf, invKc, &k0);
+  slow_k(m, G, stride, id, li, fast, kf, invKc, &k0);
   if (t) {
     const double kinf = *kf;
-    slow_troe(*t, T, kinf, k0, Mc, *dlnkf, kf, dlnkf, dkfdM);
+    slow_troe(m, *t, T, li.y, kinf, k0, Mc, *dlnkf, kf, dlnkf, dkfdM);
   }
   *kr = *kf * *invKc;
+}
+static __device__ __noinline__ void slow_rate(const Ctx& m, const double* G, int stride, int id, const FxTroe* t, double T,
+                                              bool fast, double Mc, double* kf, double* kr, double* dlnkf, double* dkfdM,
+                                              double* invKc) {
+  slow_rate(m, G, stride, id, t, T, ln_inv(T), fast, Mc, kf, kr, dlnkf, dkfdM, invKc);
 }
 
 }  // namespace fx

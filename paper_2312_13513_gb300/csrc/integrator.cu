@@ -705,7 +705,8 @@ __device__ __forceinline__ void eval_fx(const Grp<G>& g, const GxView& m, const 
   const int ns = m.ns, nr = m.nr;
   const double T = y[0];
   if (lead) {
-    const fx::Temp t = fx::temp_of(T, m, false);
+    fx::Temp t = fx::temp_of(T, m, false);
+    if (!t.fast) fx::slow_temp(t);
     if (g.tid == 0) {
       w.sc[S_L] = __longlong_as_double((long long)t.L);
       w.sc[S_IT] = __longlong_as_double((long long)t.iT);
@@ -722,7 +723,7 @@ __device__ __forceinline__ void eval_fx(const Grp<G>& g, const GxView& m, const 
   t.tau = (fx::u64)__double_as_longlong(w.sc[S_TAU]);
   t.L2 = (fx::i64)(t.L >> 1); t.iT2 = (fx::i64)(t.iT >> 1); t.tau2 = (fx::i64)(t.tau >> 1);
   t.invT = 0.0;
-  if (jac) t.invT = t.fast ? fx::to_double(t.iT2, 63 + fx::kTloExp) : 1.0 / T;
+  if (jac) t.invT = t.fast ? fx::to_double(t.iT2, 63 + fx::kTloExp) : __longlong_as_double((long long)t.iT);
 
   // species thermo (A2): g/RT (Q11.52 / ln 2 in fast cells), h/RT, cp/R
   double acc[3] = {0.0, 0.0, 0.0};
@@ -754,7 +755,8 @@ __device__ __forceinline__ void eval_fx(const Grp<G>& g, const GxView& m, const 
       }
     } else {
       const int rg = T < TMID ? 0 : 1;
-      const double lnT = log(T), invT = 1.0 / T;
+      const double2 li = fx::ln_inv_of(t);
+      const double lnT = li.x, invT = li.y;
       const double* hc = (const double*)(m.blob + m.lay->o_hc) + (rg * ns + k) * 6;
       const double* sc = (const double*)(m.blob + m.lay->o_sc) + (rg * ns + k) * 6;
       const double* cc = (const double*)(m.blob + m.lay->o_cpc) + (rg * ns + k) * 5;
@@ -836,12 +838,11 @@ __device__ __forceinline__ void eval_fx(const Grp<G>& g, const GxView& m, const 
     }
     if (!fastk) {
       if (jac) {                                            // the derivative from the FP64 constants
-        const double invT = 1.0 / T;
-        dlnkf = ((const double*)(m.blob + m.lay->o_beta))[j] * invT +
-                ((const double*)(m.blob + m.lay->o_Ta))[j] * invT * invT;
+        dlnkf = ((const double*)(m.blob + m.lay->o_beta))[j] * t.invT +
+                ((const double*)(m.blob + m.lay->o_Ta))[j] * t.invT * t.invT;
       }
-      fx::slow_rate(m, w.gRT, 1, j, ri.x == 2 ? m.troe + ri.w : nullptr, T, t.fast, Mc, &kf, &kr, &dlnkf, &dkfdM,
-                    &invKc);
+      fx::slow_rate(m, w.gRT, 1, j, ri.x == 2 ? m.troe + ri.w : nullptr, T, fx::ln_inv_of(t), t.fast, Mc, &kf,
+                    &kr, &dlnkf, &dkfdM, &invKc);
     }
     if (!jac) {
       double q = fma(kf, Pf, -(kr * Pr));

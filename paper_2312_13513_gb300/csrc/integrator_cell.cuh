@@ -35,6 +35,7 @@ namespace cell {
 
 using fx::exponent_f;
 using fx::rcp;
+using fx::slow_temp;
 using fx::Temp;
 using fx::temp_of;
 using fx::troe_fast;
@@ -90,10 +91,10 @@ __device__ __forceinline__ View bind(const unsigned char* s, const FxLayout& L, 
 struct Species64 {
   double g, h, cp, dcp;
 };
-static __device__ __noinline__ Species64 species64(const View& m, int ns, int k, double T) {
+static __device__ __noinline__ Species64 species64(const View& m, int ns, int k, double T, double2 li) {
   const MechLayout& L = *m.lay;
   const int rg = T < TMID ? 0 : 1;
-  const double lnT = log(T), invT = 1.0 / T;
+  const double lnT = li.x, invT = li.y;
   const double* hc = (const double*)(m.blob + L.o_hc) + (rg * ns + k) * 6;
   const double* sc = (const double*)(m.blob + L.o_sc) + (rg * ns + k) * 6;
   const double* cc = (const double*)(m.blob + L.o_cpc) + (rg * ns + k) * 5;
@@ -104,15 +105,18 @@ static __device__ __noinline__ Species64 species64(const View& m, int ns, int k,
   r.dcp = cc[1] + T * (2.0 * cc[2] + T * (3.0 * cc[3] + T * (4.0 * cc[4])));
   return r;
 }
+static __device__ __noinline__ Species64 species64(const View& m, int ns, int k, double T) {
+  return species64(m, ns, k, T, fx::ln_inv(T));
+}
 // all species of a cell into its workspace (cp/R with jac); sum c cp/R and its temperature
 // derivative, c = Y / W in the workspace
 template <int NS>
-__device__ __noinline__ void slow_species(const View& m, double* col, double T, double* cp_out, double* dcp_out,
+__device__ __noinline__ void slow_species(const View& m, double* col, double T, double2 li, double* cp_out, double* dcp_out,
                                           bool jac) {
   using w = Ws<NS>;
   double cps = 0.0, dcps = 0.0;
   for (int k = 0; k < NS; ++k) {
-    const Species64 r = species64(m, NS, k, T);
+    const Species64 r = species64(m, NS, k, T, li);
     col[(w::G + k) * 32] = r.g;
     col[(w::H + k) * 32] = r.h;
     const double c = col[(w::C + k) * 32];
@@ -183,7 +187,8 @@ __device__ __noinline__ void general_reaction(const View& m, double* col, double
     }
   }
   if (!fastk)
-    fx::slow_rate(m, Gc, 32, R.id, R.type == 2 ? m.troe + R.troe : nullptr, T, t.fast, Mc, &kf, &kr, &dlnkf, &dkfdM, &invKc);
+    fx::slow_rate(m, Gc, 32, R.id, R.type == 2 ? m.troe + R.troe : nullptr, T, fx::ln_inv_of(t), t.fast,
+                  Mc, &kf, &kr, &dlnkf, &dkfdM, &invKc);
   const double Pf = a[0] * a[1] * a[2], Pr = b[0] * b[1] * b[2];
   const double mult = R.type == 1 ? Mc : 1.0;
   const double fwd = kf * Pf, rev = kr * Pr, net = fwd - rev;
@@ -223,7 +228,7 @@ template <int NS, bool JAC, class YF>
 __device__ __forceinline__ void rhs(const View& m, double* col, double* Mx, double T, YF Yk, double p, double invp, int uoff) {
   using w = Ws<NS>;
   constexpr int N = w::N;
-  const Temp t = temp_of(T, m, JAC);
+  Temp t = temp_of(T, m, JAC);
   double S = 0.0, cps = 0.0, dcps = 0.0;
   double c[NS];
 #pragma unroll
@@ -265,7 +270,8 @@ __device__ __forceinline__ void rhs(const View& m, double* col, double* Mx, doub
       }
     }
   } else {
-    slow_species<NS>(m, col, T, &cps, &dcps, JAC);
+    slow_temp(t);
+    slow_species<NS>(m, col, T, fx::ln_inv_of(t), &cps, &dcps, JAC);
   }
   const double RTS = RU * T * S;
   const double rho = p * rcp(RTS), invrho = RTS * invp;
@@ -366,8 +372,8 @@ __device__ __forceinline__ void rhs(const View& m, double* col, double* Mx, doub
       const bool ok0 = in_range(Xf0, Xr0), ok1 = in_range(Xf1, Xr1);
       if (!(ok0 && ok1)) {
         double x = 0.0, y, z;
-        if (!ok0) fx::slow_rate(m, Gc, 32, R[0].id, nullptr, T, t.fast, 1.0, &kf0, &kr0, &x, &y, &z);
-        if (!ok1) fx::slow_rate(m, Gc, 32, R[1].id, nullptr, T, t.fast, 1.0, &kf1, &kr1, &x, &y, &z);
+        if (!ok0) fx::slow_rate(m, Gc, 32, R[0].id, nullptr, T, fx::ln_inv_of(t), t.fast, 1.0, &kf0, &kr0, &x, &y, &z);
+        if (!ok1) fx::slow_rate(m, Gc, 32, R[1].id, nullptr, T, fx::ln_inv_of(t), t.fast, 1.0, &kf1, &kr1, &x, &y, &z);
       }
       const double q0 = fma(kf0, *at(Cc, s0.r0) * *at(Cc, s0.r1), -(kr0 * (*at(Cc, s0.p0) * *at(Cc, s0.p1))));
       const double q1 = fma(kf1, *at(Cc, s1.r0) * *at(Cc, s1.r1), -(kr1 * (*at(Cc, s1.p0) * *at(Cc, s1.p1))));
@@ -399,7 +405,8 @@ __device__ __forceinline__ void rhs(const View& m, double* col, double* Mx, doub
       if (JAC && fastk) dlnkf = dl;
     }
     if (!fastk)
-      fx::slow_rate(m, Gc, 32, R->id, j >= n2 ? m.troe + R->troe : nullptr, T, t.fast, Mc, &kf, &kr, &dlnkf, &dkfdM, &invKc);
+      fx::slow_rate(m, Gc, 32, R->id, j >= n2 ? m.troe + R->troe : nullptr, T, fx::ln_inv_of(t), t.fast, Mc, &kf,
+                    &kr, &dlnkf, &dkfdM, &invKc);
     const bool third = j >= m.n_plain && j < n2;
     if (!JAC) {
       double q = fma(kf, a0 * a1, -(kr * (b0 * b1)));
