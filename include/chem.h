@@ -20,7 +20,7 @@
  *   - The library owns the device copies of mechanisms and models, and draws per-call
  *     temporaries from one memory pool per device (stream-ordered, on `stream`: the allocation
  *     strategy of §3.2), which keeps at most 512 MiB between calls and gives them back when the
- *     last mechanism is freed.
+ *     last mechanism and model are freed.
  */
 #ifndef CHEM_H
 #define CHEM_H

@@ -24,6 +24,15 @@ int cuda_fail(cudaError_t e, const char* what);
 // library's pool of the current device
 cudaError_t ws_alloc(void** p, size_t bytes, cudaStream_t stream);
 
+// What a call draws temporaries for (a mechanism, a model) holds one of these: the pools give their
+// memory back when the last one goes
+struct PoolUse {
+  PoolUse();
+  ~PoolUse();
+  PoolUse(const PoolUse&) = delete;
+  PoolUse& operator=(const PoolUse&) = delete;
+};
+
 #define CHEM_CUDA_TRY(call)                                   \
   do {                                                        \
     cudaError_t e_ = (call);                                  \
@@ -103,6 +112,7 @@ struct chem_mech_s {
   const unsigned long long *d_e2 = nullptr, *d_lg = nullptr;
   const unsigned int* d_rc = nullptr;
   const chem::FxEnthalpy* d_hk = nullptr; // [2][ns], null where a coefficient does not fit
+  chem::PoolUse pool;
 };
 
 namespace chem {

@@ -45,15 +45,15 @@ namespace {
 // Memory pools of the library's per-call temporaries, one per device.  The default pool gives its
 // memory back to the system at every synchronisation, so a caller that waits for each step paid the
 // physical allocation again on each call (0.2 ms for a small surrogate step, 4 ms for a
-// per-species pass); these pools keep up to kKeepBytes, and give it back when the last mechanism is
-// freed.  The pools are the driver's own, safe for any number of threads and streams.
+// per-species pass); these pools keep up to kKeepBytes, and give it back when the last mechanism and
+// model are freed.  The pools are the driver's own, safe for any number of threads and streams.
 constexpr uint64_t kKeepBytes = 512ull << 20;
 constexpr int kPoolDevices = 64;
 struct Pools {
   std::mutex mu;
   cudaMemPool_t pool[kPoolDevices] = {};
   bool tried[kPoolDevices] = {};
-  int mechanisms = 0;
+  int users = 0;
 };
 Pools& pools() {
   static Pools* p = new Pools();       // never destroyed: calls may come during process exit
@@ -81,15 +81,6 @@ cudaMemPool_t device_pool() {
     }
   }
   return P.pool[dev];
-}
-
-void count_mechanism(int d) {
-  Pools& P = pools();
-  std::lock_guard<std::mutex> lk(P.mu);
-  P.mechanisms += d;
-  if (P.mechanisms == 0)
-    for (cudaMemPool_t p : P.pool)
-      if (p) cudaMemPoolTrimTo(p, 0);
 }
 
 int align16(int x) { return (x + 15) & ~15; }
@@ -914,6 +905,19 @@ int validate(const chem_mech_desc* d) {
 
 }  // namespace
 
+PoolUse::PoolUse() {
+  Pools& P = pools();
+  std::lock_guard<std::mutex> lk(P.mu);
+  ++P.users;
+}
+PoolUse::~PoolUse() {
+  Pools& P = pools();
+  std::lock_guard<std::mutex> lk(P.mu);
+  if (--P.users == 0)
+    for (cudaMemPool_t p : P.pool)
+      if (p) cudaMemPoolTrimTo(p, 0);
+}
+
 cudaError_t ws_alloc(void** p, size_t bytes, cudaStream_t stream) {
   cudaMemPool_t pool = device_pool();
   if (pool) {
@@ -935,7 +939,6 @@ extern "C" int chem_load_mechanism_desc(const chem_mech_desc* desc, chem_mech_t*
   chem_mech_s* m = new (std::nothrow) chem_mech_s();
   if (!m) { set_error("out of host memory"); return CHEM_ENOMEM; }
   rc = build(desc, m);
-  count_mechanism(1);
   if (rc) { chem_free_mechanism(m); return rc; }
   *out = m;
   return CHEM_OK;
@@ -1021,7 +1024,6 @@ extern "C" int chem_free_mechanism(chem_mech_t m) {
   if (m->d_gx) cudaFree(m->d_gx);
   if (m->d_gxj) cudaFree(m->d_gxj);
   delete m;
-  count_mechanism(-1);
   return CHEM_OK;
 }
 

@@ -46,4 +46,5 @@ struct chem_model_s {
   int h[3] = {0, 0, 0};
   int nnet = 0;
   chem::PsNet net[chem::SUR_MAXNS];
+  chem::PoolUse pool;
 };
