@@ -24,9 +24,11 @@ int cuda_fail(cudaError_t e, const char* what);
 // library's pool of the current device
 cudaError_t ws_alloc(void** p, size_t bytes, cudaStream_t stream);
 
-// What a call draws temporaries for (a mechanism, a model) holds one of these: the pools give their
-// memory back when the last one goes
+// What a call draws temporaries for (a mechanism, a model) holds one of these: a pool gives its memory
+// back when the last one goes
 struct PoolUse {
+  int device = -1;
+  unsigned long long context = 0;
   PoolUse();
   ~PoolUse();
   PoolUse(const PoolUse&) = delete;

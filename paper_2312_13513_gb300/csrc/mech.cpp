@@ -18,6 +18,8 @@
 #include <string>
 #include <vector>
 
+#include <cuda.h>
+
 #include "chem_internal.h"
 #include "exp_table.h"
 #include "fixed.cuh"
@@ -42,45 +44,89 @@ int cuda_fail(cudaError_t e, const char* what) {
 
 namespace {
 
-// Memory pools of the library's per-call temporaries, one per device.  The default pool gives its
-// memory back to the system at every synchronisation, so a caller that waits for each step paid the
-// physical allocation again on each call (0.2 ms for a small surrogate step, 4 ms for a
-// per-species pass); these pools keep up to kKeepBytes, and give it back when the last mechanism and
-// model are freed.  The pools are the driver's own, safe for any number of threads and streams.
+// Memory pools of the library's per-call temporaries, one per device (and context of it).  The default
+// pool gives its memory back to the system at every synchronisation, so a caller that waits for each step
+// paid the physical allocation again on each call (0.2 ms for a small surrogate step, 4 ms for a
+// per-species pass); these pools keep up to kKeepBytes, and give it back when the context's last mechanism
+// and model are freed (in that context).  The pools are the driver's own, safe for any number of threads
+// and streams.  A context that is gone (a reset device) has taken its pool along: the slot's number is
+// never met again, and the handle never used.
 constexpr uint64_t kKeepBytes = 512ull << 20;
-constexpr int kPoolDevices = 64;
+struct PoolSlot {
+  int device = -1;                     // -1: free
+  unsigned long long context = 0;
+  cudaMemPool_t pool = nullptr;        // null: none could be made
+  int users = 0;
+};
 struct Pools {
   std::mutex mu;
-  cudaMemPool_t pool[kPoolDevices] = {};
-  bool tried[kPoolDevices] = {};
-  int users = 0;
+  PoolSlot slot[64];
 };
 Pools& pools() {
   static Pools* p = new Pools();       // never destroyed: calls may come during process exit
   return *p;
 }
 
+// Number of the current device's context, another one after each reset; 0 where there is none.  (Driver
+// entry points by the runtime's query: the library does not link the driver library.)
+unsigned long long context_number(int dev) {
+  typedef CUresult (*CurrentFn)(CUcontext*);
+  typedef CUresult (*IdFn)(CUcontext, unsigned long long*);
+  struct Fns {
+    CurrentFn current = nullptr;
+    IdFn id = nullptr;
+    Fns() {
+      void* p = nullptr;
+      cudaDriverEntryPointQueryResult q;
+      if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+          q == cudaDriverEntryPointSuccess)
+        current = (CurrentFn)p;
+      if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+          q == cudaDriverEntryPointSuccess)
+        id = (IdFn)p;
+    }
+  };
+  static const Fns f;
+  CUcontext c = nullptr;
+  unsigned long long n = 0;
+  if (!f.current || !f.id) return 0;
+  if (f.current(&c) != CUDA_SUCCESS || !c) {         // a host thread's first call binds it here
+    if (cudaSetDevice(dev) != cudaSuccess || f.current(&c) != CUDA_SUCCESS || !c) return 0;
+  }
+  return f.id(c, &n) == CUDA_SUCCESS ? n : 0;
+}
+
+// the slot of the current device and context, made with its pool where there is none (under the lock)
+PoolSlot* pool_slot(Pools& P, int dev) {
+  const unsigned long long c = context_number(dev);
+  PoolSlot* empty = nullptr;
+  for (PoolSlot& s : P.slot) {
+    if (s.device == dev && s.context == c) return &s;
+    if (s.device < 0 && !empty) empty = &s;
+  }
+  if (!empty) return nullptr;
+  *empty = PoolSlot{dev, c};
+  cudaMemPoolProps props{};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = dev;
+  uint64_t keep = kKeepBytes;
+  if (cudaMemPoolCreate(&empty->pool, &props) == cudaSuccess) {
+    cudaMemPoolSetAttribute(empty->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+  } else {
+    empty->pool = nullptr;
+    cudaGetLastError();
+  }
+  return empty;
+}
+
 cudaMemPool_t device_pool() {
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kPoolDevices) return nullptr;
+  if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
   Pools& P = pools();
   std::lock_guard<std::mutex> lk(P.mu);
-  if (!P.tried[dev]) {
-    P.tried[dev] = true;
-    cudaMemPoolProps props{};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = dev;
-    cudaMemPool_t pool = nullptr;
-    uint64_t keep = kKeepBytes;
-    if (cudaMemPoolCreate(&pool, &props) == cudaSuccess) {
-      cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
-      P.pool[dev] = pool;
-    } else {
-      cudaGetLastError();
-    }
-  }
-  return P.pool[dev];
+  const PoolSlot* s = pool_slot(P, dev);
+  return s ? s->pool : nullptr;
 }
 
 int align16(int x) { return (x + 15) & ~15; }
@@ -906,16 +952,30 @@ int validate(const chem_mech_desc* d) {
 }  // namespace
 
 PoolUse::PoolUse() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return; }
   Pools& P = pools();
   std::lock_guard<std::mutex> lk(P.mu);
-  ++P.users;
+  if (PoolSlot* s = pool_slot(P, dev)) {
+    device = dev;
+    context = s->context;
+    ++s->users;
+  }
 }
 PoolUse::~PoolUse() {
+  if (device < 0) return;
   Pools& P = pools();
   std::lock_guard<std::mutex> lk(P.mu);
-  if (--P.users == 0)
-    for (cudaMemPool_t p : P.pool)
-      if (p) cudaMemPoolTrimTo(p, 0);
+  for (PoolSlot& s : P.slot) {
+    if (s.device != device || s.context != context) continue;
+    if (--s.users > 0) return;
+    int here = 0;
+    if (cudaGetDevice(&here) != cudaSuccess) { cudaGetLastError(); return; }
+    if (here != device && cudaSetDevice(device) != cudaSuccess) { cudaGetLastError(); return; }
+    if (s.pool && context_number(device) == context) cudaMemPoolTrimTo(s.pool, 0);
+    if (here != device) cudaSetDevice(here);
+    return;
+  }
 }
 
 cudaError_t ws_alloc(void** p, size_t bytes, cudaStream_t stream) {
@@ -923,7 +983,7 @@ cudaError_t ws_alloc(void** p, size_t bytes, cudaStream_t stream) {
   if (pool) {
     const cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, stream);
     if (e == cudaSuccess || e == cudaErrorMemoryAllocation) return e;
-    cudaGetLastError();                // a pool of another context: the default pool serves
+    cudaGetLastError();                // the default pool serves
   }
   return cudaMallocAsync(p, bytes, stream);
 }
