@@ -206,7 +206,8 @@ struct FinishSeg {
   int splits, ld, fold;     // fold > 0: n_in of the first layer
   const double* colpart;
   float* db;
-  int cols, block0, wblocks;      // blocks block0 .. + wblocks: dW, then (cols + 7) / 8 blocks: db
+  int cols, block0, wblocks;      // blocks block0 .. + wblocks: dW (none: it is there), then (cols + 7) / 8
+                                  // blocks: db
 };
 struct FinishSet {
   FinishSeg s[MAXL];
@@ -484,11 +485,13 @@ struct chem_trainer_s {
   float* Z[MAXL];                  // pre-activations [B x out_pad]
   __nv_bfloat16* A[MAXL];          // A[0] = caller's input, A[l] = bf16(GELU(Z[l-1]))
   float* dA;
-  float* dWparts[MAXL];            // split-K partials of each layer's weight gradient (splits x W)
+  float* dWparts[MAXL];            // split-K partials of each layer's weight gradient (splits x W); null:
+                                   // the product goes straight to dW
   int splitsW[MAXL];               // K splits of each layer's weight-gradient product
   double* colpart[MAXL];           // row-block partial column sums [B / 64 x out_pad]
   double* loss_part;               // the loss gradient kernel's block sums
-  __nv_bfloat16 *dZb, *dZt, *At[MAXL];
+  __nv_bfloat16 *dZb, *dZt, *At[MAXL];   // At: one buffer for all layers where at_shared
+  bool at_shared;
   int* err;
   double* loss;
   int64_t* d_step;                 // Adam steps taken (device: a captured step advances it)
@@ -587,7 +590,8 @@ extern "C" int chem_mlp_trainer_create_layers(int n_in, int n_out, int n_hidden,
   if (!rc) rc = tr_alloc(t, &p, (size_t)batch * maxw * 4), t->dA = (float*)p;
   // weight gradients dW = dZ^T A have few output tiles and K = batch: split K over the SMs (a
   // power of two dividing the 64-wide K steps, splits x tiles at most the SM count) and add the
-  // partials in a fixed order (k_finish_grads)
+  // partials in a fixed order (k_finish_grads).  A product that is not split needs no partials, except
+  // the first layer's, which is folded
   if (!rc) {
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
@@ -598,14 +602,27 @@ extern "C" int chem_mlp_trainer_create_layers(int n_in, int n_out, int n_hidden,
       int sp = 1;
       while (nk % (2 * sp) == 0 && tiles * 2 * sp <= sms) sp *= 2;
       t->splitsW[l] = sp;
+      t->dWparts[l] = nullptr;
+      if (sp == 1 && l > 0) continue;
       rc = tr_alloc(t, &p, (size_t)sp * t->out_pad[l] * t->in_pad[l] * 4);
       t->dWparts[l] = (float*)p;
     }
   }
   const size_t nrb = (batch + kColRows - 1) / kColRows;
+  // A^T of every layer in one launch as long as all of them together are small (batch 4096 of the
+  // 512-wide network: 18 MB, where a launch is what a transpose costs); beyond that each is some
+  // microseconds of work by itself, and one buffer of the largest serves them in turn
+  size_t at_all = 0;
+  int maxin = 0;
+  for (int l = 0; l < NL; ++l) { at_all += (size_t)batch * ins[l] * 2; maxin = std::max(maxin, ins[l]); }
+  t->at_shared = at_all > ((size_t)128 << 20);
   for (int l = 0; l < NL && !rc; ++l) {
-    rc = tr_alloc(t, &p, (size_t)batch * ins[l] * 2);
-    t->At[l] = (__nv_bfloat16*)p;
+    if (t->at_shared && l > 0) {
+      t->At[l] = t->At[0];
+    } else {
+      rc = tr_alloc(t, &p, (size_t)batch * (t->at_shared ? maxin : ins[l]) * 2);
+      t->At[l] = (__nv_bfloat16*)p;
+    }
     if (rc) break;
     rc = tr_alloc(t, &p, nrb * outs[l] * 8);
     t->colpart[l] = (double*)p;
@@ -653,9 +670,11 @@ extern "C" int chem_mlp_backward(chem_trainer_t t, const float* target, double* 
   const int B = t->B, NL = t->nl;
   // A^T of every layer (batch contiguous, for the weight gradients)
   TransposeSet T{};
-  for (int l = 0; l < NL; ++l) T.j[T.n++] = TransposeJob{t->A[l], t->At[l], B, t->in_pad[l]};
-  const int trc = launch_transposes(T, st);
-  if (trc) return trc;
+  if (!t->at_shared) {
+    for (int l = 0; l < NL; ++l) T.j[T.n++] = TransposeJob{t->A[l], t->At[l], B, t->in_pad[l]};
+    const int trc = launch_transposes(T, st);
+    if (trc) return trc;
+  }
   const int nrb = (B + kColRows - 1) / kColRows;
   const dim3 mse_grid((PADIO + 63) / 64, nrb);
   CHEM_CUDA_TRY(launch_pdl(k_mse_grad, mse_grid, dim3(32, 8), 0, st, t->Z[NL - 1], target, t->dZb, t->dZt,
@@ -663,11 +682,18 @@ extern "C" int chem_mlp_backward(chem_trainer_t t, const float* target, double* 
   for (int l = NL - 1; l >= 0; --l) {
     const int nout = t->out_pad[l], nin = t->in_pad[l];
     int rc;
+    if (t->at_shared) {
+      T.j[0] = TransposeJob{t->A[l], t->At[l], B, nin};
+      T.n = 1;
+      rc = launch_transposes(T, st);
+      if (rc) return rc;
+    }
     if (t->splitsW[l] > 1)
       rc = gemm_bf16_splitk(t->dZt, B, t->At[l], B, t->dWparts[l], nin, (int64_t)nout * nin, t->splitsW[l], nout,
                             nin, B, t->err, st);
     else
-      rc = gemm_bf16(t->dZt, B, t->At[l], B, t->dWparts[l], nin, nullptr, nout, nin, B, t->err, st);
+      rc = gemm_bf16(t->dZt, B, t->At[l], B, t->dWparts[l] ? t->dWparts[l] : t->dW[l], nin, nullptr, nout, nin, B,
+                     t->err, st);
     if (rc) return rc;
     if (l > 0) {
       rc = gemm_bf16(t->dZb, nout, t->Wt[l], nout, t->dA, nin, nullptr, B, nin, nout, t->err, st);
@@ -680,7 +706,7 @@ extern "C" int chem_mlp_backward(chem_trainer_t t, const float* target, double* 
   int blocks = 0;
   for (int l = 0; l < NL; ++l) {
     const int64_t n = (int64_t)t->out_pad[l] * t->in_pad[l];
-    const int wb = (int)std::min<int64_t>((n + 255) / 256, 1024);
+    const int wb = t->dWparts[l] ? (int)std::min<int64_t>((n + 255) / 256, 1024) : 0;
     F.s[F.n++] = FinishSeg{t->dWparts[l], t->dW[l], n, t->splitsW[l], t->in_pad[l], l == 0 ? t->nin : 0,
                            t->colpart[l], t->db[l], t->out_pad[l], blocks, wb};
     blocks += wb + (t->out_pad[l] + 7) / 8;

@@ -188,3 +188,44 @@ def test_gemm_tile_widths_and_store_widths(M, N, K, ldc):
     # one BF16 rounding (2^-9 relative) and the GELU form's 5e-7
     assert torch.all((Cb[:, :N].double() - act).abs() <= 2.0 ** -8 * act.abs() + 1e-5)
     assert torch.all(C[:, N:] == 7.0) and torch.all(Cb[:, N:] == 7.0)         # nothing beyond column N
+
+
+@pytest.mark.parametrize("hidden,B", [((2048, 2048), 256), ((4096, 4096), 8192)])
+def test_trainer_with_wide_layers(hidden, B):
+    """Layers whose weight-gradient products have a tile for every SM (not split: straight to the
+    gradient), and activations beyond 128 MB (transposed one layer at a time into one buffer): gradients
+    of a batch that repeats 128 rows against those of the 128 rows, and the memory that they take."""
+    from paper_2312_13513_gb300.train import PAD, Trainer
+    rng = np.random.default_rng(43)
+    nin, nout, rep = 11, 9, B // 128
+    dims = [nin, *hidden, nout]
+    W = [rng.standard_normal((dims[i + 1], dims[i])).astype(np.float32) / np.sqrt(dims[i]) for i in range(3)]
+    b = [0.1 * rng.standard_normal(dims[i + 1]).astype(np.float32) for i in range(3)]
+    X = torch.zeros((128, PAD), dtype=torch.bfloat16, device="cuda")
+    X[:, :nin] = torch.tensor(rng.standard_normal((128, nin)), dtype=torch.float32, device="cuda").bfloat16()
+    T = torch.tensor(rng.standard_normal((128, nout)), dtype=torch.float32, device="cuda")
+    got = []
+    for n in (1, rep):
+        Xn, Tn = X.repeat(n, 1).contiguous(), T.repeat(n, 1).contiguous()
+        out = torch.empty((128 * n, nout), dtype=torch.float32, device="cuda")
+        loss = torch.zeros(1, dtype=torch.float64, device="cuda")
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        tr = Trainer(nin, nout, 128 * n, W=W, b=b, hidden=list(hidden))
+        used = free - torch.cuda.mem_get_info()[0]
+        for _ in range(2):
+            tr.forward(Xn, out)
+            tr.backward(Tn, loss)
+        got.append((*tr.get(1), loss.item(), used))
+        del tr
+    (gW, gb, gl, _), (dW, db, l1, used) = got
+    assert abs(l1 - gl) <= 1e-6 * gl
+    # the same products, scaled by a power of two: FP32 sums of up to 8192 terms in another order
+    for l in range(3):
+        assert np.linalg.norm(dW[l] - gW[l]) <= 1e-3 * np.linalg.norm(gW[l]), l
+        assert np.linalg.norm(db[l] - gb[l]) <= 1e-3 * np.linalg.norm(gb[l]), l
+    # parameters, two moments and the gradient in FP32, two BF16 copies; Z and A of each layer; three working
+    # arrays and one A^T of the widest; 96 MB for partials and the allocator's rounding
+    ins, outs = [PAD, *hidden], [*hidden, PAD]
+    need = sum(20 * i * o for i, o in zip(ins, outs)) + B * (sum(4 * o for o in outs) + sum(2 * i for i in hidden) + 10 * max(outs))
+    assert used <= need + (96 << 20), (used / 2 ** 20, need / 2 ** 20)
