@@ -229,3 +229,37 @@ def test_trainer_with_wide_layers(hidden, B):
     ins, outs = [PAD, *hidden], [*hidden, PAD]
     need = sum(20 * i * o for i, o in zip(ins, outs)) + B * (sum(4 * o for o in outs) + sum(2 * i for i in hidden) + 10 * max(outs))
     assert used <= need + (96 << 20), (used / 2 ** 20, need / 2 ** 20)
+
+
+@pytest.mark.parametrize("M,N,K,ldc,width", [(20000, 160, 64, 160, 160), (20000, 130, 128, 131, 160), (20000, 320, 128, 328, 160),
+                                             (20000, 301, 70, 301, 160), (20000, 208, 64, 208, 208)])
+def test_gemm_160_column_tiles(M, N, K, ldc, width):
+    """The 160-column tiles (five stages, ten 16-column units over four epilogue warps), and a single
+    208-column one: enough rows for a tile on every SM, whole and ragged columns, each width of store."""
+    import ctypes
+    from paper_2312_13513_gb300 import _lib
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    cost = {w: -(-N // w) * (128 + w) for w in (256, 208, 160, 128)}           # the dispatch's rule
+    assert min(cost, key=cost.get) == width and -(-M // 128) * -(-N // width) >= sms
+    g = torch.Generator(device="cuda").manual_seed(M + N)
+    lda = (K + 7) // 8 * 8
+    A = torch.randn(M, lda, device="cuda", generator=g).bfloat16()
+    B = (torch.randn(N, lda, device="cuda", generator=g) / K ** 0.5).bfloat16()
+    bias = torch.randn(N, device="cuda", generator=g)
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    st = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    p = lambda t: ctypes.c_void_p(t.data_ptr())
+    C = torch.full((M, ldc), 7.0, device="cuda")
+    Cb = torch.full((M, ldc), 7.0, device="cuda", dtype=torch.bfloat16)
+    L = _lib.load()
+    assert L.chem_gemm_bf16(p(A), lda, p(B), lda, p(C), ldc, p(bias), M, N, K, p(err), st) == 0
+    assert L.chem_gemm_bf16_act(p(A), lda, p(B), lda, p(Cb), ldc, p(bias), 1, M, N, K, p(err), st) == 0
+    torch.cuda.synchronize()
+    assert int(err.item()) == 0
+    ref = A[:, :K].double() @ B[:, :K].double().T + bias.double()
+    # FP32 accumulation of K products of size O(1 / sqrt K): K additions at 2^-24 of at most ~6
+    assert torch.allclose(C[:, :N].double(), ref, rtol=0, atol=6 * K * 2.0 ** -24)
+    act = torch.nn.functional.gelu(ref)
+    # one BF16 rounding (2^-9 relative) and the GELU form's 5e-7
+    assert torch.all((Cb[:, :N].double() - act).abs() <= 2.0 ** -8 * act.abs() + 1e-5)
+    assert torch.all(C[:, N:] == 7.0) and torch.all(Cb[:, N:] == 7.0)         # nothing beyond column N
