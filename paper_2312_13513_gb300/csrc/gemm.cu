@@ -340,34 +340,28 @@ static int gemm_launch(const void* A, int64_t lda, const void* B, int64_t ldb, f
   // tiles: 10 TB/s, 203 us = 826 TFLOP/s; on 208-wide ones 136 us = 1234 TFLOP/s), and a row block's
   // traffic is its tile count times the rows of A and B that a tile reads: the width of 256, 208, 160
   // or 128 that needs the least (800 and 400 columns: 208, four and two tiles).  128 where wider tiles
-  // would leave SMs without one (small products: more, smaller tiles finish sooner).
+  // would leave SMs without one (small products: more, smaller tiles finish sooner), and for split
+  // products, which the caller splits until the 128-wide tiles fill the SMs.
   int bn = 256;
   long long cost = -1;
   for (int w : {256, 208, 160, 128}) {
     const long long c = (long long)((N + w - 1) / w) * (BM + w);
     if (cost < 0 || c < cost) { cost = c; bn = w; }
   }
-  if (bn > 128 && (long long)((M + BM - 1) / BM) * ((N + bn - 1) / bn) * splits < sms) bn = 128;
+  if (splits > 1 || (long long)((M + BM - 1) / BM) * ((N + bn - 1) / bn) < sms) bn = 128;
   const long long ntiles = (long long)((M + BM - 1) / BM) * ((N + bn - 1) / bn) * splits;
   const unsigned grid = (unsigned)std::min<long long>(ntiles, sms);
   rc = make_tmap_bf16(&tb, B, N, K, ldb, bn, BK);
   if (rc) return rc;
-  switch (bn) {
-    case 256:
-      rc = splits > 1 ? launch_persistent<256, true>(ta, tb, g, grid, stream)
-                      : launch_persistent<256, false>(ta, tb, g, grid, stream);
-      break;
-    case 208:
-      rc = splits > 1 ? launch_persistent<208, true>(ta, tb, g, grid, stream)
-                      : launch_persistent<208, false>(ta, tb, g, grid, stream);
-      break;
-    case 160:
-      rc = splits > 1 ? launch_persistent<160, true>(ta, tb, g, grid, stream)
-                      : launch_persistent<160, false>(ta, tb, g, grid, stream);
-      break;
-    default:
-      rc = splits > 1 ? launch_persistent<128, true>(ta, tb, g, grid, stream)
-                      : launch_persistent<128, false>(ta, tb, g, grid, stream);
+  if (splits > 1) {
+    rc = launch_persistent<128, true>(ta, tb, g, grid, stream);
+  } else {
+    switch (bn) {
+      case 256: rc = launch_persistent<256, false>(ta, tb, g, grid, stream); break;
+      case 208: rc = launch_persistent<208, false>(ta, tb, g, grid, stream); break;
+      case 160: rc = launch_persistent<160, false>(ta, tb, g, grid, stream); break;
+      default: rc = launch_persistent<128, false>(ta, tb, g, grid, stream);
+    }
   }
   if (rc) return rc;
   CHEM_CUDA_TRY(cudaGetLastError());
