@@ -63,6 +63,11 @@ struct FxEnthalpy {
   float cf[5], pad[3];
 };
 
+// Species counts with instances of the kernels of one thread and of several lanes per cell, and a blob of
+// this form.  Beyond 11 fewer than three warps of cells fit in an SM's shared memory (integrator_cell.cu).
+// Below 8 none is compiled: those mechanisms keep the two-lane groups, and the two were not compared there.
+constexpr int kCellMinNs = 8, kCellMaxNs = 11;
+
 struct FxLayout {
   int ns, ntb, bytes;         // bytes = 0: no fixed-point form
   int o_exp2, o_lg, o_rcp;    // tables of fixed.cuh

@@ -410,9 +410,10 @@ int eval_t(const chem_mech_s* m, const double* T, const double* p, const double*
 
 }  // namespace
 
-// Whether the mechanism's cells run one per thread: it has a fixed-point form, its species count
-// has an instance, and at least three warps of cells fit on an SM (see shape_of).
+// Whether the mechanism's cells run one per thread: it has a fixed-point form (its species count is one
+// of the instances'), and at least three warps of cells fit on an SM (see shape_of).
 bool cell_kernel_fits(const chem_mech_s* m) {
+  static_assert(kCellMinNs == 8 && kCellMaxNs == 11, "the instances below, advance_t's and eval_t's");
   if (!m->fx.bytes) return false;
   Shape s{0, 0, 0, 0};
   int rc = CHEM_EINVAL;

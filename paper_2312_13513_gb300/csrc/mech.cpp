@@ -358,7 +358,7 @@ std::vector<unsigned char> build_fx(const chem_mech_desc* d, const chem_mech_s* 
                                     const std::vector<std::vector<int>>& nu, FxLayout* L) {
   const int ns = d->n_species, nr = d->n_reactions;
   *L = FxLayout{};
-  if (!F.ok || ns > 15 || nr > 1024) return {};
+  if (!F.ok || ns < kCellMinNs || ns > kCellMaxNs || nr > 1024) return {};
   const Partners T(d);
   Builder B;
   L->ns = ns; L->ntb = T.ntb; L->lpr0 = F.lpr0;
@@ -368,7 +368,7 @@ std::vector<unsigned char> build_fx(const chem_mech_desc* d, const chem_mech_s* 
     int nre = 0, npr = 0, nn = 0;
     for (int i = 0; i < 3; ++i) { nre += d->reac[3 * j + i] >= 0; npr += d->prod[3 * j + i] >= 0; }
     for (int k = 0; k < ns; ++k) nn += nu[j][k] != 0;
-    order[nre <= 2 && npr <= 2 && nn <= 4 && ns >= 4 ? d->rtype[j] : 3].push_back(j);
+    order[nre <= 2 && npr <= 2 && nn <= 4 ? d->rtype[j] : 3].push_back(j);
   }
   L->n_plain = (int)order[0].size(); L->n_tb = (int)order[1].size(); L->n_fo = (int)order[2].size();
   L->n_gen = (int)order[3].size();

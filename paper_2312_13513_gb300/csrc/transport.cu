@@ -529,7 +529,10 @@ extern "C" int chem_transport_eval(chem_transport_t t, const double* T, const do
     // Whole warps per sub-partition, 4 to 16 an SM as far as shared memory goes, more of them overlap one
     // warp's integer work with the others' FP64 (100003 H2 cells: a pass of the grid takes 43, 49 and
     // 80 us with up to 4, 8 and 16), but the last pass may be nearly empty: the number with the least
-    // passes times their length, max(11, warps + 4) units of 4 us.
+    // passes times their length, max(11, warps + 4) units of 4 us.  The units are those of 9 species; with
+    // 12 and 15 the rule gives 2.5 to 3 times the rate of four lanes a cell in FP64 from 30011 cells on, and
+    // 0.90 to 0.99 of it for about 1000 cells (12 species, mu alone: 43.6 us against 39.5), which use one
+    // sub-partition of 32 SMs.
     const size_t fixed = (256 + 8 * (size_t)ns + 4 * npair + 3 * (size_t)ns * ns + ns + (ns & 1)) * 8;
     const size_t per = (size_t)5 * ns * 256;
     const int64_t need = (ncells + 31) / 32;
