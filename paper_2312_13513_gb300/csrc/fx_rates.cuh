@@ -108,11 +108,15 @@ __device__ __forceinline__ double g_of(double raw, bool fast) {
   return fast ? to_double(__double_as_longlong(raw), 52) * kLn2 : raw;
 }
 
+// the exponential of the FP64 forms, out of line: six copies in them cost the cells that take none of
+// these forms 0.5 % (code size, presumably), and those that do 6 %
+static __device__ __noinline__ double exp_slow(double x, const u64* e2) { return exp_any(x, e2); }
+
 // Rate constants in FP64 for what the fixed-point path leaves out: cells whose temperature is
 // outside its range, reactions whose exponents are.  Reaction id of the FP64 form; G: the cell's
 // Gibbs energies, element k at k * stride.  kf (the high-pressure limit of a fall-off reaction),
 // 1 / Kc, and k0 of a fall-off reaction; li = ln T and 1 / T.  The exponentials run on the integer pipe
-// here too: 100003 H2 cells of 4100 to 5500 K take 718 ms (two lanes a cell: 745); with the library's,
+// here too: 100003 H2 cells of 4100 to 5500 K take 676 ms (two lanes a cell: 745); with the library's,
 // and ln T and 1 / T formed for each reaction, 1016.
 static __device__ __noinline__ void slow_k(const Ctx& m, const double* G, int stride, int id, double2 li, bool fast,
                                            double* kf, double* invKc, double* k0) {
@@ -123,10 +127,10 @@ static __device__ __noinline__ void slow_k(const Ctx& m, const double* G, int st
   const double* Ta = (const double*)(m.blob + L.o_Ta);
   const short4 re = ((const short4*)(m.blob + L.o_reac))[id], pr = ((const short4*)(m.blob + L.o_prod))[id];
   const short4 ri = ((const short4*)(m.blob + L.o_rinfo))[id];
-  *kf = exp_any(lnA[id] + beta[id] * lnT - Ta[id] * invT, m.e2);
+  *kf = exp_slow(lnA[id] + beta[id] * lnT - Ta[id] * invT, m.e2);
   if (ri.x == 2) {
     const double* tr = (const double*)(m.blob + L.o_troe) + 8 * ri.w;
-    *k0 = exp_any(tr[0] + tr[1] * lnT - tr[2] * invT, m.e2);
+    *k0 = exp_slow(tr[0] + tr[1] * lnT - tr[2] * invT, m.e2);
   }
   double x = 0.0;                                   // Delta G / RT, empty slots skipped
   if (pr.x >= 0) x = g_of(G[pr.x * stride], fast);
@@ -139,7 +143,7 @@ static __device__ __noinline__ void slow_k(const Ctx& m, const double* G, int st
     const double* cst = (const double*)(m.blob + L.o_const);
     x = fma(cst[kC_NU + 8 + ri.y], lnT - cst[kC_LNPR0], x);
   }
-  *invKc = exp_any(x, m.e2);
+  *invKc = exp_slow(x, m.e2);
 }
 
 // Troe blending in FP64 from kinf, k0 and the collision-partner sum (the general form: any value
@@ -148,11 +152,11 @@ static __device__ __noinline__ void slow_troe(const Ctx& m, const FxTroe& t, dou
                                               double Mc, double dlnkinf, double* kf, double* dlnkf, double* dkfdM) {
   *kf = 0.0; *dlnkf = 0.0; *dkfdM = 0.0;
   if (kinf == 0.0 || k0 == 0.0) return;
-  const double e3 = exp_any(-T * t.iT3, m.e2), e1 = exp_any(-T * t.iT1, m.e2);
+  const double e3 = exp_slow(-T * t.iT3, m.e2), e1 = exp_slow(-T * t.iT1, m.e2);
   double Fc = (1.0 - t.a) * e3 + t.a * e1;
   double dFc = -(1.0 - t.a) * t.iT3 * e3 - t.a * t.iT1 * e1;
   if (t.has_t2 != 0.0) {
-    const double e2 = exp_any(-t.T2 * invT, m.e2);
+    const double e2 = exp_slow(-t.T2 * invT, m.e2);
     Fc += e2;
     dFc += t.T2 * invT * invT * e2;
   }
@@ -167,7 +171,7 @@ static __device__ __noinline__ void slow_troe(const Ctx& m, const FxTroe& t, dou
   const double d = n - 0.14 * u;
   const double f1 = u / d;
   const double den = 1.0 + f1 * f1;
-  const double F = exp_any(2.302585092994046 * (L / den), m.e2);
+  const double F = exp_slow(2.302585092994046 * (L / den), m.e2);
   const double opr = 1.0 / (1.0 + Prr);
   *kf = kinf * (Prr * opr) * F;
   const double dGdlogPr = -2.0 * L * f1 / (den * den) * (n / (d * d));
